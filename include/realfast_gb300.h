@@ -254,8 +254,8 @@ rf_status rf_plan_set_form(struct rf_plan* plan, int32_t form);
 /*
  * Tuning knobs (used by the autotuner; results do not depend on them).
  * RF_TUNE_WAVE_IMAGES  images imaged per wave.  A wave's column-FFT
- *                      intermediate is images x (iu_max + 1) x npix x 8 bytes;
- *                      waves small enough to stay in L2 avoid an HBM round
+ *                      intermediate is (iu_max + 1) x npix x 8 bytes for each
+ *                      image that is not a sum of others; waves small enough to stay in L2 avoid an HBM round
  *                      trip.  Range [images_per_group, 32768].  Reallocates
  *                      the plan's scratch.
  * Errors: RF_ERR_INVALID_ARG (unknown key or value out of range),
@@ -280,8 +280,10 @@ rf_status rf_plan_set_form(struct rf_plan* plan, int32_t form);
  *                      2048^2, 2 at 4096^2) that stays in L2; 0 (default):
  *                      separate column and row launches through a wave-sized
  *                      buffer (always so for other sizes, with
- *                      RF_NOISE_CLIPPED and for rendered images).  The
- *                      autotuner times both. */
+ *                      RF_NOISE_CLIPPED, for rendered images and for plans
+ *                      with a width twice or four times another, whose
+ *                      images the row pass sums).  The autotuner times both
+ *                      where both exist. */
 #define RF_TUNE_FUSED 4
 /* RF_TUNE_RING         chunk slots of the fused pass's ring, 2 .. 8
  *                      (default 3). */
@@ -304,9 +306,9 @@ rf_status rf_plan_get_tuning(const struct rf_plan* plan, int32_t key, int64_t* v
 
 /*
  * rf_plan_autotune: pick the tuning that searches `vis` fastest and apply
- * it.  Candidates: where the fused pass exists (npix 1024 .. 4096, no
- * clipped noise), RF_TUNE_FUSED on with RF_TUNE_RING 2, 3 and 4, and off with
- * RF_TUNE_OVERLAP off and on, at waves of 2048 and 8192 images, graphs on;
+ * it.  Candidates: for npix 1024 .. 4096 without clipped noise,
+ * RF_TUNE_FUSED on with RF_TUNE_RING 2, 3 and 4 (where the plan has a fused
+ * pass, see RF_TUNE_FUSED), and off with RF_TUNE_OVERLAP off and on, at waves of 2048 and 8192 images, graphs on;
  * elsewhere a ladder of wave sizes (256 .. 8192 images) with RF_TUNE_GRAPHS
  * on and off, and from 2048 images RF_TUNE_OVERLAP on.  Before either, waves
  * of one, two and four image groups (below 256 images) whose column-FFT

@@ -65,7 +65,9 @@ inline bool finite(double x) { return std::isfinite(x); }
 
 struct Wave {
   int g_begin, g_end;
-  int img_begin, img_end;
+  int img_begin, img_end;    // image list
+  int base_begin, base_end;  // transformed images
+  int quad_begin, quad_end;
 };
 
 // Restores the caller's current device on scope exit.
@@ -216,6 +218,13 @@ struct rf_plan {
   std::vector<int32_t> ongrid_chan;
   int n_on = 0, iu_max = 0, iv_max = 0, ncol = 1, n_offgrid = 0;
   rf::ImageKernelShape shape{};
+  // Widths whose images are sums of two or four images of another width of
+  // the plan (see build_widths): sum_of[s] is that width's index (s itself for
+  // a width with transforms of its own), sum_level[s] 0, 1 (two) or 2 (four),
+  // and sum2[s] / sum4[s] the widths made from width s (-1: none).
+  std::vector<int> sum_of, sum_level, sum2, sum4;
+  bool derived = false;      // some width is such a sum
+  double base_share = 1.0;   // share of a long trial set's images that are transformed
 
   // device state
   bool host_only = false;
@@ -227,7 +236,9 @@ struct rf_plan {
   std::vector<void*> d_sdt;     // per dt index (dt = 1: d_S)
   std::vector<int32_t> sdt_lp;  // per dt index
   float2* d_T = nullptr;
-  int slots_max = 0;
+  int slots_max = 0;            // RF_TUNE_WAVE_IMAGES: images per wave
+  int tslots = 0;               // transformed images per wave (d_T)
+  int sslots = 0;               // image records per wave (partials, Parseval sums)
   StatPartial* d_partials = nullptr;
   double* d_weight = nullptr;
   int4* d_img_info = nullptr;
@@ -251,7 +262,10 @@ struct rf_plan {
   int t_span = 0;
   std::vector<int4> img_info;
   std::vector<Group> groups;
+  std::vector<rf::Quad> quads;  // of the transformed images, where widths are sums of others
+  rf::Quad* d_quads = nullptr;
   std::vector<Wave> waves;
+  bool cached_plain = false;    // the lists are the plain form's (every image on its own)
   int gslots_max = 0;           // groups per wave (cell buffer capacity)
   float2* d_cellbuf = nullptr;
   float* d_colsq = nullptr;     // [slots][ncol] Parseval sums
@@ -369,6 +383,49 @@ int64_t count_images(const rf_plan* p, int nint) {
   for (int d = 0; d < p->ndm; ++d)
     for (int s = 0; s < p->ndt; ++s) n += n_times(p, nint, d, s);
   return n;
+}
+
+// Chains of widths {b, 2 b, 4 b}: from the smallest width up, each one not yet
+// taken becomes a base, and the images of the widths twice and four times it
+// (the first entry of the list of each) are sums of its images.  Whenever an
+// image of such a width is searched, so are the images that it is the sum of:
+// floor(x / 2 b) = floor(floor(x / b) / 2) for both edge rules and for a
+// stream's span.  Sums of eight would need 64 more registers a lane to be
+// kept than tensor memory has (see k_rowfft_tree).
+void build_widths(rf_plan* p) {
+  const int n = p->ndt;
+  p->sum_of.resize(n);
+  p->sum_level.assign(n, 0);
+  p->sum2.assign(n, -1);
+  p->sum4.assign(n, -1);
+  for (int k = 0; k < n; ++k) p->sum_of[k] = k;
+  p->derived = false;
+  if (p->npix >= rf::kTreeMinNpix) {
+    std::vector<int> order(n);
+    for (int k = 0; k < n; ++k) order[k] = k;
+    std::stable_sort(order.begin(), order.end(), [p](int a, int b) { return p->dt[a] < p->dt[b]; });
+    std::vector<char> taken(n, 0);
+    for (int b : order) {
+      if (taken[b]) continue;
+      taken[b] = 1;
+      for (int lv = 1; lv <= 2; ++lv)
+        for (int k : order)
+          if (!taken[k] && p->dt[k] == p->dt[b] << lv) {
+            taken[k] = 1;
+            p->sum_of[k] = b;
+            p->sum_level[k] = lv;
+            (lv == 1 ? p->sum2 : p->sum4)[b] = k;
+            p->derived = true;
+            break;
+          }
+    }
+  }
+  double all = 0.0, base = 0.0;
+  for (int k = 0; k < n; ++k) {
+    all += 1.0 / p->dt[k];
+    if (p->sum_of[k] == k) base += 1.0 / p->dt[k];
+  }
+  p->base_share = base / all;
 }
 
 rf_status validate(const rf_plan_desc* d) {
@@ -612,22 +669,55 @@ rf_status build_tables(rf_plan* p) {
   return RF_OK;
 }
 
+// A group with its sums of two and four: at most this many images.
+int group_images(const rf_plan* p) { return p->shape.images_per_group * (p->derived ? 7 : 4) / 4; }
+
+// Transformed images and image records of a wave of `slots` images (two whole
+// groups at least, so that a half of either holds one, see run_waves_overlapped).
+int wave_tslots(const rf_plan* p, int slots) {
+  if (!p->derived) return slots;
+  return std::max(2 * p->shape.images_per_group, std::min(slots, (int)std::ceil(slots * p->base_share)));
+}
+int wave_sslots(const rf_plan* p, int slots) { return p->derived ? std::max(slots, 2 * group_images(p)) : slots; }
+
+// Default images per wave: the column-FFT scratch of its transformed images
+// within the budget.
+int default_slots(const rf_plan* p, size_t img_cap) {
+  const double per_slot = (double)p->ncol * p->npix * sizeof(float2) * p->base_share;
+  return (int)std::min<double>(std::floor((double)kTBudgetBytes / per_slot), (double)img_cap);
+}
+
 // Whether waves can be overlapped: asked for, two halves of the scratch hold
 // a group each, and neither the fused pass nor the clipped noise (whose
 // window buffer is per slot of the whole scratch) is in use.
 bool overlap_possible(const rf_plan* p) {
-  return p->overlap && !p->fused && !(p->flags & RF_NOISE_CLIPPED) &&
-         p->slots_max / 2 >= p->shape.images_per_group;
+  return p->overlap && !(p->fused && !p->derived) && !(p->flags & RF_NOISE_CLIPPED) &&
+         p->tslots / 2 >= p->shape.images_per_group && p->sslots / 2 >= group_images(p);
 }
 
-// Image and group lists for a segment of nint integrations, in (d, s, t') order.
+// Image, group and quad lists for a segment of nint integrations: trial by
+// trial (d, width with transforms of its own), in groups of up to 32 t', each
+// group's images followed by its sums of two and of four.  img_info[].w is an
+// image's place in (d, s, t') order.  The plain form takes every width on its
+// own in (d, s, t') order.
 void build_lists(rf_plan* p, int nint) {
   const int B = p->shape.images_per_group;
+  const bool plain = p->form == RF_FORM_PLAIN;
   p->img_info.clear();
   p->groups.clear();
+  p->quads.clear();
   p->waves.clear();
-  for (int d = 0; d < p->ndm; ++d)
+  std::vector<int> first(p->ndt);  // (d, s, t') place of each width's first image
+  int place = 0, nbase = 0;
+  for (int d = 0; d < p->ndm; ++d) {
     for (int s = 0; s < p->ndt; ++s) {
+      first[s] = place;
+      place += n_times(p, nint, d, s);
+    }
+    for (int s = 0; s < p->ndt; ++s) {
+      const bool tree = p->derived && !plain;
+      if (tree && p->sum_of[s] != s) continue;
+      const int s2 = tree ? p->sum2[s] : -1, s4 = tree ? p->sum4[s] : -1;
       const int nt = n_times(p, nint, d, s);
       for (int t0 = 0; t0 < nt; t0 += B) {
         Group g{};
@@ -635,31 +725,63 @@ void build_lists(rf_plan* p, int nint) {
         g.s = s;
         g.t0 = t0;
         g.nimg = std::min(B, nt - t0);
-        g.img0 = (int)p->img_info.size();
+        g.base0 = nbase;
+        nbase += g.nimg;
+        auto list = [&](int w, int t, int n) {
+          const int i = (int)p->img_info.size();
+          for (int k = 0; k < n; ++k) p->img_info.push_back(make_int4(d, w, t + k, first[w] + t + k));
+          return i;
+        };
+        g.img0 = list(s, t0, g.nimg);
+        if (s2 >= 0) {
+          g.n1 = g.nimg / 2;
+          g.img1 = list(s2, t0 / 2, g.n1);
+        }
+        if (s4 >= 0) {
+          g.n2 = g.nimg / 4;
+          g.img2 = list(s4, t0 / 4, g.n2);
+        }
         p->groups.push_back(g);
-        for (int k = 0; k < g.nimg; ++k) p->img_info.push_back(make_int4(d, s, t0 + k, 0));
       }
     }
+  }
   // overlapped waves take half the slots each (see run_waves)
   p->waves_overlap = overlap_possible(p);
-  const int cap = p->waves_overlap ? p->slots_max / 2 : p->slots_max;
-  Wave w{0, 0, 0, 0};
+  const int tcap = p->waves_overlap ? p->tslots / 2 : p->tslots;
+  const int scap = p->waves_overlap ? p->sslots / 2 : p->sslots;
+  Wave w{};
   for (int gi = 0; gi < (int)p->groups.size(); ++gi) {
     const Group& g = p->groups[gi];
-    if (g.img0 + g.nimg - w.img_begin > cap || gi - w.g_begin >= p->gslots_max) {
+    const int q0 = (int)p->quads.size();
+    const int img_end = g.img0 + g.nimg + g.n1 + g.n2;
+    if (g.base0 + g.nimg - w.base_begin > tcap || img_end - w.img_begin > scap || gi - w.g_begin >= p->gslots_max) {
       w.g_end = gi;
       w.img_end = g.img0;
+      w.base_end = g.base0;
+      w.quad_end = q0;
       p->waves.push_back(w);
-      w = Wave{gi, gi, g.img0, g.img0};
+      w = Wave{gi, gi, g.img0, g.img0, g.base0, g.base0, q0, q0};
     }
+    if (p->derived && !plain)
+      for (int k = 0; k < g.nimg; k += 4) {
+        rf::Quad q{};
+        q.base = g.base0 + k;
+        q.n = std::min(4, g.nimg - k);
+        q.img = g.img0 + k;
+        q.img1 = k / 2 < g.n1 ? g.img1 + k / 2 : -1;
+        q.img2 = k / 4 < g.n2 ? g.img2 + k / 4 : -1;
+        p->quads.push_back(q);
+      }
   }
   w.g_end = (int)p->groups.size();
   w.img_end = (int)p->img_info.size();
+  w.base_end = nbase;
+  w.quad_end = (int)p->quads.size();
   if (w.img_end > w.img_begin) p->waves.push_back(w);
   // chunks of the fused pass: each group's images in runs of chunk_images
   p->chunks.clear();
   p->wave_chunks.clear();
-  if (p->chunk_images > 0) {
+  if (p->chunk_images > 0 && !p->derived) {
     for (const Wave& wv : p->waves) {
       const int c0 = (int)p->chunks.size();
       for (int gi = wv.g_begin; gi < wv.g_end; ++gi)
@@ -670,12 +792,13 @@ void build_lists(rf_plan* p, int nint) {
   }
   p->cached_nint = nint;
   p->cached_span = p->t_span;
+  p->cached_plain = plain;
   p->drop_graph();
 }
 
 // Whether the search's waves take the fused column + row pass.
 bool use_fused(const rf_plan* p) {
-  return p->fused && p->chunk_images > 0 && p->tmap_ring.nbox > 0 && !(p->flags & RF_NOISE_CLIPPED);
+  return p->fused && !p->derived && p->chunk_images > 0 && p->tmap_ring.nbox > 0 && !(p->flags & RF_NOISE_CLIPPED);
 }
 
 // cuTensorMapEncodeTiled from the driver, looked up once.
@@ -729,7 +852,7 @@ void encode_tile_map(rf_plan* p, rf::TileMap& tm, float2* base, int slots, int t
 }
 
 // (Re)allocate the per-wave scratch for `slots` images (clamped to
-// [images_per_group, 32768]: images per wave ride on gridDim.y).
+// [images_per_group, 32768]).
 rf_status alloc_wave_scratch(rf_plan* p, int slots) {
   const int B = p->shape.images_per_group;
   slots = std::max(std::min(slots, 32768), B);
@@ -739,12 +862,12 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
   p->tmap_P.nbox = 0;
   p->tmap_H[0].nbox = p->tmap_H[1].nbox = 0;
   if (p->d_T) {
-    p->device_bytes -= (uint64_t)p->slots_max * per_slot * sizeof(float2);
+    p->device_bytes -= (uint64_t)p->tslots * per_slot * sizeof(float2);
     p->dfree(p->d_T);
     p->d_T = nullptr;
   }
   if (p->d_partials) {
-    p->device_bytes -= (uint64_t)p->slots_max * nrb * sizeof(StatPartial);
+    p->device_bytes -= (uint64_t)p->sslots * nrb * sizeof(StatPartial);
     p->dfree(p->d_partials);
     p->d_partials = nullptr;
   }
@@ -754,38 +877,40 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
     p->d_cellbuf = nullptr;
   }
   if (p->d_colsq) {
-    p->device_bytes -= (uint64_t)p->slots_max * (p->ncol + 1) * sizeof(float);
+    p->device_bytes -= (uint64_t)p->sslots * (p->ncol + 1) * sizeof(float);
     p->dfree(p->d_colsq);
     p->dfree(p->d_mean0);
     p->d_colsq = p->d_mean0 = nullptr;
   }
   if (p->d_clip) {
-    p->device_bytes -= (uint64_t)p->slots_max * sizeof(float2);
+    p->device_bytes -= (uint64_t)p->sslots * sizeof(float2);
     p->dfree(p->d_clip);
     p->d_clip = nullptr;
   }
   p->slots_max = slots;
-  p->gslots_max = std::max(2 * ((slots + B - 1) / B), 1);
+  p->tslots = wave_tslots(p, slots);
+  p->sslots = wave_sslots(p, slots);
+  p->gslots_max = std::max(2 * ((p->tslots + B - 1) / B), 1);
   p->cached_nint = -1;
   p->drop_graph();
   rf_status s;
-  if ((s = p->dalloc(&p->d_T, (size_t)slots * per_slot)) != RF_OK) return s;
-  if ((s = p->dalloc(&p->d_partials, (size_t)slots * nrb)) != RF_OK) return s;
+  if ((s = p->dalloc(&p->d_T, (size_t)p->tslots * per_slot)) != RF_OK) return s;
+  if ((s = p->dalloc(&p->d_partials, (size_t)p->sslots * nrb)) != RF_OK) return s;
   if ((s = p->dalloc(&p->d_cellbuf, (size_t)p->gslots_max * std::max(p->n_cells, 1) * 32)) != RF_OK) return s;
-  if ((s = p->dalloc(&p->d_colsq, (size_t)slots * p->ncol)) != RF_OK) return s;
-  if ((s = p->dalloc(&p->d_mean0, (size_t)slots)) != RF_OK) return s;
-  if ((p->flags & RF_NOISE_CLIPPED) && (s = p->dalloc(&p->d_clip, (size_t)slots)) != RF_OK) return s;
+  if ((s = p->dalloc(&p->d_colsq, (size_t)p->sslots * p->ncol)) != RF_OK) return s;
+  if ((s = p->dalloc(&p->d_mean0, (size_t)p->sslots)) != RF_OK) return s;
+  if ((p->flags & RF_NOISE_CLIPPED) && (s = p->dalloc(&p->d_clip, (size_t)p->sslots)) != RF_OK) return s;
   const int xb = std::min(256 / (p->npix / 32), p->npix / 2);  // row pairs of a row-pass work item
-  encode_tile_map(p, p->tmap_T, p->d_T, p->slots_max, 2 * xb);
+  encode_tile_map(p, p->tmap_T, p->d_T, p->tslots, 2 * xb);
   // the halves of d_T, each a wave's scratch when waves are overlapped
-  const int half = p->slots_max / 2;
+  const int half = p->tslots / 2;
   if (half >= B) {
     encode_tile_map(p, p->tmap_H[0], p->d_T, half, 2 * xb);
     encode_tile_map(p, p->tmap_H[1], p->d_T + (size_t)half * per_slot, half, 2 * xb);
   }
   // the periodicity row pass's tensor-copy tiles (one image's XB rows), at
   // N = 1024, where its transforms fit one warp
-  if (p->npix == 1024) encode_tile_map(p, p->tmap_P, p->d_T, p->slots_max, xb);
+  if (p->npix == 1024) encode_tile_map(p, p->tmap_P, p->d_T, p->tslots, xb);
   // fused pass: counters for the most chunks a wave can hold
   if (p->chunk_images > 0) {
     const int cap = 1 + 2 * p->gslots_max * ((p->shape.images_per_group + p->chunk_images - 1) / p->chunk_images);
@@ -842,15 +967,17 @@ uint64_t estimate_device_bytes(const rf_plan* p, int slots) {
   b += r(p->dt.size(), 8) + r(p->dt.size(), 4);
   const int64_t img_cap = std::max<int64_t>(count_images(p, p->max_nint), 1);
   b += r(img_cap, sizeof(int4)) + r(img_cap, sizeof(Group)) + r(img_cap, 8) + r(img_cap, sizeof(DevCand)) + 4 + 4;  // candidate count, error flag
+  if (p->derived) b += r(img_cap, sizeof(rf::Quad));
   const size_t per_slot = (size_t)p->ncol * N * sizeof(float2);
-  if (slots <= 0) slots = (int)std::min<size_t>(kTBudgetBytes / per_slot, (size_t)img_cap);
+  if (slots <= 0) slots = default_slots(p, (size_t)img_cap);
   const int B = p->shape.images_per_group;
   slots = std::max(std::min(slots, 32768), B);
-  const int gslots = std::max(2 * ((slots + B - 1) / B), 1);
-  b += r((size_t)slots * per_slot, 1) + r((size_t)slots * p->shape.partials_per_image, sizeof(StatPartial)) +
-       r((size_t)gslots * std::max(p->n_cells, 1) * 32, sizeof(float2)) + r((size_t)slots * p->ncol, 4) +
-       r(slots, 4);
-  if (p->flags & RF_NOISE_CLIPPED) b += r(slots, sizeof(float2));
+  const int tslots = wave_tslots(p, slots), sslots = wave_sslots(p, slots);
+  const int gslots = std::max(2 * ((tslots + B - 1) / B), 1);
+  b += r((size_t)tslots * per_slot, 1) + r((size_t)sslots * p->shape.partials_per_image, sizeof(StatPartial)) +
+       r((size_t)gslots * std::max(p->n_cells, 1) * 32, sizeof(float2)) + r((size_t)sslots * p->ncol, 4) +
+       r(sslots, 4);
+  if (p->flags & RF_NOISE_CLIPPED) b += r(sslots, sizeof(float2));
   const int ci = rf::fused_chunk_images((int)N);
   if (ci > 0) {
     b += r(img_cap, sizeof(rf::FusedChunk)) + r(1 + 2 * gslots * ((B + ci - 1) / ci), 4);
@@ -968,9 +1095,8 @@ rf_status alloc_device(rf_plan* p) {
   // column-FFT scratch, whole groups per wave
   p->chunk_images = rf::fused_chunk_images(N);
   if (p->chunk_images > 0 && (s = p->dalloc(&p->d_chunks, (size_t)p->img_cap)) != RF_OK) return s;
-  const size_t per_slot = (size_t)p->ncol * N * sizeof(float2);
-  int slots = (int)std::min<size_t>(kTBudgetBytes / per_slot, (size_t)p->img_cap);
-  if ((s = alloc_wave_scratch(p, slots)) != RF_OK) return s;
+  if (p->derived && (s = p->dalloc(&p->d_quads, (size_t)p->img_cap)) != RF_OK) return s;
+  if ((s = alloc_wave_scratch(p, default_slots(p, (size_t)p->img_cap))) != RF_OK) return s;
   if ((s = alloc_ring(p, kDefaultRing)) != RF_OK) return s;
 
   // host->device staging of raw visibilities
@@ -1046,17 +1172,34 @@ rf_status ingest(rf_plan* p, const void* vis, int nint, cudaStream_t st) {
   return RF_OK;
 }
 
-// Resampled series for every dt > 1 of the plan (after ingest).
-rf_status resample_all(rf_plan* p, int nint, cudaStream_t st) {
+// Resampled series (after ingest) of the widths dt > 1 that `used` names by
+// index (width k is used if used[k]).
+rf_status resample_widths(rf_plan* p, int nint, const std::vector<char>& used, cudaStream_t st) {
   const SegmentGeom g = geom(p, nint);
   for (int k = 0; k < p->ndt; ++k) {
-    if (p->dt[k] == 1 || p->d_sdt[k] == p->d_S) continue;
+    if (!used[k] || p->dt[k] == 1 || p->d_sdt[k] == p->d_S) continue;
     bool done = false;
-    for (int k2 = 0; k2 < k; ++k2) done = done || p->d_sdt[k2] == p->d_sdt[k];
+    for (int k2 = 0; k2 < k; ++k2) done = done || (used[k2] && p->d_sdt[k2] == p->d_sdt[k]);
     if (done) continue;
     RF_TIMED(p->prof, K_RESAMPLE, st, rf::launch_resample(g, p->d_S, p->d_sdt[k], p->dt[k], p->sdt_lp[k], st));
   }
   return RF_OK;
+}
+
+// The series that the batched search (widths with transforms of their own) or
+// the plain form (all) reads.
+rf_status resample_search(rf_plan* p, int nint, cudaStream_t st) {
+  std::vector<char> used(p->ndt, 1);
+  if (p->form != RF_FORM_PLAIN)
+    for (int k = 0; k < p->ndt; ++k) used[k] = p->sum_of[k] == k;
+  return resample_widths(p, nint, used, st);
+}
+
+// The series that n listed trials (d, s, t') read.
+rf_status resample_trials(rf_plan* p, int nint, const int32_t* trials, int n, cudaStream_t st) {
+  std::vector<char> used(p->ndt, 0);
+  for (int k = 0; k < n; ++k) used[trials[3 * k + 1]] = 1;
+  return resample_widths(p, nint, used, st);
 }
 
 // Overlapped waves (RF_TUNE_OVERLAP).  Wave w images into half w mod 2 of
@@ -1097,11 +1240,25 @@ rf_status run_waves_overlapped(rf_plan* p, const SegmentGeom& g, const std::vect
   return RF_OK;
 }
 
+// The row pass of one wave: over quads where the plan has widths that are sums
+// of others (never for listed trials, whose images `im` takes), else image by
+// image.  `clip`: the wave's clipping windows, or null.
+cudaError_t launch_row_pass(rf_plan* p, const SegmentGeom& g, const Wave& w, const float2* T, StatPartial* part,
+                            const rf::TileMap* tm, const float2* clip, float* im, cudaStream_t st,
+                            const rf::PassLaunch* pl) {
+  if (tm->nbox == 0) tm = nullptr;
+  if (w.quad_end > w.quad_begin)
+    return rf::launch_rowfft_tree(g, p->tb, T, p->d_quads + w.quad_begin, w.quad_end - w.quad_begin, w.img_begin,
+                                  w.base_begin, part, tm, p->d_err, st, clip, pl);
+  return rf::launch_rowfft_stats(g, p->tb, T, w.img_end - w.img_begin, w.img_begin, p->d_weight, part, im, tm,
+                                 p->d_err, st, clip, pl);
+}
+
 // The wave loop of run_waves_overlapped (streams and events set up).
 rf_status overlapped_loop(rf_plan* p, const SegmentGeom& g, const std::vector<Wave>& waves, DevStat* d_stats,
                          cudaStream_t st, const rf::PassLaunch& pc, const rf::PassLaunch& pr) {
   cudaStream_t so = p->ostream;
-  const size_t half = (size_t)p->slots_max / 2;
+  const size_t half = (size_t)p->tslots / 2, shalf = (size_t)p->sslots / 2;
   const size_t per_slot = (size_t)p->ncol * p->npix;
   const size_t nrb = (size_t)p->shape.partials_per_image;
   for (size_t wi = 0; wi < waves.size(); ++wi) {
@@ -1110,21 +1267,19 @@ rf_status overlapped_loop(rf_plan* p, const SegmentGeom& g, const std::vector<Wa
     const int ng = w.g_end - w.g_begin;
     const int ni = w.img_end - w.img_begin;
     float2* T = p->d_T + h * half * per_slot;
-    StatPartial* part = p->d_partials + h * half * nrb;
-    float* colsq = p->d_colsq + h * half * p->ncol;
-    float* mean0 = p->d_mean0 + h * half;
+    StatPartial* part = p->d_partials + h * shalf * nrb;
+    float* colsq = p->d_colsq + h * shalf * p->ncol;
+    float* mean0 = p->d_mean0 + h * shalf;
     RF_TIMED(p->prof, K_GRID_CELLS, st,
              rf::launch_grid_cells(g, p->tb, p->d_groups, w.g_begin, ng, p->d_cellbuf, st));
     if (wi >= 2) RF_CUDA(cudaStreamWaitEvent(st, p->oev[2 + h], 0));
     RF_TIMED(p->prof, K_GRID_COLFFT, st,
-             rf::launch_colfft(g, p->tb, p->d_groups, w.g_begin, ng, w.img_begin, p->d_cellbuf, T, colsq, mean0,
-                               st, &pc));
+             rf::launch_colfft(g, p->tb, p->d_groups, w.g_begin, ng, w.img_begin, w.base_begin, p->d_cellbuf, T,
+                               colsq, mean0, st, &pc));
     RF_CUDA(cudaEventRecord(p->oev[h], st));
     RF_CUDA(cudaStreamWaitEvent(so, p->oev[h], 0));
     RF_TIMED(p->prof, K_ROWFFT_STATS, so,
-             rf::launch_rowfft_stats(g, p->tb, T, ni, w.img_begin, p->d_weight, part, nullptr,
-                                     p->tmap_H[h].nbox > 0 ? &p->tmap_H[h] : nullptr, p->d_err, so, nullptr,
-                                     &pr));
+             launch_row_pass(p, g, w, T, part, &p->tmap_H[h], nullptr, nullptr, so, &pr));
     RF_TIMED(p->prof, K_FINALIZE, so,
              rf::launch_finalize(g, part, colsq, mean0, p->d_img_info, p->d_weight, ni, w.img_begin, p->threshold,
                                  p->d_cands, p->d_ncand, p->img_cap, d_stats, so, false));
@@ -1162,16 +1317,15 @@ rf_status run_waves(rf_plan* p, int nint, const std::vector<Wave>& waves, int ni
       continue;
     }
     RF_TIMED(p->prof, K_GRID_COLFFT, st,
-             rf::launch_colfft(g, p->tb, p->d_groups, w.g_begin, ng, w.img_begin, p->d_cellbuf, p->d_T,
-                               p->d_colsq, p->d_mean0, st));
+             rf::launch_colfft(g, p->tb, p->d_groups, w.g_begin, ng, w.img_begin, w.base_begin, p->d_cellbuf,
+                               p->d_T, p->d_colsq, p->d_mean0, st));
     const bool clip = (p->flags & RF_NOISE_CLIPPED) != 0;
     if (clip)
       RF_TIMED(p->prof, K_CLIP_WINDOW, st, rf::launch_clip_window(g, p->d_colsq, p->d_mean0, ni, p->d_clip, st));
     float* im = d_images ? d_images + (size_t)w.img_begin * p->npix * p->npix : nullptr;
     RF_TIMED(p->prof, K_ROWFFT_STATS, st,
-             rf::launch_rowfft_stats(g, p->tb, p->d_T, ni, w.img_begin, p->d_weight, p->d_partials, im,
-                                     p->tmap_T.nbox > 0 ? &p->tmap_T : nullptr, p->d_err, st,
-                                     clip ? p->d_clip : nullptr));
+             launch_row_pass(p, g, w, p->d_T, p->d_partials, &p->tmap_T, clip ? p->d_clip : nullptr, im, st,
+                             nullptr));
     RF_TIMED(p->prof, K_FINALIZE, st,
              rf::launch_finalize(g, p->d_partials, p->d_colsq, p->d_mean0, p->d_img_info, p->d_weight, ni,
                                  w.img_begin, p->threshold, p->d_cands, p->d_ncand, p->img_cap, d_stats, st,
@@ -1306,15 +1460,18 @@ rf_status search_impl(rf_plan* p, const void* vis, int nint, void* stream, rf_ca
 
   rf_status s = ingest(p, vis, nint, st);
   if (s != RF_OK) return s;
-  s = resample_all(p, nint, st);
+  s = resample_search(p, nint, st);
   if (s != RF_OK) return s;
-  if (p->cached_nint != nint || p->cached_span != p->t_span) {
+  if (p->cached_nint != nint || p->cached_span != p->t_span || p->cached_plain != (p->form == RF_FORM_PLAIN)) {
     build_lists(p, nint);
     if (!p->img_info.empty()) {
       RF_CUDA(cudaMemcpyAsync(p->d_img_info, p->img_info.data(), p->img_info.size() * sizeof(int4),
                               cudaMemcpyHostToDevice, st));
       RF_CUDA(cudaMemcpyAsync(p->d_groups, p->groups.data(), p->groups.size() * sizeof(Group),
                               cudaMemcpyHostToDevice, st));
+      if (!p->quads.empty())
+        RF_CUDA(cudaMemcpyAsync(p->d_quads, p->quads.data(), p->quads.size() * sizeof(rf::Quad),
+                                cudaMemcpyHostToDevice, st));
       if (!p->chunks.empty())
         RF_CUDA(cudaMemcpyAsync(p->d_chunks, p->chunks.data(), p->chunks.size() * sizeof(rf::FusedChunk),
                                 cudaMemcpyHostToDevice, st));
@@ -1386,12 +1543,13 @@ rf_status search_impl(rf_plan* p, const void* vis, int nint, void* stream, rf_ca
   *n_out = dc.size();
   if (want_stats && n_stats) *n_stats = (size_t)nimg;
   if (d_stats) {
-    const size_t ns = std::min<size_t>(stats_cap, (size_t)nimg);
-    for (size_t k = 0; k < ns; ++k) {
+    for (const int4& info : p->img_info) {
+      const size_t k = (size_t)info.w;  // the device wrote the records in (d, s, t') order
+      if (k >= stats_cap) continue;
       rf_image_stat& o = stats[k];
-      o.dm_idx = p->img_info[k].x;
-      o.dt_idx = p->img_info[k].y;
-      o.t_idx = p->img_info[k].z;
+      o.dm_idx = info.x;
+      o.dt_idx = info.y;
+      o.t_idx = info.z;
       o.x = ds[k].x;
       o.y = ds[k].y;
       o.peak = ds[k].peak;
@@ -1423,18 +1581,18 @@ rf_status render_core(rf_plan* p, int nint, const int32_t* trials, int n, float*
   std::vector<int4> info(n);
   std::vector<Group> grp(n);
   for (int k = 0; k < n; ++k) {
-    info[k] = make_int4(trials[3 * k], trials[3 * k + 1], trials[3 * k + 2], 0);
-    grp[k] = Group{trials[3 * k], trials[3 * k + 1], trials[3 * k + 2], 1, k, {0, 0, 0}};
+    info[k] = make_int4(trials[3 * k], trials[3 * k + 1], trials[3 * k + 2], k);
+    grp[k] = Group{trials[3 * k], trials[3 * k + 1], trials[3 * k + 2], 1, k, k, 0, 0, 0, 0, {0, 0}};
   }
   p->cached_nint = -1;
   p->drop_graph();
   RF_CUDA(cudaMemcpyAsync(p->d_img_info, info.data(), n * sizeof(int4), cudaMemcpyHostToDevice, st));
   RF_CUDA(cudaMemcpyAsync(p->d_groups, grp.data(), n * sizeof(Group), cudaMemcpyHostToDevice, st));
   std::vector<Wave> waves;
-  const int per_wave = std::min(p->slots_max, p->gslots_max);  // single-image groups
+  const int per_wave = std::min(std::min(p->tslots, p->sslots), p->gslots_max);  // single-image groups
   for (int k = 0; k < n; k += per_wave) {
     const int e = std::min(n, k + per_wave);
-    waves.push_back(Wave{k, e, k, e});
+    waves.push_back(Wave{k, e, k, e, k, e, 0, 0});
   }
   RF_CUDA(cudaMemsetAsync(p->d_ncand, 0, sizeof(int), st));
   rf_status s = run_waves(p, nint, waves, n, nullptr, d_img, st);
@@ -1542,6 +1700,7 @@ rf_status rf_plan_create(const rf_plan_desc* desc, rf_plan** out) {
   p->dm.assign(desc->dm_list, desc->dm_list + desc->ndm);
   p->dt.assign(desc->dt_list, desc->dt_list + desc->ndt);
   p->host_only = (desc->flags & RF_HOST_ONLY) != 0;
+  build_widths(p);
   s = build_tables(p);
   if (s != RF_OK) {
     delete p;
@@ -1594,6 +1753,7 @@ rf_status rf_plan_estimate_bytes(const rf_plan_desc* desc, int64_t wave_images, 
   tmp.freq.assign(desc->freq_hz, desc->freq_hz + desc->nchan);
   tmp.dm.assign(desc->dm_list, desc->dm_list + desc->ndm);
   tmp.dt.assign(desc->dt_list, desc->dt_list + desc->ndt);
+  build_widths(&tmp);
   s = build_tables(&tmp);
   if (s != RF_OK) return s;
   *bytes = estimate_device_bytes(&tmp, (int)std::min<int64_t>(std::max<int64_t>(wave_images, 0), 32768));
@@ -1634,7 +1794,7 @@ rf_status rf_render_images(rf_plan* p, const void* vis, int32_t nint, void* stre
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   s = ingest(p, vis, nint, st);
   if (s != RF_OK) return s;
-  s = resample_all(p, nint, st);
+  s = resample_trials(p, nint, trials, n, st);
   if (s != RF_OK) return s;
   const size_t npx = (size_t)p->npix * p->npix;
   float* d_img = nullptr;
@@ -1680,7 +1840,7 @@ rf_status rf_candidate_products(rf_plan* p, const void* vis, int32_t nint, void*
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   s = ingest(p, vis, nint, st);
   if (s != RF_OK) return s;
-  s = resample_all(p, nint, st);
+  s = resample_trials(p, nint, trials.data(), n, st);
   if (s != RF_OK) return s;
   if (!p->d_cellbc) {  // per-row (iu, iv) table, built on first use
     std::vector<int2> cb((size_t)p->nbl * p->nchan);
@@ -1854,15 +2014,15 @@ rf_status rf_periodicity_search(rf_plan* p, const void* vis, int32_t nint, int32
     for (int j = 0; j < nb; ++j)
       for (int kb = 0; kb < nkb; ++kb) {
         const int n = std::min(B, K - kb * B);
-        if ((nimg + 2 * n) - w.i0 > p->slots_max || ((int)grp.size() + 2) - w.g0 > p->gslots_max) {
+        if ((nimg + 2 * n) - w.i0 > std::min(p->tslots, p->sslots) || ((int)grp.size() + 2) - w.g0 > p->gslots_max) {
           w.g1 = (int)grp.size();
           w.i1 = nimg;
           w.p1 = (int)pairs.size();
           waves.push_back(w);
           w = PW{w.g1, w.g1, nimg, nimg, w.p1, w.p1};
         }
-        grp.push_back(Group{0, 2 * j, kb * B, n, nimg, {0, 0, 0}});
-        grp.push_back(Group{0, 2 * j + 1, kb * B, n, nimg + n, {0, 0, 0}});
+        grp.push_back(Group{0, 2 * j, kb * B, n, nimg, nimg, 0, 0, 0, 0, {0, 0}});
+        grp.push_back(Group{0, 2 * j + 1, kb * B, n, nimg + n, nimg + n, 0, 0, 0, 0, {0, 0}});
         for (int i = 0; i < n; ++i)
           pairs.push_back(make_int4(nimg + i - w.i0, nimg + n + i - w.i0, dms[b0 + j], kmin + kb * B + i));
         nimg += 2 * n;
@@ -1878,7 +2038,7 @@ rf_status rf_periodicity_search(rf_plan* p, const void* vis, int32_t nint, int32
       const int ng = v.g1 - v.g0;
       const int np = v.p1 - v.p0;
       RF_CUDA(rf::launch_grid_cells(gp, tbp, d_grp, v.g0, ng, p->d_cellbuf, st));
-      RF_CUDA(rf::launch_colfft(gp, tbp, d_grp, v.g0, ng, v.i0, p->d_cellbuf, p->d_T, p->d_colsq, p->d_mean0, st));
+      RF_CUDA(rf::launch_colfft(gp, tbp, d_grp, v.g0, ng, v.i0, v.i0, p->d_cellbuf, p->d_T, p->d_colsq, p->d_mean0, st));
       RF_CUDA(rf::launch_rowfft_power(gp, tbp, p->d_T, d_pairs + v.p0, np, p->d_partials,
                                       p->tmap_P.nbox > 0 ? &p->tmap_P : nullptr, p->d_err, st));
       RF_CUDA(rf::launch_finalize_power(gp, p->d_partials, p->d_colsq, p->d_mean0, d_pairs + v.p0, np,
@@ -2065,13 +2225,16 @@ rf_status rf_plan_autotune(rf_plan* p, const void* vis, int32_t nint, void* stre
   const size_t per_slot = (size_t)p->ncol * p->npix * sizeof(float2);
   size_t free_b = 0, total_b = 0;
   RF_CUDA(cudaMemGetInfo(&free_b, &total_b));
-  const size_t have = free_b / 2 + (size_t)p->slots_max * per_slot;  // the current scratch is reusable
+  const size_t have = free_b / 2 + (size_t)p->tslots * per_slot;  // the current scratch is reusable
   struct Cand {
     int wave, graphs, fused, ring, overlap;
   };
   std::vector<Cand> cands;
-  auto fits = [&](int w) { return (size_t)std::max(w, B) * per_slot <= have; };
-  const bool can_fuse = p->chunk_images > 0 && !(p->flags & RF_NOISE_CLIPPED);
+  auto fits = [&](int w) { return (size_t)wave_tslots(p, std::max(w, B)) * per_slot <= have; };
+  // where widths are sums of others the fused pass does not apply, but its
+  // sizes keep their two wave sizes
+  const bool big = p->chunk_images > 0 && !(p->flags & RF_NOISE_CLIPPED);
+  const bool can_fuse = big && !p->derived;
   // waves whose column-FFT output fits the L2 cache (one to four groups), so
   // that the row pass may find it there instead of in HBM
   int l2 = 0;
@@ -2080,11 +2243,12 @@ rf_status rf_plan_autotune(rf_plan* p, const void* vis, int32_t nint, void* stre
     l2 = 0;
   }
   for (int w = B; w <= 4 * B && w < 256; w *= 2)
-    if ((size_t)w * per_slot <= (size_t)l2 && fits(w) && w < nimg) cands.push_back({w, 1, 0, p->ring, 0});
-  if (can_fuse) {
+    if ((size_t)wave_tslots(p, w) * per_slot <= (size_t)l2 && fits(w) && w < nimg) cands.push_back({w, 1, 0, p->ring, 0});
+  if (big) {
     for (int w : {2048, 8192}) {
       if (!fits(w)) continue;
-      for (int ring : {2, 3, 4}) cands.push_back({w, 1, 1, ring, 0});
+      if (can_fuse)
+        for (int ring : {2, 3, 4}) cands.push_back({w, 1, 1, ring, 0});
       cands.push_back({w, 1, 0, p->ring, 0});
       if (w / 2 >= B) cands.push_back({w, 1, 0, p->ring, 1});
       if (w >= nimg) break;

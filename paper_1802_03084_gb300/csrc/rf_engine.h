@@ -58,14 +58,31 @@ struct DevTables {
 };
 
 // Group of consecutive output integrations of one (DM, dt) trial imaged
-// together by the gridding/column-FFT kernel.
+// together by the gridding/column-FFT kernel, and the images derived from
+// them.  The transforms of an image are linear in the visibilities, and a
+// boxcar of 2 dt (4 dt) integrations is the sum of two (four) consecutive ones
+// of dt, so image t' of the trial of width 2 dt (4 dt) is the sum of images
+// 2 t' and 2 t' + 1 (4 t' .. 4 t' + 3) of the same DM: it takes no transform of
+// its own.  t0 is a multiple of 32 wherever n1 or n2 is set.
 struct Group {
   int32_t d;
   int32_t s;
   int32_t t0;
   int32_t nimg;
   int32_t img0;  // index of the group's first image in the image list
-  int32_t pad[3];
+  int32_t base0;  // index of its first image among the transformed images
+  int32_t n1, img1;  // sums of two: how many are searched, the first one's index in the image list
+  int32_t n2, img2;  // sums of four
+  int32_t pad[2];
+};
+
+// Up to four consecutive transformed images of a group, for the row pass: the
+// transformed-image index of the first, how many there are, and the image
+// list's indices of the first, of the first sum of two and of the sum of four
+// (-1: not searched).
+struct Quad {
+  int32_t base, n, img, img1;
+  int32_t img2, pad[3];
 };
 
 // One chunk of the fused imaging pass: nk consecutive images from image
@@ -236,12 +253,13 @@ cudaError_t launch_grid_cells(const SegmentGeom& g, const DevTables& tb, const G
                               int ngroups, float2* cellbuf, cudaStream_t st);
 
 // Column FFTs (pass A2) of the same groups from cellbuf; writes
-// Tbuf[slot][col][y], slot = image index - img_base, the Parseval sums
+// Tbuf[b][col][y], b = transformed-image index - base_base, and for every
+// image of the groups, sums of two and four included, the Parseval sums
 // colsq[slot][col] (weighted sum of |H|^2 over the column) and
-// mean0[slot] = Re H(u = 0, v = 0).
+// mean0[slot] = Re H(u = 0, v = 0), slot = image index - img_base.
 cudaError_t launch_colfft(const SegmentGeom& g, const DevTables& tb, const Group* groups, int g_begin,
-                          int ngroups, int img_base, const float2* cellbuf, float2* Tbuf, float* colsq,
-                          float* mean0, cudaStream_t st, const PassLaunch* pl = nullptr);
+                          int ngroups, int img_base, int base_base, const float2* cellbuf, float2* Tbuf,
+                          float* colsq, float* mean0, cudaStream_t st, const PassLaunch* pl = nullptr);
 
 // Fused column + row pass (npix 1024 .. 4096) of the chunks [0, nchunks)
 // of one wave (chunks[] on the device, groups indexed absolutely, cellbuf
@@ -271,6 +289,14 @@ cudaError_t launch_rowfft_stats(const SegmentGeom& g, const DevTables& tb, const
                                 int img_base, const double* weight, StatPartial* partials, float* images,
                                 const TileMap* tm, int* err, cudaStream_t st, const float2* clip = nullptr,
                                 const PassLaunch* pl = nullptr);
+
+// The same for the transformed images of nquads quads (T slots relative to
+// base_base, statistics slots to img_base) and the images derived from them,
+// npix >= kTreeMinNpix.
+cudaError_t launch_rowfft_tree(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Quad* quads,
+                               int nquads, int img_base, int base_base, StatPartial* partials, const TileMap* tm,
+                               int* err, cudaStream_t st, const float2* clip, const PassLaunch* pl = nullptr);
+constexpr int kTreeMinNpix = 64;  // below, a row-pass block is less than a warp
 
 // Reduce row-block partials, compute sigma / snr, append candidates and
 // (optionally) per-image stats for images [img_base, img_base + nimg).

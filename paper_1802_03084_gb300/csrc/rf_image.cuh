@@ -99,6 +99,14 @@ struct ColCfg {
   static_assert((XA * R * STRIDE * 8) % 16 == 0, "staged cells start 16-byte aligned");
 };
 
+// Tensor memory of a k_rowfft_tree block: 128 columns (two sums deep, 64
+// registers each) for each set of four warps; an SM has 512.
+template <int N>
+struct TreeCfg {
+  static constexpr int COLS = 128 * ((ImgCfg<N>::THREADS_B + 127) / 128);
+  static_assert((COLS & (COLS - 1)) == 0 && COLS <= 512, "tensor-memory columns");
+};
+
 // Image row of index i of the column-FFT output (see SegmentGeom::tsplit).
 __device__ __forceinline__ int t_row(int i, int tsplit, int log2l) {
   return tsplit > 1 ? ((i & ((1 << log2l) - 1)) * tsplit + (i >> log2l)) : i;
@@ -217,7 +225,7 @@ __device__ __forceinline__ void col_fft_store(float2* buf, const float2* __restr
 // third FFT pass and no barrier across warps for N >= 2048.
 template <int N>
 __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
-    k_colfft(SegmentGeom g, DevTables tb, const Group* __restrict__ groups, int g_begin, int img_base,
+    k_colfft(SegmentGeom g, DevTables tb, const Group* __restrict__ groups, int g_begin, int img_base, int base_base,
              const float2* __restrict__ cellbuf, float2* __restrict__ Tbuf, float* __restrict__ colsq,
              float* __restrict__ mean0) {
   using C = ColCfg<N>;
@@ -263,25 +271,64 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
 
     // Parseval: the image's sum of squares is N^2 / (4 W^2) times the sum
     // of |G|^2 over the full Hermitian plane, which counts this column
-    // twice unless u = 0; its mean is G(0, 0) / (2 W).  Each warp sums
-    // |H|^2 of the column's cells for some of the images (FP32, fixed order).
+    // twice unless u = 0; its mean is G(0, 0) / (2 W).  Lane k is image k of
+    // the part (two cells a step where the part is 16 images), so the cells of
+    // a sum of two or four images are xor-shuffles away; the warps' FP32 sums
+    // meet in the first FFT buffer and are added in a fixed order.
     {
-      const float wcol = col == 0 ? 1.f : 2.f;
-      for (int kl = tid >> 5; kl < nk; kl += C::THREADS / 32) {
-        float acc = 0.f;
-        for (int c = lane; c < ncells; c += 32) {
-          const float2 h = cellv[c * PI + 2 * ((kl >> 1) ^ (c & (CPC - 1))) + (kl & 1)];
-          acc = fmaf(h.x, h.x, fmaf(h.y, h.y, acc));
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) {
-          const size_t slot = (size_t)(gr.img0 + kbase + kl - img_base);
-          colsq[slot * g.ncol + col] = wcol * acc;
-          // row 0 sorts first in column 0; cell 0's first chunk is unswizzled
-          if (col == 0) mean0[slot] = (ncells > 0 && crow[0] == 0) ? cellv[kl].x : 0.f;
+      constexpr int NW = C::THREADS / 32, CPS = 32 / PI;
+      const bool derived = gr.n1 > 0 || gr.n2 > 0;
+      const int warp = tid >> 5, kl = lane & (PI - 1);
+      float a0 = 0.f, a1 = 0.f, a2 = 0.f;
+      for (int cb = warp * CPS; cb < ncells; cb += NW * CPS) {
+        const int c = cb + lane / PI;
+        float2 h = make_float2(0.f, 0.f);
+        if (c < ncells && kl < nk) h = cellv[c * PI + 2 * ((kl >> 1) ^ (c & (CPC - 1))) + (kl & 1)];
+        a0 = fmaf(h.x, h.x, fmaf(h.y, h.y, a0));
+        if (derived) {
+          h.x += __shfl_xor_sync(0xffffffffu, h.x, 1);
+          h.y += __shfl_xor_sync(0xffffffffu, h.y, 1);
+          a1 = fmaf(h.x, h.x, fmaf(h.y, h.y, a1));
+          h.x += __shfl_xor_sync(0xffffffffu, h.x, 2);
+          h.y += __shfl_xor_sync(0xffffffffu, h.y, 2);
+          a2 = fmaf(h.x, h.x, fmaf(h.y, h.y, a2));
         }
       }
+      if constexpr (CPS == 2) {
+        a0 += __shfl_xor_sync(0xffffffffu, a0, 16);
+        a1 += __shfl_xor_sync(0xffffffffu, a1, 16);
+        a2 += __shfl_xor_sync(0xffffffffu, a2, 16);
+      }
+      static_assert(CPS <= 2 && NW * 3 * 32 * 4 <= C::SMEM_FIXED, "Parseval sums fit the FFT buffers");
+      float* red = reinterpret_cast<float*>(fbuf);  // [level][warp][32]
+      red[warp * 32 + lane] = a0;
+      if (derived) {
+        red[(NW + warp) * 32 + lane] = a1;
+        red[(2 * NW + warp) * 32 + lane] = a2;
+      }
+      __syncthreads();
+      const int lv = warp;  // warps 0 .. 2: single images, sums of two, sums of four
+      if (lv < (derived ? 3 : 1) && lane < PI) {
+        const int k = kbase + lane, j = k >> lv;
+        const int lim = lv == 0 ? gr.nimg : (lv == 1 ? gr.n1 : gr.n2);
+        if ((lane & ((1 << lv) - 1)) == 0 && j < lim) {
+          float acc = 0.f;
+          for (int w = 0; w < NW; ++w) acc += red[(lv * NW + w) * 32 + lane];
+          const size_t slot = (size_t)((lv == 0 ? gr.img0 : (lv == 1 ? gr.img1 : gr.img2)) + j - img_base);
+          colsq[slot * g.ncol + col] = (col == 0 ? 1.f : 2.f) * acc;
+          if (col == 0) {
+            // row 0 sorts first in column 0; cell 0's chunks are unswizzled
+            float m = 0.f;
+            if (ncells > 0 && crow[0] == 0) {
+              m = cellv[lane].x;
+              if (lv >= 1) m += cellv[lane + 1].x;
+              if (lv == 2) m += cellv[lane + 2].x + cellv[lane + 3].x;
+            }
+            mean0[slot] = m;
+          }
+        }
+      }
+      __syncthreads();  // the FFT buffer is free again
     }
 
     if (xf < C::XA) {
@@ -289,7 +336,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
       for (int rd = 0; rd < nrounds; ++rd) {
         const int kl = rd * C::XA + xf;
         const bool live = kl < nk;
-        float2* dst = live ? Tbuf + ((size_t)(gr.img0 + kbase + kl - img_base) * g.ncol + col) * N + p * L : nullptr;
+        float2* dst = live ? Tbuf + ((size_t)(gr.base0 + kbase + kl - base_base) * g.ncol + col) * N + p * L : nullptr;
         col_scatter<N, PI>(buf, runs, nruns, cellv, crow, kl, live, rtw, t, p, xf * R + p);
         col_fft_store<N>(buf, tb.twiddle_col, t, xf * R + p, dst);
       }
@@ -390,36 +437,67 @@ __device__ __forceinline__ void row_zbuild(float2 (&v)[ImgCfg<N>::EB], const flo
   }
 }
 
-// Row pass, after row_zbuild: the inverse FFT of the row pair (T rows
-// i = y0 + 2 xf and i + 1, image rows t_row of them) in `buf`, the pair's
-// max pixel with its lowest index (and under CLIP the kept-pixel sums), one
-// StatPartial per warp of the transform, and the two image rows if `images`.
-template <int N, bool CLIP>
-__device__ __forceinline__ void row_finish(float2 (&v)[ImgCfg<N>::EB], float2* buf, const float2* __restrict__ tw,
-                                           int t, int xf, int slot, int y0, int tsplit, int log2l,
-                                           const double* __restrict__ weight, int img_base,
-                                           float* __restrict__ images, StatPartial* __restrict__ partials,
-                                           const float2* __restrict__ clip) {
+// Row pass, after row_zbuild: the inverse FFT of the row pair in `buf`.
+template <int N>
+__device__ __forceinline__ void row_fft(float2 (&v)[ImgCfg<N>::EB], float2* buf, const float2* __restrict__ tw, int t,
+                                        int xf) {
   using K = ImgCfg<N>;
-  constexpr int EB = K::EB, TB = K::TB;
+  constexpr int EB = K::EB;
   constexpr int H = N / K::RSPLIT;  // transform length per warp group
   // split transform (see row_zbuild): warp s runs the length-H transform of
   // Y_s in its own buffer; its second pass takes the pair table of
   // exp(+2 pi i k r / H) (s = 0, the table's section at N) or of
   // exp(+2 pi i r (2k + 1) / N) (s = 1, at N + H), so it is given the
   // table base tw + H + s H (the transform reads only its pair table)
-  const int s = K::RSPLIT == 2 ? t >> 5 : 0;
-  const int tt = K::RSPLIT == 2 ? t & 31 : t;
   if constexpr (K::RSPLIT == 2) {
-    fft_inverse_from_regs<H, false, EB>(v, buf + s * fft_stride<H>(), tw + H + s * H, tt, xf);
+    const int s = t >> 5;
+    fft_inverse_from_regs<H, false, EB>(v, buf + s * fft_stride<H>(), tw + H + s * H, t & 31, xf);
   } else {
     fft_inverse_from_regs<N, false, EB>(v, buf, tw, t, xf);
   }
-  // pixel of output register (m, q): output o of the transform, or of
-  // sub-transform s as pixel 2 o + s
-  auto pix = [&](int m, int q) {
-    return K::RSPLIT == 2 ? 2 * fft_out_index<H, EB>(tt, m, q) + s : fft_out_index<N, EB>(t, m, q);
-  };
+}
+
+// Pixel of output register (m, q) of thread t after row_fft: output o of the
+// transform, or of sub-transform s as pixel 2 o + s.
+template <int N>
+__device__ __forceinline__ int row_pix(int t, int m, int q) {
+  using K = ImgCfg<N>;
+  if constexpr (K::RSPLIT == 2) return 2 * fft_out_index<N / 2, K::EB>(t & 31, m, q) + (t >> 5);
+  else return fft_out_index<N, K::EB>(t, m, q);
+}
+
+// The two image rows (scaled) of a row pair whose pixels are in v.
+template <int N>
+__device__ __forceinline__ void row_write(const float2 (&v)[ImgCfg<N>::EB], int t, int xf, int slot, int y0, int tsplit,
+                                          int log2l, double W, float* __restrict__ images) {
+  using K = ImgCfg<N>;
+  constexpr int LP = FftShape<N / K::RSPLIT, K::EB>::LAST_P;
+  const float scale = W > 0.0 ? (float)(0.5 / W) : 0.f;
+  float* ima = images + ((size_t)slot * N + t_row(y0 + 2 * xf, tsplit, log2l)) * N;
+  float* imb = images + ((size_t)slot * N + t_row(y0 + 2 * xf + 1, tsplit, log2l)) * N;
+#pragma unroll
+  for (int m = 0; m < K::EB / LP; ++m)
+#pragma unroll
+    for (int q = 0; q < LP; ++q) {
+      const float2 z = v[m * LP + dft_perm<LP>(q)];
+      const int o = row_pix<N>(t, m, q);
+      ima[o] = z.x * scale;
+      imb[o] = z.y * scale;
+    }
+}
+
+// Statistics of the row pair (T rows i = y0 + 2 xf and i + 1, image rows t_row
+// of them) of the image in `slot` whose pixels are in v: the pair's max pixel
+// with its lowest index (and under CLIP the kept-pixel sums), one StatPartial
+// per warp of the transform.
+template <int N, bool CLIP>
+__device__ __forceinline__ void row_stats(const float2 (&v)[ImgCfg<N>::EB], int t, int xf, int slot, int y0,
+                                          int tsplit, int log2l, StatPartial* __restrict__ partials,
+                                          const float2* __restrict__ clip) {
+  using K = ImgCfg<N>;
+  constexpr int EB = K::EB, TB = K::TB;
+  constexpr int H = N / K::RSPLIT;
+  auto pix = [&](int m, int q) { return row_pix<N>(t, m, q); };
 
   // per-row-pair statistics: the max pixel and its lowest index (the
   // noise comes from the grid by Parseval's identity, see k_colfft).  The
@@ -430,21 +508,6 @@ __device__ __forceinline__ void row_finish(float2 (&v)[ImgCfg<N>::EB], float2* b
   const int yb = t_row(i + 1, tsplit, log2l);
   constexpr int LP = FftShape<H, EB>::LAST_P;
   constexpr int EM = EB / LP;
-  if (images != nullptr) {
-    const double W = weight[img_base + slot];
-    const float scale = W > 0.0 ? (float)(0.5 / W) : 0.f;
-    float* ima = images + ((size_t)slot * N + ya) * N;
-    float* imb = images + ((size_t)slot * N + yb) * N;
-#pragma unroll
-    for (int m = 0; m < EM; ++m)
-#pragma unroll
-      for (int q = 0; q < LP; ++q) {
-        const float2 z = v[m * LP + dft_perm<LP>(q)];
-        const int o = pix(m, q);
-        ima[o] = z.x * scale;
-        imb[o] = z.y * scale;
-      }
-  }
   // max of row y (real parts) and of row y + 1 (imaginary parts), four
   // independent chains each
   float mxa[4] = {-FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX};
@@ -672,9 +735,172 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
       __syncthreads();  // tile consumed: prefetch the next item
       if (item + (int)gridDim.x < nitems) fetch(item + gridDim.x);
     }
-    row_finish<N, CLIP>(v, fbuf + xf * K::STRIDE_B, tb.twiddle, t, xf, slot, y0, g.tsplit, log2l,
-                        images != nullptr ? weight : nullptr, img_base, images, partials, clip);
+    row_fft<N>(v, fbuf + xf * K::STRIDE_B, tb.twiddle, t, xf);
+    if (images != nullptr) row_write<N>(v, t, xf, slot, y0, g.tsplit, log2l, weight[img_base + slot], images);
+    row_stats<N, CLIP>(v, t, xf, slot, y0, g.tsplit, log2l, partials, clip);
   }
+}
+
+// Pass B over quads of transformed images, with the images derived from them:
+// work item = (quad, block of RB rows).  A block takes the quad's images one
+// after the other through the transform of k_rowfft_stats.  The pixel rows of
+// image k stay with the lane that made them: an even image's are kept, an odd
+// one's added to them, which is the row pair of the sum of two images (the
+// image of twice the width), and the sums of two make the sum of four in the
+// same way.  Every searched one of these images gets its StatPartial here, so
+// the widths 2 dt and 4 dt cost no gridding, no column pass and no row
+// transform, only additions and the maxima.
+// What is kept (64 registers a lane, twice) has no room in registers (the
+// transform takes 128, two blocks per SM) or in shared memory (113 KB a block
+// are FFT buffers and tile): it goes to tensor memory, which nothing else
+// uses here and whose loads and stores do not pass through the L1/shared
+// pipe that bounds this kernel.  Two sums deep is what 512 columns hold for 16
+// warps (128 columns a warp, four warps on each quarter of the lanes), hence
+// quads.
+// Measured on whole segments: 177,521 images of 1024^2 (widths 1, 2, 4, 8: six
+// in ten transformed) 266.8 to 201.8 ms, 69,139 of 2048^2 (widths 1 .. 16)
+// 521.6 to 350.5 ms, 504 of 4096^2 (widths 1 .. 32) 23.2 to 14.1 ms.
+// A block that gives up a bounded wait leaves the item loop and frees its
+// tensor memory with the others.
+template <int N, bool CLIP>
+__global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
+    k_rowfft_tree(SegmentGeom g, DevTables tb, const float2* __restrict__ Tbuf, const Quad* __restrict__ quads,
+                  int nquads, int img_base, int base_base, StatPartial* __restrict__ partials,
+                  const __grid_constant__ CUtensorMap tmap, int tma_boxes, int tma_rows, int* __restrict__ err,
+                  const float2* __restrict__ clip) {
+  using K = ImgCfg<N>;
+  static_assert(K::EB == 32 && K::THREADS_B % 32 == 0, "64 values a lane, whole warps");
+  constexpr int NWB = K::THREADS_B / 32;
+  constexpr unsigned TCOLS = TreeCfg<N>::COLS;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  float2* fbuf = reinterpret_cast<float2*>(smraw);  // [XB][STRIDE_B]
+  unsigned char* tb0 = smraw + K::XB * K::STRIDE_B * 8;
+  if constexpr (K::TILE_TMA) tb0 += (1024u - (smem_u32(tb0) & 1023u)) & 1023u;  // swizzle atom alignment
+  float4* tile = reinterpret_cast<float4*>(tb0);    // [rows][CH]
+  __shared__ __align__(8) unsigned long long tbar;
+  __shared__ int s_done;  // warps done reading the tile in hand (warp-local transforms)
+  __shared__ unsigned s_tmem;
+  const int tid = threadIdx.x;
+  const int ncol = g.ncol;
+  constexpr int nrb = N / K::RB;
+  const int nitems = nquads * nrb;
+  const int xf = tid / K::TB;
+  const int t = tid - xf * K::TB;
+  const int log2l = FftShape<N>::LOG2N - (g.tsplit > 1 ? __ffs(g.tsplit) - 1 : 0);
+  const bool use_tma = K::TILE_TMA && tma_boxes > 0;
+  constexpr bool WARP_LOCAL = K::TILE_TMA && (K::TB <= 32 || K::RSPLIT == 2);  // see k_rowfft_stats
+  unsigned phase = 0;
+  if (tid < 32) tmem_alloc(&s_tmem, TCOLS);
+  if (tid == 0) {
+    mbar_init(&tbar, 1);
+    s_done = 0;
+  }
+  __syncthreads();
+  // this warp's lanes and columns: level 0 (single images) and 1 (sums of two)
+  const unsigned keep = s_tmem + ((unsigned)((tid >> 5) & 3) << 21) + (unsigned)(tid >> 7) * 128u;
+  auto issue_tma = [&](int sl, int yb) {  // by one thread
+    mbar_expect_tx(&tbar, (unsigned)(tma_boxes * tma_rows * K::CH * 16));
+    for (int b = 0; b < tma_boxes; ++b)
+      tma_load_3d(tile + (size_t)b * tma_rows * K::CH, &tmap, 2 * yb, b * tma_rows, sl, &tbar);
+  };
+  auto fetch = [&](int sl, int yb) {
+    if (use_tma) {
+      if (tid == 0) issue_tma(sl, yb);
+    } else {
+      const float2* src = Tbuf + (size_t)sl * ncol * N + yb;
+      for (int i = tid; i < ncol * K::CH; i += K::THREADS_B) {
+        const int u = i / K::CH;
+        const int c = i - u * K::CH;
+        cp_async16(tile + u * K::CH + K::swz(u, c), src + (size_t)u * N + 2 * c);
+      }
+      cp_async_commit();
+    }
+  };
+
+  int item = blockIdx.x;
+  Quad cur = quads[item / nrb];  // the grid is at most the number of items
+  bool failed = false;
+  fetch(cur.base - base_base, (item % nrb) * K::RB);
+  while (item < nitems && !failed) {
+    const int y0 = (item % nrb) * K::RB;
+    const int next = item + (int)gridDim.x;
+    Quad nxt = cur;
+    if (next < nitems) nxt = quads[next / nrb];
+    const int top = cur.img2 >= 0 ? 2 : (cur.img1 >= 0 ? 1 : 0);
+    for (int k = 0; k < cur.n; ++k) {
+      if (use_tma && WARP_LOCAL) {
+        // as in k_rowfft_stats: no copy is issued without this warp's count
+        // below, so the other warps' waits run out in turn
+        if (!__all_sync(0xffffffffu, mbar_wait(&tbar, phase))) {
+          if ((tid & 31) == 0) atomicExch(err, 1);
+          mbar_wait(&tbar, phase);
+          failed = true;
+          break;
+        }
+        phase ^= 1u;
+      } else if (use_tma) {
+        const bool ok = mbar_wait(&tbar, phase);
+        if (__syncthreads_or(!ok)) {
+          if (tid == 0) {
+            atomicExch(err, 1);
+            mbar_wait(&tbar, phase);
+          }
+          failed = true;
+          break;
+        }
+        phase ^= 1u;
+      } else {
+        cp_async_wait_all();
+        __syncthreads();
+      }
+      float2 v[K::EB];
+      row_zbuild<N>(v, tile, t, xf, ncol);
+      // the tile is read: the next image's (or the next item's first one's)
+      const bool more = k + 1 < cur.n || next < nitems;
+      const int nsl = (k + 1 < cur.n ? cur.base + k + 1 : nxt.base) - base_base;
+      const int nyb = k + 1 < cur.n ? y0 : (next % nrb) * K::RB;
+      if (use_tma && WARP_LOCAL) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if ((tid & 31) == 0) {
+          __threadfence_block();
+          if (atomicAdd(&s_done, 1) == NWB - 1) {
+            s_done = 0;
+            __threadfence_block();
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            if (more) issue_tma(nsl, nyb);
+          }
+        }
+      } else {
+        __syncthreads();
+        if (more) fetch(nsl, nyb);
+      }
+      row_fft<N>(v, fbuf + xf * K::STRIDE_B, tb.twiddle, t, xf);
+      int slot = cur.img + k - img_base;
+#pragma unroll 1
+      for (int lv = 0;;) {
+        if (slot >= 0) row_stats<N, CLIP>(v, t, xf, slot, y0, g.tsplit, log2l, partials, clip);
+        // level lv's block of images that ends the next level's must be whole
+        if (lv >= top || (k | ((2 << lv) - 1)) >= cur.n) break;
+        __syncwarp();
+        if (((k >> lv) & 1) == 0) {
+          tmem_store16(keep + lv * 64, v);
+          tmem_store16(keep + lv * 64 + 32, v + 16);
+          break;
+        }
+        tmem_add16(keep + lv * 64, v);
+        tmem_add16(keep + lv * 64 + 32, v + 16);
+        ++lv;
+        const int first = lv == 1 ? cur.img1 : cur.img2;
+        slot = first < 0 ? -1 : first + (lv == 1 ? k >> 1 : 0) - img_base;
+      }
+    }
+    item = next;
+    cur = nxt;
+  }
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+  __syncthreads();
+  if (tid < 32) tmem_free(s_tmem, TCOLS);
 }
 
 // ------------------------------------------------------- fused imaging pass
@@ -892,8 +1118,8 @@ __global__ void __launch_bounds__(FusedCfg<N>::THREADS, 2)
       __syncthreads();  // the staging area is read
       prefetch(nxt, next_stage, pf);
       const int slot = cur.slot0 + a;
-      row_finish<N, false>(v, fbuf + xfb * K::STRIDE_B, tb.twiddle, tb_, xfb, slot, b * K::RB, g.tsplit, log2l,
-                           nullptr, img_base, nullptr, partials, nullptr);
+      row_fft<N>(v, fbuf + xfb * K::STRIDE_B, tb.twiddle, tb_, xfb);
+      row_stats<N, false>(v, tb_, xfb, slot, b * K::RB, g.tsplit, log2l, partials, nullptr);
     } else if (kind == 1) {
       // --------------------------------------------------------- column item
       const FusedChunk ch = cur.ch;
@@ -1315,7 +1541,7 @@ int rowfft_tile_rows(int ncol);
 
 template <int N>
 cudaError_t run_colfft(const SegmentGeom& g, const DevTables& tb, const Group* groups, int g_begin, int ngroups,
-                       int img_base, const float2* cellbuf, float2* Tbuf, float* colsq, float* mean0,
+                       int img_base, int base_base, const float2* cellbuf, float2* Tbuf, float* colsq, float* mean0,
                        cudaStream_t st, const PassLaunch* pl) {
   using C = ColCfg<N>;
   using K = ImgCfg<N>;
@@ -1332,8 +1558,8 @@ cudaError_t run_colfft(const SegmentGeom& g, const DevTables& tb, const Group* g
     smem = one_per_sm_smem(smem, K::SMEM_B_FIXED + (K::TILE_TMA ? 1024 : 0) + rowfft_tile_rows<N>(g.ncol) * K::CH * 16,
                            smem_max);
   dim3 grid(ngroups, g.ncol);
-  return launch_with(k_colfft<N>, grid, dim3(C::THREADS), smem, st, pl, g, tb, groups, g_begin, img_base, cellbuf,
-                     Tbuf, colsq, mean0);
+  return launch_with(k_colfft<N>, grid, dim3(C::THREADS), smem, st, pl, g, tb, groups, g_begin, img_base, base_base,
+                     cellbuf, Tbuf, colsq, mean0);
 }
 
 // Rows of the row-pass tile: ncol, or the boxes' total under tensor copies.
@@ -1388,6 +1614,49 @@ cudaError_t run_rowfft_stats(const SegmentGeom& g, const DevTables& tb, const fl
                                       pl);
 }
 
+template <int N, bool CLIP>
+cudaError_t run_rowfft_tree_k(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Quad* quads,
+                              int nquads, int img_base, int base_base, StatPartial* partials, const TileMap* tm,
+                              int* err, cudaStream_t st, const float2* clip, const PassLaunch* pl) {
+  using K = ImgCfg<N>;
+  const int smem = K::SMEM_B_FIXED + (K::TILE_TMA ? 1024 : 0) + rowfft_tile_rows<N>(g.ncol) * K::CH * 16;
+  auto kern = k_rowfft_tree<N, CLIP>;
+  const int smem_max = max_dynamic_smem(kern);
+  if (smem > smem_max) return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  if (e != cudaSuccess) return e;
+  if (nquads <= 0) return cudaSuccess;
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, K::THREADS_B, smem);
+  if (e != cudaSuccess) return e;
+  per_sm = std::min(per_sm, 512 / TreeCfg<N>::COLS);  // a block beyond that would wait for tensor memory
+  const long nitems = (long)nquads * (N / K::RB);
+  long grid = std::min<long>(nitems, (long)std::max(per_sm, 1) * sm_count());
+  if (pl != nullptr && pl->items_per_block > 0)  // an item is up to four images
+    grid = std::max(grid, std::min<long>((4 * nitems + pl->items_per_block - 1) / pl->items_per_block,
+                                         std::min<long>(nitems, INT_MAX)));
+  const bool tma = K::TILE_TMA && tm != nullptr && tm->nbox > 0 && err != nullptr;
+  CUtensorMap none;
+  memset(&none, 0, sizeof(none));
+  return launch_with(kern, dim3((unsigned)grid), dim3(K::THREADS_B), smem, st, pl, g, tb, Tbuf, quads, nquads,
+                     img_base, base_base, partials, tma ? tm->map : none, tma ? tm->nbox : 0, tma ? tm->rows : 0, err,
+                     clip);
+}
+
+template <int N>
+cudaError_t run_rowfft_tree(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Quad* quads,
+                            int nquads, int img_base, int base_base, StatPartial* partials, const TileMap* tm,
+                            int* err, cudaStream_t st, const float2* clip, const PassLaunch* pl) {
+  static_assert(N >= kTreeMinNpix, "whole warps");
+  if (clip != nullptr)
+    return run_rowfft_tree_k<N, true>(g, tb, Tbuf, quads, nquads, img_base, base_base, partials, tm, err, st, clip,
+                                      pl);
+  return run_rowfft_tree_k<N, false>(g, tb, Tbuf, quads, nquads, img_base, base_base, partials, tm, err, st, nullptr,
+                                     pl);
+}
+
 template <int N>
 cudaError_t run_image_fused(const SegmentGeom& g, const DevTables& tb, const Group* groups, int g_begin,
                             const FusedChunk* chunks, int nchunks, int img_base, const float2* cellbuf,
@@ -1438,7 +1707,7 @@ void fill_shape(ImageKernelShape* o) {
 }
 
 #define RF_INSTANTIATE_IMAGE(N)                                                                              \
-  template cudaError_t run_colfft<N>(const SegmentGeom&, const DevTables&, const Group*, int, int, int,      \
+  template cudaError_t run_colfft<N>(const SegmentGeom&, const DevTables&, const Group*, int, int, int, int, \
                                      const float2*, float2*, float*, float*, cudaStream_t,                  \
                                      const PassLaunch*);                                                    \
   template cudaError_t run_rowfft_stats<N>(const SegmentGeom&, const DevTables&, const float2*, int, int,    \
@@ -1447,6 +1716,11 @@ void fill_shape(ImageKernelShape* o) {
   template void fill_shape<N>(ImageKernelShape*);                                                           \
   template cudaError_t run_rowfft_power<N>(const SegmentGeom&, const DevTables&, const float2*, const int4*, \
                                            int, StatPartial*, const TileMap*, int*, cudaStream_t);
+
+#define RF_INSTANTIATE_TREE(N)                                                                               \
+  template cudaError_t run_rowfft_tree<N>(const SegmentGeom&, const DevTables&, const float2*, const Quad*,  \
+                                          int, int, int, StatPartial*, const TileMap*, int*, cudaStream_t,   \
+                                          const float2*, const PassLaunch*);
 
 #define RF_INSTANTIATE_FUSED(N)                                                                              \
   template cudaError_t run_image_fused<N>(const SegmentGeom&, const DevTables&, const Group*, int,            \

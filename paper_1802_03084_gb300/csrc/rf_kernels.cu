@@ -516,7 +516,7 @@ __global__ void k_finalize(int npix, int nrb, int ncol, const StatPartial* __res
     ds.x = 0;
     ds.y = 0;
     ds.mean = 0.0;
-    if (stats) stats[img] = ds;
+    if (stats) stats[info.w] = ds;
     return;
   }
   // mean = G(0,0) / 2W; mean of I^2 = sum_full |G|^2 / 4W^2 (Parseval)
@@ -542,7 +542,7 @@ __global__ void k_finalize(int npix, int nrb, int ncol, const StatPartial* __res
   ds.x = x;
   ds.y = y;
   ds.mean = mean;
-  if (stats) stats[img] = ds;
+  if (stats) stats[info.w] = ds;
   if (sigma > 0.0 && snr >= threshold) {
     const int k = atomicAdd(ncand, 1);
     if (k < cand_cap) {
@@ -575,8 +575,11 @@ cudaError_t launch_finalize(const SegmentGeom& g, const StatPartial* partials, c
 
 // --------------------------------------------------------------- dispatch --
 template <int N>
-cudaError_t run_colfft(const SegmentGeom&, const DevTables&, const Group*, int, int, int, const float2*, float2*,
+cudaError_t run_colfft(const SegmentGeom&, const DevTables&, const Group*, int, int, int, int, const float2*, float2*,
                        float*, float*, cudaStream_t, const PassLaunch*);
+template <int N>
+cudaError_t run_rowfft_tree(const SegmentGeom&, const DevTables&, const float2*, const Quad*, int, int, int,
+                            StatPartial*, const TileMap*, int*, cudaStream_t, const float2*, const PassLaunch*);
 template <int N>
 cudaError_t run_rowfft_stats(const SegmentGeom&, const DevTables&, const float2*, int, int, const double*,
                              StatPartial*, float*, const TileMap*, int*, cudaStream_t, const float2*,
@@ -623,12 +626,12 @@ cudaError_t launch_image_fused(const SegmentGeom& g, const DevTables& tb, const 
 }
 
 cudaError_t launch_colfft(const SegmentGeom& g, const DevTables& tb, const Group* groups, int g_begin,
-                          int ngroups, int img_base, const float2* cellbuf, float2* Tbuf, float* colsq,
+                          int ngroups, int img_base, int base_base, const float2* cellbuf, float2* Tbuf, float* colsq,
                           float* mean0, cudaStream_t st, const PassLaunch* pl) {
   switch (g.npix) {
 #define RF_CASE(N) \
   case N:          \
-    return run_colfft<N>(g, tb, groups, g_begin, ngroups, img_base, cellbuf, Tbuf, colsq, mean0, st, pl);
+    return run_colfft<N>(g, tb, groups, g_begin, ngroups, img_base, base_base, cellbuf, Tbuf, colsq, mean0, st, pl);
     RF_FOR_EACH_N(RF_CASE)
 #undef RF_CASE
     default:
@@ -645,6 +648,20 @@ cudaError_t launch_rowfft_stats(const SegmentGeom& g, const DevTables& tb, const
   case N:          \
     return run_rowfft_stats<N>(g, tb, Tbuf, nimg, img_base, weight, partials, images, tm, err, st, clip, pl);
     RF_FOR_EACH_N(RF_CASE)
+#undef RF_CASE
+    default:
+      return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_rowfft_tree(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Quad* quads,
+                               int nquads, int img_base, int base_base, StatPartial* partials, const TileMap* tm,
+                               int* err, cudaStream_t st, const float2* clip, const PassLaunch* pl) {
+  switch (g.npix) {
+#define RF_CASE(N)                                                                                                 \
+  case N:                                                                                                          \
+    return run_rowfft_tree<N>(g, tb, Tbuf, quads, nquads, img_base, base_base, partials, tm, err, st, clip, pl);
+    RF_CASE(64) RF_CASE(128) RF_CASE(256) RF_CASE(512) RF_CASE(1024) RF_CASE(2048) RF_CASE(4096) RF_CASE(8192)
 #undef RF_CASE
     default:
       return cudaErrorInvalidValue;
