@@ -758,8 +758,9 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
 // warps (128 columns a warp, four warps on each quarter of the lanes), hence
 // quads.
 // Measured on whole segments: 177,521 images of 1024^2 (widths 1, 2, 4, 8: six
-// in ten transformed) 266.8 to 201.8 ms, 69,139 of 2048^2 (widths 1 .. 16)
-// 521.6 to 350.5 ms, 504 of 4096^2 (widths 1 .. 32) 23.2 to 14.1 ms.
+// in ten transformed) 266.8 to 171.5 ms, 69,139 of 2048^2 (widths 1 .. 16)
+// 521.6 to 308.9 ms, 504 of 4096^2 (widths 1 .. 32) 23.2 to 14.1 ms.  Of the
+// 1024^2 row passes' 91 ms, keeping and adding take 3 and the sums' maxima 9.
 // A block that gives up a bounded wait leaves the item loop and frees its
 // tensor memory with the others.
 template <int N, bool CLIP>
@@ -1215,6 +1216,27 @@ int max_dynamic_smem(Kernel kern) {
   return optin - (int)fa.sharedSizeBytes;
 }
 
+// Blocks of `kern` an SM holds at once, for a kernel that allocates `cols`
+// columns of tensor memory: the occupancy query answers 1 for any kernel with
+// an allocation, whatever its size, but blocks whose columns fit together do
+// run together (one block per SM made the 1024^2 row pass 1.5 times slower).
+// Registers are given to warps in units of 256.
+template <class Kernel>
+cudaError_t tmem_blocks_per_sm(int* out, Kernel kern, int threads, int smem, int cols) {
+  cudaFuncAttributes fa;
+  int dev = 0, regs = 0, sm_smem = 0, reserved = 0;
+  cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&regs, cudaDevAttrMaxRegistersPerMultiprocessor, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+  if (e != cudaSuccess) return e;
+  const int by_regs = regs / std::max((threads + 31) / 32 * ((fa.numRegs * 32 + 255) / 256 * 256), 1);
+  const int by_smem = sm_smem / std::max(smem + (int)fa.sharedSizeBytes + reserved, 1);
+  *out = std::max(1, std::min(std::min(by_regs, by_smem), 512 / cols));
+  return cudaSuccess;
+}
+
 // Launch `kern`, with the scheduling priority of `pl` where it sets one (a
 // launch attribute, so that a captured graph keeps it on the kernel node).
 template <class... P, class... A>
@@ -1629,9 +1651,8 @@ cudaError_t run_rowfft_tree_k(const SegmentGeom& g, const DevTables& tb, const f
   if (e != cudaSuccess) return e;
   if (nquads <= 0) return cudaSuccess;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, K::THREADS_B, smem);
+  e = tmem_blocks_per_sm(&per_sm, kern, K::THREADS_B, smem, TreeCfg<N>::COLS);
   if (e != cudaSuccess) return e;
-  per_sm = std::min(per_sm, 512 / TreeCfg<N>::COLS);  // a block beyond that would wait for tensor memory
   const long nitems = (long)nquads * (N / K::RB);
   long grid = std::min<long>(nitems, (long)std::max(per_sm, 1) * sm_count());
   if (pl != nullptr && pl->items_per_block > 0)  // an item is up to four images
