@@ -317,7 +317,7 @@ def load_traffic(kernel, images_per_launch):
 
 
 KERNEL_SOURCES = ("rf_async.cuh", "rf_fft.cuh", "rf_image.cuh", "rf_image_small.cu", "rf_image_large.cu",
-                  "rf_image_fused.cu", "rf_kernels.cu")
+                  "rf_image_tree.cu", "rf_kernels.cu")
 
 
 def source_hash():

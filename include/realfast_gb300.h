@@ -272,21 +272,13 @@ rf_status rf_plan_set_form(struct rf_plan* plan, int32_t form);
  *                      the same images; the knob lets a test run the 64-bit
  *                      variant on a small plan. */
 #define RF_TUNE_WIDE_INDEX 3
-/* RF_TUNE_FUSED        1: for npix 1024 .. 4096 the search runs
- *                      each wave's column and row FFTs as one persistent
- *                      launch whose column-FFT output passes through a small
- *                      ring of chunk slots (RF_TUNE_RING of them, each one
- *                      round of column transforms: 8 images at 1024^2, 4 at
- *                      2048^2, 2 at 4096^2) that stays in L2; 0 (default):
- *                      separate column and row launches through a wave-sized
- *                      buffer (always so for other sizes, with
- *                      RF_NOISE_CLIPPED, for rendered images and for plans
- *                      with a width twice or four times another, whose
- *                      images the row pass sums).  The autotuner times both
- *                      where both exist. */
+/* RF_TUNE_FUSED        0 (default) or 1, kept and reported.  It once chose one
+ *                      persistent launch for a wave's column and row FFTs,
+ *                      1.3 to 1.5 times slower than the separate passes on
+ *                      every workload; the separate passes always run. */
 #define RF_TUNE_FUSED 4
-/* RF_TUNE_RING         chunk slots of the fused pass's ring, 2 .. 8
- *                      (default 3). */
+/* RF_TUNE_RING         2 .. 8 (default 3), kept and reported: the depth of
+ *                      that launch's buffer, without effect. */
 #define RF_TUNE_RING 5
 /* RF_TUNE_OVERLAP      1: waves hold at most half of RF_TUNE_WAVE_IMAGES
  *                      images and alternate between the two halves of the
@@ -307,8 +299,7 @@ rf_status rf_plan_get_tuning(const struct rf_plan* plan, int32_t key, int64_t* v
 /*
  * rf_plan_autotune: pick the tuning that searches `vis` fastest and apply
  * it.  Candidates: for npix 1024 .. 4096 without clipped noise,
- * RF_TUNE_FUSED on with RF_TUNE_RING 2, 3 and 4 (where the plan has a fused
- * pass, see RF_TUNE_FUSED), and off with RF_TUNE_OVERLAP off and on, at waves of 2048 and 8192 images, graphs on;
+ * RF_TUNE_OVERLAP off and on, at waves of 2048 and 8192 images, graphs on;
  * elsewhere a ladder of wave sizes (256 .. 8192 images) with RF_TUNE_GRAPHS
  * on and off, and from 2048 images RF_TUNE_OVERLAP on.  Before either, waves
  * of one, two and four image groups (below 256 images) whose column-FFT
@@ -619,8 +610,7 @@ rf_status rf_stream_destroy(struct rf_stream* s);
 /* Check of the bounded device-side waits (no counterpart in the paper): one
  * block waits, at most `polls` polls (1 .. 2^20) each, on an mbarrier that
  * nothing arrives at, as the row pass waits for its tile copies, and on a
- * global count that nothing raises, as the fused imaging pass waits for
- * work items of other blocks.  Both waits must give up and report it
+ * global count that nothing raises.  Both waits must give up and report it
  * instead of hanging: *gave_up = 1.  The device stays usable afterwards.
  * Errors: RF_ERR_INVALID_ARG, RF_ERR_NO_DEVICE, RF_ERR_CUDA. */
 rf_status rf_selftest_bounded_wait(int32_t device, int32_t polls, int32_t* gave_up);

@@ -653,11 +653,11 @@ class Plan:
         rf_plan_set_tuning(self.handle, RF_TUNE_WIDE_INDEX, 1 if enable else 0)
 
     def set_fused(self, enable: bool):
-        """The fused column + row pass (npix 1024 .. 4096) on or off."""
+        """Kept and reported, without effect (see RF_TUNE_FUSED)."""
         rf_plan_set_tuning(self.handle, RF_TUNE_FUSED, 1 if enable else 0)
 
     def set_ring(self, slots: int):
-        """Chunk slots of the fused pass's L2-resident ring (2 .. 8)."""
+        """Kept and reported, without effect (2 .. 8)."""
         rf_plan_set_tuning(self.handle, RF_TUNE_RING, slots)
 
     def set_overlap(self, enable: bool):

@@ -55,7 +55,7 @@ constexpr size_t kTBudgetBytes = 4096ull << 20;  // column-FFT scratch per wave
 constexpr int kRangeEntries = 64;                // target entries per gridding warp
 constexpr size_t kPeriodicBudgetBytes = 1ull << 30;  // transformed series per DM batch
 constexpr size_t kPlainBudgetBytes = 4096ull << 20;  // plain form: intermediates of one chunk
-constexpr int kDefaultRing = 3;                      // fused pass: chunk slots of the ring
+constexpr int kDefaultRing = 3;                      // RF_TUNE_RING
 constexpr int kOverlapRowItems = 16;                 // overlapped waves: work items per row-pass block
 
 // Round half away from zero: sign(x) floor(|x| + 1/2).
@@ -273,19 +273,9 @@ struct rf_plan {
   float2* d_clip = nullptr;     // [slots] clipping window (RF_NOISE_CLIPPED only)
   rf::PlainBuffers plain{};     // allocated on the first plain-form search
 
-  // fused column + row pass (npix 1024 .. 4096): chunks of the image list,
-  // the chunks of each wave, and the L2-resident ring of column-FFT output
-  bool fused = false;           // RF_TUNE_FUSED (the autotuner turns it on where it wins)
-  int ring = kDefaultRing;      // RF_TUNE_RING
-  int chunk_images = 0;         // images per chunk (0: no fused pass at this size)
-  std::vector<rf::FusedChunk> chunks;
-  std::vector<int2> wave_chunks;  // per wave: [first, last) chunk
-  rf::FusedChunk* d_chunks = nullptr;
-  int* d_fcount = nullptr;      // 1 + 2 x (most chunks of a wave) counters
-  int fcount_cap = 0;
-  float2* d_Tring = nullptr;
-  int ring_alloc = 0;
-  rf::TileMap tmap_ring{};
+  // RF_TUNE_FUSED and RF_TUNE_RING: kept and reported, without effect
+  bool fused = false;
+  int ring = kDefaultRing;
 
   // overlapped waves (RF_TUNE_OVERLAP): waves of at most half the slots
   // alternate between the halves of the scratch; wave w + 1's gridding and
@@ -688,10 +678,10 @@ int default_slots(const rf_plan* p, size_t img_cap) {
 }
 
 // Whether waves can be overlapped: asked for, two halves of the scratch hold
-// a group each, and neither the fused pass nor the clipped noise (whose
-// window buffer is per slot of the whole scratch) is in use.
+// a group each, and the clipped noise (whose window buffer is per slot of the
+// whole scratch) is not in use.
 bool overlap_possible(const rf_plan* p) {
-  return p->overlap && !(p->fused && !p->derived) && !(p->flags & RF_NOISE_CLIPPED) &&
+  return p->overlap && !(p->flags & RF_NOISE_CLIPPED) &&
          p->tslots / 2 >= p->shape.images_per_group && p->sslots / 2 >= group_images(p);
 }
 
@@ -778,27 +768,10 @@ void build_lists(rf_plan* p, int nint) {
   w.base_end = nbase;
   w.quad_end = (int)p->quads.size();
   if (w.img_end > w.img_begin) p->waves.push_back(w);
-  // chunks of the fused pass: each group's images in runs of chunk_images
-  p->chunks.clear();
-  p->wave_chunks.clear();
-  if (p->chunk_images > 0 && !p->derived) {
-    for (const Wave& wv : p->waves) {
-      const int c0 = (int)p->chunks.size();
-      for (int gi = wv.g_begin; gi < wv.g_end; ++gi)
-        for (int k = 0; k < p->groups[gi].nimg; k += p->chunk_images)
-          p->chunks.push_back({gi, k, std::min(p->chunk_images, p->groups[gi].nimg - k), 0});
-      p->wave_chunks.push_back(make_int2(c0, (int)p->chunks.size()));
-    }
-  }
   p->cached_nint = nint;
   p->cached_span = p->t_span;
   p->cached_plain = plain;
   p->drop_graph();
-}
-
-// Whether the search's waves take the fused column + row pass.
-bool use_fused(const rf_plan* p) {
-  return p->fused && !p->derived && p->chunk_images > 0 && p->tmap_ring.nbox > 0 && !(p->flags & RF_NOISE_CLIPPED);
 }
 
 // cuTensorMapEncodeTiled from the driver, looked up once.
@@ -911,36 +884,6 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
   // the periodicity row pass's tensor-copy tiles (one image's XB rows), at
   // N = 1024, where its transforms fit one warp
   if (p->npix == 1024) encode_tile_map(p, p->tmap_P, p->d_T, p->tslots, xb);
-  // fused pass: counters for the most chunks a wave can hold
-  if (p->chunk_images > 0) {
-    const int cap = 1 + 2 * p->gslots_max * ((p->shape.images_per_group + p->chunk_images - 1) / p->chunk_images);
-    if (p->d_fcount) {
-      p->device_bytes -= (uint64_t)p->fcount_cap * sizeof(int);
-      p->dfree(p->d_fcount);
-      p->d_fcount = nullptr;
-    }
-    if ((s = p->dalloc(&p->d_fcount, (size_t)cap)) != RF_OK) return s;
-    p->fcount_cap = cap;
-  }
-  return RF_OK;
-}
-
-// (Re)allocate the fused pass's ring of `ring` chunk slots and its tensor map.
-rf_status alloc_ring(rf_plan* p, int ring) {
-  if (p->chunk_images <= 0) return RF_OK;
-  const size_t per_ring = (size_t)p->chunk_images * p->ncol * p->npix;
-  p->tmap_ring.nbox = 0;
-  p->drop_graph();
-  if (p->d_Tring) {
-    p->device_bytes -= (uint64_t)p->ring_alloc * per_ring * sizeof(float2);
-    p->dfree(p->d_Tring);
-    p->d_Tring = nullptr;
-  }
-  rf_status s = p->dalloc(&p->d_Tring, (size_t)ring * per_ring);
-  if (s != RF_OK) return s;
-  p->ring = p->ring_alloc = ring;
-  encode_tile_map(p, p->tmap_ring, p->d_Tring, ring * p->chunk_images,
-                  2 * std::min(256 / (p->npix / 32), p->npix / 2));
   return RF_OK;
 }
 
@@ -978,11 +921,6 @@ uint64_t estimate_device_bytes(const rf_plan* p, int slots) {
        r((size_t)gslots * std::max(p->n_cells, 1) * 32, sizeof(float2)) + r((size_t)sslots * p->ncol, 4) +
        r(sslots, 4);
   if (p->flags & RF_NOISE_CLIPPED) b += r(sslots, sizeof(float2));
-  const int ci = rf::fused_chunk_images((int)N);
-  if (ci > 0) {
-    b += r(img_cap, sizeof(rf::FusedChunk)) + r(1 + 2 * gslots * ((B + ci - 1) / ci), 4);
-    b += r((size_t)kDefaultRing * ci * per_slot, 1);
-  }
   const size_t per_int = rows * p->npol * sizeof(float2);
   const size_t stage_nint = std::max<size_t>(1, std::min<size_t>(kStageBytes / per_int, (size_t)p->max_nint));
   b += r(stage_nint * per_int, 1);
@@ -1093,11 +1031,8 @@ rf_status alloc_device(rf_plan* p) {
   RF_CUDA(cudaMemset(p->d_err, 0, sizeof(int)));
 
   // column-FFT scratch, whole groups per wave
-  p->chunk_images = rf::fused_chunk_images(N);
-  if (p->chunk_images > 0 && (s = p->dalloc(&p->d_chunks, (size_t)p->img_cap)) != RF_OK) return s;
   if (p->derived && (s = p->dalloc(&p->d_quads, (size_t)p->img_cap)) != RF_OK) return s;
   if ((s = alloc_wave_scratch(p, default_slots(p, (size_t)p->img_cap))) != RF_OK) return s;
-  if ((s = alloc_ring(p, kDefaultRing)) != RF_OK) return s;
 
   // host->device staging of raw visibilities
   const size_t per_int = (size_t)p->nbl * p->nchan * p->npol * sizeof(float2);
@@ -1295,8 +1230,7 @@ rf_status run_waves(rf_plan* p, int nint, const std::vector<Wave>& waves, int ni
   RF_TIMED(p->prof, K_WEIGHTS, st,
            rf::launch_weights(p->d_img_info, nimg_total, (p->flags & RF_EDGE_PARTIAL) != 0, g, p->tb,
                               (double)p->n_on, p->d_weight, st));
-  const bool fused = d_images == nullptr && &waves == &p->waves && use_fused(p);
-  if (!fused && d_images == nullptr && &waves == &p->waves && p->waves_overlap && overlap_possible(p))
+  if (d_images == nullptr && &waves == &p->waves && p->waves_overlap && overlap_possible(p))
     return run_waves_overlapped(p, g, waves, d_stats, st);
   for (size_t wi = 0; wi < waves.size(); ++wi) {
     const Wave& w = waves[wi];
@@ -1304,18 +1238,6 @@ rf_status run_waves(rf_plan* p, int nint, const std::vector<Wave>& waves, int ni
     const int ni = w.img_end - w.img_begin;
     RF_TIMED(p->prof, K_GRID_CELLS, st,
              rf::launch_grid_cells(g, p->tb, p->d_groups, w.g_begin, ng, p->d_cellbuf, st));
-    if (fused) {
-      const int2 wc = p->wave_chunks[wi];
-      RF_TIMED(p->prof, K_IMAGE_FUSED, st,
-               rf::launch_image_fused(g, p->tb, p->d_groups, w.g_begin, p->d_chunks + wc.x, wc.y - wc.x,
-                                      w.img_begin, p->d_cellbuf, p->d_Tring, p->ring, p->tmap_ring, p->d_colsq,
-                                      p->d_mean0, p->d_partials, p->d_fcount, p->d_err, st));
-      RF_TIMED(p->prof, K_FINALIZE, st,
-               rf::launch_finalize(g, p->d_partials, p->d_colsq, p->d_mean0, p->d_img_info, p->d_weight, ni,
-                                   w.img_begin, p->threshold, p->d_cands, p->d_ncand, p->img_cap, d_stats, st,
-                                   false));
-      continue;
-    }
     RF_TIMED(p->prof, K_GRID_COLFFT, st,
              rf::launch_colfft(g, p->tb, p->d_groups, w.g_begin, ng, w.img_begin, w.base_begin, p->d_cellbuf,
                                p->d_T, p->d_colsq, p->d_mean0, st));
@@ -1472,9 +1394,6 @@ rf_status search_impl(rf_plan* p, const void* vis, int nint, void* stream, rf_ca
       if (!p->quads.empty())
         RF_CUDA(cudaMemcpyAsync(p->d_quads, p->quads.data(), p->quads.size() * sizeof(rf::Quad),
                                 cudaMemcpyHostToDevice, st));
-      if (!p->chunks.empty())
-        RF_CUDA(cudaMemcpyAsync(p->d_chunks, p->chunks.data(), p->chunks.size() * sizeof(rf::FusedChunk),
-                                cudaMemcpyHostToDevice, st));
     }
   }
   const int nimg = (int)p->img_info.size();
@@ -1502,7 +1421,7 @@ rf_status search_impl(rf_plan* p, const void* vis, int nint, void* stream, rf_ca
   RF_CUDA(cudaStreamSynchronize(st));
   if (kerr) {
     cudaMemset(p->d_err, 0, sizeof(int));
-    return fail(RF_ERR_TIMEOUT, "a bounded device-side wait (a tile copy, or a fused-pass dependency) gave up");
+    return fail(RF_ERR_TIMEOUT, "a bounded device-side wait for a tile copy gave up");
   }
   ncand = std::min(ncand, p->img_cap);
   std::vector<DevCand> dc(ncand);
@@ -2176,8 +2095,6 @@ rf_status rf_plan_set_tuning(rf_plan* p, int32_t key, int64_t value) {
     if (!bg.owned) return fail(RF_ERR_BUSY, "plan is in use by another call");
     DeviceGuard dg(p->device);
     p->fused = value != 0;
-    p->cached_nint = -1;  // overlapped waves (half size) are built only without the fused pass
-    p->drop_graph();
     return RF_OK;
   }
   if (key == RF_TUNE_OVERLAP) {
@@ -2196,11 +2113,8 @@ rf_status rf_plan_set_tuning(rf_plan* p, int32_t key, int64_t value) {
     BusyGuard bg(&p->busy);
     if (!bg.owned) return fail(RF_ERR_BUSY, "plan is in use by another call");
     DeviceGuard dg(p->device);
-    if (p->chunk_images <= 0) {
-      p->ring = (int)value;
-      return RF_OK;
-    }
-    return alloc_ring(p, (int)value);
+    p->ring = (int)value;
+    return RF_OK;
   }
   if (key != RF_TUNE_WAVE_IMAGES) return fail(RF_ERR_INVALID_ARG, "unknown tuning key %d", key);
   if (p->host_only) return fail(RF_ERR_INVALID_ARG, "plan was created with RF_HOST_ONLY");
@@ -2227,14 +2141,13 @@ rf_status rf_plan_autotune(rf_plan* p, const void* vis, int32_t nint, void* stre
   RF_CUDA(cudaMemGetInfo(&free_b, &total_b));
   const size_t have = free_b / 2 + (size_t)p->tslots * per_slot;  // the current scratch is reusable
   struct Cand {
-    int wave, graphs, fused, ring, overlap;
+    int wave, graphs, overlap;
   };
   std::vector<Cand> cands;
   auto fits = [&](int w) { return (size_t)wave_tslots(p, std::max(w, B)) * per_slot <= have; };
-  // where widths are sums of others the fused pass does not apply, but its
-  // sizes keep their two wave sizes
-  const bool big = p->chunk_images > 0 && !(p->flags & RF_NOISE_CLIPPED);
-  const bool can_fuse = big && !p->derived;
+  // from 1024^2 up a wave has work for every SM at two sizes; smaller images
+  // take a ladder
+  const bool big = p->npix >= 1024 && p->npix <= 4096 && !(p->flags & RF_NOISE_CLIPPED);
   // waves whose column-FFT output fits the L2 cache (one to four groups), so
   // that the row pass may find it there instead of in HBM
   int l2 = 0;
@@ -2243,14 +2156,12 @@ rf_status rf_plan_autotune(rf_plan* p, const void* vis, int32_t nint, void* stre
     l2 = 0;
   }
   for (int w = B; w <= 4 * B && w < 256; w *= 2)
-    if ((size_t)wave_tslots(p, w) * per_slot <= (size_t)l2 && fits(w) && w < nimg) cands.push_back({w, 1, 0, p->ring, 0});
+    if ((size_t)wave_tslots(p, w) * per_slot <= (size_t)l2 && fits(w) && w < nimg) cands.push_back({w, 1, 0});
   if (big) {
     for (int w : {2048, 8192}) {
       if (!fits(w)) continue;
-      if (can_fuse)
-        for (int ring : {2, 3, 4}) cands.push_back({w, 1, 1, ring, 0});
-      cands.push_back({w, 1, 0, p->ring, 0});
-      if (w / 2 >= B) cands.push_back({w, 1, 0, p->ring, 1});
+      cands.push_back({w, 1, 0});
+      if (w / 2 >= B) cands.push_back({w, 1, 1});
       if (w >= nimg) break;
     }
   } else {
@@ -2258,13 +2169,13 @@ rf_status rf_plan_autotune(rf_plan* p, const void* vis, int32_t nint, void* stre
       const int wc = std::max(w, B);
       if (!fits(wc)) continue;
       if (!cands.empty() && cands.back().wave >= nimg) break;
-      cands.push_back({wc, 1, 0, p->ring, 0});
-      cands.push_back({wc, 0, 0, p->ring, 0});
-      if (wc >= 2048 && wc / 2 >= B && !(p->flags & RF_NOISE_CLIPPED)) cands.push_back({wc, 1, 0, p->ring, 1});
+      cands.push_back({wc, 1, 0});
+      cands.push_back({wc, 0, 0});
+      if (wc >= 2048 && wc / 2 >= B && !(p->flags & RF_NOISE_CLIPPED)) cands.push_back({wc, 1, 1});
     }
   }
   if (cands.empty())
-    cands.push_back({p->slots_max, p->use_graphs ? 1 : 0, p->fused ? 1 : 0, p->ring, p->overlap ? 1 : 0});
+    cands.push_back({p->slots_max, p->use_graphs ? 1 : 0, p->overlap ? 1 : 0});
 
   // timing search: every (DM, dt) limited to its first nint/4 integrations
   const int span = nint >= 256 ? nint / 4 : 0;
@@ -2286,9 +2197,7 @@ rf_status rf_plan_autotune(rf_plan* p, const void* vis, int32_t nint, void* stre
         break;
       }
       if (p->slots_max != c.wave) s = alloc_wave_scratch(p, c.wave);
-      if (s == RF_OK && c.fused && p->ring != c.ring) s = alloc_ring(p, c.ring);
       p->use_graphs = c.graphs != 0;
-      p->fused = c.fused != 0;
       p->overlap = c.overlap != 0;
       p->cached_nint = -1;
       p->drop_graph();
@@ -2314,8 +2223,8 @@ rf_status rf_plan_autotune(rf_plan* p, const void* vis, int32_t nint, void* stre
     if (ntried < 16 && report) {
       report->tried_wave_images[ntried] = c.wave;
       report->tried_graphs[ntried] = c.graphs;
-      report->tried_fused[ntried] = c.fused;
-      report->tried_ring[ntried] = c.ring;
+      report->tried_fused[ntried] = 0;
+      report->tried_ring[ntried] = p->ring;
       report->tried_overlap[ntried] = c.overlap;
       report->tried_ms[ntried] = ms;
     }
@@ -2332,9 +2241,7 @@ rf_status rf_plan_autotune(rf_plan* p, const void* vis, int32_t nint, void* stre
   {
     BusyGuard bg(&p->busy);
     if (p->slots_max != best.wave && (s = alloc_wave_scratch(p, best.wave)) != RF_OK) return s;
-    if (best.fused && p->ring != best.ring && (s = alloc_ring(p, best.ring)) != RF_OK) return s;
     p->use_graphs = best.graphs != 0;
-    p->fused = best.fused != 0;
     p->overlap = best.overlap != 0;
     p->cached_nint = -1;
     p->drop_graph();
@@ -2342,7 +2249,7 @@ rf_status rf_plan_autotune(rf_plan* p, const void* vis, int32_t nint, void* stre
   if (report) {
     report->best_wave_images = best.wave;
     report->best_graphs = best.graphs;
-    report->best_fused = best.fused;
+    report->best_fused = 0;
     report->best_overlap = best.overlap;
     report->best_ring = p->ring;
     report->ntried = std::min(ntried, 16);

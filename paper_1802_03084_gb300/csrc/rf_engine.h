@@ -85,16 +85,6 @@ struct Quad {
   int32_t img2, pad[3];
 };
 
-// One chunk of the fused imaging pass: nk consecutive images from image
-// kbase of group g (absolute group index), whose column-FFT output shares one
-// slot of the ring.
-struct FusedChunk {
-  int32_t g;
-  int32_t kbase;
-  int32_t nk;
-  int32_t pad;
-};
-
 // Tensor map of a column-FFT output buffer T[slot][u][N] (as FP32 pairs) for
 // the row pass's tile copies: nbox boxes of `rows` u rows each cover ncol.
 struct TileMap {
@@ -222,8 +212,7 @@ constexpr int col_split(int n) { return n >= 2048 ? n / 1024 : 1; }
 // row pair, 256-thread blocks) or 16 (128 threads per row pair, 512-thread
 // blocks: twice the warps in the same shared memory, at 64 registers a
 // thread).  Both give the same images; 16 measured 36% slower on GB300
-// (48.0 against 35.2 ms per 8134-image launch), so 32 is built.  The fused
-// pass exists at 2048 only with 32.
+// (48.0 against 35.2 ms per 8134-image launch), so 32 is built.
 #define RF_ROW_VALUES_2048 32
 
 // ---------------------------------------------------------------- launchers
@@ -260,20 +249,6 @@ cudaError_t launch_grid_cells(const SegmentGeom& g, const DevTables& tb, const G
 cudaError_t launch_colfft(const SegmentGeom& g, const DevTables& tb, const Group* groups, int g_begin,
                           int ngroups, int img_base, int base_base, const float2* cellbuf, float2* Tbuf,
                           float* colsq, float* mean0, cudaStream_t st, const PassLaunch* pl = nullptr);
-
-// Fused column + row pass (npix 1024 .. 4096) of the chunks [0, nchunks)
-// of one wave (chunks[] on the device, groups indexed absolutely, cellbuf
-// holding groups from g_begin): column FFTs into the ring Tring (ring slots
-// of fused_chunk_images(N) images, tensor map tm), row FFTs and statistics
-// into partials, Parseval sums into colsq/mean0 (slots relative to
-// img_base).  counters: 1 + 2 nchunks ints (zeroed here).  err: set when a
-// bounded wait gave up.
-cudaError_t launch_image_fused(const SegmentGeom& g, const DevTables& tb, const Group* groups, int g_begin,
-                               const FusedChunk* chunks, int nchunks, int img_base, const float2* cellbuf,
-                               float2* Tring, int ring, const TileMap& tm, float* colsq, float* mean0,
-                               StatPartial* partials, int* counters, int* err, cudaStream_t st);
-// Images per chunk of the fused pass (0: no fused pass at this size).
-int fused_chunk_images(int npix);
 
 // Clipping window of each of `nimg` slots for the clipped noise, in raw
 // pixel units (the image times 2W): clip[i] = {mean0[i], kClipSigmas *

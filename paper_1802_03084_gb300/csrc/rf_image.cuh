@@ -904,300 +904,6 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
   if (tid < 32) tmem_free(s_tmem, TCOLS);
 }
 
-// ------------------------------------------------------- fused imaging pass
-// Launch shape of the fused column + row pass (N = 1024 .. 4096): one block
-// shape serves both roles; a chunk is CI = ColCfg<N>::XA images, one column
-// round.
-template <int N>
-struct FusedCfg {
-  using K = ImgCfg<N>;
-  using C = ColCfg<N>;
-  static constexpr int CI = C::XA;                    // images per chunk
-  static constexpr int NRB = N / K::RB;               // row items per image
-  static constexpr int FB = cmax(K::XB * K::STRIDE_B, C::XA * C::R * C::STRIDE);  // float2 of FFT buffers
-  static constexpr int THREADS = K::THREADS_B;
-  static_assert(K::THREADS_B == C::THREADS, "one block shape for both roles");
-  static_assert(K::TILE_TMA && CI >= 2, "fused pass: N = 1024 .. 4096");
-};
-
-// The fused imaging pass of one wave: the column FFTs and the row FFTs with
-// statistics in one persistent launch, the column-FFT output staying in an
-// L2-resident ring of `ring` chunk slots instead of a wave-sized buffer in
-// HBM.  Blocks take work items in order from one counter (two ahead of the
-// item in hand, so the counter's latency is hidden).  Step s holds the ncol
-// column items of chunk s (u = 0 .. ncol-1: stage the column's row map,
-// rows and cells for the chunk's images, Parseval sums, one round of column
-// transforms, store into ring slot s mod ring), then the row items of chunk
-// s - 1 (image, block of RB rows: tensor-copy tile, row FFTs, statistics,
-// as in k_rowfft_stats).  A row item waits until every warp of its chunk's
-// ncol column items has stored; a warp of a column item of chunk s >= ring
-// waits, before it stores, until the row items of chunk s - ring have read
-// the slot.  Every wait is on items taken from the counter earlier, and a
-// block finishes its item before it starts the next one it took, so the
-// smallest unfinished item always has its inputs: the order cannot
-// deadlock.  Each wait is bounded; one that gives up sets *err (the other
-// blocks then stop at their next wait or item) and the block leaves after
-// its copies in flight have landed.  The staging area (a row item's tile, or
-// a column item's map, rows and cells) is filled for the next item as soon
-// as the current one has read it.
-// counters: [0] work counter, [1 + c] warps of chunk c's column items that
-// stored, [1 + nchunks + c] row items that read chunk c's slot; zero at launch.
-template <int N>
-__global__ void __launch_bounds__(FusedCfg<N>::THREADS, 2)
-    k_image_fused(SegmentGeom g, DevTables tb, const Group* __restrict__ groups, int g_begin,
-                  const FusedChunk* __restrict__ chunks, int nchunks, int img_base,
-                  const float2* __restrict__ cellbuf, float2* __restrict__ Tring, int ring,
-                  float* __restrict__ colsq, float* __restrict__ mean0, StatPartial* __restrict__ partials,
-                  const __grid_constant__ CUtensorMap tmap, int tma_boxes, int tma_rows, int* __restrict__ counters,
-                  int* __restrict__ err) {
-  using K = ImgCfg<N>;
-  using C = ColCfg<N>;
-  using F = FusedCfg<N>;
-  constexpr int CI = F::CI;
-  constexpr int CPC = CI / 2;       // 16-byte chunks per staged cell row
-  constexpr int NRB = F::NRB;
-  constexpr int WPB = F::THREADS / 32;
-  constexpr int L = C::L, R = C::R, TL = C::TL;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  float2* fbuf = reinterpret_cast<float2*>(smraw);
-  unsigned char* st0 = smraw + F::FB * 8;
-  st0 += (1024u - (smem_u32(st0) & 1023u)) & 1023u;  // swizzle atom alignment of the tile
-  float4* tile = reinterpret_cast<float4*>(st0);                           // row role: [rows][CH]
-  float2* cellv = reinterpret_cast<float2*>(st0);                          // column role: [max_cells][CI]
-  float2* rtw = cellv + (size_t)g.max_cells * CI;                           // [max_cells][R - 1]
-  int* crow = reinterpret_cast<int*>(rtw + (size_t)g.max_cells * (R - 1));  // [max_cells]
-  int* runs = crow + g.max_cells;                                           // [max_cells]
-  __shared__ __align__(8) unsigned long long tbar;
-  __shared__ int s_q;     // the item after next
-  __shared__ int s_fail;  // a wait gave up, or another block reported one
-  __shared__ int s_pf;    // the next item's tile copy was issued
-  const int tid = threadIdx.x;
-  const int lane = tid & 31;
-  const int warp = tid >> 5;
-  const int ncol = g.ncol;
-  const int ips = ncol + CI * NRB;  // items per step
-  const long total = (long)(nchunks + 1) * ips;
-  int* const work = counters;
-  int* const colcnt = counters + 1;
-  int* const rowcnt = counters + 1 + nchunks;
-  const int log2l = FftShape<N>::LOG2N - (g.tsplit > 1 ? __ffs(g.tsplit) - 1 : 0);
-  const unsigned tile_bytes = (unsigned)(tma_boxes * tma_rows * K::CH * 16);
-  // roles' thread layouts
-  const int xfb = tid / K::TB, tb_ = tid - xfb * K::TB;                // row role
-  const int xfa = tid / (R * TL), pa = (tid / TL) % R, ta = tid % TL;  // column role
-
-  // An item's place in the order: kind 0 none, 1 column (chunk c, column a),
-  // 2 row (chunk c, image a, block b), with its chunk and the wave slot of the
-  // chunk's first image.  The chunk and group loads are issued one item ahead.
-  struct Item {
-    int kind, c, a, b, slot0;
-    FusedChunk ch;
-  };
-  auto locate = [&](long qq) -> Item {  // arithmetic, then the chunk's loads
-    Item it{0, 0, 0, 0, 0, {0, 0, 0, 0}};
-    if (qq >= total) return it;
-    const int st = (int)(qq / ips), o = (int)(qq - (long)st * ips);
-    if (o < ncol) {
-      it.c = st;
-      it.a = o;
-      it.kind = st < nchunks ? 1 : 0;
-    } else {
-      it.c = st - 1;
-      const int j = o - ncol;
-      it.a = j / NRB;
-      it.b = j - it.a * NRB;
-      it.kind = (it.c >= 0 && it.c < nchunks) ? 2 : 0;
-    }
-    if (it.kind != 0) {
-      it.ch = chunks[it.c];
-      it.slot0 = groups[it.ch.g].img0 + it.ch.kbase - img_base;
-    }
-    return it;
-  };
-  // the kind once the chunk is known: a row item past the chunk's images is none
-  auto kind_of = [&](const Item& it) { return (it.kind == 2 && it.a >= it.ch.nk) ? 0 : it.kind; };
-  auto ring_slot = [&](int c, int jj) { return (c % ring) * CI + jj; };
-  auto issue_tile = [&](int c, int jj, int rb) {  // thread 0
-    fence_proxy_async_global();
-    mbar_expect_tx(&tbar, tile_bytes);
-    for (int bx = 0; bx < tma_boxes; ++bx)
-      tma_load_3d(tile + (size_t)bx * tma_rows * K::CH, &tmap, 2 * rb * K::RB, bx * tma_rows, ring_slot(c, jj),
-                  &tbar);
-  };
-  auto issue_stage = [&](const FusedChunk& ch, int u) {  // all threads: the column's rows, runs and cells
-    const int cell0 = tb.col_cell_ptr[u];
-    const int nc = tb.col_cell_ptr[u + 1] - cell0;
-    const int run0 = tb.col_run_ptr[u];
-    const int nr = tb.col_run_ptr[u + 1] - run0;
-    for (int cc = tid; cc < nc; cc += F::THREADS) cp_async4(crow + cc, tb.cell_row + cell0 + cc);
-    for (int j = tid; j < nr; j += F::THREADS) cp_async4(runs + j, tb.col_runs + run0 + j);
-    if constexpr (R > 1)
-      for (int i = tid; i < nr * (R - 1); i += F::THREADS) cp_async8(rtw + i, tb.col_run_tw + (size_t)run0 * (R - 1) + i);
-    const float2* src = cellbuf + ((size_t)(ch.g - g_begin) * g.ncells + cell0) * 32 + ch.kbase;
-    for (int i = tid; i < nc * CPC; i += F::THREADS) {
-      const int cc = i / CPC;
-      const int j = i - cc * CPC;
-      cp_async16(cellv + cc * CI + 2 * (j ^ (cc & (CPC - 1))), src + cc * 32 + 2 * j);
-    }
-    cp_async_commit();
-  };
-  // fill the staging area for item qn after the current item has read it:
-  // a column item's stage (all threads), or a row item's tile if its chunk is
-  // complete (thread 0; *pf tells)
-  auto prefetch = [&](const Item& nx, bool& stage_ready, int& pf) {
-    const int k2 = kind_of(nx);
-    stage_ready = false;
-    if (k2 == 2) {
-      if (tid == 0 && ld_acquire_gpu(colcnt + nx.c) >= ncol * WPB) {
-        issue_tile(nx.c, nx.a, nx.b);
-        pf = 1;
-      }
-    } else if (k2 == 1) {
-      issue_stage(nx.ch, nx.a);
-      stage_ready = true;
-    }
-  };
-
-  if (tid == 0) {
-    mbar_init(&tbar, 1);
-    s_fail = 0;
-    s_pf = 0;
-    s_q = atomicAdd(work, 1);
-  }
-  __syncthreads();
-  long q = s_q;
-  __syncthreads();
-  if (tid == 0) s_q = atomicAdd(work, 1);
-  __syncthreads();
-  long qn = s_q;
-  unsigned phase = 0;
-  bool tile_ready = false;   // a tile copy for item q is in flight
-  bool stage_ready = false;  // item q's column stage is in flight (cp.async)
-  Item cur = locate(q);
-
-  while (q < total) {
-    int qf = 0;
-    if (tid == 0) qf = atomicAdd(work, 1);  // the item after next, used at the item's end
-    const Item nxt = locate(qn);             // its loads complete during this item
-    int pf = 0;                              // thread 0: a tile copy for item qn was issued
-    bool next_stage = false;
-    const int kind = kind_of(cur);
-    const int c = cur.c, a = cur.a, b = cur.b;
-    if (kind == 2) {
-      // ------------------------------------------------------------ row item
-      if (!tile_ready) {
-        bool bad = false;
-        if (tid == 0) {
-          if (wait_count(colcnt + c, ncol * WPB, err)) issue_tile(c, a, b);
-          else bad = true;
-        }
-        if (__syncthreads_or(bad)) {
-          if (tid == 0) atomicExch(err, 1);
-          cp_async_wait_all();
-          __syncthreads();
-          return;
-        }
-      }
-      const bool ok = mbar_wait(&tbar, phase);
-      if (__syncthreads_or(!ok)) {
-        if (tid == 0) {
-          atomicExch(err, 1);
-          mbar_wait(&tbar, phase);  // once more, so the copy does not land after the block has left
-        }
-        cp_async_wait_all();
-        __syncthreads();
-        return;
-      }
-      phase ^= 1u;
-      if (tid == 0) {  // the tile's reads of the ring slot are complete
-        fence_proxy_async_global();
-        __threadfence();
-        atomicAdd(rowcnt + c, 1);
-      }
-      float2 v[K::EB];
-      row_zbuild<N>(v, tile, tb_, xfb, ncol);
-      __syncthreads();  // the staging area is read
-      prefetch(nxt, next_stage, pf);
-      const int slot = cur.slot0 + a;
-      row_fft<N>(v, fbuf + xfb * K::STRIDE_B, tb.twiddle, tb_, xfb);
-      row_stats<N, false>(v, tb_, xfb, slot, b * K::RB, g.tsplit, log2l, partials, nullptr);
-    } else if (kind == 1) {
-      // --------------------------------------------------------- column item
-      const FusedChunk ch = cur.ch;
-      const int u = a;
-      const int ncells = tb.col_cell_ptr[u + 1] - tb.col_cell_ptr[u];
-      const int nruns = tb.col_run_ptr[u + 1] - tb.col_run_ptr[u];
-      if (!stage_ready) issue_stage(ch, u);
-      cp_async_wait_all();
-      __syncthreads();
-      const int wslot0 = cur.slot0;
-      // Parseval sums of the column, one warp per image
-      if (warp < ch.nk) {
-        const int kl = warp;
-        float acc = 0.f;
-        for (int cc = lane; cc < ncells; cc += 32) {
-          const float2 h = cellv[cc * CI + 2 * ((kl >> 1) ^ (cc & (CPC - 1))) + (kl & 1)];
-          acc = fmaf(h.x, h.x, fmaf(h.y, h.y, acc));
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) {
-          colsq[(size_t)(wslot0 + kl) * ncol + u] = (u == 0 ? 1.f : 2.f) * acc;
-          if (u == 0) mean0[wslot0 + kl] = (ncells > 0 && crow[0] == 0) ? cellv[kl].x : 0.f;
-        }
-      }
-      float2* buf = fbuf + (xfa * R + pa) * C::STRIDE;
-      col_scatter<N, CI>(buf, runs, nruns, cellv, crow, xfa, xfa < ch.nk, rtw, ta, pa, xfa * R + pa);
-      __syncthreads();  // the staging area is read
-      prefetch(nxt, next_stage, pf);
-      // this warp's slot rows are free once the row items of chunk c - ring have read them
-      bool ok = true;
-      if (c >= ring) {
-        if (lane == 0) ok = wait_count(rowcnt + (c - ring), chunks[c - ring].nk * NRB, err);
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        if (!ok && lane == 0) atomicExch(err, 1);
-      }
-      float2* dst = (ok && xfa < ch.nk) ? Tring + ((size_t)ring_slot(c, xfa) * ncol + u) * N + pa * L : nullptr;
-      col_fft_store<N>(buf, tb.twiddle_col, ta, xfa * R + pa, dst);
-      if (ok) {
-        // the warp's stores, then one cumulative fence and the count (the
-        // row items read the slot through the async proxy)
-        __syncwarp();
-        if (lane == 0) {
-          fence_proxy_async_global();
-          __threadfence();
-          atomicAdd(colcnt + c, 1);
-        }
-      }
-    } else {
-      // an empty place of the order (a missing image of a short chunk, the
-      // first and last steps): nothing was staged for it
-      __syncthreads();
-      prefetch(nxt, next_stage, pf);
-    }
-    // end of the item: publish the item after next and the prefetch; stop
-    // if any block has given up
-    if (tid == 0) {
-      s_q = qf;
-      s_pf = pf;
-      s_fail = ld_acquire_gpu(err) != 0;
-    }
-    __syncthreads();
-    tile_ready = s_pf != 0;
-    stage_ready = next_stage;
-    q = qn;
-    qn = s_q;
-    cur = nxt;
-    if (s_fail) {
-      if (tid == 0 && tile_ready) mbar_wait(&tbar, phase);
-      cp_async_wait_all();
-      __syncthreads();
-      return;
-    }
-  }
-  cp_async_wait_all();
-}
-
 // The most dynamic shared memory a block of `kern` can have: the device's
 // opt-in per-block limit (227 KB on sm_103a) less the kernel's static shared
 // memory.  Kernels whose request depends on the plan set their attribute to
@@ -1679,38 +1385,6 @@ cudaError_t run_rowfft_tree(const SegmentGeom& g, const DevTables& tb, const flo
 }
 
 template <int N>
-cudaError_t run_image_fused(const SegmentGeom& g, const DevTables& tb, const Group* groups, int g_begin,
-                            const FusedChunk* chunks, int nchunks, int img_base, const float2* cellbuf,
-                            float2* Tring, int ring, const TileMap& tm, float* colsq, float* mean0,
-                            StatPartial* partials, int* counters, int* err, cudaStream_t st) {
-  using K = ImgCfg<N>;
-  using C = ColCfg<N>;
-  using F = FusedCfg<N>;
-  if (nchunks <= 0) return cudaSuccess;
-  if (tm.nbox <= 0 || ring < 2) return cudaErrorInvalidValue;
-  const int tile = rowfft_tile_rows<N>(g.ncol) * K::CH * 16;
-  const int cols = g.max_cells * (F::CI * 8 + 8 + (C::R - 1) * 8);
-  const int smem = F::FB * 8 + 1024 + std::max(tile, cols);
-  auto kern = k_image_fused<N>;
-  const int smem_max = max_dynamic_smem(kern);
-  if (smem > smem_max) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(counters, 0, (size_t)(1 + 2 * nchunks) * sizeof(int), st);
-  if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, F::THREADS, smem);
-  if (e != cudaSuccess) return e;
-  const long items = (long)(nchunks + 1) * (g.ncol + F::CI * F::NRB);
-  const long grid = std::min<long>(items, (long)std::max(per_sm, 1) * sm_count());
-  kern<<<(int)grid, F::THREADS, smem, st>>>(g, tb, groups, g_begin, chunks, nchunks, img_base, cellbuf, Tring, ring,
-                                           colsq, mean0, partials, tm.map, tm.nbox, tm.rows, counters, err);
-  return cudaGetLastError();
-}
-
-template <int N>
 void fill_shape(ImageKernelShape* o) {
   using K = ImgCfg<N>;
   o->images_per_group = K::B;
@@ -1742,10 +1416,5 @@ void fill_shape(ImageKernelShape* o) {
   template cudaError_t run_rowfft_tree<N>(const SegmentGeom&, const DevTables&, const float2*, const Quad*,  \
                                           int, int, int, StatPartial*, const TileMap*, int*, cudaStream_t,   \
                                           const float2*, const PassLaunch*);
-
-#define RF_INSTANTIATE_FUSED(N)                                                                              \
-  template cudaError_t run_image_fused<N>(const SegmentGeom&, const DevTables&, const Group*, int,            \
-                                          const FusedChunk*, int, int, const float2*, float2*, int,         \
-                                          const TileMap&, float*, float*, StatPartial*, int*, int*, cudaStream_t);
 
 }  // namespace rf
