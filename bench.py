@@ -607,7 +607,7 @@ def run_next_rows(args):
     cms_, cc = timed(lambda: plan_c.search(vis, nint), 3)
     line["noise_clipped"] = {"ms": cms_, "overhead_ms": cms_ - ms, "candidates": int(len(cc)),
                              "candidates_plain_noise": int(len(cands)),
-                             "clip_window_kernel_ms": kernel_ms(plan_c, "clip_window"),
+                             "clip_window_kernel_ms": kernel_ms(plan_c, "image_noise"),
                              "rowfft_stats_kernel_ms": kernel_ms(plan_c, "rowfft_stats")}
     plan_c.close()
     # stream: segments of nint integrations overlapping by the longest sweep,

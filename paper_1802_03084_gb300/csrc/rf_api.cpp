@@ -97,12 +97,12 @@ struct BusyGuard {
 
 enum KernelKind {
   K_H2D = 0, K_INGEST, K_RESAMPLE, K_WEIGHTS, K_GRID_CELLS, K_GRID_COLFFT, K_ROWFFT_STATS, K_FINALIZE,
-  K_PLAIN_TRIAL, K_MEAN_SUBTRACT, K_CLIP_WINDOW, K_IMAGE_FUSED, K_NKINDS
+  K_PLAIN_TRIAL, K_MEAN_SUBTRACT, K_IMAGE_NOISE, K_IMAGE_FUSED, K_NKINDS
 };
 const char* const kKindNames[K_NKINDS] = {"h2d_copy",    "ingest",       "resample",
                                            "weights",     "grid_cells",   "grid_colfft",
                                            "rowfft_stats", "finalize",    "plain_trial_chunk",
-                                           "mean_subtract", "clip_window", "image_fused"};
+                                           "mean_subtract", "image_noise", "image_fused"};
 
 // Event-pair timing of every launch a plan issues while profiling is on.
 struct Profiler {
@@ -270,7 +270,10 @@ struct rf_plan {
   float2* d_cellbuf = nullptr;
   float* d_colsq = nullptr;     // [slots][ncol] Parseval sums
   float* d_mean0 = nullptr;     // [slots] Re H(0, 0)
-  float2* d_clip = nullptr;     // [slots] clipping window (RF_NOISE_CLIPPED only)
+  rf::ImgNoise* d_noise = nullptr;  // [sslots] mean and noise from the Parseval sums
+  float* d_gate = nullptr;      // [sslots] least raw maximum of a candidate
+  float2* d_clip = nullptr;     // [sslots] clipping window (RF_NOISE_CLIPPED only)
+  rf::ClipPartial* d_cparts = nullptr;  // kept-pixel partials (RF_NOISE_CLIPPED only)
   rf::PlainBuffers plain{};     // allocated on the first plain-form search
 
   // RF_TUNE_FUSED and RF_TUNE_RING: kept and reported, without effect
@@ -855,10 +858,25 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
     p->dfree(p->d_mean0);
     p->d_colsq = p->d_mean0 = nullptr;
   }
+  if (p->d_noise) {
+    p->device_bytes -= (uint64_t)p->sslots * sizeof(rf::ImgNoise);
+    p->dfree(p->d_noise);
+    p->d_noise = nullptr;
+  }
+  if (p->d_gate) {
+    p->device_bytes -= (uint64_t)p->sslots * sizeof(float);
+    p->dfree(p->d_gate);
+    p->d_gate = nullptr;
+  }
   if (p->d_clip) {
     p->device_bytes -= (uint64_t)p->sslots * sizeof(float2);
     p->dfree(p->d_clip);
     p->d_clip = nullptr;
+  }
+  if (p->d_cparts) {
+    p->device_bytes -= (uint64_t)p->sslots * nrb * sizeof(rf::ClipPartial);
+    p->dfree(p->d_cparts);
+    p->d_cparts = nullptr;
   }
   p->slots_max = slots;
   p->tslots = wave_tslots(p, slots);
@@ -872,7 +890,13 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
   if ((s = p->dalloc(&p->d_cellbuf, (size_t)p->gslots_max * std::max(p->n_cells, 1) * 32)) != RF_OK) return s;
   if ((s = p->dalloc(&p->d_colsq, (size_t)p->sslots * p->ncol)) != RF_OK) return s;
   if ((s = p->dalloc(&p->d_mean0, (size_t)p->sslots)) != RF_OK) return s;
-  if ((p->flags & RF_NOISE_CLIPPED) && (s = p->dalloc(&p->d_clip, (size_t)p->sslots)) != RF_OK) return s;
+  if ((s = p->dalloc(&p->d_noise, (size_t)p->sslots)) != RF_OK) return s;
+  if (p->flags & RF_NOISE_CLIPPED) {
+    if ((s = p->dalloc(&p->d_clip, (size_t)p->sslots)) != RF_OK) return s;
+    if ((s = p->dalloc(&p->d_cparts, (size_t)p->sslots * nrb)) != RF_OK) return s;
+  } else if ((s = p->dalloc(&p->d_gate, (size_t)p->sslots)) != RF_OK) {
+    return s;
+  }
   const int xb = std::min(256 / (p->npix / 32), p->npix / 2);  // row pairs of a row-pass work item
   encode_tile_map(p, p->tmap_T, p->d_T, p->tslots, 2 * xb);
   // the halves of d_T, each a wave's scratch when waves are overlapped
@@ -919,8 +943,11 @@ uint64_t estimate_device_bytes(const rf_plan* p, int slots) {
   const int gslots = std::max(2 * ((tslots + B - 1) / B), 1);
   b += r((size_t)tslots * per_slot, 1) + r((size_t)sslots * p->shape.partials_per_image, sizeof(StatPartial)) +
        r((size_t)gslots * std::max(p->n_cells, 1) * 32, sizeof(float2)) + r((size_t)sslots * p->ncol, 4) +
-       r(sslots, 4);
-  if (p->flags & RF_NOISE_CLIPPED) b += r(sslots, sizeof(float2));
+       r(sslots, 4) + r(sslots, sizeof(rf::ImgNoise));
+  if (p->flags & RF_NOISE_CLIPPED)
+    b += r(sslots, sizeof(float2)) + r((size_t)sslots * p->shape.partials_per_image, sizeof(rf::ClipPartial));
+  else
+    b += r(sslots, sizeof(float));
   const size_t per_int = rows * p->npol * sizeof(float2);
   const size_t stage_nint = std::max<size_t>(1, std::min<size_t>(kStageBytes / per_int, (size_t)p->max_nint));
   b += r(stage_nint * per_int, 1);
@@ -1177,16 +1204,46 @@ rf_status run_waves_overlapped(rf_plan* p, const SegmentGeom& g, const std::vect
 
 // The row pass of one wave: over quads where the plan has widths that are sums
 // of others (never for listed trials, whose images `im` takes), else image by
-// image.  `clip`: the wave's clipping windows, or null.
-cudaError_t launch_row_pass(rf_plan* p, const SegmentGeom& g, const Wave& w, const float2* T, StatPartial* part,
-                            const rf::TileMap* tm, const float2* clip, float* im, cudaStream_t st,
-                            const rf::PassLaunch* pl) {
+// image.
+cudaError_t launch_row_pass(rf_plan* p, const SegmentGeom& g, const Wave& w, const float2* T, const rf::PassStats& ps,
+                            const rf::TileMap* tm, float* im, cudaStream_t st, const rf::PassLaunch* pl) {
   if (tm->nbox == 0) tm = nullptr;
   if (w.quad_end > w.quad_begin)
     return rf::launch_rowfft_tree(g, p->tb, T, p->d_quads + w.quad_begin, w.quad_end - w.quad_begin, w.img_begin,
-                                  w.base_begin, part, tm, p->d_err, st, clip, pl);
-  return rf::launch_rowfft_stats(g, p->tb, T, w.img_end - w.img_begin, w.img_begin, p->d_weight, part, im, tm,
-                                 p->d_err, st, clip, pl);
+                                  w.base_begin, ps, tm, p->d_err, st, pl);
+  return rf::launch_rowfft_stats(g, p->tb, T, w.img_end - w.img_begin, w.img_begin, p->d_weight, ps, im, tm, p->d_err,
+                                 st, pl);
+}
+
+// Everything after a wave's column pass, on `st`: the images' noise, the row
+// pass and the finalisation, with the wave's slots of the scratch starting at
+// slot0 (colsq, mean0 and the statistics' buffers).  Every image's peak
+// position is wanted where statistics or images are returned; else the row
+// pass looks for it only in what can become a candidate (not under the clipped
+// noise, which is known only after the row pass).
+rf_status finish_wave(rf_plan* p, const SegmentGeom& g, const Wave& w, const float2* T, size_t slot0,
+                      const rf::TileMap* tm, DevStat* d_stats, float* im, cudaStream_t st,
+                      const rf::PassLaunch* pl) {
+  const size_t nrb = (size_t)p->shape.partials_per_image;
+  const int ni = w.img_end - w.img_begin;
+  const float* colsq = p->d_colsq + slot0 * p->ncol;
+  const float* mean0 = p->d_mean0 + slot0;
+  rf::ImgNoise* noise = p->d_noise + slot0;
+  const bool clip = (p->flags & RF_NOISE_CLIPPED) != 0;
+  float2* cw = clip ? p->d_clip + slot0 : nullptr;
+  float* gate = clip || d_stats || im ? nullptr : p->d_gate + slot0;
+  RF_TIMED(p->prof, K_IMAGE_NOISE, st,
+           rf::launch_image_noise(g, colsq, mean0, p->d_weight, ni, w.img_begin, p->threshold, noise, gate, cw, st));
+  rf::PassStats ps;
+  ps.partials = p->d_partials + slot0 * nrb;
+  ps.gate = gate;
+  ps.clip = cw;
+  ps.cparts = clip ? p->d_cparts + slot0 * nrb : nullptr;
+  RF_TIMED(p->prof, K_ROWFFT_STATS, st, launch_row_pass(p, g, w, T, ps, tm, im, st, pl));
+  RF_TIMED(p->prof, K_FINALIZE, st,
+           rf::launch_finalize(g, ps, noise, mean0, p->d_img_info, p->d_weight, ni, w.img_begin, p->threshold,
+                               p->d_cands, p->d_ncand, p->img_cap, d_stats, st));
+  return RF_OK;
 }
 
 // The wave loop of run_waves_overlapped (streams and events set up).
@@ -1195,14 +1252,11 @@ rf_status overlapped_loop(rf_plan* p, const SegmentGeom& g, const std::vector<Wa
   cudaStream_t so = p->ostream;
   const size_t half = (size_t)p->tslots / 2, shalf = (size_t)p->sslots / 2;
   const size_t per_slot = (size_t)p->ncol * p->npix;
-  const size_t nrb = (size_t)p->shape.partials_per_image;
   for (size_t wi = 0; wi < waves.size(); ++wi) {
     const Wave& w = waves[wi];
     const int h = (int)(wi & 1);
     const int ng = w.g_end - w.g_begin;
-    const int ni = w.img_end - w.img_begin;
     float2* T = p->d_T + h * half * per_slot;
-    StatPartial* part = p->d_partials + h * shalf * nrb;
     float* colsq = p->d_colsq + h * shalf * p->ncol;
     float* mean0 = p->d_mean0 + h * shalf;
     RF_TIMED(p->prof, K_GRID_CELLS, st,
@@ -1213,11 +1267,8 @@ rf_status overlapped_loop(rf_plan* p, const SegmentGeom& g, const std::vector<Wa
                                colsq, mean0, st, &pc));
     RF_CUDA(cudaEventRecord(p->oev[h], st));
     RF_CUDA(cudaStreamWaitEvent(so, p->oev[h], 0));
-    RF_TIMED(p->prof, K_ROWFFT_STATS, so,
-             launch_row_pass(p, g, w, T, part, &p->tmap_H[h], nullptr, nullptr, so, &pr));
-    RF_TIMED(p->prof, K_FINALIZE, so,
-             rf::launch_finalize(g, part, colsq, mean0, p->d_img_info, p->d_weight, ni, w.img_begin, p->threshold,
-                                 p->d_cands, p->d_ncand, p->img_cap, d_stats, so, false));
+    const rf_status s = finish_wave(p, g, w, T, h * shalf, &p->tmap_H[h], d_stats, nullptr, so, &pr);
+    if (s != RF_OK) return s;
     RF_CUDA(cudaEventRecord(p->oev[2 + h], so));
   }
   return RF_OK;
@@ -1235,23 +1286,14 @@ rf_status run_waves(rf_plan* p, int nint, const std::vector<Wave>& waves, int ni
   for (size_t wi = 0; wi < waves.size(); ++wi) {
     const Wave& w = waves[wi];
     const int ng = w.g_end - w.g_begin;
-    const int ni = w.img_end - w.img_begin;
     RF_TIMED(p->prof, K_GRID_CELLS, st,
              rf::launch_grid_cells(g, p->tb, p->d_groups, w.g_begin, ng, p->d_cellbuf, st));
     RF_TIMED(p->prof, K_GRID_COLFFT, st,
              rf::launch_colfft(g, p->tb, p->d_groups, w.g_begin, ng, w.img_begin, w.base_begin, p->d_cellbuf,
                                p->d_T, p->d_colsq, p->d_mean0, st));
-    const bool clip = (p->flags & RF_NOISE_CLIPPED) != 0;
-    if (clip)
-      RF_TIMED(p->prof, K_CLIP_WINDOW, st, rf::launch_clip_window(g, p->d_colsq, p->d_mean0, ni, p->d_clip, st));
     float* im = d_images ? d_images + (size_t)w.img_begin * p->npix * p->npix : nullptr;
-    RF_TIMED(p->prof, K_ROWFFT_STATS, st,
-             launch_row_pass(p, g, w, p->d_T, p->d_partials, &p->tmap_T, clip ? p->d_clip : nullptr, im, st,
-                             nullptr));
-    RF_TIMED(p->prof, K_FINALIZE, st,
-             rf::launch_finalize(g, p->d_partials, p->d_colsq, p->d_mean0, p->d_img_info, p->d_weight, ni,
-                                 w.img_begin, p->threshold, p->d_cands, p->d_ncand, p->img_cap, d_stats, st,
-                                 clip));
+    const rf_status s = finish_wave(p, g, w, p->d_T, 0, &p->tmap_T, d_stats, im, st, nullptr);
+    if (s != RF_OK) return s;
   }
   return RF_OK;
 }

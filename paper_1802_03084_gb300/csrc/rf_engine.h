@@ -150,16 +150,35 @@ void fft_twiddle_table(int n, float2* out);
 // Cell of an off-grid (baseline, channel) in the per-row cell table.
 constexpr int kOffGrid = -2147483647 - 1;
 
-// Row-block partial statistics of one image (raw pixel units).  With the
-// clipped noise, sum and sumsq hold the sums of d = J - mean0 and d^2 over
-// the `kept` pixels J of the block with |d| <= clip sigmas (else zero).
+// Largest pixel of a part of one image (raw pixel units).
 struct StatPartial {
-  double sum;
-  double sumsq;
   float max;
-  int32_t idx;  // y * N + x of max (lowest on ties)
+  int32_t idx;  // y * N + x of max (lowest on ties); INT_MAX where the max is below the image's gate
+};
+
+// With the clipped noise, of the same part: the sums of d = J - mean0 and d^2
+// over its `kept` pixels J with |d| <= clip sigmas.
+struct ClipPartial {
+  float sum;
+  float sumsq;
   int32_t kept;
   int32_t pad;
+};
+
+// Mean and noise of one image over all its pixels, from the Parseval sums.
+struct ImgNoise {
+  double mean;
+  double sigma;
+};
+
+// Statistics of the row pass, per slot of a wave.  clip and cparts are set
+// together (the clipped noise).  gate: an image's maxima below its gate are
+// written without their index (null: every index is wanted).
+struct PassStats {
+  StatPartial* partials = nullptr;  // [slot][partials per image]
+  const float* gate = nullptr;
+  const float2* clip = nullptr;
+  ClipPartial* cparts = nullptr;    // [slot][partials per image]
 };
 
 // Clipping radius of the optional one-pass clipped noise, in units of the
@@ -250,37 +269,37 @@ cudaError_t launch_colfft(const SegmentGeom& g, const DevTables& tb, const Group
                           int ngroups, int img_base, int base_base, const float2* cellbuf, float2* Tbuf,
                           float* colsq, float* mean0, cudaStream_t st, const PassLaunch* pl = nullptr);
 
-// Clipping window of each of `nimg` slots for the clipped noise, in raw
-// pixel units (the image times 2W): clip[i] = {mean0[i], kClipSigmas *
-// sigma over all pixels}, the sigma from the Parseval sums colsq.
-cudaError_t launch_clip_window(const SegmentGeom& g, const float* colsq, const float* mean0, int nimg,
-                               float2* clip, cudaStream_t st);
+// Noise of each of `nimg` slots (first image img_base) from the Parseval sums
+// colsq, before the row pass.  gate[i] (if not null): the raw pixel value below
+// which a maximum cannot make image i a candidate.  clip[i] (if not null): the
+// clipping window of the clipped noise in raw pixel units (the image times
+// 2W), {mean0[i], kClipSigmas * sigma over all pixels}.
+cudaError_t launch_image_noise(const SegmentGeom& g, const float* colsq, const float* mean0, const double* weight,
+                               int nimg, int img_base, double threshold, ImgNoise* noise, float* gate, float2* clip,
+                               cudaStream_t st);
 
 // Row C2R (pass B) + statistics of `nimg` images in slots [0, nimg) whose
 // first image index is img_base.  Optionally writes the scaled images.
-// With `clip` (per slot, from launch_clip_window) the partials also carry
-// the kept-pixel sums of the clipped noise.
+// `ps` names the per-slot inputs and outputs of the statistics.
 cudaError_t launch_rowfft_stats(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, int nimg,
-                                int img_base, const double* weight, StatPartial* partials, float* images,
-                                const TileMap* tm, int* err, cudaStream_t st, const float2* clip = nullptr,
-                                const PassLaunch* pl = nullptr);
+                                int img_base, const double* weight, const PassStats& ps, float* images,
+                                const TileMap* tm, int* err, cudaStream_t st, const PassLaunch* pl = nullptr);
 
 // The same for the transformed images of nquads quads (T slots relative to
 // base_base, statistics slots to img_base) and the images derived from them,
 // npix >= kTreeMinNpix.
 cudaError_t launch_rowfft_tree(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Quad* quads,
-                               int nquads, int img_base, int base_base, StatPartial* partials, const TileMap* tm,
-                               int* err, cudaStream_t st, const float2* clip, const PassLaunch* pl = nullptr);
+                               int nquads, int img_base, int base_base, const PassStats& ps, const TileMap* tm,
+                               int* err, cudaStream_t st, const PassLaunch* pl = nullptr);
 constexpr int kTreeMinNpix = 64;  // below, a row-pass block is less than a warp
 
 // Reduce row-block partials, compute sigma / snr, append candidates and
 // (optionally) per-image stats for images [img_base, img_base + nimg).
-// With `clip` the mean and sigma are those of the kept pixels, from the
+// Under ps.clip the mean and sigma are those of the kept pixels, from the
 // partials' sums around mean0.
-cudaError_t launch_finalize(const SegmentGeom& g, const StatPartial* partials, const float* colsq,
-                            const float* mean0, const int4* img_info, const double* weight, int nimg, int img_base,
-                            double threshold, DevCand* cands, int* ncand, int cand_cap, DevStat* stats,
-                            cudaStream_t st, bool clip = false);
+cudaError_t launch_finalize(const SegmentGeom& g, const PassStats& ps, const ImgNoise* noise, const float* mean0,
+                            const int4* img_info, const double* weight, int nimg, int img_base, double threshold,
+                            DevCand* cands, int* ncand, int cand_cap, DevStat* stats, cudaStream_t st);
 
 // Buffers of the plain per-trial form (chunks of up to `cap` images).
 struct PlainBuffers {

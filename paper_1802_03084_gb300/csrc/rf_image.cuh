@@ -344,6 +344,31 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
   }
 }
 
+// Maximum and minimum over aligned groups of W lanes (every lane has its
+// group's): one reduction instruction over a whole warp.
+template <int W>
+__device__ __forceinline__ float warp_max(float v) {
+  if constexpr (W == 32) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+  } else {
+#pragma unroll
+    for (int off = W / 2; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
+    return v;
+  }
+}
+template <int W>
+__device__ __forceinline__ int warp_min(int v) {
+  if constexpr (W == 32) {
+    return __reduce_min_sync(0xffffffffu, v);
+  } else {
+#pragma unroll
+    for (int off = W / 2; off > 0; off >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, off));
+    return v;
+  }
+}
+
 __device__ __forceinline__ void max_merge(float& m, int& i, float m2, int i2) {
   if (m2 > m || (m2 == m && i2 < i)) {
     m = m2;
@@ -489,11 +514,15 @@ __device__ __forceinline__ void row_write(const float2 (&v)[ImgCfg<N>::EB], int 
 // Statistics of the row pair (T rows i = y0 + 2 xf and i + 1, image rows t_row
 // of them) of the image in `slot` whose pixels are in v: the pair's max pixel
 // with its lowest index (and under CLIP the kept-pixel sums), one StatPartial
-// per warp of the transform.
+// per warp of the transform.  The index is looked for only where the max is
+// not below `gate`, the image's least raw value that can make it a candidate:
+// finding it (a search through the lane's 64 values and a second reduction)
+// costs as much as the maximum itself, and nearly every image of a segment is
+// noise: 1024^2 realtime row passes 91.0 -> 84.2 ms, 2048^2 batching 175.7 ->
+// 163.1, 4096^2 stress subset 8.41 -> 8.01, 512^2 serving 5.37 -> 4.67.
 template <int N, bool CLIP>
 __device__ __forceinline__ void row_stats(const float2 (&v)[ImgCfg<N>::EB], int t, int xf, int slot, int y0,
-                                          int tsplit, int log2l, StatPartial* __restrict__ partials,
-                                          const float2* __restrict__ clip) {
+                                          int tsplit, int log2l, float gate, const PassStats& ps) {
   using K = ImgCfg<N>;
   constexpr int EB = K::EB, TB = K::TB;
   constexpr int H = N / K::RSPLIT;
@@ -524,13 +553,12 @@ __device__ __forceinline__ void row_stats(const float2 (&v)[ImgCfg<N>::EB], int 
   // several warps joined through shared memory)
   constexpr int WL = TB < 32 ? TB : 32;
   constexpr unsigned MASK = 0xffffffffu;
-  float wmax = lmax;
-#pragma unroll
-  for (int off = WL / 2; off > 0; off >>= 1) wmax = fmaxf(wmax, __shfl_xor_sync(MASK, wmax, off));
+  const float wmax = warp_max<WL>(lmax);
   // a lane holding the maximum finds its lowest index: row ya comes before
   // row yb, and within a row the lane's outputs ascend with (q, m)
   int best = INT_MAX;
-  if (lmax == wmax) {
+  const bool want = CLIP || !(wmax < gate);
+  if (want && lmax == wmax) {
     if (mx == wmax) {
 #pragma unroll
       for (int q = 0; q < LP; ++q)
@@ -552,14 +580,13 @@ __device__ __forceinline__ void row_stats(const float2 (&v)[ImgCfg<N>::EB], int 
     }
   found:;
   }
-#pragma unroll
-  for (int off = WL / 2; off > 0; off >>= 1) best = min(best, __shfl_xor_sync(MASK, best, off));
+  if (CLIP || __any_sync(MASK, want)) best = warp_min<WL>(best);
   // clipped noise: sums of the kept pixels' deviations from mean0, rows y
   // and y + 1 in separate chains
   float s1 = 0.f, s2 = 0.f;
   int cn = 0;
   if constexpr (CLIP) {
-    const float2 cw = clip[slot];
+    const float2 cw = ps.clip[slot];
     float ax = 0.f, qx = 0.f, ay = 0.f, qy = 0.f;
     int nx = 0, ny = 0;
 #pragma unroll
@@ -591,14 +618,9 @@ __device__ __forceinline__ void row_stats(const float2 (&v)[ImgCfg<N>::EB], int 
   // spans several warps; the finalisation combines them): no barrier
   if ((t & 31) == 0) {
     constexpr int WPT = TB > 32 ? TB / 32 : 1;
-    StatPartial sp;
-    sp.sum = s1;
-    sp.sumsq = s2;
-    sp.kept = cn;
-    sp.max = wmax;
-    sp.idx = best;
-    sp.pad = 0;
-    partials[(size_t)slot * K::PARTIALS + ((y0 >> 1) + xf) * WPT + (t >> 5)] = sp;  // by T row pair
+    const size_t o = (size_t)slot * K::PARTIALS + ((y0 >> 1) + xf) * WPT + (t >> 5);  // by T row pair
+    ps.partials[o] = StatPartial{wmax, best};
+    if constexpr (CLIP) ps.cparts[o] = ClipPartial{s1, s2, cn, 0};
   }
 }
 
@@ -624,9 +646,8 @@ __device__ __forceinline__ void row_stats(const float2 (&v)[ImgCfg<N>::EB], int 
 template <int N, bool CLIP>
 __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
     k_rowfft_stats(SegmentGeom g, DevTables tb, const float2* __restrict__ Tbuf, int nimg, int img_base,
-                   const double* __restrict__ weight, StatPartial* __restrict__ partials,
-                   float* __restrict__ images, const __grid_constant__ CUtensorMap tmap, int tma_boxes,
-                   int tma_rows, int* __restrict__ err, const float2* __restrict__ clip) {
+                   const double* __restrict__ weight, const PassStats ps, float* __restrict__ images,
+                   const __grid_constant__ CUtensorMap tmap, int tma_boxes, int tma_rows, int* __restrict__ err) {
   using K = ImgCfg<N>;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* fbuf = reinterpret_cast<float2*>(smraw);  // [XB][STRIDE_B]
@@ -714,6 +735,7 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
     }
     const int slot = item / nrb;
     const int y0 = (item - slot * nrb) * K::RB;
+    const float gate = !CLIP && ps.gate != nullptr ? ps.gate[slot] : -FLT_MAX;
     float2 v[K::EB];
     row_zbuild<N>(v, tile, t, xf, ncol);
     if (use_tma && WARP_LOCAL) {
@@ -737,7 +759,7 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
     }
     row_fft<N>(v, fbuf + xf * K::STRIDE_B, tb.twiddle, t, xf);
     if (images != nullptr) row_write<N>(v, t, xf, slot, y0, g.tsplit, log2l, weight[img_base + slot], images);
-    row_stats<N, CLIP>(v, t, xf, slot, y0, g.tsplit, log2l, partials, clip);
+    row_stats<N, CLIP>(v, t, xf, slot, y0, g.tsplit, log2l, gate, ps);
   }
 }
 
@@ -766,9 +788,8 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
 template <int N, bool CLIP>
 __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
     k_rowfft_tree(SegmentGeom g, DevTables tb, const float2* __restrict__ Tbuf, const Quad* __restrict__ quads,
-                  int nquads, int img_base, int base_base, StatPartial* __restrict__ partials,
-                  const __grid_constant__ CUtensorMap tmap, int tma_boxes, int tma_rows, int* __restrict__ err,
-                  const float2* __restrict__ clip) {
+                  int nquads, int img_base, int base_base, const PassStats ps,
+                  const __grid_constant__ CUtensorMap tmap, int tma_boxes, int tma_rows, int* __restrict__ err) {
   using K = ImgCfg<N>;
   static_assert(K::EB == 32 && K::THREADS_B % 32 == 0, "64 values a lane, whole warps");
   constexpr int NWB = K::THREADS_B / 32;
@@ -828,6 +849,16 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
     Quad nxt = cur;
     if (next < nitems) nxt = quads[next / nrb];
     const int top = cur.img2 >= 0 ? 2 : (cur.img1 >= 0 ? 1 : 0);
+    // lanes 0 .. 3 hold the gates of the quad's images, 4 and 5 those of the
+    // sums of two, 6 that of the sum of four
+    float gates = -FLT_MAX;
+    if (!CLIP && ps.gate != nullptr) {
+      const int lane = tid & 31;
+      int sl = lane < cur.n ? cur.img + lane : -1;
+      if (lane >= 4) sl = lane < 6 && cur.img1 >= 0 && 2 * (lane - 4) + 1 < cur.n ? cur.img1 + lane - 4 : -1;
+      if (lane == 6) sl = cur.img2;
+      if (sl >= 0) gates = ps.gate[sl - img_base];
+    }
     for (int k = 0; k < cur.n; ++k) {
       if (use_tma && WARP_LOCAL) {
         // as in k_rowfft_stats: no copy is issued without this warp's count
@@ -880,7 +911,8 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
       int slot = cur.img + k - img_base;
 #pragma unroll 1
       for (int lv = 0;;) {
-        if (slot >= 0) row_stats<N, CLIP>(v, t, xf, slot, y0, g.tsplit, log2l, partials, clip);
+        const float gate = __shfl_sync(0xffffffffu, gates, lv == 0 ? k : (lv == 1 ? 4 + (k >> 1) : 6));
+        if (slot >= 0) row_stats<N, CLIP>(v, t, xf, slot, y0, g.tsplit, log2l, gate, ps);
         // level lv's block of images that ends the next level's must be whole
         if (lv >= top || (k | ((2 << lv) - 1)) >= cur.n) break;
         __syncwarp();
@@ -1222,14 +1254,7 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
       fft_sync<TB>(xf);
     }
     if (t == 0) {
-      StatPartial sp;
-      sp.sum = 0.0;
-      sp.sumsq = 0.0;
-      sp.max = mx;
-      sp.idx = mi;
-      sp.kept = 0;
-      sp.pad = 0;
-      partials[(size_t)pj * N + iy] = sp;
+      partials[(size_t)pj * N + iy] = StatPartial{mx, mi};
     }
   }
 }
@@ -1301,9 +1326,8 @@ int rowfft_tile_rows(int ncol) {
 
 template <int N, bool CLIP>
 cudaError_t run_rowfft_stats_k(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, int nimg,
-                               int img_base, const double* weight, StatPartial* partials, float* images,
-                               const TileMap* tm, int* err, cudaStream_t st, const float2* clip,
-                               const PassLaunch* pl) {
+                               int img_base, const double* weight, const PassStats& ps, float* images,
+                               const TileMap* tm, int* err, cudaStream_t st, const PassLaunch* pl) {
   using K = ImgCfg<N>;
   const int smem = K::SMEM_B_FIXED + (K::TILE_TMA ? 1024 : 0) + rowfft_tile_rows<N>(g.ncol) * K::CH * 16;
   auto kern = k_rowfft_stats<N, CLIP>;
@@ -1326,26 +1350,22 @@ cudaError_t run_rowfft_stats_k(const SegmentGeom& g, const DevTables& tb, const 
   CUtensorMap none;
   memset(&none, 0, sizeof(none));
   return launch_with(kern, dim3((unsigned)grid), dim3(K::THREADS_B), smem, st, pl, g, tb, Tbuf, nimg, img_base,
-                     weight, partials, images, tma ? tm->map : none, tma ? tm->nbox : 0, tma ? tm->rows : 0, err,
-                     clip);
+                     weight, ps, images, tma ? tm->map : none, tma ? tm->nbox : 0, tma ? tm->rows : 0, err);
 }
 
 template <int N>
 cudaError_t run_rowfft_stats(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, int nimg,
-                             int img_base, const double* weight, StatPartial* partials, float* images,
-                             const TileMap* tm, int* err, cudaStream_t st, const float2* clip,
-                             const PassLaunch* pl) {
-  if (clip != nullptr)
-    return run_rowfft_stats_k<N, true>(g, tb, Tbuf, nimg, img_base, weight, partials, images, tm, err, st, clip,
-                                       pl);
-  return run_rowfft_stats_k<N, false>(g, tb, Tbuf, nimg, img_base, weight, partials, images, tm, err, st, nullptr,
-                                      pl);
+                             int img_base, const double* weight, const PassStats& ps, float* images,
+                             const TileMap* tm, int* err, cudaStream_t st, const PassLaunch* pl) {
+  if (ps.clip != nullptr)
+    return run_rowfft_stats_k<N, true>(g, tb, Tbuf, nimg, img_base, weight, ps, images, tm, err, st, pl);
+  return run_rowfft_stats_k<N, false>(g, tb, Tbuf, nimg, img_base, weight, ps, images, tm, err, st, pl);
 }
 
 template <int N, bool CLIP>
 cudaError_t run_rowfft_tree_k(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Quad* quads,
-                              int nquads, int img_base, int base_base, StatPartial* partials, const TileMap* tm,
-                              int* err, cudaStream_t st, const float2* clip, const PassLaunch* pl) {
+                              int nquads, int img_base, int base_base, const PassStats& ps, const TileMap* tm,
+                              int* err, cudaStream_t st, const PassLaunch* pl) {
   using K = ImgCfg<N>;
   const int smem = K::SMEM_B_FIXED + (K::TILE_TMA ? 1024 : 0) + rowfft_tile_rows<N>(g.ncol) * K::CH * 16;
   auto kern = k_rowfft_tree<N, CLIP>;
@@ -1368,20 +1388,17 @@ cudaError_t run_rowfft_tree_k(const SegmentGeom& g, const DevTables& tb, const f
   CUtensorMap none;
   memset(&none, 0, sizeof(none));
   return launch_with(kern, dim3((unsigned)grid), dim3(K::THREADS_B), smem, st, pl, g, tb, Tbuf, quads, nquads,
-                     img_base, base_base, partials, tma ? tm->map : none, tma ? tm->nbox : 0, tma ? tm->rows : 0, err,
-                     clip);
+                     img_base, base_base, ps, tma ? tm->map : none, tma ? tm->nbox : 0, tma ? tm->rows : 0, err);
 }
 
 template <int N>
 cudaError_t run_rowfft_tree(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Quad* quads,
-                            int nquads, int img_base, int base_base, StatPartial* partials, const TileMap* tm,
-                            int* err, cudaStream_t st, const float2* clip, const PassLaunch* pl) {
+                            int nquads, int img_base, int base_base, const PassStats& ps, const TileMap* tm,
+                            int* err, cudaStream_t st, const PassLaunch* pl) {
   static_assert(N >= kTreeMinNpix, "whole warps");
-  if (clip != nullptr)
-    return run_rowfft_tree_k<N, true>(g, tb, Tbuf, quads, nquads, img_base, base_base, partials, tm, err, st, clip,
-                                      pl);
-  return run_rowfft_tree_k<N, false>(g, tb, Tbuf, quads, nquads, img_base, base_base, partials, tm, err, st, nullptr,
-                                     pl);
+  if (ps.clip != nullptr)
+    return run_rowfft_tree_k<N, true>(g, tb, Tbuf, quads, nquads, img_base, base_base, ps, tm, err, st, pl);
+  return run_rowfft_tree_k<N, false>(g, tb, Tbuf, quads, nquads, img_base, base_base, ps, tm, err, st, pl);
 }
 
 template <int N>
@@ -1406,15 +1423,15 @@ void fill_shape(ImageKernelShape* o) {
                                      const float2*, float2*, float*, float*, cudaStream_t,                  \
                                      const PassLaunch*);                                                    \
   template cudaError_t run_rowfft_stats<N>(const SegmentGeom&, const DevTables&, const float2*, int, int,    \
-                                           const double*, StatPartial*, float*, const TileMap*, int*,       \
-                                           cudaStream_t, const float2*, const PassLaunch*);                 \
+                                           const double*, const PassStats&, float*, const TileMap*, int*,   \
+                                           cudaStream_t, const PassLaunch*);                                \
   template void fill_shape<N>(ImageKernelShape*);                                                           \
   template cudaError_t run_rowfft_power<N>(const SegmentGeom&, const DevTables&, const float2*, const int4*, \
                                            int, StatPartial*, const TileMap*, int*, cudaStream_t);
 
 #define RF_INSTANTIATE_TREE(N)                                                                               \
   template cudaError_t run_rowfft_tree<N>(const SegmentGeom&, const DevTables&, const float2*, const Quad*,  \
-                                          int, int, int, StatPartial*, const TileMap*, int*, cudaStream_t,   \
-                                          const float2*, const PassLaunch*);
+                                          int, int, int, const PassStats&, const TileMap*, int*,             \
+                                          cudaStream_t, const PassLaunch*);
 
 }  // namespace rf

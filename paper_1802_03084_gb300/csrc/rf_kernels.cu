@@ -420,11 +420,11 @@ cudaError_t launch_weights(const int4* img_info, int nimg, bool partial, const S
 }
 
 // --------------------------------------------------------------- finalize --
-// Per image: reduce the row-block partials (FP64), then
-//   mean = sum / N^2,  sigma = sqrt(sum_sq / N^2 - mean^2)  (population),
+// Per image: mean and sigma = sqrt(mean of I^2 - mean^2) (population) come
+// from k_image_noise, or with the clipped noise from the kept-pixel partials;
 //   peak = max pixel (lowest y N + x on ties),  snr = peak / sigma,
-// and append a candidate iff snr >= threshold (Sec. 3.1).  Raw pixel sums are
-// scaled by 1 / (2 W) here.
+// and a candidate is appended iff snr >= threshold (Sec. 3.1).  Raw pixel
+// values are scaled by 1 / (2 W) here.
 __device__ __forceinline__ void fmax_merge(float& m, int& i, float m2, int i2) {
   if (m2 > m || (m2 == m && i2 < i)) {
     m = m2;
@@ -442,56 +442,78 @@ __device__ __forceinline__ double parseval_sum(const float* __restrict__ cs, int
   return sq;
 }
 
-// One warp per image slot: the clipping window {mean, kClipSigmas sigma} of
-// the raw image J = 2W I.  mean(J) = Re G(0, 0) and mean(J^2) = the sum of
-// |G|^2 over the full plane (Parseval), so var(J) = sum - mean^2.
-__global__ void k_clip_window(int ncol, const float* __restrict__ colsq, const float* __restrict__ mean0, int nimg,
-                              float2* __restrict__ clip) {
+// One warp per image slot: mean and noise of the image from its Parseval sums
+// (mean = G(0, 0) / 2W; mean of I^2 = sum over the full plane of |G|^2 /
+// 4W^2), so that they are known before the row pass.  gate[i]: no raw maximum
+// below it reaches the threshold (threshold * sigma in raw units, lowered by
+// far more than its rounding).  clip[i]: the clipping window {mean, kClipSigmas
+// sigma} of the raw image J = 2W I.
+__global__ void k_image_noise(int ncol, const float* __restrict__ colsq, const float* __restrict__ mean0,
+                              const double* __restrict__ weight, int nimg, int img_base, double threshold,
+                              ImgNoise* __restrict__ noise, float* __restrict__ gate, float2* __restrict__ clip) {
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (i >= nimg) return;
   const double sq = parseval_sum(colsq + (size_t)i * ncol, ncol, lane);
   if (lane != 0) return;
   const float m = mean0[i];
-  double var = sq - (double)m * (double)m;
+  const double W = weight[img_base + i];
+  const double inv = W > 0.0 ? 0.5 / W : 0.0;
+  const double mean = (double)m * inv;
+  double var = sq * inv * inv - mean * mean;
   var = var > 0.0 ? var : 0.0;
-  clip[i] = make_float2(m, (float)(kClipSigmas * sqrt(var)));
+  const double sigma = sqrt(var);
+  noise[i] = ImgNoise{mean, sigma};
+  if (gate != nullptr) gate[i] = (float)(threshold * sigma * (2.0 * W) * (1.0 - 1e-5));
+  if (clip != nullptr) {
+    double raw = sq - (double)m * (double)m;
+    raw = raw > 0.0 ? raw : 0.0;
+    clip[i] = make_float2(m, (float)(kClipSigmas * sqrt(raw)));
+  }
 }
 
-cudaError_t launch_clip_window(const SegmentGeom& g, const float* colsq, const float* mean0, int nimg, float2* clip,
+cudaError_t launch_image_noise(const SegmentGeom& g, const float* colsq, const float* mean0, const double* weight,
+                               int nimg, int img_base, double threshold, ImgNoise* noise, float* gate, float2* clip,
                                cudaStream_t st) {
   if (nimg <= 0) return cudaSuccess;
-  k_clip_window<<<(nimg + 7) / 8, 256, 0, st>>>(g.ncol, colsq, mean0, nimg, clip);
+  k_image_noise<<<(nimg + 7) / 8, 256, 0, st>>>(g.ncol, colsq, mean0, weight, nimg, img_base, threshold, noise, gate,
+                                                clip);
   return cudaGetLastError();
 }
 
-__global__ void k_finalize(int npix, int nrb, int ncol, const StatPartial* __restrict__ partials,
-                           const float* __restrict__ colsq, const float* __restrict__ mean0,
-                           const int4* __restrict__ img_info, const double* __restrict__ weight, int nimg,
-                           int img_base, double threshold, DevCand* __restrict__ cands, int* __restrict__ ncand,
-                           int cand_cap, DevStat* __restrict__ stats, int clip) {
+__global__ void k_finalize(int npix, int nrb, const PassStats ps, const ImgNoise* __restrict__ noise,
+                           const float* __restrict__ mean0, const int4* __restrict__ img_info,
+                           const double* __restrict__ weight, int nimg, int img_base, double threshold,
+                           DevCand* __restrict__ cands, int* __restrict__ ncand, int cand_cap,
+                           DevStat* __restrict__ stats) {
   // one warp per image; lanes stride over the row-pair partials (peak, and
-  // the kept-pixel sums of the clipped noise) and the per-column Parseval
-  // sums (FP64), then an xor-tree (fixed order) combines them
+  // the kept-pixel sums of the clipped noise, FP64), then an xor-tree (fixed
+  // order) combines them
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (i >= nimg) return;
   const int img = img_base + i;
-  const StatPartial* pp = partials + (size_t)i * nrb;
+  const bool clip = ps.clip != nullptr;
+  const StatPartial* __restrict__ pp = ps.partials + (size_t)i * nrb;
   float mx = -FLT_MAX;
   int mi = INT_MAX;
-  double ks1 = 0.0, ks2 = 0.0;
-  long long kn = 0;
+#pragma unroll 4
   for (int r = lane; r < nrb; r += 32) {
     const StatPartial p = pp[r];
     fmax_merge(mx, mi, p.max, p.idx);
-    if (clip) {
+  }
+  double ks1 = 0.0, ks2 = 0.0;
+  long long kn = 0;
+  if (clip) {
+    const ClipPartial* __restrict__ cp = ps.cparts + (size_t)i * nrb;
+#pragma unroll 4
+    for (int r = lane; r < nrb; r += 32) {
+      const ClipPartial p = cp[r];
       ks1 += p.sum;
       ks2 += p.sumsq;
       kn += p.kept;
     }
   }
-  const double sq = parseval_sum(colsq + (size_t)i * ncol, ncol, lane);
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     const float om = __shfl_xor_sync(0xffffffffu, mx, off);
@@ -519,19 +541,17 @@ __global__ void k_finalize(int npix, int nrb, int ncol, const StatPartial* __res
     if (stats) stats[info.w] = ds;
     return;
   }
-  // mean = G(0,0) / 2W; mean of I^2 = sum_full |G|^2 / 4W^2 (Parseval)
   const double inv = 0.5 / W;
-  double mean = (double)mean0[i] * inv;
-  double var = sq * inv * inv - mean * mean;
+  double mean = noise[i].mean;
+  double sigma = noise[i].sigma;
   if (clip) {
     // clipped noise: the kept pixels' deviations d from mean0 (raw units)
     const double n = kn > 0 ? (double)kn : 1.0;
     const double m1 = ks1 / n;
     mean = ((double)mean0[i] + m1) * inv;
-    var = (ks2 / n - m1 * m1) * inv * inv;
+    const double var = (ks2 / n - m1 * m1) * inv * inv;
+    sigma = sqrt(var > 0.0 ? var : 0.0);
   }
-  var = var > 0.0 ? var : 0.0;
-  const double sigma = sqrt(var);
   const double peak = (double)mx * inv;
   const double snr = sigma > 0.0 ? peak / sigma : 0.0;
   const int y = mi / npix;
@@ -560,16 +580,14 @@ __global__ void k_finalize(int npix, int nrb, int ncol, const StatPartial* __res
   }
 }
 
-cudaError_t launch_finalize(const SegmentGeom& g, const StatPartial* partials, const float* colsq,
-                            const float* mean0, const int4* img_info, const double* weight, int nimg, int img_base,
-                            double threshold, DevCand* cands, int* ncand, int cand_cap, DevStat* stats,
-                            cudaStream_t st, bool clip) {
+cudaError_t launch_finalize(const SegmentGeom& g, const PassStats& ps, const ImgNoise* noise, const float* mean0,
+                            const int4* img_info, const double* weight, int nimg, int img_base, double threshold,
+                            DevCand* cands, int* ncand, int cand_cap, DevStat* stats, cudaStream_t st) {
   if (nimg <= 0) return cudaSuccess;
   ImageKernelShape sh;
   if (!image_kernel_shape(g.npix, &sh)) return cudaErrorInvalidValue;
-  const int nrb = sh.partials_per_image;
-  k_finalize<<<(nimg + 7) / 8, 256, 0, st>>>(g.npix, nrb, g.ncol, partials, colsq, mean0, img_info, weight, nimg,
-                                              img_base, threshold, cands, ncand, cand_cap, stats, clip ? 1 : 0);
+  k_finalize<<<(nimg + 7) / 8, 256, 0, st>>>(g.npix, sh.partials_per_image, ps, noise, mean0, img_info, weight, nimg,
+                                              img_base, threshold, cands, ncand, cand_cap, stats);
   return cudaGetLastError();
 }
 
@@ -579,11 +597,10 @@ cudaError_t run_colfft(const SegmentGeom&, const DevTables&, const Group*, int, 
                        float*, float*, cudaStream_t, const PassLaunch*);
 template <int N>
 cudaError_t run_rowfft_tree(const SegmentGeom&, const DevTables&, const float2*, const Quad*, int, int, int,
-                            StatPartial*, const TileMap*, int*, cudaStream_t, const float2*, const PassLaunch*);
+                            const PassStats&, const TileMap*, int*, cudaStream_t, const PassLaunch*);
 template <int N>
 cudaError_t run_rowfft_stats(const SegmentGeom&, const DevTables&, const float2*, int, int, const double*,
-                             StatPartial*, float*, const TileMap*, int*, cudaStream_t, const float2*,
-                             const PassLaunch*);
+                             const PassStats&, float*, const TileMap*, int*, cudaStream_t, const PassLaunch*);
 template <int N>
 void fill_shape(ImageKernelShape*);
 template <int N>
@@ -607,13 +624,12 @@ cudaError_t launch_colfft(const SegmentGeom& g, const DevTables& tb, const Group
 }
 
 cudaError_t launch_rowfft_stats(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, int nimg,
-                                int img_base, const double* weight, StatPartial* partials, float* images,
-                                const TileMap* tm, int* err, cudaStream_t st, const float2* clip,
-                                const PassLaunch* pl) {
+                                int img_base, const double* weight, const PassStats& ps, float* images,
+                                const TileMap* tm, int* err, cudaStream_t st, const PassLaunch* pl) {
   switch (g.npix) {
 #define RF_CASE(N) \
   case N:          \
-    return run_rowfft_stats<N>(g, tb, Tbuf, nimg, img_base, weight, partials, images, tm, err, st, clip, pl);
+    return run_rowfft_stats<N>(g, tb, Tbuf, nimg, img_base, weight, ps, images, tm, err, st, pl);
     RF_FOR_EACH_N(RF_CASE)
 #undef RF_CASE
     default:
@@ -622,12 +638,12 @@ cudaError_t launch_rowfft_stats(const SegmentGeom& g, const DevTables& tb, const
 }
 
 cudaError_t launch_rowfft_tree(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Quad* quads,
-                               int nquads, int img_base, int base_base, StatPartial* partials, const TileMap* tm,
-                               int* err, cudaStream_t st, const float2* clip, const PassLaunch* pl) {
+                               int nquads, int img_base, int base_base, const PassStats& ps, const TileMap* tm,
+                               int* err, cudaStream_t st, const PassLaunch* pl) {
   switch (g.npix) {
 #define RF_CASE(N)                                                                                                 \
   case N:                                                                                                          \
-    return run_rowfft_tree<N>(g, tb, Tbuf, quads, nquads, img_base, base_base, partials, tm, err, st, clip, pl);
+    return run_rowfft_tree<N>(g, tb, Tbuf, quads, nquads, img_base, base_base, ps, tm, err, st, pl);
     RF_CASE(64) RF_CASE(128) RF_CASE(256) RF_CASE(512) RF_CASE(1024) RF_CASE(2048) RF_CASE(4096) RF_CASE(8192)
 #undef RF_CASE
     default:

@@ -207,7 +207,9 @@ cudaError_t run_noalloc(const float2* grid, double weight, const DeviceSetup& d,
   DevTables tb{};
   tb.twiddle = tw;
   tb.twiddle_col = tw;
-  e = launch_rowfft_stats(g, tb, T, 1, 0, nullptr, partials, nullptr, nullptr, nullptr, st);
+  PassStats ps;
+  ps.partials = partials;
+  e = launch_rowfft_stats(g, tb, T, 1, 0, nullptr, ps, nullptr, nullptr, nullptr, st);
   if (e != cudaSuccess) return e;
   k_noalloc_finalize<<<1, 32, 0, st>>>(partials, K::PARTIALS, colsq, mean0, N, weight, out);
   return cudaGetLastError();
