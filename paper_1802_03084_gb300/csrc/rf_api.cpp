@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <cmath>
 #include <cstdarg>
@@ -67,7 +68,7 @@ struct Wave {
   int g_begin, g_end;
   int img_begin, img_end;    // image list
   int base_begin, base_end;  // transformed images
-  int quad_begin, quad_end;
+  int unit_begin, unit_end;
 };
 
 // Restores the caller's current device on scope exit.
@@ -220,10 +221,12 @@ struct rf_plan {
   rf::ImageKernelShape shape{};
   // Widths whose images are sums of two or four images of another width of
   // the plan (see build_widths): sum_of[s] is that width's index (s itself for
-  // a width with transforms of its own), sum_level[s] 0, 1 (two) or 2 (four),
-  // and sum2[s] / sum4[s] the widths made from width s (-1: none).
-  std::vector<int> sum_of, sum_level, sum2, sum4;
+  // a width with transforms of its own), and sums[s][L - 1] the width made of
+  // 2^L images of width s (-1: none).
+  std::vector<int> sum_of;
+  std::vector<std::array<int, 4>> sums;
   bool derived = false;      // some width is such a sum
+  bool pairs = false;        // some width is a sum of 8 or 16 (see pairs_possible)
   double base_share = 1.0;   // share of a long trial set's images that are transformed
 
   // device state
@@ -252,6 +255,8 @@ struct rf_plan {
   rf::TileMap tmap_T{};         // tensor map of d_T for the row pass (nbox 0: none)
   rf::TileMap tmap_P{};         // tensor map of d_T for the periodicity row pass (N = 1024)
   rf::TileMap tmap_H[2]{};      // tensor maps of the two halves of d_T (overlapped waves)
+  rf::TileMap tmap_D{};         // tensor maps of d_T and its halves in duo order, for units of image pairs
+  rf::TileMap tmap_DH[2]{};
   float2* d_stage = nullptr;
   int stage_nint = 0;
 
@@ -262,8 +267,8 @@ struct rf_plan {
   int t_span = 0;
   std::vector<int4> img_info;
   std::vector<Group> groups;
-  std::vector<rf::Quad> quads;  // of the transformed images, where widths are sums of others
-  rf::Quad* d_quads = nullptr;
+  std::vector<rf::Unit> units;  // of the transformed images, where widths are sums of others
+  rf::Unit* d_units = nullptr;
   std::vector<Wave> waves;
   bool cached_plain = false;    // the lists are the plain form's (every image on its own)
   int gslots_max = 0;           // groups per wave (cell buffer capacity)
@@ -272,6 +277,7 @@ struct rf_plan {
   float* d_mean0 = nullptr;     // [slots] Re H(0, 0)
   rf::ImgNoise* d_noise = nullptr;  // [sslots] mean and noise from the Parseval sums
   float* d_gate = nullptr;      // [sslots] least raw maximum of a candidate
+  unsigned long long* d_best = nullptr;  // [sslots] largest pixel that reaches it
   float2* d_clip = nullptr;     // [sslots] clipping window (RF_NOISE_CLIPPED only)
   rf::ClipPartial* d_cparts = nullptr;  // kept-pixel partials (RF_NOISE_CLIPPED only)
   rf::PlainBuffers plain{};     // allocated on the first plain-form search
@@ -388,11 +394,9 @@ int64_t count_images(const rf_plan* p, int nint) {
 void build_widths(rf_plan* p) {
   const int n = p->ndt;
   p->sum_of.resize(n);
-  p->sum_level.assign(n, 0);
-  p->sum2.assign(n, -1);
-  p->sum4.assign(n, -1);
+  p->sums.assign(n, {-1, -1, -1, -1});
   for (int k = 0; k < n; ++k) p->sum_of[k] = k;
-  p->derived = false;
+  p->derived = p->pairs = false;
   if (p->npix >= rf::kTreeMinNpix) {
     std::vector<int> order(n);
     for (int k = 0; k < n; ++k) order[k] = k;
@@ -401,14 +405,14 @@ void build_widths(rf_plan* p) {
     for (int b : order) {
       if (taken[b]) continue;
       taken[b] = 1;
-      for (int lv = 1; lv <= 2; ++lv)
+      for (int lv = 1; lv <= (rf::pairs_possible(p->npix) ? 4 : 2); ++lv)
         for (int k : order)
           if (!taken[k] && p->dt[k] == p->dt[b] << lv) {
             taken[k] = 1;
             p->sum_of[k] = b;
-            p->sum_level[k] = lv;
-            (lv == 1 ? p->sum2 : p->sum4)[b] = k;
+            p->sums[b][lv - 1] = k;
             p->derived = true;
+            p->pairs |= lv > 2;
             break;
           }
     }
@@ -662,8 +666,13 @@ rf_status build_tables(rf_plan* p) {
   return RF_OK;
 }
 
-// A group with its sums of two and four: at most this many images.
-int group_images(const rf_plan* p) { return p->shape.images_per_group * (p->derived ? 7 : 4) / 4; }
+// A group with its sums: at most this many images.
+int group_images(const rf_plan* p) { return p->shape.images_per_group * (p->derived ? 2 : 1); }
+
+// Row-pass partials per image: the most that any of the plan's row passes writes.
+size_t plan_partials(const rf_plan* p) {
+  return rf::unit_partials(p->shape, p->pairs);
+}
 
 // Transformed images and image records of a wave of `slots` images (two whole
 // groups at least, so that a half of either holds one, see run_waves_overlapped).
@@ -688,9 +697,9 @@ bool overlap_possible(const rf_plan* p) {
          p->tslots / 2 >= p->shape.images_per_group && p->sslots / 2 >= group_images(p);
 }
 
-// Image, group and quad lists for a segment of nint integrations: trial by
+// Image, group and unit lists for a segment of nint integrations: trial by
 // trial (d, width with transforms of its own), in groups of up to 32 t', each
-// group's images followed by its sums of two and of four.  img_info[].w is an
+// group's images followed by its sums of two, of four and so on.  img_info[].w is an
 // image's place in (d, s, t') order.  The plain form takes every width on its
 // own in (d, s, t') order.
 void build_lists(rf_plan* p, int nint) {
@@ -698,7 +707,7 @@ void build_lists(rf_plan* p, int nint) {
   const bool plain = p->form == RF_FORM_PLAIN;
   p->img_info.clear();
   p->groups.clear();
-  p->quads.clear();
+  p->units.clear();
   p->waves.clear();
   std::vector<int> first(p->ndt);  // (d, s, t') place of each width's first image
   int place = 0, nbase = 0;
@@ -710,7 +719,6 @@ void build_lists(rf_plan* p, int nint) {
     for (int s = 0; s < p->ndt; ++s) {
       const bool tree = p->derived && !plain;
       if (tree && p->sum_of[s] != s) continue;
-      const int s2 = tree ? p->sum2[s] : -1, s4 = tree ? p->sum4[s] : -1;
       const int nt = n_times(p, nint, d, s);
       for (int t0 = 0; t0 < nt; t0 += B) {
         Group g{};
@@ -726,14 +734,11 @@ void build_lists(rf_plan* p, int nint) {
           return i;
         };
         g.img0 = list(s, t0, g.nimg);
-        if (s2 >= 0) {
-          g.n1 = g.nimg / 2;
-          g.img1 = list(s2, t0 / 2, g.n1);
-        }
-        if (s4 >= 0) {
-          g.n2 = g.nimg / 4;
-          g.img2 = list(s4, t0 / 4, g.n2);
-        }
+        for (int lv = 1; tree && lv <= 4; ++lv)
+          if (p->sums[s][lv - 1] >= 0) {
+            g.nsum[lv - 1] = g.nimg >> lv;
+            g.isum[lv - 1] = list(p->sums[s][lv - 1], t0 >> lv, g.nimg >> lv);
+          }
         p->groups.push_back(g);
       }
     }
@@ -745,31 +750,31 @@ void build_lists(rf_plan* p, int nint) {
   Wave w{};
   for (int gi = 0; gi < (int)p->groups.size(); ++gi) {
     const Group& g = p->groups[gi];
-    const int q0 = (int)p->quads.size();
-    const int img_end = g.img0 + g.nimg + g.n1 + g.n2;
+    const int q0 = (int)p->units.size();
+    const int img_end = g.img0 + g.nimg + g.nsum[0] + g.nsum[1] + g.nsum[2] + g.nsum[3];
     if (g.base0 + g.nimg - w.base_begin > tcap || img_end - w.img_begin > scap || gi - w.g_begin >= p->gslots_max) {
       w.g_end = gi;
       w.img_end = g.img0;
       w.base_end = g.base0;
-      w.quad_end = q0;
+      w.unit_end = q0;
       p->waves.push_back(w);
       w = Wave{gi, gi, g.img0, g.img0, g.base0, g.base0, q0, q0};
     }
     if (p->derived && !plain)
-      for (int k = 0; k < g.nimg; k += 4) {
-        rf::Quad q{};
+      for (int k = 0, step = rf::unit_images(p->pairs); k < g.nimg; k += step) {
+        rf::Unit q{};
         q.base = g.base0 + k;
-        q.n = std::min(4, g.nimg - k);
-        q.img = g.img0 + k;
-        q.img1 = k / 2 < g.n1 ? g.img1 + k / 2 : -1;
-        q.img2 = k / 4 < g.n2 ? g.img2 + k / 4 : -1;
-        p->quads.push_back(q);
+        q.n = std::min(step, g.nimg - k);
+        q.img[0] = g.img0 + k;
+        for (int lv = 1; lv <= 4; ++lv)
+          q.img[lv] = k >> lv < g.nsum[lv - 1] ? g.isum[lv - 1] + (k >> lv) : -1;
+        p->units.push_back(q);
       }
   }
   w.g_end = (int)p->groups.size();
   w.img_end = (int)p->img_info.size();
   w.base_end = nbase;
-  w.quad_end = (int)p->quads.size();
+  w.unit_end = (int)p->units.size();
   if (w.img_end > w.img_begin) p->waves.push_back(w);
   p->cached_nint = nint;
   p->cached_span = p->t_span;
@@ -801,7 +806,8 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 // `rows` u rows; box rows of 128, 64 or 32 bytes are swizzled in that mode.
 // The search's row pass takes the 2 XB rows of a work item (trows = 2 XB),
 // the periodicity row pass the XB rows of one image (trows = XB).
-void encode_tile_map(rf_plan* p, rf::TileMap& tm, float2* base, int slots, int trows) {
+// `duo`: not swizzled, T is in duo order.
+void encode_tile_map(rf_plan* p, rf::TileMap& tm, float2* base, int slots, int trows, bool duo = false) {
   tm.nbox = 0;
   const int N = p->npix;
   if (N < 1024 || !base || slots <= 0) return;
@@ -814,7 +820,8 @@ void encode_tile_map(rf_plan* p, rf::TileMap& tm, float2* base, int slots, int t
   const cuuint64_t strides[2] = {(cuuint64_t)N * 8, (cuuint64_t)p->ncol * N * 8};
   const cuuint32_t box[3] = {(cuuint32_t)(2 * trows), (cuuint32_t)rows, 1};
   const cuuint32_t es[3] = {1, 1, 1};
-  const CUtensorMapSwizzle sw = row_bytes == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
+  const CUtensorMapSwizzle sw = duo                ? CU_TENSOR_MAP_SWIZZLE_NONE
+                                : row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
                                 : row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
                                 : row_bytes == 32 ? CU_TENSOR_MAP_SWIZZLE_32B
                                                   : CU_TENSOR_MAP_SWIZZLE_NONE;
@@ -833,10 +840,11 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
   const int B = p->shape.images_per_group;
   slots = std::max(std::min(slots, 32768), B);
   const size_t per_slot = (size_t)p->ncol * p->npix;
-  const int nrb = p->shape.partials_per_image;
+  const size_t nrb = plan_partials(p);
   p->tmap_T.nbox = 0;  // the maps describe d_T, about to be freed
   p->tmap_P.nbox = 0;
   p->tmap_H[0].nbox = p->tmap_H[1].nbox = 0;
+  p->tmap_D.nbox = p->tmap_DH[0].nbox = p->tmap_DH[1].nbox = 0;
   if (p->d_T) {
     p->device_bytes -= (uint64_t)p->tslots * per_slot * sizeof(float2);
     p->dfree(p->d_T);
@@ -868,6 +876,11 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
     p->dfree(p->d_gate);
     p->d_gate = nullptr;
   }
+  if (p->d_best) {
+    p->device_bytes -= (uint64_t)p->sslots * 8;
+    p->dfree(p->d_best);
+    p->d_best = nullptr;
+  }
   if (p->d_clip) {
     p->device_bytes -= (uint64_t)p->sslots * sizeof(float2);
     p->dfree(p->d_clip);
@@ -894,8 +907,9 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
   if (p->flags & RF_NOISE_CLIPPED) {
     if ((s = p->dalloc(&p->d_clip, (size_t)p->sslots)) != RF_OK) return s;
     if ((s = p->dalloc(&p->d_cparts, (size_t)p->sslots * nrb)) != RF_OK) return s;
-  } else if ((s = p->dalloc(&p->d_gate, (size_t)p->sslots)) != RF_OK) {
-    return s;
+  } else {
+    if ((s = p->dalloc(&p->d_gate, (size_t)p->sslots)) != RF_OK) return s;
+    if ((s = p->dalloc(&p->d_best, (size_t)p->sslots)) != RF_OK) return s;
   }
   const int xb = std::min(256 / (p->npix / 32), p->npix / 2);  // row pairs of a row-pass work item
   encode_tile_map(p, p->tmap_T, p->d_T, p->tslots, 2 * xb);
@@ -908,6 +922,13 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
   // the periodicity row pass's tensor-copy tiles (one image's XB rows), at
   // N = 1024, where its transforms fit one warp
   if (p->npix == 1024) encode_tile_map(p, p->tmap_P, p->d_T, p->tslots, xb);
+  if (p->pairs) {
+    encode_tile_map(p, p->tmap_D, p->d_T, p->tslots, xb, true);
+    if (half >= B) {
+      encode_tile_map(p, p->tmap_DH[0], p->d_T, half, xb, true);
+      encode_tile_map(p, p->tmap_DH[1], p->d_T + (size_t)half * per_slot, half, xb, true);
+    }
+  }
   return RF_OK;
 }
 
@@ -934,20 +955,20 @@ uint64_t estimate_device_bytes(const rf_plan* p, int slots) {
   b += r(p->dt.size(), 8) + r(p->dt.size(), 4);
   const int64_t img_cap = std::max<int64_t>(count_images(p, p->max_nint), 1);
   b += r(img_cap, sizeof(int4)) + r(img_cap, sizeof(Group)) + r(img_cap, 8) + r(img_cap, sizeof(DevCand)) + 4 + 4;  // candidate count, error flag
-  if (p->derived) b += r(img_cap, sizeof(rf::Quad));
+  if (p->derived) b += r(img_cap, sizeof(rf::Unit));
   const size_t per_slot = (size_t)p->ncol * N * sizeof(float2);
   if (slots <= 0) slots = default_slots(p, (size_t)img_cap);
   const int B = p->shape.images_per_group;
   slots = std::max(std::min(slots, 32768), B);
   const int tslots = wave_tslots(p, slots), sslots = wave_sslots(p, slots);
   const int gslots = std::max(2 * ((tslots + B - 1) / B), 1);
-  b += r((size_t)tslots * per_slot, 1) + r((size_t)sslots * p->shape.partials_per_image, sizeof(StatPartial)) +
+  b += r((size_t)tslots * per_slot, 1) + r((size_t)sslots * plan_partials(p), sizeof(StatPartial)) +
        r((size_t)gslots * std::max(p->n_cells, 1) * 32, sizeof(float2)) + r((size_t)sslots * p->ncol, 4) +
        r(sslots, 4) + r(sslots, sizeof(rf::ImgNoise));
   if (p->flags & RF_NOISE_CLIPPED)
-    b += r(sslots, sizeof(float2)) + r((size_t)sslots * p->shape.partials_per_image, sizeof(rf::ClipPartial));
+    b += r(sslots, sizeof(float2)) + r((size_t)sslots * plan_partials(p), sizeof(rf::ClipPartial));
   else
-    b += r(sslots, sizeof(float));
+    b += r(sslots, sizeof(float)) + r(sslots, 8);
   const size_t per_int = rows * p->npol * sizeof(float2);
   const size_t stage_nint = std::max<size_t>(1, std::min<size_t>(kStageBytes / per_int, (size_t)p->max_nint));
   b += r(stage_nint * per_int, 1);
@@ -1058,7 +1079,7 @@ rf_status alloc_device(rf_plan* p) {
   RF_CUDA(cudaMemset(p->d_err, 0, sizeof(int)));
 
   // column-FFT scratch, whole groups per wave
-  if (p->derived && (s = p->dalloc(&p->d_quads, (size_t)p->img_cap)) != RF_OK) return s;
+  if (p->derived && (s = p->dalloc(&p->d_units, (size_t)p->img_cap)) != RF_OK) return s;
   if ((s = alloc_wave_scratch(p, default_slots(p, (size_t)p->img_cap))) != RF_OK) return s;
 
   // host->device staging of raw visibilities
@@ -1202,46 +1223,55 @@ rf_status run_waves_overlapped(rf_plan* p, const SegmentGeom& g, const std::vect
   return RF_OK;
 }
 
-// The row pass of one wave: over quads where the plan has widths that are sums
+// The row pass of one wave: over units where the plan has widths that are sums
 // of others (never for listed trials, whose images `im` takes), else image by
 // image.
 cudaError_t launch_row_pass(rf_plan* p, const SegmentGeom& g, const Wave& w, const float2* T, const rf::PassStats& ps,
                             const rf::TileMap* tm, float* im, cudaStream_t st, const rf::PassLaunch* pl) {
   if (tm->nbox == 0) tm = nullptr;
-  if (w.quad_end > w.quad_begin)
-    return rf::launch_rowfft_tree(g, p->tb, T, p->d_quads + w.quad_begin, w.quad_end - w.quad_begin, w.img_begin,
-                                  w.base_begin, ps, tm, p->d_err, st, pl);
+  if (w.unit_end > w.unit_begin)
+    return rf::launch_rowfft_tree(g, p->tb, T, p->d_units + w.unit_begin, w.unit_end - w.unit_begin, p->pairs,
+                                  w.img_begin, w.base_begin, ps, tm, p->d_err, st, pl);
   return rf::launch_rowfft_stats(g, p->tb, T, w.img_end - w.img_begin, w.img_begin, p->d_weight, ps, im, tm, p->d_err,
                                  st, pl);
 }
 
+// Whether a wave's column-FFT output is in duo order.
+bool wave_duo(const rf_plan* p, const Wave& w) { return w.unit_end > w.unit_begin && p->pairs; }
+
 // Everything after a wave's column pass, on `st`: the images' noise, the row
 // pass and the finalisation, with the wave's slots of the scratch starting at
-// slot0 (colsq, mean0 and the statistics' buffers).  Every image's peak
-// position is wanted where statistics or images are returned; else the row
-// pass looks for it only in what can become a candidate (not under the clipped
-// noise, which is known only after the row pass).
+// slot0 (colsq, mean0 and the statistics' buffers).  Every image's peak is
+// wanted where statistics or images are returned; else the row pass keeps only
+// what can become a candidate (not under the clipped noise, which is known only
+// after the row pass).
 rf_status finish_wave(rf_plan* p, const SegmentGeom& g, const Wave& w, const float2* T, size_t slot0,
-                      const rf::TileMap* tm, DevStat* d_stats, float* im, cudaStream_t st,
+                      const rf::TileMap* tm_rows, const rf::TileMap* tm_duo, DevStat* d_stats, float* im, cudaStream_t st,
                       const rf::PassLaunch* pl) {
-  const size_t nrb = (size_t)p->shape.partials_per_image;
+  const bool units = w.unit_end > w.unit_begin;
+  const rf::TileMap* tm = wave_duo(p, w) ? tm_duo : tm_rows;
+  const size_t nparts = units ? plan_partials(p) : p->shape.partials_per_image;
   const int ni = w.img_end - w.img_begin;
   const float* colsq = p->d_colsq + slot0 * p->ncol;
   const float* mean0 = p->d_mean0 + slot0;
   rf::ImgNoise* noise = p->d_noise + slot0;
   const bool clip = (p->flags & RF_NOISE_CLIPPED) != 0;
   float2* cw = clip ? p->d_clip + slot0 : nullptr;
-  float* gate = clip || d_stats || im ? nullptr : p->d_gate + slot0;
+  const bool only_cands = !clip && !d_stats && !im;
+  float* gate = only_cands ? p->d_gate + slot0 : nullptr;
+  unsigned long long* best = only_cands ? p->d_best + slot0 : nullptr;
   RF_TIMED(p->prof, K_IMAGE_NOISE, st,
-           rf::launch_image_noise(g, colsq, mean0, p->d_weight, ni, w.img_begin, p->threshold, noise, gate, cw, st));
+           rf::launch_image_noise(g, colsq, mean0, p->d_weight, ni, w.img_begin, p->threshold, noise, gate, best,
+                                  cw, st));
   rf::PassStats ps;
-  ps.partials = p->d_partials + slot0 * nrb;
+  ps.partials = p->d_partials + slot0 * plan_partials(p);
   ps.gate = gate;
+  ps.best = best;
   ps.clip = cw;
-  ps.cparts = clip ? p->d_cparts + slot0 * nrb : nullptr;
+  ps.cparts = clip ? p->d_cparts + slot0 * plan_partials(p) : nullptr;
   RF_TIMED(p->prof, K_ROWFFT_STATS, st, launch_row_pass(p, g, w, T, ps, tm, im, st, pl));
   RF_TIMED(p->prof, K_FINALIZE, st,
-           rf::launch_finalize(g, ps, noise, mean0, p->d_img_info, p->d_weight, ni, w.img_begin, p->threshold,
+           rf::launch_finalize(g, ps, (int)nparts, noise, mean0, p->d_img_info, p->d_weight, ni, w.img_begin, p->threshold,
                                p->d_cands, p->d_ncand, p->img_cap, d_stats, st));
   return RF_OK;
 }
@@ -1264,10 +1294,10 @@ rf_status overlapped_loop(rf_plan* p, const SegmentGeom& g, const std::vector<Wa
     if (wi >= 2) RF_CUDA(cudaStreamWaitEvent(st, p->oev[2 + h], 0));
     RF_TIMED(p->prof, K_GRID_COLFFT, st,
              rf::launch_colfft(g, p->tb, p->d_groups, w.g_begin, ng, w.img_begin, w.base_begin, p->d_cellbuf, T,
-                               colsq, mean0, st, &pc));
+                               colsq, mean0, wave_duo(p, w), st, &pc));
     RF_CUDA(cudaEventRecord(p->oev[h], st));
     RF_CUDA(cudaStreamWaitEvent(so, p->oev[h], 0));
-    const rf_status s = finish_wave(p, g, w, T, h * shalf, &p->tmap_H[h], d_stats, nullptr, so, &pr);
+    const rf_status s = finish_wave(p, g, w, T, h * shalf, &p->tmap_H[h], &p->tmap_DH[h], d_stats, nullptr, so, &pr);
     if (s != RF_OK) return s;
     RF_CUDA(cudaEventRecord(p->oev[2 + h], so));
   }
@@ -1290,9 +1320,9 @@ rf_status run_waves(rf_plan* p, int nint, const std::vector<Wave>& waves, int ni
              rf::launch_grid_cells(g, p->tb, p->d_groups, w.g_begin, ng, p->d_cellbuf, st));
     RF_TIMED(p->prof, K_GRID_COLFFT, st,
              rf::launch_colfft(g, p->tb, p->d_groups, w.g_begin, ng, w.img_begin, w.base_begin, p->d_cellbuf,
-                               p->d_T, p->d_colsq, p->d_mean0, st));
+                               p->d_T, p->d_colsq, p->d_mean0, wave_duo(p, w), st));
     float* im = d_images ? d_images + (size_t)w.img_begin * p->npix * p->npix : nullptr;
-    const rf_status s = finish_wave(p, g, w, p->d_T, 0, &p->tmap_T, d_stats, im, st, nullptr);
+    const rf_status s = finish_wave(p, g, w, p->d_T, 0, &p->tmap_T, &p->tmap_D, d_stats, im, st, nullptr);
     if (s != RF_OK) return s;
   }
   return RF_OK;
@@ -1433,8 +1463,8 @@ rf_status search_impl(rf_plan* p, const void* vis, int nint, void* stream, rf_ca
                               cudaMemcpyHostToDevice, st));
       RF_CUDA(cudaMemcpyAsync(p->d_groups, p->groups.data(), p->groups.size() * sizeof(Group),
                               cudaMemcpyHostToDevice, st));
-      if (!p->quads.empty())
-        RF_CUDA(cudaMemcpyAsync(p->d_quads, p->quads.data(), p->quads.size() * sizeof(rf::Quad),
+      if (!p->units.empty())
+        RF_CUDA(cudaMemcpyAsync(p->d_units, p->units.data(), p->units.size() * sizeof(rf::Unit),
                                 cudaMemcpyHostToDevice, st));
     }
   }
@@ -1543,7 +1573,7 @@ rf_status render_core(rf_plan* p, int nint, const int32_t* trials, int n, float*
   std::vector<Group> grp(n);
   for (int k = 0; k < n; ++k) {
     info[k] = make_int4(trials[3 * k], trials[3 * k + 1], trials[3 * k + 2], k);
-    grp[k] = Group{trials[3 * k], trials[3 * k + 1], trials[3 * k + 2], 1, k, k, 0, 0, 0, 0, {0, 0}};
+    grp[k] = Group{trials[3 * k], trials[3 * k + 1], trials[3 * k + 2], 1, k, k, {}, {}, {}};
   }
   p->cached_nint = -1;
   p->drop_graph();
@@ -1982,8 +2012,8 @@ rf_status rf_periodicity_search(rf_plan* p, const void* vis, int32_t nint, int32
           waves.push_back(w);
           w = PW{w.g1, w.g1, nimg, nimg, w.p1, w.p1};
         }
-        grp.push_back(Group{0, 2 * j, kb * B, n, nimg, nimg, 0, 0, 0, 0, {0, 0}});
-        grp.push_back(Group{0, 2 * j + 1, kb * B, n, nimg + n, nimg + n, 0, 0, 0, 0, {0, 0}});
+        grp.push_back(Group{0, 2 * j, kb * B, n, nimg, nimg, {}, {}, {}});
+        grp.push_back(Group{0, 2 * j + 1, kb * B, n, nimg + n, nimg + n, {}, {}, {}});
         for (int i = 0; i < n; ++i)
           pairs.push_back(make_int4(nimg + i - w.i0, nimg + n + i - w.i0, dms[b0 + j], kmin + kb * B + i));
         nimg += 2 * n;
@@ -1999,7 +2029,8 @@ rf_status rf_periodicity_search(rf_plan* p, const void* vis, int32_t nint, int32
       const int ng = v.g1 - v.g0;
       const int np = v.p1 - v.p0;
       RF_CUDA(rf::launch_grid_cells(gp, tbp, d_grp, v.g0, ng, p->d_cellbuf, st));
-      RF_CUDA(rf::launch_colfft(gp, tbp, d_grp, v.g0, ng, v.i0, v.i0, p->d_cellbuf, p->d_T, p->d_colsq, p->d_mean0, st));
+      RF_CUDA(rf::launch_colfft(gp, tbp, d_grp, v.g0, ng, v.i0, v.i0, p->d_cellbuf, p->d_T, p->d_colsq, p->d_mean0, false,
+                                st));
       RF_CUDA(rf::launch_rowfft_power(gp, tbp, p->d_T, d_pairs + v.p0, np, p->d_partials,
                                       p->tmap_P.nbox > 0 ? &p->tmap_P : nullptr, p->d_err, st));
       RF_CUDA(rf::launch_finalize_power(gp, p->d_partials, p->d_colsq, p->d_mean0, d_pairs + v.p0, np,

@@ -60,10 +60,10 @@ struct DevTables {
 // Group of consecutive output integrations of one (DM, dt) trial imaged
 // together by the gridding/column-FFT kernel, and the images derived from
 // them.  The transforms of an image are linear in the visibilities, and a
-// boxcar of 2 dt (4 dt) integrations is the sum of two (four) consecutive ones
-// of dt, so image t' of the trial of width 2 dt (4 dt) is the sum of images
-// 2 t' and 2 t' + 1 (4 t' .. 4 t' + 3) of the same DM: it takes no transform of
-// its own.  t0 is a multiple of 32 wherever n1 or n2 is set.
+// boxcar of 2^L dt integrations is the sum of 2^L consecutive ones of dt, so
+// image t' of the trial of width 2^L dt is the sum of images 2^L t' ..
+// 2^L t' + 2^L - 1 of the same DM: it takes no transform of its own.  t0 is a
+// multiple of 32 wherever a sum is searched.
 struct Group {
   int32_t d;
   int32_t s;
@@ -71,19 +71,37 @@ struct Group {
   int32_t nimg;
   int32_t img0;  // index of the group's first image in the image list
   int32_t base0;  // index of its first image among the transformed images
-  int32_t n1, img1;  // sums of two: how many are searched, the first one's index in the image list
-  int32_t n2, img2;  // sums of four
+  // sums of 2, 4, 8 and 16: how many are searched, the first one's index in
+  // the image list
+  int32_t nsum[4], isum[4];
   int32_t pad[2];
 };
 
-// Up to four consecutive transformed images of a group, for the row pass: the
-// transformed-image index of the first, how many there are, and the image
-// list's indices of the first, of the first sum of two and of the sum of four
-// (-1: not searched).
-struct Quad {
-  int32_t base, n, img, img1;
-  int32_t img2, pad[3];
+// Up to unit_images(pairs) consecutive transformed images of a group, for the
+// row pass: the transformed-image index of the first, how many there are, and
+// the image list's indices of the first one and of the first sum of 2, 4, 8
+// and 16 of them (-1: not searched).
+struct Unit {
+  int32_t base, n, img[5], pad;
 };
+// Sums of 8 and 16 images take the row pass that transforms images in pairs
+// (k_rowfft_duo: four levels of sums), which goes up to 2048^2.  Plans without
+// them, or above that size, take k_rowfft_tree (two rows of one image a
+// transform, two levels): per transform it is the faster one (2048^2, widths
+// 1 .. 16: 3.90 us an image against 4.13; 512^2 with clipped noise, widths 1,
+// 2, 4: 4.05 ms against 4.41), but each width more that is a sum saves the
+// gridding, column pass and row transforms of its images (2048^2, widths 1 ..
+// 16: 291 ms against 262).
+constexpr bool pairs_possible(int npix) { return npix <= 2048; }
+constexpr int unit_images(bool pairs) { return pairs ? 16 : 4; }
+// Position of image row r of column u within its block of XB rows in the
+// column-FFT output that k_rowfft_duo reads: r ^ duo_swizzle(npix, u), so that
+// the 16 lanes which read 8-byte values of consecutive columns from shared
+// memory at once (or of several rows, where a transform has fewer lanes)
+// meet 16 different bank pairs.
+__host__ __device__ constexpr int duo_swizzle(int npix, int u) {
+  return npix >= 512 ? (u / (npix / 512)) & (npix >= 1024 ? 8192 / npix - 1 : 15) : (u * (512 / npix)) & 15;
+}
 
 // Tensor map of a column-FFT output buffer T[slot][u][N] (as FP32 pairs) for
 // the row pass's tile copies: nbox boxes of `rows` u rows each cover ncol.
@@ -153,7 +171,7 @@ constexpr int kOffGrid = -2147483647 - 1;
 // Largest pixel of a part of one image (raw pixel units).
 struct StatPartial {
   float max;
-  int32_t idx;  // y * N + x of max (lowest on ties); INT_MAX where the max is below the image's gate
+  int32_t idx;  // y * N + x of max (lowest on ties)
 };
 
 // With the clipped noise, of the same part: the sums of d = J - mean0 and d^2
@@ -171,15 +189,35 @@ struct ImgNoise {
   double sigma;
 };
 
-// Statistics of the row pass, per slot of a wave.  clip and cparts are set
-// together (the clipped noise).  gate: an image's maxima below its gate are
-// written without their index (null: every index is wanted).
+// Statistics of the row pass, per slot of a wave: the maximum of every part of
+// an image (partials), with the clipped noise also the kept-pixel sums (clip
+// and cparts are set together); or, where only candidates are wanted (best and
+// gate are set together), each image's largest pixel if it is not below its
+// gate: best[slot] starts at 0 and ends as the largest best_key of such pixels.
 struct PassStats {
   StatPartial* partials = nullptr;  // [slot][partials per image]
-  const float* gate = nullptr;
   const float2* clip = nullptr;
   ClipPartial* cparts = nullptr;    // [slot][partials per image]
+  unsigned long long* best = nullptr;
+  const float* gate = nullptr;
 };
+
+// A pixel as a key: of two pixels the larger value has the larger key, of two
+// equal ones the lower index.  Never 0 (the value is not NaN).
+#ifdef __CUDACC__
+__device__ __forceinline__ unsigned best_order(float v) {
+  const unsigned b = __float_as_uint(v);
+  return b & 0x80000000u ? ~b : b | 0x80000000u;
+}
+__device__ __forceinline__ unsigned long long best_key(float v, int pixel) {
+  return (unsigned long long)best_order(v) << 32 | (0xffffffffu - (unsigned)pixel);
+}
+__device__ __forceinline__ float best_max(unsigned long long key) {
+  const unsigned b = (unsigned)(key >> 32);
+  return __uint_as_float(b & 0x80000000u ? b & 0x7fffffffu : ~b);
+}
+__device__ __forceinline__ int best_pixel(unsigned long long key) { return (int)(0xffffffffu - (unsigned)key); }
+#endif
 
 // Clipping radius of the optional one-pass clipped noise, in units of the
 // noise over all pixels.
@@ -264,19 +302,20 @@ cudaError_t launch_grid_cells(const SegmentGeom& g, const DevTables& tb, const G
 // Tbuf[b][col][y], b = transformed-image index - base_base, and for every
 // image of the groups, sums of two and four included, the Parseval sums
 // colsq[slot][col] (weighted sum of |H|^2 over the column) and
-// mean0[slot] = Re H(u = 0, v = 0), slot = image index - img_base.
+// mean0[slot] = Re H(u = 0, v = 0), slot = image index - img_base.  `duo`: in
+// the row order of k_rowfft_duo (duo_swizzle).
 cudaError_t launch_colfft(const SegmentGeom& g, const DevTables& tb, const Group* groups, int g_begin,
                           int ngroups, int img_base, int base_base, const float2* cellbuf, float2* Tbuf,
-                          float* colsq, float* mean0, cudaStream_t st, const PassLaunch* pl = nullptr);
+                          float* colsq, float* mean0, bool duo, cudaStream_t st, const PassLaunch* pl = nullptr);
 
 // Noise of each of `nimg` slots (first image img_base) from the Parseval sums
-// colsq, before the row pass.  gate[i] (if not null): the raw pixel value below
-// which a maximum cannot make image i a candidate.  clip[i] (if not null): the
+// colsq, before the row pass.  gate[i] and best[i] (if not null): the raw pixel
+// value below which a maximum cannot make image i a candidate, and 0.  clip[i] (if not null): the
 // clipping window of the clipped noise in raw pixel units (the image times
 // 2W), {mean0[i], kClipSigmas * sigma over all pixels}.
 cudaError_t launch_image_noise(const SegmentGeom& g, const float* colsq, const float* mean0, const double* weight,
-                               int nimg, int img_base, double threshold, ImgNoise* noise, float* gate, float2* clip,
-                               cudaStream_t st);
+                               int nimg, int img_base, double threshold, ImgNoise* noise, float* gate,
+                               unsigned long long* best, float2* clip, cudaStream_t st);
 
 // Row C2R (pass B) + statistics of `nimg` images in slots [0, nimg) whose
 // first image index is img_base.  Optionally writes the scaled images.
@@ -285,20 +324,22 @@ cudaError_t launch_rowfft_stats(const SegmentGeom& g, const DevTables& tb, const
                                 int img_base, const double* weight, const PassStats& ps, float* images,
                                 const TileMap* tm, int* err, cudaStream_t st, const PassLaunch* pl = nullptr);
 
-// The same for the transformed images of nquads quads (T slots relative to
+// The same for the transformed images of nunits units (T slots relative to
 // base_base, statistics slots to img_base) and the images derived from them,
-// npix >= kTreeMinNpix.
-cudaError_t launch_rowfft_tree(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Quad* quads,
-                               int nquads, int img_base, int base_base, const PassStats& ps, const TileMap* tm,
-                               int* err, cudaStream_t st, const PassLaunch* pl = nullptr);
+// npix >= kTreeMinNpix.  With `pairs` (npix <= 2048) T is in duo order and tm
+// maps boxes of one image's XB rows; unit_partials(shape, pairs) partials per
+// image.
+cudaError_t launch_rowfft_tree(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Unit* units,
+                               int nunits, bool pairs, int img_base, int base_base, const PassStats& ps,
+                               const TileMap* tm, int* err, cudaStream_t st, const PassLaunch* pl = nullptr);
 constexpr int kTreeMinNpix = 64;  // below, a row-pass block is less than a warp
 
-// Reduce row-block partials, compute sigma / snr, append candidates and
+// Reduce nparts partials per image (or take ps.best), compute sigma / snr, append candidates and
 // (optionally) per-image stats for images [img_base, img_base + nimg).
 // Under ps.clip the mean and sigma are those of the kept pixels, from the
 // partials' sums around mean0.
-cudaError_t launch_finalize(const SegmentGeom& g, const PassStats& ps, const ImgNoise* noise, const float* mean0,
-                            const int4* img_info, const double* weight, int nimg, int img_base, double threshold,
+cudaError_t launch_finalize(const SegmentGeom& g, const PassStats& ps, int nparts, const ImgNoise* noise,
+                            const float* mean0, const int4* img_info, const double* weight, int nimg, int img_base, double threshold,
                             DevCand* cands, int* ncand, int cand_cap, DevStat* stats, cudaStream_t st);
 
 // Buffers of the plain per-trial form (chunks of up to `cap` images).
@@ -339,6 +380,9 @@ struct ImageKernelShape {
   bool tile_tma;        // row-pass tiles arrive by tensor copies (boxes, 1 KB alignment)
 };
 bool image_kernel_shape(int npix, ImageKernelShape* out);
+// Partials per image of launch_rowfft_tree: one per row where images are
+// transformed in pairs, else as launch_rowfft_stats, one per row pair.
+inline int unit_partials(const ImageKernelShape& s, bool pairs) { return s.partials_per_image * (pairs ? 2 : 1); }
 
 // Streaming multiprocessors of the current device (cached per device: launch
 // shapes are sized from it, and another GPU of the process may differ).

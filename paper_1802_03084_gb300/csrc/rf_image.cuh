@@ -192,10 +192,11 @@ __device__ __forceinline__ void col_scatter(float2* buf, const int* __restrict__
 }
 
 // The length-L inverse FFT of the inputs col_scatter put in `buf`
-// (sub-transform xsub of the block), written to dst[0 .. L) if dst.
+// (sub-transform xsub of the block), written to dst[0 .. L) if dst, output o at
+// o ^ sw.
 template <int N>
 __device__ __forceinline__ void col_fft_store(float2* buf, const float2* __restrict__ twc, int t, int xsub,
-                                              float2* __restrict__ dst) {
+                                              float2* __restrict__ dst, int sw) {
   using C = ColCfg<N>;
   constexpr int L = C::L, TL = C::TL, EL = C::EL;
   float2 v[EL];
@@ -205,7 +206,11 @@ __device__ __forceinline__ void col_fft_store(float2* buf, const float2* __restr
 #pragma unroll
     for (int m = 0; m < EL / LP; ++m)
 #pragma unroll
-      for (int q = 0; q < LP; ++q) dst[fft_out_index<L>(t, m, q)] = v[m * LP + dft_perm<LP>(q)];
+      for (int q = 0; q < LP; ++q) {
+        // sw < 16, and outputs of 16 lanes or more differ from t by multiples of 16
+        const int o = TL >= 16 ? fft_out_index<L>(t ^ sw, m, q) : fft_out_index<L>(t, m, q) ^ sw;
+        dst[o] = v[m * LP + dft_perm<LP>(q)];
+      }
   }
   fft_sync<TL>(xsub);  // the buffer is reused by the next transform
 }
@@ -227,7 +232,7 @@ template <int N>
 __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
     k_colfft(SegmentGeom g, DevTables tb, const Group* __restrict__ groups, int g_begin, int img_base, int base_base,
              const float2* __restrict__ cellbuf, float2* __restrict__ Tbuf, float* __restrict__ colsq,
-             float* __restrict__ mean0) {
+             float* __restrict__ mean0, int duo) {
   using C = ColCfg<N>;
   constexpr int PI = C::PI;          // images staged at a time
   constexpr int CPC = PI / 2;        // 16-byte chunks per cell row
@@ -240,7 +245,8 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
   int* runs = crow + g.max_cells;                                           // [max_cells]
   const int tid = threadIdx.x;
   const int lane = tid & 31;
-  const Group gr = groups[g_begin + blockIdx.x];
+  const Group* __restrict__ gp = groups + g_begin + blockIdx.x;
+  const Group gr = *gp;
   const int col = blockIdx.y;
   const int cell0 = tb.col_cell_ptr[col];
   const int ncells = tb.col_cell_ptr[col + 1] - cell0;
@@ -257,6 +263,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
   const int p = (tid / TL) % R;           // sub-transform: output rows y = p mod R
   const int t = tid % TL;
   float2* buf = fbuf + (xf * R + p) * C::STRIDE;
+  const int sw = duo ? duo_swizzle(N, col) : 0;
   for (int kbase = 0; kbase < gr.nimg; kbase += PI) {
     if (kbase > 0) __syncthreads();  // the previous part's cells are consumed
     for (int i = tid; i < ncells * CPC; i += C::THREADS) {
@@ -273,56 +280,54 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
     // of |G|^2 over the full Hermitian plane, which counts this column
     // twice unless u = 0; its mean is G(0, 0) / (2 W).  Lane k is image k of
     // the part (two cells a step where the part is 16 images), so the cells of
-    // a sum of two or four images are xor-shuffles away; the warps' FP32 sums
-    // meet in the first FFT buffer and are added in a fixed order.
+    // a sum of 2, 4, 8 or 16 images are xor-shuffles away; the warps' FP32
+    // sums meet in the first FFT buffer and are added in a fixed order.
     {
       constexpr int NW = C::THREADS / 32, CPS = 32 / PI;
-      const bool derived = gr.n1 > 0 || gr.n2 > 0;
+      constexpr int NL = N < kTreeMinNpix ? 0 : (pairs_possible(N) ? 4 : 2);
+      int top = 0;
+#pragma unroll
+      for (int lv = 1; lv <= NL; ++lv)
+        if (gp->nsum[lv - 1] > 0) top = lv;
       const int warp = tid >> 5, kl = lane & (PI - 1);
-      float a0 = 0.f, a1 = 0.f, a2 = 0.f;
+      float a[NL + 1] = {};
       for (int cb = warp * CPS; cb < ncells; cb += NW * CPS) {
         const int c = cb + lane / PI;
         float2 h = make_float2(0.f, 0.f);
         if (c < ncells && kl < nk) h = cellv[c * PI + 2 * ((kl >> 1) ^ (c & (CPC - 1))) + (kl & 1)];
-        a0 = fmaf(h.x, h.x, fmaf(h.y, h.y, a0));
-        if (derived) {
-          h.x += __shfl_xor_sync(0xffffffffu, h.x, 1);
-          h.y += __shfl_xor_sync(0xffffffffu, h.y, 1);
-          a1 = fmaf(h.x, h.x, fmaf(h.y, h.y, a1));
-          h.x += __shfl_xor_sync(0xffffffffu, h.x, 2);
-          h.y += __shfl_xor_sync(0xffffffffu, h.y, 2);
-          a2 = fmaf(h.x, h.x, fmaf(h.y, h.y, a2));
-        }
+        a[0] = fmaf(h.x, h.x, fmaf(h.y, h.y, a[0]));
+#pragma unroll
+        for (int lv = 1; lv <= NL; ++lv)
+          if (lv <= top) {
+            h.x += __shfl_xor_sync(0xffffffffu, h.x, 1 << (lv - 1));
+            h.y += __shfl_xor_sync(0xffffffffu, h.y, 1 << (lv - 1));
+            a[lv] = fmaf(h.x, h.x, fmaf(h.y, h.y, a[lv]));
+          }
       }
-      if constexpr (CPS == 2) {
-        a0 += __shfl_xor_sync(0xffffffffu, a0, 16);
-        a1 += __shfl_xor_sync(0xffffffffu, a1, 16);
-        a2 += __shfl_xor_sync(0xffffffffu, a2, 16);
-      }
-      static_assert(CPS <= 2 && NW * 3 * 32 * 4 <= C::SMEM_FIXED, "Parseval sums fit the FFT buffers");
+      static_assert(CPS <= 2 && (1 << NL) <= PI && NL < NW && NW * (NL + 1) * 32 * 4 <= C::SMEM_FIXED,
+                    "Parseval sums fit the FFT buffers, the sums' images one part, their levels the warps");
       float* red = reinterpret_cast<float*>(fbuf);  // [level][warp][32]
-      red[warp * 32 + lane] = a0;
-      if (derived) {
-        red[(NW + warp) * 32 + lane] = a1;
-        red[(2 * NW + warp) * 32 + lane] = a2;
-      }
+#pragma unroll
+      for (int lv = 0; lv <= NL; ++lv)
+        if (lv <= top) {
+          if constexpr (CPS == 2) a[lv] += __shfl_xor_sync(0xffffffffu, a[lv], 16);
+          red[(lv * NW + warp) * 32 + lane] = a[lv];
+        }
       __syncthreads();
-      const int lv = warp;  // warps 0 .. 2: single images, sums of two, sums of four
-      if (lv < (derived ? 3 : 1) && lane < PI) {
+      const int lv = warp;  // warp 0: single images, warp lv: sums of 2^lv
+      if (lv <= top && lane < PI) {
         const int k = kbase + lane, j = k >> lv;
-        const int lim = lv == 0 ? gr.nimg : (lv == 1 ? gr.n1 : gr.n2);
+        const int lim = lv == 0 ? gr.nimg : gp->nsum[lv - 1];
         if ((lane & ((1 << lv) - 1)) == 0 && j < lim) {
           float acc = 0.f;
           for (int w = 0; w < NW; ++w) acc += red[(lv * NW + w) * 32 + lane];
-          const size_t slot = (size_t)((lv == 0 ? gr.img0 : (lv == 1 ? gr.img1 : gr.img2)) + j - img_base);
+          const size_t slot = (size_t)((lv == 0 ? gr.img0 : gp->isum[lv - 1]) + j - img_base);
           colsq[slot * g.ncol + col] = (col == 0 ? 1.f : 2.f) * acc;
           if (col == 0) {
             // row 0 sorts first in column 0; cell 0's chunks are unswizzled
             float m = 0.f;
             if (ncells > 0 && crow[0] == 0) {
-              m = cellv[lane].x;
-              if (lv >= 1) m += cellv[lane + 1].x;
-              if (lv == 2) m += cellv[lane + 2].x + cellv[lane + 3].x;
+              for (int i = 0; i < 1 << lv; ++i) m += cellv[lane + i].x;
             }
             mean0[slot] = m;
           }
@@ -338,7 +343,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
         const bool live = kl < nk;
         float2* dst = live ? Tbuf + ((size_t)(gr.base0 + kbase + kl - base_base) * g.ncol + col) * N + p * L : nullptr;
         col_scatter<N, PI>(buf, runs, nruns, cellv, crow, kl, live, rtw, t, p, xf * R + p);
-        col_fft_store<N>(buf, tb.twiddle_col, t, xf * R + p, dst);
+        col_fft_store<N>(buf, tb.twiddle_col, t, xf * R + p, dst, sw);
       }
     }
   }
@@ -511,30 +516,70 @@ __device__ __forceinline__ void row_write(const float2 (&v)[ImgCfg<N>::EB], int 
     }
 }
 
+// What a row pass keeps of an image (see PassStats).
+enum RowMode { kBest, kParts, kClip };
+
+// An image row's (or row pair's) maximum into the image's best, called where
+// some lane's maximum lmax is not below the gate (all lanes call; groups of WL
+// lanes share an image row): where the group's maximum beats what the image
+// has, a lane that holds it finds its lowest index and offers it.  Nearly every
+// image of a segment is noise and never gets here.
+template <int WL, class Find>
+__device__ __forceinline__ void row_best(float lmax, float gate, unsigned long long* __restrict__ best, Find find) {
+  const float wmax = warp_max<WL>(lmax);
+  if (lmax == wmax && !(lmax < gate)) {
+    unsigned long long have;
+    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(have) : "l"(best) : "memory");
+    if (best_order(lmax) >= (unsigned)(have >> 32)) atomicMax(best, best_key(lmax, find(lmax)));
+  }
+}
+
+// Kept-pixel sums of the clipped noise: deviations d from cw.x of the lane's
+// values with |d| <= cw.y.
+struct KeptSums {
+  float s = 0.f, q = 0.f;
+  int n = 0;
+  __device__ __forceinline__ void add(float v, float2 cw) {
+    const float d = v - cw.x;
+    if (fabsf(d) <= cw.y) {
+      s += d;
+      q = fmaf(d, d, q);
+      ++n;
+    }
+  }
+};
+template <int WL>
+__device__ __forceinline__ ClipPartial kept_reduce(const KeptSums& a, const KeptSums& b) {
+  float s = a.s + b.s, q = a.q + b.q;
+  int n = a.n + b.n;
+#pragma unroll
+  for (int off = WL / 2; off > 0; off >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, off);
+    q += __shfl_xor_sync(0xffffffffu, q, off);
+    n += __shfl_xor_sync(0xffffffffu, n, off);
+  }
+  return ClipPartial{s, q, n, 0};
+}
+
 // Statistics of the row pair (T rows i = y0 + 2 xf and i + 1, image rows t_row
 // of them) of the image in `slot` whose pixels are in v: the pair's max pixel
-// with its lowest index (and under CLIP the kept-pixel sums), one StatPartial
-// per warp of the transform.  The index is looked for only where the max is
-// not below `gate`, the image's least raw value that can make it a candidate:
-// finding it (a search through the lane's 64 values and a second reduction)
-// costs as much as the maximum itself, and nearly every image of a segment is
-// noise: 1024^2 realtime row passes 91.0 -> 84.2 ms, 2048^2 batching 175.7 ->
-// 163.1, 4096^2 stress subset 8.41 -> 8.01, 512^2 serving 5.37 -> 4.67.
-template <int N, bool CLIP>
+// with its lowest index (and under kClip the kept-pixel sums), one StatPartial
+// per warp of the transform; under kBest only the image's best.  Finding the
+// index and writing a partial cost as much as the maximum itself, and this
+// kernel is bound by instruction issue: leaving them out
+// (kBest against kParts with the index gated) took the 1024^2 realtime row
+// passes from 85.0 to 75.2 ms, 2048^2 batching from 186 to 147, 4096^2 stress
+// subset from 8.01 to 7.60.
+template <int N, RowMode M>
 __device__ __forceinline__ void row_stats(const float2 (&v)[ImgCfg<N>::EB], int t, int xf, int slot, int y0,
                                           int tsplit, int log2l, float gate, const PassStats& ps) {
   using K = ImgCfg<N>;
   constexpr int EB = K::EB, TB = K::TB;
   constexpr int H = N / K::RSPLIT;
-  auto pix = [&](int m, int q) { return row_pix<N>(t, m, q); };
-
-  // per-row-pair statistics: the max pixel and its lowest index (the
-  // noise comes from the grid by Parseval's identity, see k_colfft).  The
+  // the noise comes from the grid by Parseval's identity, see k_colfft.  The
   // pair is T rows i, i + 1, image rows ya < yb (adjacent unless the
   // column pass split its transforms: then R apart)
   const int i = y0 + 2 * xf;
-  const int ya = t_row(i, tsplit, log2l);
-  const int yb = t_row(i + 1, tsplit, log2l);
   constexpr int LP = FftShape<H, EB>::LAST_P;
   constexpr int EM = EB / LP;
   // max of row y (real parts) and of row y + 1 (imaginary parts), four
@@ -549,23 +594,17 @@ __device__ __forceinline__ void row_stats(const float2 (&v)[ImgCfg<N>::EB], int 
   const float mx = fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3]));
   const float my = fmaxf(fmaxf(mya[0], mya[1]), fmaxf(mya[2], mya[3]));
   const float lmax = fmaxf(mx, my);
-  // reduce over the transform's T threads (a warp, a part of one, or
-  // several warps joined through shared memory)
-  constexpr int WL = TB < 32 ? TB : 32;
-  constexpr unsigned MASK = 0xffffffffu;
-  const float wmax = warp_max<WL>(lmax);
-  // a lane holding the maximum finds its lowest index: row ya comes before
+  // the lowest index of the lane's pixels equal to `top`: row ya comes before
   // row yb, and within a row the lane's outputs ascend with (q, m)
-  int best = INT_MAX;
-  const bool want = CLIP || !(wmax < gate);
-  if (want && lmax == wmax) {
-    if (mx == wmax) {
+  auto find = [&](float top) {
+    int best = INT_MAX;
+    if (mx == top) {
 #pragma unroll
       for (int q = 0; q < LP; ++q)
 #pragma unroll
         for (int m = 0; m < EM; ++m)
-          if (v[m * LP + dft_perm<LP>(q)].x == wmax) {
-            best = ya * N + pix(m, q);
+          if (v[m * LP + dft_perm<LP>(q)].x == top) {
+            best = t_row(i, tsplit, log2l) * N + row_pix<N>(t, m, q);
             goto found;
           }
     } else {
@@ -573,54 +612,41 @@ __device__ __forceinline__ void row_stats(const float2 (&v)[ImgCfg<N>::EB], int 
       for (int q = 0; q < LP; ++q)
 #pragma unroll
         for (int m = 0; m < EM; ++m)
-          if (v[m * LP + dft_perm<LP>(q)].y == wmax) {
-            best = yb * N + pix(m, q);
+          if (v[m * LP + dft_perm<LP>(q)].y == top) {
+            best = t_row(i + 1, tsplit, log2l) * N + row_pix<N>(t, m, q);
             goto found;
           }
     }
-  found:;
+  found:
+    return best;
+  };
+  constexpr int WL = TB < 32 ? TB : 32;
+  if constexpr (M == kBest) {
+    if (__any_sync(0xffffffffu, !(lmax < gate))) row_best<WL>(lmax, gate, ps.best + slot, find);
+    return;
   }
-  if (CLIP || __any_sync(MASK, want)) best = warp_min<WL>(best);
-  // clipped noise: sums of the kept pixels' deviations from mean0, rows y
-  // and y + 1 in separate chains
-  float s1 = 0.f, s2 = 0.f;
-  int cn = 0;
-  if constexpr (CLIP) {
+  // reduce over the transform's T threads (a warp, a part of one, or several
+  // warps, one partial each, which the finalisation combines: no barrier)
+  const float wmax = warp_max<WL>(lmax);
+  int best = INT_MAX;
+  if (lmax == wmax) best = find(wmax);
+  best = warp_min<WL>(best);
+  ClipPartial cp{};
+  if constexpr (M == kClip) {
     const float2 cw = ps.clip[slot];
-    float ax = 0.f, qx = 0.f, ay = 0.f, qy = 0.f;
-    int nx = 0, ny = 0;
+    KeptSums a, b;  // rows y and y + 1 in separate chains
 #pragma unroll
     for (int e = 0; e < EB; ++e) {
-      const float dx = v[e].x - cw.x;
-      const float dy = v[e].y - cw.x;
-      if (fabsf(dx) <= cw.y) {
-        ax += dx;
-        qx = fmaf(dx, dx, qx);
-        ++nx;
-      }
-      if (fabsf(dy) <= cw.y) {
-        ay += dy;
-        qy = fmaf(dy, dy, qy);
-        ++ny;
-      }
+      a.add(v[e].x, cw);
+      b.add(v[e].y, cw);
     }
-    s1 = ax + ay;
-    s2 = qx + qy;
-    cn = nx + ny;
-#pragma unroll
-    for (int off = WL / 2; off > 0; off >>= 1) {
-      s1 += __shfl_xor_sync(MASK, s1, off);
-      s2 += __shfl_xor_sync(MASK, s2, off);
-      cn += __shfl_xor_sync(MASK, cn, off);
-    }
+    cp = kept_reduce<WL>(a, b);
   }
-  // one partial per warp of the transform (WPT of them when a transform
-  // spans several warps; the finalisation combines them): no barrier
   if ((t & 31) == 0) {
     constexpr int WPT = TB > 32 ? TB / 32 : 1;
     const size_t o = (size_t)slot * K::PARTIALS + ((y0 >> 1) + xf) * WPT + (t >> 5);  // by T row pair
     ps.partials[o] = StatPartial{wmax, best};
-    if constexpr (CLIP) ps.cparts[o] = ClipPartial{s1, s2, cn, 0};
+    if constexpr (M == kClip) ps.cparts[o] = cp;
   }
 }
 
@@ -632,18 +658,18 @@ __device__ __forceinline__ void row_stats(const float2 (&v)[ImgCfg<N>::EB], int 
 // warp of a row pair's transform writes one StatPartial (one per row pair
 // when the transform fits a warp, T/32 of them when it spans several): the
 // max pixel of its part of the two rows with its lowest index, and under
-// CLIP the kept-pixel sums (FP32 per thread and across the warp's lanes; the
+// kClip the kept-pixel sums (FP32 per thread and across the warp's lanes; the
 // finalisation combines an image's partials in FP64).
 // With tma_boxes > 0 (N >= 1024 only) thread 0 fetches each item's tile with
 // tma_boxes tensor copies of tma_rows u rows from `tmap` ([slot][u][2N
 // floats]) and every thread waits on an mbarrier; a wait that gives up sets
 // *err, waits once more (bounded) for the copy in flight, and the block
 // returns.  Otherwise the threads copy it with cp.async.
-// CLIP (the one-pass clipped noise): clip[slot] = {mean0, r} in raw pixel
+// kClip (the one-pass clipped noise): clip[slot] = {mean0, r} in raw pixel
 // units, and each row pair also sums d = J - mean0 and d^2 over its pixels J
 // with |d| <= r and counts them (FP32 per thread and across the transform's
 // threads in a fixed order).
-template <int N, bool CLIP>
+template <int N, RowMode M>
 __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
     k_rowfft_stats(SegmentGeom g, DevTables tb, const float2* __restrict__ Tbuf, int nimg, int img_base,
                    const double* __restrict__ weight, const PassStats ps, float* __restrict__ images,
@@ -735,7 +761,7 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
     }
     const int slot = item / nrb;
     const int y0 = (item - slot * nrb) * K::RB;
-    const float gate = !CLIP && ps.gate != nullptr ? ps.gate[slot] : -FLT_MAX;
+    const float gate = M == kBest ? ps.gate[slot] : 0.f;
     float2 v[K::EB];
     row_zbuild<N>(v, tile, t, xf, ncol);
     if (use_tma && WARP_LOCAL) {
@@ -759,12 +785,12 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
     }
     row_fft<N>(v, fbuf + xf * K::STRIDE_B, tb.twiddle, t, xf);
     if (images != nullptr) row_write<N>(v, t, xf, slot, y0, g.tsplit, log2l, weight[img_base + slot], images);
-    row_stats<N, CLIP>(v, t, xf, slot, y0, g.tsplit, log2l, gate, ps);
+    row_stats<N, M>(v, t, xf, slot, y0, g.tsplit, log2l, gate, ps);
   }
 }
 
-// Pass B over quads of transformed images, with the images derived from them:
-// work item = (quad, block of RB rows).  A block takes the quad's images one
+// Pass B over units of up to four transformed images (quads), with the images
+// derived from them (sums of two and four): work item = (quad, block of RB rows).  A block takes the quad's images one
 // after the other through the transform of k_rowfft_stats.  The pixel rows of
 // image k stay with the lane that made them: an even image's are kept, an odd
 // one's added to them, which is the row pair of the sum of two images (the
@@ -785,10 +811,10 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
 // 1024^2 row passes' 91 ms, keeping and adding take 3 and the sums' maxima 9.
 // A block that gives up a bounded wait leaves the item loop and frees its
 // tensor memory with the others.
-template <int N, bool CLIP>
+template <int N, RowMode M>
 __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
-    k_rowfft_tree(SegmentGeom g, DevTables tb, const float2* __restrict__ Tbuf, const Quad* __restrict__ quads,
-                  int nquads, int img_base, int base_base, const PassStats ps,
+    k_rowfft_tree(SegmentGeom g, DevTables tb, const float2* __restrict__ Tbuf, const Unit* __restrict__ units,
+                  int nunits, int img_base, int base_base, const PassStats ps,
                   const __grid_constant__ CUtensorMap tmap, int tma_boxes, int tma_rows, int* __restrict__ err) {
   using K = ImgCfg<N>;
   static_assert(K::EB == 32 && K::THREADS_B % 32 == 0, "64 values a lane, whole warps");
@@ -805,7 +831,7 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
   const int tid = threadIdx.x;
   const int ncol = g.ncol;
   constexpr int nrb = N / K::RB;
-  const int nitems = nquads * nrb;
+  const int nitems = nunits * nrb;
   const int xf = tid / K::TB;
   const int t = tid - xf * K::TB;
   const int log2l = FftShape<N>::LOG2N - (g.tsplit > 1 ? __ffs(g.tsplit) - 1 : 0);
@@ -840,23 +866,23 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
   };
 
   int item = blockIdx.x;
-  Quad cur = quads[item / nrb];  // the grid is at most the number of items
+  Unit cur = units[item / nrb];  // the grid is at most the number of items
   bool failed = false;
   fetch(cur.base - base_base, (item % nrb) * K::RB);
   while (item < nitems && !failed) {
     const int y0 = (item % nrb) * K::RB;
     const int next = item + (int)gridDim.x;
-    Quad nxt = cur;
-    if (next < nitems) nxt = quads[next / nrb];
-    const int top = cur.img2 >= 0 ? 2 : (cur.img1 >= 0 ? 1 : 0);
+    Unit nxt = cur;
+    if (next < nitems) nxt = units[next / nrb];
+    const int top = cur.img[2] >= 0 ? 2 : (cur.img[1] >= 0 ? 1 : 0);
     // lanes 0 .. 3 hold the gates of the quad's images, 4 and 5 those of the
     // sums of two, 6 that of the sum of four
-    float gates = -FLT_MAX;
-    if (!CLIP && ps.gate != nullptr) {
+    float gates = 0.f;
+    if (M == kBest) {
       const int lane = tid & 31;
-      int sl = lane < cur.n ? cur.img + lane : -1;
-      if (lane >= 4) sl = lane < 6 && cur.img1 >= 0 && 2 * (lane - 4) + 1 < cur.n ? cur.img1 + lane - 4 : -1;
-      if (lane == 6) sl = cur.img2;
+      int sl = lane < cur.n ? cur.img[0] + lane : -1;
+      if (lane >= 4) sl = lane < 6 && cur.img[1] >= 0 && 2 * (lane - 4) + 1 < cur.n ? cur.img[1] + lane - 4 : -1;
+      if (lane == 6) sl = cur.img[2];
       if (sl >= 0) gates = ps.gate[sl - img_base];
     }
     for (int k = 0; k < cur.n; ++k) {
@@ -908,11 +934,11 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
         if (more) fetch(nsl, nyb);
       }
       row_fft<N>(v, fbuf + xf * K::STRIDE_B, tb.twiddle, t, xf);
-      int slot = cur.img + k - img_base;
+      int slot = cur.img[0] + k - img_base;
 #pragma unroll 1
       for (int lv = 0;;) {
         const float gate = __shfl_sync(0xffffffffu, gates, lv == 0 ? k : (lv == 1 ? 4 + (k >> 1) : 6));
-        if (slot >= 0) row_stats<N, CLIP>(v, t, xf, slot, y0, g.tsplit, log2l, gate, ps);
+        if (slot >= 0) row_stats<N, M>(v, t, xf, slot, y0, g.tsplit, log2l, gate, ps);
         // level lv's block of images that ends the next level's must be whole
         if (lv >= top || (k | ((2 << lv) - 1)) >= cur.n) break;
         __syncwarp();
@@ -924,7 +950,7 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
         tmem_add16(keep + lv * 64, v);
         tmem_add16(keep + lv * 64 + 32, v + 16);
         ++lv;
-        const int first = lv == 1 ? cur.img1 : cur.img2;
+        const int first = lv == 1 ? cur.img[1] : cur.img[2];
         slot = first < 0 ? -1 : first + (lv == 1 ? k >> 1 : 0) - img_base;
       }
     }
@@ -934,6 +960,316 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
   __syncthreads();
   if (tid < 32) tmem_free(s_tmem, TCOLS);
+}
+
+// Row pass of image pairs, the first-pass inputs of image row xf of the item:
+// Z[u] = T_A[u] + i T_B[u] of two images' tiles, Hermitian-extended as in
+// row_zbuild with the images in the place of the rows.
+// Tiles are [u][XB] complex values, row r of column u at r ^ duo_swizzle(N, u),
+// the same for all columns a lane reads directly and for all it mirrors.
+template <int N>
+__device__ __forceinline__ void row_zbuild_duo(float2 (&v)[ImgCfg<N>::EB], const float2* __restrict__ tileA,
+                                               const float2* __restrict__ tileB, int t, int xf, int ncol) {
+  using K = ImgCfg<N>;
+  constexpr int EB = K::EB, TB = K::TB, XB = K::XB;
+  const float2 zero = make_float2(0.f, 0.f);
+  if constexpr (K::RSPLIT == 2) {  // see row_zbuild
+    constexpr int H = N / 2;
+    static_assert(EB == 32 && TB == 64 && duo_swizzle(N, 32) == 0, "split row transform layout");
+    const int s = t >> 5, j = t & 31;
+    const int rd_end = ncol > j ? (ncol - j + 31) / 32 : 0;
+    const int xm = H - j - ncol;
+    const int rm_beg = xm < 0 ? 0 : xm / 32 + 1;
+    const int od = j * XB + (xf ^ duo_swizzle(N, j)), om = (H - j) * XB + (xf ^ duo_swizzle(N, H - j));
+    const float2 pm1 = make_float2(s == 0 ? 1.f : -1.f, s == 0 ? -1.f : 1.f);
+#pragma unroll
+    for (int r = 0; r < 32; ++r) {
+      float2 a = zero, b = zero, c = zero, d = zero;
+      if (r < rd_end) {
+        a = tileA[od + r * 32 * XB];
+        b = tileB[od + r * 32 * XB];
+      }
+      if (r >= rm_beg) {
+        c = tileA[om - r * 32 * XB];
+        d = tileB[om - r * 32 * XB];
+      }
+      const float2 P = f2_fma(c, pm1, a);
+      const float2 Q = f2_fma(d, pm1, b);
+      float2 z = make_float2(P.x - Q.y, P.y + Q.x);
+      if (r == 0 && j == 0) {
+        const float sg = s == 0 ? 1.f : -1.f;
+        z = make_float2(fmaf(sg, c.x + d.y, a.x), fmaf(sg, d.x - c.y, b.x));
+      }
+      if (s != 0 && r > 0) z = r == 16 ? cmul_i(z) : cmul_c<false>(z, cos_r64(r), sin_r64(r));
+      v[r] = z;
+    }
+  } else {
+    static_assert(duo_swizzle(N, TB) == 0, "one swizzle per lane");
+    const int rd_end = ncol > t ? (ncol - t + TB - 1) / TB : 0;
+    const int rm_beg = (N - ncol - t) / TB + 1;
+    const int od = t * XB + (xf ^ duo_swizzle(N, t)), om = (N - t) * XB + (xf ^ duo_swizzle(N, N - t));
+#pragma unroll
+    for (int r = 0; r < EB / 2; ++r) {
+      float2 a = zero, b = zero;
+      if (r < rd_end) {
+        a = tileA[od + r * TB * XB];
+        b = tileB[od + r * TB * XB];
+      }
+      v[r] = (r == 0 && t == 0) ? make_float2(a.x, b.x) : make_float2(a.x - b.y, a.y + b.x);
+    }
+#pragma unroll
+    for (int r = EB / 2; r < EB; ++r) {
+      float2 a = zero, b = zero;
+      if (r >= rm_beg) {
+        a = tileA[om - r * TB * XB];
+        b = tileB[om - r * TB * XB];
+      }
+      v[r] = make_float2(a.x + b.y, b.x - a.y);
+    }
+  }
+}
+
+// Statistics of one image row (T row i) of the image in `slot`, output e of the
+// lane's registers read by val(e): one partial per warp of the transform, as
+// row_stats writes for a row pair.
+template <int N, RowMode M, class F>
+__device__ __forceinline__ void row_stats_one(F val, int t, int i, int slot, int tsplit, int log2l, float gate,
+                                              const PassStats& ps) {
+  using K = ImgCfg<N>;
+  constexpr int EB = K::EB, TB = K::TB;
+  constexpr int LP = FftShape<N / K::RSPLIT, EB>::LAST_P;
+  constexpr int EM = EB / LP;
+  constexpr int WL = TB < 32 ? TB : 32;
+  float m4[4] = {-FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX};
+#pragma unroll
+  for (int e = 0; e < EB; e += 2) m4[(e >> 1) & 3] = fmax3f(m4[(e >> 1) & 3], val(e), val(e + 1));
+  const float lmax = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+  auto find = [&](float top) {
+    int best = INT_MAX;
+#pragma unroll
+    for (int q = 0; q < LP; ++q)
+#pragma unroll
+      for (int m = 0; m < EM; ++m)
+        if (val(m * LP + dft_perm<LP>(q)) == top) {
+          best = t_row(i, tsplit, log2l) * N + row_pix<N>(t, m, q);
+          goto found;
+        }
+  found:
+    return best;
+  };
+  if constexpr (M == kBest) {
+    if (__any_sync(0xffffffffu, !(lmax < gate))) row_best<WL>(lmax, gate, ps.best + slot, find);
+    return;
+  }
+  const float wmax = warp_max<WL>(lmax);
+  int best = INT_MAX;
+  if (lmax == wmax) best = find(wmax);
+  best = warp_min<WL>(best);
+  ClipPartial cp{};
+  if constexpr (M == kClip) {
+    const float2 cw = ps.clip[slot];
+    KeptSums k[2];
+#pragma unroll
+    for (int e = 0; e < EB; ++e) k[e & 1].add(val(e), cw);
+    cp = kept_reduce<WL>(k[0], k[1]);
+  }
+  if ((t & 31) == 0) {
+    constexpr int WPT = TB > 32 ? TB / 32 : 1;
+    const size_t o = (size_t)slot * (2 * K::PARTIALS) + i * WPT + (t >> 5);
+    ps.partials[o] = StatPartial{wmax, best};
+    if constexpr (M == kClip) ps.cparts[o] = cp;
+  }
+}
+
+// Pass B over units of up to 16 consecutive transformed images, with the images
+// derived from them (sums of 2, 4, 8 and 16), N <= 2048: work item = (unit,
+// block of XB rows).  A block takes the unit's images two at a time through
+// the transform of k_rowfft_stats, one image row of both per transform (A in
+// the real parts, B in the imaginary parts; an odd last image alone), so a
+// lane holds the same pixels of both and their sum is one addition, with
+// nothing kept.  Longer sums form as a binary counter does: a sum of an even
+// place is kept, the next one is added to it and goes a level up.  What is
+// kept, 32 registers a lane and level, goes to tensor memory, which nothing else
+// uses here and whose loads and stores do not pass through the L1/shared pipe;
+// three levels take 96 of the 128 columns that 16 warps of an SM can have each.
+// Two rows of one image a transform (k_rowfft_tree) keep 64 registers a level
+// and one level more, which fits two levels of sums.  1024^2 realtime (widths 1,
+// 2, 4, 8): 94,700 images transformed and not 106,500, 164.3 -> 147.4 ms with
+// kBest; 2048^2 batching (1 .. 16) 295.3 -> 261.9 ms.
+// T is read in duo order: with the tiles' rows of XB 8-byte values permuted by
+// column, a half-warp's loads meet 16 bank pairs (the hardware's swizzles move
+// 16-byte chunks: two-way conflicts).
+template <int N, RowMode M>
+__global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
+    k_rowfft_duo(SegmentGeom g, DevTables tb, const float2* __restrict__ Tbuf, const Unit* __restrict__ units,
+                 int nunits, int img_base, int base_base, const PassStats ps,
+                 const __grid_constant__ CUtensorMap tmap, int tma_boxes, int tma_rows, int* __restrict__ err) {
+  using K = ImgCfg<N>;
+  constexpr int EB = K::EB, XB = K::XB, NL = 4;
+  static_assert(EB == 32 && K::THREADS_B % 32 == 0 && pairs_possible(N) && (1 << NL) == unit_images(true), "32 values a lane, whole warps");
+  static_assert(sizeof(Unit) == 32, "eight words, one a lane");
+  constexpr bool WARP_LOCAL = K::TILE_TMA && (K::TB <= 32 || K::RSPLIT == 2);  // see k_rowfft_stats
+  static_assert(WARP_LOCAL == K::TILE_TMA, "tensor copies only where no barrier crosses a warp");
+  constexpr int NWB = K::THREADS_B / 32;
+  constexpr unsigned TCOLS = TreeCfg<N>::COLS;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  float2* fbuf = reinterpret_cast<float2*>(smraw);  // [XB][STRIDE_B]
+  unsigned char* tb0 = smraw + XB * K::STRIDE_B * 8;
+  if constexpr (K::TILE_TMA) tb0 += (1024u - (smem_u32(tb0) & 1023u)) & 1023u;
+  const bool use_tma = K::TILE_TMA && tma_boxes > 0;
+  const int trows = use_tma ? tma_boxes * tma_rows : g.ncol;
+  float2* tileA = reinterpret_cast<float2*>(tb0);  // [rows][XB]
+  float2* tileB = tileA + (size_t)trows * XB;
+  __shared__ __align__(8) unsigned long long tbar;
+  __shared__ int s_done;  // warps done reading the tiles in hand
+  __shared__ unsigned s_tmem;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int ncol = g.ncol;
+  constexpr int nrb = N / XB;
+  const int nitems = nunits * nrb;
+  const int xf = tid / K::TB;
+  const int t = tid - xf * K::TB;
+  const int log2l = FftShape<N>::LOG2N - (g.tsplit > 1 ? __ffs(g.tsplit) - 1 : 0);
+  unsigned phase = 0;
+  if (tid < 32) tmem_alloc(&s_tmem, TCOLS);
+  if (tid == 0) {
+    mbar_init(&tbar, 1);
+    s_done = 0;
+  }
+  __syncthreads();
+  // this warp's lanes and columns: 32 for each level that is kept
+  const unsigned keep = s_tmem + ((unsigned)((tid >> 5) & 3) << 21) + (unsigned)(tid >> 7) * 128u;
+  // lanes 0 .. 15 stand for a unit's images, 16 .. 23 for its sums of two,
+  // 24 .. 27 of four, 28 and 29 of eight, 30 of sixteen: place lj of level ll
+  const int ll = lane < 16 ? 0 : (lane < 24 ? 1 : (lane < 28 ? 2 : (lane < 30 ? 3 : 4)));
+  const int lj = lane - (32 - (32 >> ll));
+
+  // tiles of rows yb .. yb + XB of the image in T slot sl, and of the next one if `two`
+  auto issue_tma = [&](int sl, bool two, int yb) {  // by one thread
+    const int n = two ? 2 : 1;
+    mbar_expect_tx(&tbar, (unsigned)(n * tma_boxes * tma_rows * XB * 8));
+    for (int i = 0; i < n; ++i)
+      for (int b = 0; b < tma_boxes; ++b)
+        tma_load_3d((i ? tileB : tileA) + (size_t)b * tma_rows * XB, &tmap, 2 * yb, b * tma_rows, sl + i, &tbar);
+  };
+  auto fetch = [&](int sl, bool two, int yb) {
+    if (use_tma) {
+      if (tid == 0) issue_tma(sl, two, yb);
+      return;
+    }
+    constexpr int CH = XB / 2;  // 16-byte chunks per column
+    const float2* src = Tbuf + (size_t)sl * ncol * N + yb;
+    const int n = (two ? 2 : 1) * ncol * CH;
+    for (int i = tid; i < n; i += K::THREADS_B) {
+      const int u = i / CH;  // columns of A, then of B
+      const int c = i - u * CH;
+      cp_async16(tileA + (size_t)u * XB + 2 * c, src + (size_t)u * N + 2 * c);
+    }
+    cp_async_commit();
+  };
+
+  int item = blockIdx.x;
+  // a unit's words, one a lane: base, n, img[0 .. 4]
+  auto load_unit = [&](int it) { return reinterpret_cast<const int*>(units + it / nrb)[lane & 7]; };
+  int cur = load_unit(item);  // the grid is at most the number of items
+  bool failed = false;
+  fetch(__shfl_sync(0xffffffffu, cur, 0) - base_base, __shfl_sync(0xffffffffu, cur, 1) > 1, (item % nrb) * XB);
+  while (item < nitems && !failed) {
+    const int y0 = (item % nrb) * XB;
+    const int next = item + (int)gridDim.x;
+    const int nxt = next < nitems ? load_unit(next) : cur;
+    const int base = __shfl_sync(0xffffffffu, cur, 0), n = __shfl_sync(0xffffffffu, cur, 1);
+    const int first = __shfl_sync(0xffffffffu, cur, 2 + ll);
+    // this lane's image: its slot (-1: not searched) and gate; the highest level searched
+    const int slots = first >= 0 && (lj + 1) << ll <= n ? first + lj - img_base : -1;
+    const int top = 31 - __clz((int)(__ballot_sync(0xffffffffu, cur >= 0) >> 2 & 31u) | 1);
+    float gates = 0.f;
+    if (M == kBest && slots >= 0) gates = ps.gate[slots];
+    const int i = y0 + xf;
+    for (int k = 0; k < n; k += 2) {
+      if (use_tma) {
+        // as in k_rowfft_stats: no copy is issued without this warp's count
+        // below, so the other warps' waits run out in turn
+        if (!__all_sync(0xffffffffu, mbar_wait(&tbar, phase))) {
+          if (lane == 0) atomicExch(err, 1);
+          mbar_wait(&tbar, phase);
+          failed = true;
+          break;
+        }
+        phase ^= 1u;
+      } else {
+        cp_async_wait_all();
+        __syncthreads();
+      }
+      const bool two = k + 1 < n;
+      float2 v[EB];
+      row_zbuild_duo<N>(v, tileA, two ? tileB : tileA, t, xf, ncol);  // A alone: beside itself
+      // the tiles are read: the unit's next images' (or the next item's first ones')
+      const bool here = k + 2 < n;
+      const int nbase = __shfl_sync(0xffffffffu, nxt, 0), nn = __shfl_sync(0xffffffffu, nxt, 1);
+      const int nsl = (here ? base + k + 2 : nbase) - base_base;
+      const bool ntwo = here ? k + 3 < n : nn > 1;
+      const int nyb = here ? y0 : (next % nrb) * XB;
+      const bool more = here || next < nitems;
+      if (use_tma) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) {
+          __threadfence_block();
+          if (atomicAdd(&s_done, 1) == NWB - 1) {
+            s_done = 0;
+            __threadfence_block();
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            if (more) issue_tma(nsl, ntwo, nyb);
+          }
+        }
+      } else {
+        __syncthreads();
+        if (more) fetch(nsl, ntwo, nyb);
+      }
+      row_fft<N>(v, fbuf + xf * K::STRIDE_B, tb.twiddle, t, xf);
+      {
+        const int sa = __shfl_sync(0xffffffffu, slots, k), sb = __shfl_sync(0xffffffffu, slots, k + 1);
+        const float ga = __shfl_sync(0xffffffffu, gates, k), gb = __shfl_sync(0xffffffffu, gates, k + 1);
+        row_stats_one<N, M>([&](int e) { return v[e].x; }, t, i, sa, g.tsplit, log2l, ga, ps);
+        if (two) row_stats_one<N, M>([&](int e) { return v[e].y; }, t, i, sb, g.tsplit, log2l, gb, ps);
+      }
+      if (!two || top == 0) continue;
+      float2 s[EB / 2];
+#pragma unroll
+      for (int e = 0; e < EB / 2; ++e)
+        s[e] = make_float2(v[2 * e].x + v[2 * e].y, v[2 * e + 1].x + v[2 * e + 1].y);
+#pragma unroll 1
+      for (int lv = 1;; ++lv) {
+        const int j = k >> lv;  // s is sum j of this level
+        const int sl = __shfl_sync(0xffffffffu, slots, 32 - (32 >> lv) + j);
+        const float gt = __shfl_sync(0xffffffffu, gates, 32 - (32 >> lv) + j);
+        if (sl >= 0)
+          row_stats_one<N, M>([&](int e) { return e & 1 ? s[e >> 1].y : s[e >> 1].x; }, t, i, sl, g.tsplit, log2l,
+                                 gt, ps);
+        // the next level's block of images must be whole
+        if (lv >= top || ((j | 1) + 1) << lv > n) break;
+        __syncwarp();
+        if ((j & 1) == 0) {
+          tmem_store16(keep + (lv - 1) * 32, s);
+          break;
+        }
+        tmem_add16(keep + (lv - 1) * 32, s);
+      }
+    }
+    item = next;
+    cur = nxt;
+  }
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+  __syncthreads();
+  if (tid < 32) tmem_free(s_tmem, TCOLS);
+}
+
+// The row-pass kernel of units at side N.
+template <int N, RowMode M, bool PAIRS>
+constexpr auto tree_kernel() {
+  if constexpr (PAIRS) return k_rowfft_duo<N, M>;
+  else return k_rowfft_tree<N, M>;
 }
 
 // The most dynamic shared memory a block of `kern` can have: the device's
@@ -1295,7 +1631,7 @@ int rowfft_tile_rows(int ncol);
 template <int N>
 cudaError_t run_colfft(const SegmentGeom& g, const DevTables& tb, const Group* groups, int g_begin, int ngroups,
                        int img_base, int base_base, const float2* cellbuf, float2* Tbuf, float* colsq, float* mean0,
-                       cudaStream_t st, const PassLaunch* pl) {
+                       bool duo, cudaStream_t st, const PassLaunch* pl) {
   using C = ColCfg<N>;
   using K = ImgCfg<N>;
   int smem = C::SMEM_FIXED + g.max_cells * C::SMEM_PER_CELL;
@@ -1312,7 +1648,7 @@ cudaError_t run_colfft(const SegmentGeom& g, const DevTables& tb, const Group* g
                            smem_max);
   dim3 grid(ngroups, g.ncol);
   return launch_with(k_colfft<N>, grid, dim3(C::THREADS), smem, st, pl, g, tb, groups, g_begin, img_base, base_base,
-                     cellbuf, Tbuf, colsq, mean0);
+                     cellbuf, Tbuf, colsq, mean0, duo ? 1 : 0);
 }
 
 // Rows of the row-pass tile: ncol, or the boxes' total under tensor copies.
@@ -1324,13 +1660,13 @@ int rowfft_tile_rows(int ncol) {
   return nbox * rows;
 }
 
-template <int N, bool CLIP>
+template <int N, RowMode M>
 cudaError_t run_rowfft_stats_k(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, int nimg,
                                int img_base, const double* weight, const PassStats& ps, float* images,
                                const TileMap* tm, int* err, cudaStream_t st, const PassLaunch* pl) {
   using K = ImgCfg<N>;
   const int smem = K::SMEM_B_FIXED + (K::TILE_TMA ? 1024 : 0) + rowfft_tile_rows<N>(g.ncol) * K::CH * 16;
-  auto kern = k_rowfft_stats<N, CLIP>;
+  auto kern = k_rowfft_stats<N, M>;
   const int smem_max = max_dynamic_smem(kern);
   if (smem > smem_max) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
@@ -1358,47 +1694,56 @@ cudaError_t run_rowfft_stats(const SegmentGeom& g, const DevTables& tb, const fl
                              int img_base, const double* weight, const PassStats& ps, float* images,
                              const TileMap* tm, int* err, cudaStream_t st, const PassLaunch* pl) {
   if (ps.clip != nullptr)
-    return run_rowfft_stats_k<N, true>(g, tb, Tbuf, nimg, img_base, weight, ps, images, tm, err, st, pl);
-  return run_rowfft_stats_k<N, false>(g, tb, Tbuf, nimg, img_base, weight, ps, images, tm, err, st, pl);
+    return run_rowfft_stats_k<N, kClip>(g, tb, Tbuf, nimg, img_base, weight, ps, images, tm, err, st, pl);
+  if (ps.best != nullptr)
+    return run_rowfft_stats_k<N, kBest>(g, tb, Tbuf, nimg, img_base, weight, ps, images, tm, err, st, pl);
+  return run_rowfft_stats_k<N, kParts>(g, tb, Tbuf, nimg, img_base, weight, ps, images, tm, err, st, pl);
 }
 
-template <int N, bool CLIP>
-cudaError_t run_rowfft_tree_k(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Quad* quads,
-                              int nquads, int img_base, int base_base, const PassStats& ps, const TileMap* tm,
+template <int N, RowMode M, bool PAIRS>
+cudaError_t run_rowfft_tree_k(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Unit* units,
+                              int nunits, int img_base, int base_base, const PassStats& ps, const TileMap* tm,
                               int* err, cudaStream_t st, const PassLaunch* pl) {
   using K = ImgCfg<N>;
   const int smem = K::SMEM_B_FIXED + (K::TILE_TMA ? 1024 : 0) + rowfft_tile_rows<N>(g.ncol) * K::CH * 16;
-  auto kern = k_rowfft_tree<N, CLIP>;
+  auto kern = tree_kernel<N, M, PAIRS>();
   const int smem_max = max_dynamic_smem(kern);
   if (smem > smem_max) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;
-  if (nquads <= 0) return cudaSuccess;
+  if (nunits <= 0) return cudaSuccess;
   int per_sm = 0;
   e = tmem_blocks_per_sm(&per_sm, kern, K::THREADS_B, smem, TreeCfg<N>::COLS);
   if (e != cudaSuccess) return e;
-  const long nitems = (long)nquads * (N / K::RB);
+  // an item is up to unit_images(PAIRS) images, two of them a transform where they are paired
+  const long nitems = (long)nunits * (N / (PAIRS ? K::XB : K::RB));
+  const long steps = unit_images(PAIRS) / (PAIRS ? 2 : 1);
   long grid = std::min<long>(nitems, (long)std::max(per_sm, 1) * sm_count());
-  if (pl != nullptr && pl->items_per_block > 0)  // an item is up to four images
-    grid = std::max(grid, std::min<long>((4 * nitems + pl->items_per_block - 1) / pl->items_per_block,
+  if (pl != nullptr && pl->items_per_block > 0)
+    grid = std::max(grid, std::min<long>((steps * nitems + pl->items_per_block - 1) / pl->items_per_block,
                                          std::min<long>(nitems, INT_MAX)));
   const bool tma = K::TILE_TMA && tm != nullptr && tm->nbox > 0 && err != nullptr;
   CUtensorMap none;
   memset(&none, 0, sizeof(none));
-  return launch_with(kern, dim3((unsigned)grid), dim3(K::THREADS_B), smem, st, pl, g, tb, Tbuf, quads, nquads,
+  return launch_with(kern, dim3((unsigned)grid), dim3(K::THREADS_B), smem, st, pl, g, tb, Tbuf, units, nunits,
                      img_base, base_base, ps, tma ? tm->map : none, tma ? tm->nbox : 0, tma ? tm->rows : 0, err);
 }
 
 template <int N>
-cudaError_t run_rowfft_tree(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Quad* quads,
-                            int nquads, int img_base, int base_base, const PassStats& ps, const TileMap* tm,
-                            int* err, cudaStream_t st, const PassLaunch* pl) {
+cudaError_t run_rowfft_tree(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Unit* units,
+                            int nunits, bool pairs, int img_base, int base_base, const PassStats& ps,
+                            const TileMap* tm, int* err, cudaStream_t st, const PassLaunch* pl) {
   static_assert(N >= kTreeMinNpix, "whole warps");
-  if (ps.clip != nullptr)
-    return run_rowfft_tree_k<N, true>(g, tb, Tbuf, quads, nquads, img_base, base_base, ps, tm, err, st, pl);
-  return run_rowfft_tree_k<N, false>(g, tb, Tbuf, quads, nquads, img_base, base_base, ps, tm, err, st, pl);
+#define RF_UNITS(M, P) run_rowfft_tree_k<N, M, P>(g, tb, Tbuf, units, nunits, img_base, base_base, ps, tm, err, st, pl)
+  if (pairs) {
+    if constexpr (pairs_possible(N))
+      return ps.clip ? RF_UNITS(kClip, true) : (ps.best ? RF_UNITS(kBest, true) : RF_UNITS(kParts, true));
+    return cudaErrorInvalidValue;
+  }
+  return ps.clip ? RF_UNITS(kClip, false) : (ps.best ? RF_UNITS(kBest, false) : RF_UNITS(kParts, false));
+#undef RF_UNITS
 }
 
 template <int N>
@@ -1420,7 +1765,7 @@ void fill_shape(ImageKernelShape* o) {
 
 #define RF_INSTANTIATE_IMAGE(N)                                                                              \
   template cudaError_t run_colfft<N>(const SegmentGeom&, const DevTables&, const Group*, int, int, int, int, \
-                                     const float2*, float2*, float*, float*, cudaStream_t,                  \
+                                     const float2*, float2*, float*, float*, bool, cudaStream_t,            \
                                      const PassLaunch*);                                                    \
   template cudaError_t run_rowfft_stats<N>(const SegmentGeom&, const DevTables&, const float2*, int, int,    \
                                            const double*, const PassStats&, float*, const TileMap*, int*,   \
@@ -1430,8 +1775,8 @@ void fill_shape(ImageKernelShape* o) {
                                            int, StatPartial*, const TileMap*, int*, cudaStream_t);
 
 #define RF_INSTANTIATE_TREE(N)                                                                               \
-  template cudaError_t run_rowfft_tree<N>(const SegmentGeom&, const DevTables&, const float2*, const Quad*,  \
-                                          int, int, int, const PassStats&, const TileMap*, int*,             \
+  template cudaError_t run_rowfft_tree<N>(const SegmentGeom&, const DevTables&, const float2*, const Unit*,  \
+                                          int, bool, int, int, const PassStats&, const TileMap*, int*,       \
                                           cudaStream_t, const PassLaunch*);
 
 }  // namespace rf

@@ -1,4 +1,4 @@
-// Row pass with derived images (sums of two and four) for image sides 64 .. 8192.
+// Row pass with derived images (sums of 2 .. 16 images) for image sides 64 .. 8192.
 #include "rf_image.cuh"
 
 namespace rf {

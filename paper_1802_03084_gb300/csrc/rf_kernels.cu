@@ -450,7 +450,8 @@ __device__ __forceinline__ double parseval_sum(const float* __restrict__ cs, int
 // sigma} of the raw image J = 2W I.
 __global__ void k_image_noise(int ncol, const float* __restrict__ colsq, const float* __restrict__ mean0,
                               const double* __restrict__ weight, int nimg, int img_base, double threshold,
-                              ImgNoise* __restrict__ noise, float* __restrict__ gate, float2* __restrict__ clip) {
+                              ImgNoise* __restrict__ noise, float* __restrict__ gate,
+                              unsigned long long* __restrict__ best, float2* __restrict__ clip) {
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (i >= nimg) return;
@@ -464,7 +465,10 @@ __global__ void k_image_noise(int ncol, const float* __restrict__ colsq, const f
   var = var > 0.0 ? var : 0.0;
   const double sigma = sqrt(var);
   noise[i] = ImgNoise{mean, sigma};
-  if (gate != nullptr) gate[i] = (float)(threshold * sigma * (2.0 * W) * (1.0 - 1e-5));
+  if (gate != nullptr) {
+    gate[i] = (float)(threshold * sigma * (2.0 * W) * (1.0 - 1e-5));
+    best[i] = 0;
+  }
   if (clip != nullptr) {
     double raw = sq - (double)m * (double)m;
     raw = raw > 0.0 ? raw : 0.0;
@@ -473,13 +477,76 @@ __global__ void k_image_noise(int ncol, const float* __restrict__ colsq, const f
 }
 
 cudaError_t launch_image_noise(const SegmentGeom& g, const float* colsq, const float* mean0, const double* weight,
-                               int nimg, int img_base, double threshold, ImgNoise* noise, float* gate, float2* clip,
-                               cudaStream_t st) {
+                               int nimg, int img_base, double threshold, ImgNoise* noise, float* gate,
+                               unsigned long long* best, float2* clip, cudaStream_t st) {
   if (nimg <= 0) return cudaSuccess;
   k_image_noise<<<(nimg + 7) / 8, 256, 0, st>>>(g.ncol, colsq, mean0, weight, nimg, img_base, threshold, noise, gate,
-                                                clip);
+                                                best, clip);
   return cudaGetLastError();
 }
+
+// Sigma, S/N, threshold and record of one image with raw maximum mx at pixel
+// mi; under the clipped noise from the kept pixels' deviations d from mean0 (raw
+// units): kn of them, sums ks1 of d and ks2 of d^2.
+__device__ __forceinline__ void finalize_image(int npix, float mx, int mi, bool clip, long long kn, double ks1,
+                                               double ks2, int i, int img, const ImgNoise* __restrict__ noise,
+                                               const float* __restrict__ mean0, const int4* __restrict__ img_info,
+                                               const double* __restrict__ weight, double threshold,
+                                               DevCand* __restrict__ cands, int* __restrict__ ncand, int cand_cap,
+                                               DevStat* __restrict__ stats) {
+  const double W = weight[img];
+  const int4 info = img_info[img];
+  DevStat ds;
+  ds.pad = 0;
+  ds.weight = W;
+  if (!(W > 0.0)) {
+    ds.peak = 0.f;
+    ds.sigma = 0.f;
+    ds.snr = 0.f;
+    ds.x = 0;
+    ds.y = 0;
+    ds.mean = 0.0;
+    if (stats) stats[info.w] = ds;
+    return;
+  }
+  const double inv = 0.5 / W;
+  double mean = noise[i].mean;
+  double sigma = noise[i].sigma;
+  if (clip) {
+    const double n = kn > 0 ? (double)kn : 1.0;
+    const double m1 = ks1 / n;
+    mean = ((double)mean0[i] + m1) * inv;
+    const double var = (ks2 / n - m1 * m1) * inv * inv;
+    sigma = sqrt(var > 0.0 ? var : 0.0);
+  }
+  const double peak = (double)mx * inv;
+  const double snr = sigma > 0.0 ? peak / sigma : 0.0;
+  const int y = mi / npix;
+  const int x = mi - y * npix;
+  ds.peak = (float)peak;
+  ds.sigma = (float)sigma;
+  ds.snr = (float)snr;
+  ds.x = x;
+  ds.y = y;
+  ds.mean = mean;
+  if (stats) stats[info.w] = ds;
+  if (sigma > 0.0 && snr >= threshold) {
+    const int k = atomicAdd(ncand, 1);
+    if (k < cand_cap) {
+      DevCand c;
+      c.d = info.x;
+      c.s = info.y;
+      c.t = info.z;
+      c.x = x;
+      c.y = y;
+      c.snr = (float)snr;
+      c.peak = (float)peak;
+      c.sigma = (float)sigma;
+      cands[k] = c;
+    }
+  }
+}
+
 
 __global__ void k_finalize(int npix, int nrb, const PassStats ps, const ImgNoise* __restrict__ noise,
                            const float* __restrict__ mean0, const int4* __restrict__ img_info,
@@ -526,67 +593,33 @@ __global__ void k_finalize(int npix, int nrb, const PassStats ps, const ImgNoise
     }
   }
   if (lane != 0) return;
-  const double W = weight[img];
-  const int4 info = img_info[img];
-  DevStat ds;
-  ds.pad = 0;
-  ds.weight = W;
-  if (!(W > 0.0)) {
-    ds.peak = 0.f;
-    ds.sigma = 0.f;
-    ds.snr = 0.f;
-    ds.x = 0;
-    ds.y = 0;
-    ds.mean = 0.0;
-    if (stats) stats[info.w] = ds;
-    return;
-  }
-  const double inv = 0.5 / W;
-  double mean = noise[i].mean;
-  double sigma = noise[i].sigma;
-  if (clip) {
-    // clipped noise: the kept pixels' deviations d from mean0 (raw units)
-    const double n = kn > 0 ? (double)kn : 1.0;
-    const double m1 = ks1 / n;
-    mean = ((double)mean0[i] + m1) * inv;
-    const double var = (ks2 / n - m1 * m1) * inv * inv;
-    sigma = sqrt(var > 0.0 ? var : 0.0);
-  }
-  const double peak = (double)mx * inv;
-  const double snr = sigma > 0.0 ? peak / sigma : 0.0;
-  const int y = mi / npix;
-  const int x = mi - y * npix;
-  ds.peak = (float)peak;
-  ds.sigma = (float)sigma;
-  ds.snr = (float)snr;
-  ds.x = x;
-  ds.y = y;
-  ds.mean = mean;
-  if (stats) stats[info.w] = ds;
-  if (sigma > 0.0 && snr >= threshold) {
-    const int k = atomicAdd(ncand, 1);
-    if (k < cand_cap) {
-      DevCand c;
-      c.d = info.x;
-      c.s = info.y;
-      c.t = info.z;
-      c.x = x;
-      c.y = y;
-      c.snr = (float)snr;
-      c.peak = (float)peak;
-      c.sigma = (float)sigma;
-      cands[k] = c;
-    }
-  }
+  finalize_image(npix, mx, mi, clip, kn, ks1, ks2, i, img, noise, mean0, img_info, weight, threshold, cands, ncand,
+                 cand_cap, stats);
 }
 
-cudaError_t launch_finalize(const SegmentGeom& g, const PassStats& ps, const ImgNoise* noise, const float* mean0,
-                            const int4* img_info, const double* weight, int nimg, int img_base, double threshold,
+// The same where the row pass kept each image's largest pixel only if it can be
+// a candidate's: one thread per image.
+__global__ void k_finalize_best(int npix, const unsigned long long* __restrict__ best,
+                                const ImgNoise* __restrict__ noise, const float* __restrict__ mean0,
+                                const int4* __restrict__ img_info, const double* __restrict__ weight, int nimg,
+                                int img_base, double threshold, DevCand* __restrict__ cands, int* __restrict__ ncand,
+                                int cand_cap) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nimg || best[i] == 0) return;
+  finalize_image(npix, best_max(best[i]), best_pixel(best[i]), false, 0, 0.0, 0.0, i, img_base + i, noise, mean0,
+                 img_info, weight, threshold, cands, ncand, cand_cap, nullptr);
+}
+
+cudaError_t launch_finalize(const SegmentGeom& g, const PassStats& ps, int nparts, const ImgNoise* noise,
+                            const float* mean0, const int4* img_info, const double* weight, int nimg, int img_base, double threshold,
                             DevCand* cands, int* ncand, int cand_cap, DevStat* stats, cudaStream_t st) {
   if (nimg <= 0) return cudaSuccess;
-  ImageKernelShape sh;
-  if (!image_kernel_shape(g.npix, &sh)) return cudaErrorInvalidValue;
-  k_finalize<<<(nimg + 7) / 8, 256, 0, st>>>(g.npix, sh.partials_per_image, ps, noise, mean0, img_info, weight, nimg,
+  if (ps.best != nullptr && stats == nullptr) {
+    k_finalize_best<<<(nimg + 127) / 128, 128, 0, st>>>(g.npix, ps.best, noise, mean0, img_info, weight, nimg,
+                                                        img_base, threshold, cands, ncand, cand_cap);
+    return cudaGetLastError();
+  }
+  k_finalize<<<(nimg + 7) / 8, 256, 0, st>>>(g.npix, nparts, ps, noise, mean0, img_info, weight, nimg,
                                               img_base, threshold, cands, ncand, cand_cap, stats);
   return cudaGetLastError();
 }
@@ -594,9 +627,9 @@ cudaError_t launch_finalize(const SegmentGeom& g, const PassStats& ps, const Img
 // --------------------------------------------------------------- dispatch --
 template <int N>
 cudaError_t run_colfft(const SegmentGeom&, const DevTables&, const Group*, int, int, int, int, const float2*, float2*,
-                       float*, float*, cudaStream_t, const PassLaunch*);
+                       float*, float*, bool, cudaStream_t, const PassLaunch*);
 template <int N>
-cudaError_t run_rowfft_tree(const SegmentGeom&, const DevTables&, const float2*, const Quad*, int, int, int,
+cudaError_t run_rowfft_tree(const SegmentGeom&, const DevTables&, const float2*, const Unit*, int, bool, int, int,
                             const PassStats&, const TileMap*, int*, cudaStream_t, const PassLaunch*);
 template <int N>
 cudaError_t run_rowfft_stats(const SegmentGeom&, const DevTables&, const float2*, int, int, const double*,
@@ -611,11 +644,12 @@ cudaError_t run_rowfft_power(const SegmentGeom&, const DevTables&, const float2*
 
 cudaError_t launch_colfft(const SegmentGeom& g, const DevTables& tb, const Group* groups, int g_begin,
                           int ngroups, int img_base, int base_base, const float2* cellbuf, float2* Tbuf, float* colsq,
-                          float* mean0, cudaStream_t st, const PassLaunch* pl) {
+                          float* mean0, bool duo, cudaStream_t st, const PassLaunch* pl) {
   switch (g.npix) {
 #define RF_CASE(N) \
   case N:          \
-    return run_colfft<N>(g, tb, groups, g_begin, ngroups, img_base, base_base, cellbuf, Tbuf, colsq, mean0, st, pl);
+    return run_colfft<N>(g, tb, groups, g_begin, ngroups, img_base, base_base, cellbuf, Tbuf, colsq, mean0, duo, st, \
+                         pl);
     RF_FOR_EACH_N(RF_CASE)
 #undef RF_CASE
     default:
@@ -637,13 +671,13 @@ cudaError_t launch_rowfft_stats(const SegmentGeom& g, const DevTables& tb, const
   }
 }
 
-cudaError_t launch_rowfft_tree(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Quad* quads,
-                               int nquads, int img_base, int base_base, const PassStats& ps, const TileMap* tm,
-                               int* err, cudaStream_t st, const PassLaunch* pl) {
+cudaError_t launch_rowfft_tree(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Unit* units,
+                               int nunits, bool pairs, int img_base, int base_base, const PassStats& ps,
+                               const TileMap* tm, int* err, cudaStream_t st, const PassLaunch* pl) {
   switch (g.npix) {
 #define RF_CASE(N)                                                                                                 \
   case N:                                                                                                          \
-    return run_rowfft_tree<N>(g, tb, Tbuf, quads, nquads, img_base, base_base, ps, tm, err, st, pl);
+    return run_rowfft_tree<N>(g, tb, Tbuf, units, nunits, pairs, img_base, base_base, ps, tm, err, st, pl);
     RF_CASE(64) RF_CASE(128) RF_CASE(256) RF_CASE(512) RF_CASE(1024) RF_CASE(2048) RF_CASE(4096) RF_CASE(8192)
 #undef RF_CASE
     default:

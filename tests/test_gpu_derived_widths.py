@@ -1,8 +1,8 @@
 """Widths whose images are sums of another width's images against plans that
 search each width alone.
 
-In a plan whose widths hold {b, 2b, 4b}, only the images of width b are
-transformed; a plan of one width transforms every image.  Both must give the
+In a plan whose widths hold {b, 2b, 4b, 8b, 16b}, only the images of width b are
+transformed (two levels above 2048^2); a plan of one width transforms every image.  Both must give the
 same statistics.  An image's FP32 error is of order 3e-7 sigma RMS and 6 times
 that over a few million pixels, on either side, and a peak is at least 3
 sigma, so peaks agree to 1e-6 relative; 2e-5 is asked for.  Where the pixel
@@ -51,6 +51,14 @@ def engine():
     (2048, 18, [1, 4], True, rf.RF_NOISE_CLIPPED),
     (4096, 14, [1, 2, 4], True, 0),
     (8192, 7, [1, 2, 4], True, 0),
+    (64, 66, [1, 16], False, 0),
+    (128, 47, [1, 2, 4, 8, 16], True, rf.RF_NOISE_CLIPPED),
+    (256, 100, [3, 6, 12, 24, 48], False, 0),
+    (512, 37, [1, 8, 3], True, rf.RF_STORE_FP16),
+    (1024, 49, [16, 1, 2, 8], False, 0),
+    (1024, 32, [1, 16], True, rf.RF_NOISE_CLIPPED),
+    (2048, 33, [1, 4, 16, 8], True, rf.RF_STORE_FP16),
+    (2048, 17, [1, 8, 2], False, rf.RF_NOISE_CLIPPED),
 ])
 def test_derived_widths_equal_widths_alone(npix, nint, dts, partial, flags):
     rng = np.random.default_rng(npix + nint)
