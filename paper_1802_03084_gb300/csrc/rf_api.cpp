@@ -212,6 +212,7 @@ struct rf_plan {
   std::vector<int32_t> col_ent_ptr, col_cell_ptr, cell_row;
   std::vector<int32_t> col_run_ptr, col_runs;  // runs of each column (see DevTables::col_runs)
   std::vector<float2> col_run_tw;              // their twiddles (see DevTables::col_run_tw)
+  std::vector<int2> col_lane;     // runs of each lane of a column sub-transform (see DevTables)
   std::vector<int2> ranges;
   std::vector<int4> plain_ent;  // {bc, col, row, flags} for the plain form
   std::vector<GridEntry> ent;
@@ -527,8 +528,23 @@ rf_status build_tables(rf_plan* p) {
     }
 
   // half-plane columns 0..iu_max: entries sorted by (col, row, bc, flags)
+  // Within a column, rows sort by (v1 mod TL, v1 div TL, v div L), v1 = v mod
+  // L, L = N / col_split(N), TL = col_lanes(L): the batched column pass finds
+  // the rows that share v1 (combined by its decimation-in-frequency step) next
+  // to each other, and those that one of its lanes takes in that lane's order.
+  const int Lc = N / rf::col_split(N), TLc = rf::col_lanes(Lc);
+  std::vector<int> place(N);  // order of the rows of a column
+  for (int v = 0; v < N; ++v) {
+    const int v1 = v % Lc;
+    place[v] = (v1 % TLc * (Lc / TLc) + v1 / TLc) * (N / Lc) + v / Lc;
+  }
   struct E {
     int col, row, bc, flags;
+    uint64_t key;  // column, then place of the row, then bc and flags
+  };
+  auto entry = [&](int col, int row, int bc, int flags) {
+    return E{col, row, bc, flags,
+             ((uint64_t)col * N + place[row]) << 31 | (uint64_t)bc << 2 | (uint64_t)flags};
   };
   std::vector<E> es;
   es.reserve((size_t)p->n_on + nbl);
@@ -541,27 +557,15 @@ rf_status build_tables(rf_plan* p) {
       const int neg = ((u + v) & 1) ? rf::ENT_NEG : 0;
       const int bc = c * nbl + bb;
       if (u > 0) {
-        es.push_back({u, mod(v), bc, neg});
+        es.push_back(entry(u, mod(v), bc, neg));
       } else if (u < 0) {
-        es.push_back({-u, mod(-v), bc, rf::ENT_CONJ | neg});
+        es.push_back(entry(-u, mod(-v), bc, rf::ENT_CONJ | neg));
       } else {
-        es.push_back({0, mod(v), bc, neg});
-        es.push_back({0, mod(-v), bc, rf::ENT_CONJ | neg});
+        es.push_back(entry(0, mod(v), bc, neg));
+        es.push_back(entry(0, mod(-v), bc, rf::ENT_CONJ | neg));
       }
     }
-  // Within a column, rows sort by (v mod L, v div L), L = N / col_split(N):
-  // the batched column pass finds the rows that share v mod L (combined by
-  // its decimation-in-frequency gather) next to each other.  For N <= 1024,
-  // L = N and this is plain row order.
-  const int Lc = N / rf::col_split(N);
-  std::sort(es.begin(), es.end(), [Lc](const E& a, const E& b2) {
-    if (a.col != b2.col) return a.col < b2.col;
-    const int ka = a.row % Lc, kb = b2.row % Lc;
-    if (ka != kb) return ka < kb;
-    if (a.row != b2.row) return a.row < b2.row;
-    if (a.bc != b2.bc) return a.bc < b2.bc;
-    return a.flags < b2.flags;
-  });
+  std::sort(es.begin(), es.end(), [](const E& a, const E& b2) { return a.key < b2.key; });
   p->ncol = p->n_on > 0 ? p->iu_max + 1 : 1;
   if (!rf::image_kernel_shape(N, &p->shape)) return fail(RF_ERR_INVALID_ARG, "npix %d has no kernel", N);
   p->plain_ent.clear();
@@ -600,6 +604,7 @@ rf_status build_tables(rf_plan* p) {
   // runs of each column for the column pass's scatter
   p->col_run_ptr.assign(p->ncol + 1, 0);
   p->col_runs.clear();
+  p->col_lane.assign((size_t)p->ncol * TLc, make_int2(0, 0));
   for (int col = 0; col < p->ncol; ++col) {
     const int c0 = p->col_cell_ptr[col], c1 = p->col_cell_ptr[col + 1];
     p->col_run_ptr[col] = (int)p->col_runs.size();
@@ -607,6 +612,9 @@ rf_status build_tables(rf_plan* p) {
       const int v1 = p->cell_row[c] % Lc;
       int n = 1;
       while (c + n < c1 && p->cell_row[c + n] % Lc == v1) ++n;
+      int2& lane = p->col_lane[(size_t)col * TLc + v1 % TLc];
+      if (lane.x == 0) lane.y = (int)p->col_runs.size() - p->col_run_ptr[col];
+      lane.x = (int)((unsigned)lane.x | 1u << (v1 / TLc));
       p->col_runs.push_back(((c - c0) << 4) | n);
       c += n;
     }
@@ -940,7 +948,7 @@ uint64_t estimate_device_bytes(const rf_plan* p, int slots) {
   auto r = [](size_t n, size_t sz) { return (uint64_t)std::max<size_t>(n, 1) * sz; };
   uint64_t b = 0;
   b += r(p->delays.size(), 4) + r(p->dt.size(), 4) + r(p->ranges.size(), 8) + r(p->col_cell_ptr.size(), 4) +
-       r(p->cell_row.size(), 4) + r(p->col_run_ptr.size(), 4) + r(p->col_runs.size(), 4) + r(p->col_run_tw.size(), 8) + r(p->ent.size(), sizeof(GridEntry)) + r(p->ongrid_chan.size(), 4) + r(rf::fft_twiddle_len((int)N), 8);
+       r(p->cell_row.size(), 4) + r(p->col_run_ptr.size(), 4) + r(p->col_runs.size(), 4) + r(p->col_lane.size(), 8) + r(p->col_run_tw.size(), 8) + r(p->ent.size(), sizeof(GridEntry)) + r(p->ongrid_chan.size(), 4) + r(rf::fft_twiddle_len((int)N), 8);
   if (rf::col_split((int)N) > 1) b += r(rf::fft_twiddle_len((int)N / rf::col_split((int)N)), 8);
   const size_t nint_pad = (p->max_nint + 31) / 32 * 32;
   const size_t esz = (p->flags & RF_STORE_FP16) ? 4 : 8;
@@ -989,6 +997,7 @@ rf_status alloc_device(rf_plan* p) {
   int32_t *d_delays = nullptr, *d_dt = nullptr, *d_ogc = nullptr, *d_ccp = nullptr, *d_crow = nullptr,
           *d_rptr = nullptr, *d_runs = nullptr;
   float2* d_rtw = nullptr;
+  int2* d_clane = nullptr;
   int2* d_ranges = nullptr;
   GridEntry* d_ent = nullptr;
   rf_status s;
@@ -1001,6 +1010,7 @@ rf_status alloc_device(rf_plan* p) {
   if ((s = up(&d_rptr, p->col_run_ptr)) != RF_OK) return s;
   if ((s = up(&d_runs, p->col_runs)) != RF_OK) return s;
   if ((s = up(&d_rtw, p->col_run_tw)) != RF_OK) return s;
+  if ((s = up(&d_clane, p->col_lane)) != RF_OK) return s;
   if ((s = up(&d_ent, p->ent)) != RF_OK) return s;
   if ((s = up(&d_ogc, p->ongrid_chan)) != RF_OK) return s;
   std::vector<float2> tw(rf::fft_twiddle_len(N));
@@ -1022,6 +1032,7 @@ rf_status alloc_device(rf_plan* p) {
   p->tb.col_run_ptr = d_rptr;
   p->tb.col_runs = d_runs;
   p->tb.col_run_tw = d_rtw;
+  p->tb.col_lane = d_clane;
   p->tb.ent = d_ent;
   p->tb.ongrid_chan = d_ogc;
   p->tb.twiddle = d_tw;

@@ -41,11 +41,15 @@ struct DevTables {
   // with L = N / col_split(N) (the same table as `twiddle` when N <= 1024)
   const float2* twiddle_col;
   // runs of every imaged column: the column's cells at rows v1 + L v2 for one
-  // v1 (cells sort by (v mod L, v div L) within a column, so a run is
+  // v1 (cells sort by (v1 mod TL, v1 div TL, v2) within a column, so a run is
   // consecutive); col_runs[col_run_ptr[col] + j] = (first cell << 4) | cells,
   // the first cell counted within the column
   const int32_t* col_run_ptr;   // [ncol + 1]
   const int32_t* col_runs;
+  // per column and lane t of the TL lanes of a column sub-transform (E = L / TL
+  // values a lane): x = bits r for which row t + r TL is occupied (any v2), y =
+  // the lane's first run within the column; runs sort by (lane, r)
+  const int2* col_lane;         // [ncol][TL]
   // per run j and sub-transform p = 1 .. R-1 (R = col_split(N) > 1): the
   // decimation-in-frequency twiddle w_N^(v1 p) of the run's row v1, at
   // col_run_tw[j (R - 1) + p - 1] (computed in FP64, rounded once)
@@ -387,6 +391,9 @@ inline int unit_partials(const ImageKernelShape& s, bool pairs) { return s.parti
 // Streaming multiprocessors of the current device (cached per device: launch
 // shapes are sized from it, and another GPU of the process may differ).
 int sm_count();
+
+// Lanes of one column sub-transform of length l, and values each takes.
+constexpr int col_lanes(int l) { return l >= 32 ? l / 32 : 1; }
 
 // Sets the thread-local message returned by rf_last_error().
 void set_last_error(const char* msg);

@@ -94,6 +94,10 @@ struct ColCfg {
   // values (PI images), its row and (at most) one run with its R - 1 twiddles
   static constexpr int SMEM_FIXED = XA * R * STRIDE * 8;
   static constexpr int SMEM_PER_CELL = PI * 8 + 4 + 4 + (R - 1) * 8;
+  // staged values per cell: one of padding for R = 1 (in the place of the row and run)
+  static constexpr int CELL_PITCH = R > 1 ? PI : PI + 1;
+  // the Parseval sums are reduced before the transforms, not after them
+  static constexpr bool EARLY = R >= 2;
   static_assert(TL <= 32, "column sub-transforms fit one warp");
   static_assert(R <= 8, "at most eight sub-transforms per column");
   static_assert((XA * R * STRIDE * 8) % 16 == 0, "staged cells start 16-byte aligned");
@@ -128,16 +132,6 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 
-// Column pass: the first-pass inputs of sub-transform p (of R) of staged
-// image kl, through the sub-transform's own buffer.  Its lanes zero the
-// buffer and scatter the column's runs into it: run j (cells at rows
-// v1 + L v2 for one v1) puts, for R > 1 with the decimation-in-frequency
-// step folded in,
-//   Y_p[v1] = w_N^(v1 p) sum_{v2 < R} H[v1 + L v2] w_R^(v2 p)
-// at row v1 (the run's cells in ascending v2, a fixed order; R = 1: the one
-// cell's value).  Only the sub-transform's lanes synchronise.  runs[j] =
-// (first cell << 4) | cells; cellv holds PI images per staged cell, 16-byte
-// chunks swizzled by the cell.  Not live: the buffer stays zero.
 // a times w_R^k, k < R <= 8: exact for the powers of i, the sqrt(1/2)
 // constant for the odd eighths.
 template <int R>
@@ -153,54 +147,77 @@ __device__ __forceinline__ float2 mul_wR(float2 a, int k) {
   }
 }
 
-template <int N, int PI>
-__device__ __forceinline__ void col_scatter(float2* buf, const int* __restrict__ runs, int nruns,
-                                            const float2* __restrict__ cellv, const int* __restrict__ crow, int kl,
-                                            bool live, const float2* __restrict__ rtw, int t, int p, int xsub) {
+// Column pass: the first-pass inputs v[r] = Y_p[t + r TL] of sub-transform p
+// (of R) of staged image kl.  A column has some 50 occupied rows of 1024, so
+// its runs are sorted by the lane that takes them and then by r, and a lane
+// holds a mask of its r (see DevTables::col_lane): it reads its own runs one
+// after the other, and the rows that are empty cost neither a store nor a
+// load.  Zeroing the sub-transform's buffer, scattering the runs into it and
+// loading it took some 140 of a transform's 315 shared-memory wavefronts: column
+// passes of 512^2 serving 3.64 -> 3.10 ms, 1024^2 realtime 58.5 -> 54.0, 2048^2
+// batching 92.3 -> 89.2, 4096^2 stress subset 4.31 -> 4.23.
+// R = 1: a run is a cell, read where it was staged.  R > 1: the lanes first put
+//   Y_p[v1] = w_N^(v1 p) sum_{v2 < R} H[v1 + L v2] w_R^(v2 p)
+// of every run (its cells in ascending v2, a fixed order) at the start of the
+// sub-transform's own buffer.  runs[j] = (first cell << 4) | cells; cellv holds
+// PI images per staged cell in rows of CELL_PITCH, for R > 1 with 16-byte chunks
+// swizzled by the cell.  Only the sub-transform's lanes synchronise.
+template <int N>
+__device__ __forceinline__ void col_gather(float2 (&v)[ColCfg<N>::EL], float2* buf, const int* __restrict__ runs,
+                                           int nruns, const float2* __restrict__ cellv, const int* __restrict__ crow,
+                                           int kl, bool live, const float2* __restrict__ rtw, int t, int p, int xsub,
+                                           int2 mine) {
   using C = ColCfg<N>;
-  constexpr int CPC = PI > 1 ? PI / 2 : 1;
-  constexpr int L = C::L, R = C::R, TL = C::TL, STRIDE = C::STRIDE;
-  if constexpr (STRIDE % 2 == 0) {  // 16 bytes at a time (every buffer then starts 16-byte aligned)
-    float4* buf4 = reinterpret_cast<float4*>(buf);
-    for (int i = t; i < STRIDE / 2; i += TL) buf4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  } else {
-    for (int i = t; i < STRIDE; i += TL) buf[i] = make_float2(0.f, 0.f);
-  }
-  fft_sync<TL>(xsub);
-  if (live) {
-    const int kc = kl >> 1, ko = kl & 1;
-    for (int j = t; j < nruns; j += TL) {
-      const int m = runs[j];
-      const int c0 = m >> 4;
-      const int v1 = crow[c0] & (L - 1);
-      float2 a = cellv[c0 * PI + 2 * (kc ^ (c0 & (CPC - 1))) + ko];
-      if constexpr (R > 1) {
+  constexpr int PI = C::PI, CPC = PI / 2;
+  constexpr int L = C::L, R = C::R, TL = C::TL, EL = C::EL;
+  const unsigned mask = live ? (unsigned)mine.x : 0u;
+  const float2* q;
+  constexpr int STEP = R > 1 ? 1 : C::CELL_PITCH;
+  if constexpr (R > 1) {
+    if (live) {
+      const int kc = kl >> 1, ko = kl & 1;
+      for (int j = t; j < nruns; j += TL) {
+        const int m = runs[j];
+        const int c0 = m >> 4;
+        float2 a = cellv[c0 * PI + 2 * (kc ^ (c0 & (CPC - 1))) + ko];
         const int n = m & 15;
         if (p > 0) a = mul_wR<R>(a, ((crow[c0] >> C::LOG2L) * p) & (R - 1));
-        for (int q = 1; q < n; ++q) {
-          const int c = c0 + q;
+        for (int i = 1; i < n; ++i) {
+          const int c = c0 + i;
           float2 h = cellv[c * PI + 2 * (kc ^ (c & (CPC - 1))) + ko];
           if (p > 0) h = mul_wR<R>(h, ((crow[c] >> C::LOG2L) * p) & (R - 1));
           a = cadd(a, h);
         }
         if (p > 0) a = cmul(a, rtw[j * (R - 1) + p - 1]);  // w_N^(v1 p), staged per run
+        buf[j] = a;
       }
-      buf[padx(v1)] = a;
+    }
+    static_assert(L <= C::STRIDE, "runs fit the buffer");
+    fft_sync<TL>(xsub);
+    q = buf + mine.y;
+  } else {
+    q = cellv + mine.y * STEP + kl;
+  }
+#pragma unroll
+  for (int r = 0; r < EL; ++r) {
+    v[r] = make_float2(0.f, 0.f);
+    if (mask >> r & 1u) {
+      v[r] = *q;
+      q += STEP;
     }
   }
-  fft_sync<TL>(xsub);
+  if constexpr (R > 1) fft_sync<TL>(xsub);  // all runs are read before the first pass stores
 }
 
-// The length-L inverse FFT of the inputs col_scatter put in `buf`
+// The length-L inverse FFT of the inputs v through `buf`
 // (sub-transform xsub of the block), written to dst[0 .. L) if dst, output o at
 // o ^ sw.
 template <int N>
-__device__ __forceinline__ void col_fft_store(float2* buf, const float2* __restrict__ twc, int t, int xsub,
+__device__ __forceinline__ void col_fft_store(float2 (&v)[ColCfg<N>::EL], float2* buf, const float2* __restrict__ twc, int t, int xsub,
                                               float2* __restrict__ dst, int sw) {
   using C = ColCfg<N>;
   constexpr int L = C::L, TL = C::TL, EL = C::EL;
-  float2 v[EL];
-  fft_inverse_to_regs<L, true>(v, buf, twc, t, xsub);  // packed style (see rf_fft.cuh)
+  fft_inverse_from_regs<L, true>(v, buf, twc, t, xsub);  // packed style (see rf_fft.cuh)
   if (dst != nullptr) {
     constexpr int LP = FftShape<L>::LAST_P;
 #pragma unroll
@@ -218,11 +235,10 @@ __device__ __forceinline__ void col_fft_store(float2* buf, const float2* __restr
 // Pass A2: the column FFTs of one group (up to 32 consecutive t' of a
 // trial) and one half-plane column u.  The column's cell sums for the
 // group's images (cellbuf row per cell, 32 images) are copied to shared
-// memory with cp.async (16-byte chunks XOR-swizzled by cell), PI images at a
-// time.  Each column is R = col_split(N) sub-transforms of length L = N/R.
-// In rounds of XA images, each sub-transform zeroes its own buffer and
-// scatters the column's runs into it (col_scatter), which for R > 1 folds in
-// one decimation-in-frequency step: sub-transform p takes
+// memory with cp.async, PI images at a time.  Each column is R = col_split(N)
+// sub-transforms of length L = N/R.  In rounds of XA images, each
+// sub-transform takes the column's runs (col_gather), which for R > 1 folds
+// in one decimation-in-frequency step: sub-transform p takes
 //   Y_p[v1] = w_N^(v1 p) sum_{v2 < R} H[v1 + L v2] w_R^(v2 p),
 // and its length-L inverse FFT is column output y = R k + p at k, stored at
 // T[slot][u][p L + k] (see SegmentGeom::tsplit).  A sub-transform
@@ -239,7 +255,8 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
   constexpr int L = C::L, R = C::R, TL = C::TL;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* fbuf = reinterpret_cast<float2*>(smraw);                       // [XA][R][STRIDE]
-  float2* cellv = reinterpret_cast<float2*>(fbuf + C::XA * R * C::STRIDE);  // [max_cells][PI], swizzled
+  float2* cellv = reinterpret_cast<float2*>(fbuf + C::XA * R * C::STRIDE);  // [max_cells][CELL_PITCH]
+  // R > 1 only
   float2* rtw = cellv + (size_t)g.max_cells * PI;                           // [max_cells][R - 1]
   int* crow = reinterpret_cast<int*>(rtw + (size_t)g.max_cells * (R - 1));  // [max_cells]
   int* runs = crow + g.max_cells;                                           // [max_cells]
@@ -255,21 +272,32 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
   // and barrier below
   const int run0 = tb.col_run_ptr[col];
   const int nruns = tb.col_run_ptr[col + 1] - run0;
-  for (int c = tid; c < ncells; c += C::THREADS) crow[c] = tb.cell_row[cell0 + c];
-  for (int j = tid; j < nruns; j += C::THREADS) runs[j] = tb.col_runs[run0 + j];
-  if constexpr (R > 1)
+  if constexpr (R > 1) {
+    for (int c = tid; c < ncells; c += C::THREADS) crow[c] = tb.cell_row[cell0 + c];
+    for (int j = tid; j < nruns; j += C::THREADS) runs[j] = tb.col_runs[run0 + j];
     for (int i = tid; i < nruns * (R - 1); i += C::THREADS) rtw[i] = tb.col_run_tw[(size_t)run0 * (R - 1) + i];
+  }
+  const bool dc = col == 0 && ncells > 0 && tb.cell_row[cell0] == 0;  // row 0 sorts first
   const int xf = tid / (R * TL);          // image of the round
   const int p = (tid / TL) % R;           // sub-transform: output rows y = p mod R
   const int t = tid % TL;
+  const int2 mine = tb.col_lane[(size_t)col * TL + t];
   float2* buf = fbuf + (xf * R + p) * C::STRIDE;
   const int sw = duo ? duo_swizzle(N, col) : 0;
   for (int kbase = 0; kbase < gr.nimg; kbase += PI) {
     if (kbase > 0) __syncthreads();  // the previous part's cells are consumed
-    for (int i = tid; i < ncells * CPC; i += C::THREADS) {
-      const int c = i / CPC;
-      const int j = i - c * CPC;
-      cp_async16(cellv + c * PI + 2 * (j ^ (c & (CPC - 1))), src + c * 32 + kbase + 2 * j);
+    if constexpr (R > 1) {
+      for (int i = tid; i < ncells * CPC; i += C::THREADS) {
+        const int c = i / CPC;
+        const int j = i - c * CPC;
+        cp_async16(cellv + c * PI + 2 * (j ^ (c & (CPC - 1))), src + c * 32 + kbase + 2 * j);
+      }
+    } else {
+      for (int i = tid; i < ncells * PI; i += C::THREADS) {
+        const int c = i / PI;
+        const int j = i - c * PI;
+        cp_async8(cellv + c * C::CELL_PITCH + j, src + c * 32 + kbase + j);
+      }
     }
     cp_async_commit();
     cp_async_wait_all();
@@ -281,20 +309,26 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
     // twice unless u = 0; its mean is G(0, 0) / (2 W).  Lane k is image k of
     // the part (two cells a step where the part is 16 images), so the cells of
     // a sum of 2, 4, 8 or 16 images are xor-shuffles away; the warps' FP32
-    // sums meet in the first FFT buffer and are added in a fixed order.
+    // sums meet in the first FFT buffer and are added in a fixed order: after
+    // the transforms, so that no barrier stands before those, unless the
+    // sums' registers would spill there (C::EARLY).
+    constexpr int NL = N < kTreeMinNpix ? 0 : (pairs_possible(N) ? 4 : 2);
+    constexpr int NW = C::THREADS / 32, CPS = 32 / PI;
+    const int warp = tid >> 5, kp = lane & (PI - 1);
+    auto at = [&](int c, int k) {
+      return R > 1 ? c * PI + 2 * ((k >> 1) ^ (c & (CPC - 1))) + (k & 1) : c * C::CELL_PITCH + k;
+    };
+    float a[NL + 1] = {};
+    int top = 0;
     {
-      constexpr int NW = C::THREADS / 32, CPS = 32 / PI;
-      constexpr int NL = N < kTreeMinNpix ? 0 : (pairs_possible(N) ? 4 : 2);
-      int top = 0;
 #pragma unroll
       for (int lv = 1; lv <= NL; ++lv)
         if (gp->nsum[lv - 1] > 0) top = lv;
-      const int warp = tid >> 5, kl = lane & (PI - 1);
-      float a[NL + 1] = {};
+#pragma unroll 2
       for (int cb = warp * CPS; cb < ncells; cb += NW * CPS) {
         const int c = cb + lane / PI;
         float2 h = make_float2(0.f, 0.f);
-        if (c < ncells && kl < nk) h = cellv[c * PI + 2 * ((kl >> 1) ^ (c & (CPC - 1))) + (kl & 1)];
+        if (c < ncells && kp < nk) h = cellv[at(c, kp)];
         a[0] = fmaf(h.x, h.x, fmaf(h.y, h.y, a[0]));
 #pragma unroll
         for (int lv = 1; lv <= NL; ++lv)
@@ -306,6 +340,9 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
       }
       static_assert(CPS <= 2 && (1 << NL) <= PI && NL < NW && NW * (NL + 1) * 32 * 4 <= C::SMEM_FIXED,
                     "Parseval sums fit the FFT buffers, the sums' images one part, their levels the warps");
+    }
+
+    auto reduce = [&] {
       float* red = reinterpret_cast<float*>(fbuf);  // [level][warp][32]
 #pragma unroll
       for (int lv = 0; lv <= NL; ++lv)
@@ -324,16 +361,17 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
           const size_t slot = (size_t)((lv == 0 ? gr.img0 : gp->isum[lv - 1]) + j - img_base);
           colsq[slot * g.ncol + col] = (col == 0 ? 1.f : 2.f) * acc;
           if (col == 0) {
-            // row 0 sorts first in column 0; cell 0's chunks are unswizzled
             float m = 0.f;
-            if (ncells > 0 && crow[0] == 0) {
-              for (int i = 0; i < 1 << lv; ++i) m += cellv[lane + i].x;
-            }
+            if (dc)
+              for (int i = 0; i < 1 << lv; ++i) m += cellv[at(0, lane + i)].x;
             mean0[slot] = m;
           }
         }
       }
-      __syncthreads();  // the FFT buffer is free again
+    };
+    if constexpr (C::EARLY) {
+      reduce();
+      __syncthreads();  // the FFT buffers are free again
     }
 
     if (xf < C::XA) {
@@ -342,9 +380,15 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
         const int kl = rd * C::XA + xf;
         const bool live = kl < nk;
         float2* dst = live ? Tbuf + ((size_t)(gr.base0 + kbase + kl - base_base) * g.ncol + col) * N + p * L : nullptr;
-        col_scatter<N, PI>(buf, runs, nruns, cellv, crow, kl, live, rtw, t, p, xf * R + p);
-        col_fft_store<N>(buf, tb.twiddle_col, t, xf * R + p, dst, sw);
+        float2 v[C::EL];
+        col_gather<N>(v, buf, runs, nruns, cellv, crow, kl, live, rtw, t, p, xf * R + p, mine);
+        col_fft_store<N>(v, buf, tb.twiddle_col, t, xf * R + p, dst, sw);
       }
+    }
+
+    if constexpr (!C::EARLY) {
+      __syncthreads();  // the FFT buffers are free
+      reduce();
     }
   }
 }
