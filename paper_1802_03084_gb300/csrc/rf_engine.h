@@ -302,6 +302,11 @@ cudaError_t launch_weights(const int4* img_info, int nimg, bool partial, const S
 cudaError_t launch_grid_cells(const SegmentGeom& g, const DevTables& tb, const Group* groups, int g_begin,
                               int ngroups, float2* cellbuf, cudaStream_t st);
 
+// The same for groups of one image each, of any trials: from the series
+// resampled to each one's width, or, with `direct`, from S (bitwise the same).
+cudaError_t launch_grid_single(const SegmentGeom& g, const DevTables& tb, const Group* groups, int g_begin,
+                               int ngroups, const void* S, bool direct, float2* cellbuf, cudaStream_t st);
+
 // Column FFTs (pass A2) of the same groups from cellbuf; writes
 // Tbuf[b][col][y], b = transformed-image index - base_base, and for every
 // image of the groups, sums of two and four included, the Parseval sums
