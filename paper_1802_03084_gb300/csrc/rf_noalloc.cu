@@ -33,7 +33,7 @@ constexpr int kMaxDevices = 64;
 // the same call first, so nothing has to start at zero.
 constexpr size_t kTBytes = (size_t)kMaxN * (kMaxN / 2) * sizeof(float2);
 constexpr size_t kPartialBytes = (size_t)ImgCfg<kMaxN>::PARTIALS * sizeof(StatPartial);
-constexpr size_t kColsqBytes = (kMaxN / 2 + 64) * sizeof(float);  // Parseval column sums + mean term
+constexpr size_t kColsqBytes = (kMaxN / 2 + 64) * sizeof(float);  // Parseval column sums, mean term, block count
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kTBytes + kPartialBytes + kColsqBytes];
 
 // Twiddle tables of the length-N transforms (fft_twiddle_table) for N = 16,
@@ -139,15 +139,16 @@ __global__ void __launch_bounds__(ImgCfg<N>::T * ImgCfg<N>::XA)
   }
 }
 
-// Reduce the row-block partials and the Parseval column sums of one image into
-// an rf_image_stat: one block, its threads strided over both, then a fixed
-// tree of the lanes and of the warps.  One thread walking them in turn waits
-// for a load after a load: a call at 1024^2 took 73.7 us so, 41.0 this way.
-constexpr int kFinalThreads = 256;
-__global__ void __launch_bounds__(kFinalThreads)
-    k_noalloc_finalize(const StatPartial* __restrict__ partials, int nrb, const float* __restrict__ colsq,
-                       const float* __restrict__ mean0, int npix, double weight, rf_image_stat* __restrict__ out) {
-  constexpr int NW = kFinalThreads / 32;
+// Reduce the row partials and the Parseval column sums of one image into an
+// rf_image_stat by the THREADS threads of one block: strided over both, then a
+// fixed tree of the lanes and of the warps.  (One thread walking them in turn
+// waits for a load after a load: a call at 1024^2 took 73.7 us so, 41.0 this
+// way.)
+template <int THREADS>
+__device__ __forceinline__ void noalloc_finalize(const StatPartial* __restrict__ partials, int nparts,
+                                                 const float* __restrict__ colsq, const float* __restrict__ mean0,
+                                                 int npix, double weight, rf_image_stat* __restrict__ out) {
+  constexpr int NW = THREADS / 32;
   __shared__ double w_sq[NW];
   __shared__ float w_max[NW];
   __shared__ int w_idx[NW];
@@ -155,11 +156,14 @@ __global__ void __launch_bounds__(kFinalThreads)
   double sq = 0.0;
   float mx = -FLT_MAX;
   int mi = INT_MAX;
-  for (int r = tid; r < nrb; r += kFinalThreads) {
-    const StatPartial p = partials[r];
-    max_merge(mx, mi, p.max, p.idx);
+  // read past the first level cache: other blocks of the same launch wrote them
+#pragma unroll 8
+  for (int r = tid; r < nparts; r += THREADS) {
+    const float2 p = __ldcg(reinterpret_cast<const float2*>(partials) + r);
+    max_merge(mx, mi, p.x, __float_as_int(p.y));
   }
-  for (int c = tid; c < npix / 2; c += kFinalThreads) sq += (double)colsq[c];
+#pragma unroll 8
+  for (int c = tid; c < npix / 2; c += THREADS) sq += (double)__ldcg(colsq + c);
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     sq += __shfl_xor_sync(0xffffffffu, sq, off);
@@ -180,7 +184,7 @@ __global__ void __launch_bounds__(kFinalThreads)
   }
   // mean = G(0,0) / 2W; mean of I^2 = sum_full |G|^2 / 4W^2 (Parseval)
   const double inv = 0.5 / weight;
-  const double mean = (double)*mean0 * inv;
+  const double mean = (double)__ldcg(mean0) * inv;
   double var = sq * inv * inv - mean * mean;
   var = var > 0.0 ? var : 0.0;
   const double sigma = sqrt(var);
@@ -199,6 +203,108 @@ __global__ void __launch_bounds__(kFinalThreads)
   *out = o;
 }
 
+
+__global__ void __launch_bounds__(256)
+    k_noalloc_finalize(const StatPartial* __restrict__ partials, int nparts, const float* __restrict__ colsq,
+                       const float* __restrict__ mean0, int npix, double weight, rf_image_stat* __restrict__ out) {
+  noalloc_finalize<256>(partials, nparts, colsq, mean0, npix, weight, out);
+}
+
+// N >= 64: two launches, shaped for one image.  The imaging kernels' blocks
+// (32 columns or row pairs at 256^2, a tile in shared memory) suit thousands
+// of images; one image then runs on four SMs and waits for its staging loops.
+// Here a block is a few transforms, which load their inputs straight into
+// registers (every load in flight at once; the other half of a sector is its
+// neighbour's), and the last row block to finish reduces the image.
+// 256^2: 34.3 to 27.9 us a call, 1024^2: 41.0 to 35.5, most of it host time now.
+template <int N>
+struct SingleCfg {
+  static constexpr int T = ImgCfg<N>::T, E = ImgCfg<N>::E;
+  static constexpr int XC = cmax(4, 32 / T);   // columns per block: 32-byte sectors
+  static constexpr int XR = cmax(2, 32 / T);   // row pairs per block
+  static constexpr int NC = N / 2;
+  static_assert(T >= 2 && T <= 32 && E == 32 && NC % XC == 0 && NC % XR == 0, "whole warps, whole blocks");
+};
+
+// Column u of the half plane: the (-1)^(u + v) phase-centre shift, the Parseval
+// sum and the inverse FFT along v into T[u][.].  Also zeroes the row launch's
+// count of finished blocks.
+template <int N>
+__global__ void __launch_bounds__(SingleCfg<N>::T * SingleCfg<N>::XC)
+    k_single_columns(const float2* __restrict__ grid, float2* __restrict__ T, const float2* __restrict__ tw,
+                     float* __restrict__ colsq, float* __restrict__ mean0, unsigned* __restrict__ done) {
+  using C = SingleCfg<N>;
+  constexpr int TT = C::T, E = C::E;
+  __shared__ float2 sm[C::XC * fft_stride<N>()];
+  const int xf = threadIdx.x / TT, t = threadIdx.x % TT;
+  const int u = blockIdx.x * C::XC + xf;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *done = 0;
+  float2 v[E];
+  const float2* src = grid + (size_t)t * (N / 2 + 1) + u;
+#pragma unroll
+  for (int r = 0; r < E; ++r) v[r] = __ldg(src + (size_t)r * TT * (N / 2 + 1));
+  if ((u + t) & 1)  // rows t + r TT, TT even
+#pragma unroll
+    for (int r = 0; r < E; ++r) v[r] = make_float2(-v[r].x, -v[r].y);
+  float acc = 0.f;
+#pragma unroll
+  for (int r = 0; r < E; ++r) acc = fmaf(v[r].x, v[r].x, fmaf(v[r].y, v[r].y, acc));
+#pragma unroll
+  for (int off = TT / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+  if (t == 0) {
+    colsq[u] = (u == 0 ? 1.f : 2.f) * acc;  // twice for u > 0
+    if (u == 0) *mean0 = v[0].x;
+  }
+  fft_inverse_from_regs<N>(v, sm + xf * fft_stride<N>(), tw, t, xf);
+  float2* dst = T + (size_t)u * N;
+  constexpr int LP = FftShape<N>::LAST_P;
+#pragma unroll
+  for (int m = 0; m < E / LP; ++m)
+#pragma unroll
+    for (int q = 0; q < LP; ++q) dst[fft_out_index<N>(t, m, q)] = v[m * LP + dft_perm<LP>(q)];
+}
+
+// Rows y, y + 1 from T (as row_zbuild), their maximum into partials[y / 2], and
+// the image's record by the block that finishes last.
+template <int N>
+__global__ void __launch_bounds__(SingleCfg<N>::T * SingleCfg<N>::XR)
+    k_single_rows(const float2* __restrict__ T, const float2* __restrict__ tw, StatPartial* __restrict__ partials,
+                  const float* __restrict__ colsq, const float* __restrict__ mean0, unsigned* __restrict__ done,
+                  double weight, rf_image_stat* __restrict__ out) {
+  using C = SingleCfg<N>;
+  constexpr int TT = C::T, E = C::E;
+  __shared__ float2 sm[C::XR * fft_stride<N>()];
+  __shared__ bool last;
+  const int xf = threadIdx.x / TT, t = threadIdx.x % TT;
+  const int pair = blockIdx.x * C::XR + xf;
+  float2 v[E];
+  // rows 2 pair, 2 pair + 1 of column u: one 16-byte load
+  const float4* col = reinterpret_cast<const float4*>(T) + pair;
+#pragma unroll
+  for (int r = 0; r < E / 2; ++r) {
+    const float4 ab = col[(size_t)(t + r * TT) * (N / 2)];
+    v[r] = (r == 0 && t == 0) ? make_float2(ab.x, ab.z) : make_float2(ab.x - ab.w, ab.y + ab.z);
+  }
+#pragma unroll
+  for (int r = E / 2; r < E; ++r) {
+    // column N - u; u = N / 2 has none
+    float4 ab = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r > E / 2 || t > 0) ab = col[(size_t)(N - t - r * TT) * (N / 2)];
+    v[r] = make_float2(ab.x + ab.w, ab.z - ab.y);
+  }
+  fft_inverse_from_regs<N>(v, sm + xf * fft_stride<N>(), tw, t, xf);
+  PassStats ps;
+  ps.partials = partials;
+  row_stats<N, kParts>(v, t, pair, 0, 0, 1, 0, 0.f, ps);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  noalloc_finalize<SingleCfg<N>::T * SingleCfg<N>::XR>(partials, N / 2, colsq, mean0, N, weight, out);
+}
+
 template <int N>
 cudaError_t run_noalloc(const float2* grid, double weight, const DeviceSetup& d, cudaStream_t st,
                         rf_image_stat* out) {
@@ -210,32 +316,42 @@ cudaError_t run_noalloc(const float2* grid, double weight, const DeviceSetup& d,
   static_assert(N <= kMaxN, "image larger than the static scratch");
   static_assert(K::PARTIALS <= ImgCfg<kMaxN>::PARTIALS, "partials area too small");
   static_assert(K::T <= 32, "the Parseval reduction of k_colfft_dense spans one warp");
-  // set on every call: the attribute belongs to the current device's context
-  const cudaError_t attr =
-      cudaFuncSetAttribute(k_colfft_dense<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, K::SMEM_A_FIXED);
-  if (attr != cudaSuccess) return attr;
   float2* T = reinterpret_cast<float2*>(d.scratch);
   StatPartial* partials = reinterpret_cast<StatPartial*>(d.scratch + kTBytes);
   float* colsq = reinterpret_cast<float*>(d.scratch + kTBytes + kPartialBytes);
   float* mean0 = colsq + kMaxN / 2;
   const float2* tw = d.twiddle + twiddle_offset(N);
   constexpr int NC = N / 2;
-  k_colfft_dense<N><<<(NC + K::XA - 1) / K::XA, K::T * K::XA, K::SMEM_A_FIXED, st>>>(grid, T, tw, colsq, mean0);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  SegmentGeom g{};
-  g.npix = N;
-  g.ncol = NC;
-  g.tsplit = 1;  // k_colfft_dense stores T in natural row order
-  DevTables tb{};
-  tb.twiddle = tw;
-  tb.twiddle_col = tw;
-  PassStats ps;
-  ps.partials = partials;
-  e = launch_rowfft_stats(g, tb, T, 1, 0, nullptr, ps, nullptr, nullptr, nullptr, st);
-  if (e != cudaSuccess) return e;
-  k_noalloc_finalize<<<1, kFinalThreads, 0, st>>>(partials, K::PARTIALS, colsq, mean0, N, weight, out);
-  return cudaGetLastError();
+  if constexpr (N >= 64) {
+    using C = SingleCfg<N>;
+    unsigned* done = reinterpret_cast<unsigned*>(mean0 + 1);
+    k_single_columns<N><<<NC / C::XC, C::T * C::XC, 0, st>>>(grid, T, tw, colsq, mean0, done);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_single_rows<N><<<NC / C::XR, C::T * C::XR, 0, st>>>(T, tw, partials, colsq, mean0, done, weight, out);
+    return cudaGetLastError();
+  } else {
+    // set on every call: the attribute belongs to the current device's context
+    const cudaError_t attr =
+        cudaFuncSetAttribute(k_colfft_dense<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, K::SMEM_A_FIXED);
+    if (attr != cudaSuccess) return attr;
+    k_colfft_dense<N><<<(NC + K::XA - 1) / K::XA, K::T * K::XA, K::SMEM_A_FIXED, st>>>(grid, T, tw, colsq, mean0);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    SegmentGeom g{};
+    g.npix = N;
+    g.ncol = NC;
+    g.tsplit = 1;  // k_colfft_dense stores T in natural row order
+    DevTables tb{};
+    tb.twiddle = tw;
+    tb.twiddle_col = tw;
+    PassStats ps;
+    ps.partials = partials;
+    e = launch_rowfft_stats(g, tb, T, 1, 0, nullptr, ps, nullptr, nullptr, nullptr, st);
+    if (e != cudaSuccess) return e;
+    k_noalloc_finalize<<<1, 256, 0, st>>>(partials, K::PARTIALS, colsq, mean0, N, weight, out);
+    return cudaGetLastError();
+  }
 }
 
 
