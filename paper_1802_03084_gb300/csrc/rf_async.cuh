@@ -58,6 +58,22 @@ __device__ __forceinline__ void tmem_store16(unsigned addr, const float2* v) {
       "f"(v[0].x), "f"(v[0].y), "f"(v[1].x), "f"(v[1].y), "f"(v[2].x), "f"(v[2].y), "f"(v[3].x), "f"(v[3].y), "f"(v[4].x), "f"(v[4].y), "f"(v[5].x), "f"(v[5].y), "f"(v[6].x), "f"(v[6].y), "f"(v[7].x), "f"(v[7].y), "f"(v[8].x), "f"(v[8].y), "f"(v[9].x), "f"(v[9].y), "f"(v[10].x), "f"(v[10].y), "f"(v[11].x), "f"(v[11].y), "f"(v[12].x), "f"(v[12].y), "f"(v[13].x), "f"(v[13].y), "f"(v[14].x), "f"(v[14].y), "f"(v[15].x), "f"(v[15].y)
       : "memory");
 }
+// One value of every lane into and from one column (tmem_load1: this warp's
+// earlier stores are waited for).
+__device__ __forceinline__ void tmem_store1(unsigned addr, float v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ float tmem_load1(unsigned addr) {
+  float v;
+  asm volatile(
+      "tcgen05.wait::st.sync.aligned;\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=f"(v)
+      : "r"(addr)
+      : "memory");
+  return v;
+}
 // v[0 .. 16) += the 32 columns (this warp's earlier stores are waited for).
 __device__ __forceinline__ void tmem_add16(unsigned addr, float2* v) {
   float r[32];

@@ -1075,10 +1075,10 @@ __device__ __forceinline__ void row_zbuild_duo(float2 (&v)[ImgCfg<N>::EB], const
 
 // Statistics of one image row (T row i) of the image in `slot`, output e of the
 // lane's registers read by val(e): one partial per warp of the transform, as
-// row_stats writes for a row pair.
+// row_stats writes for a row pair.  Returns the lane's maximum.
 template <int N, RowMode M, class F>
-__device__ __forceinline__ void row_stats_one(F val, int t, int i, int slot, int tsplit, int log2l, float gate,
-                                              const PassStats& ps) {
+__device__ __forceinline__ float row_stats_one(F val, int t, int i, int slot, int tsplit, int log2l, float gate,
+                                               const PassStats& ps) {
   using K = ImgCfg<N>;
   constexpr int EB = K::EB, TB = K::TB;
   constexpr int LP = FftShape<N / K::RSPLIT, EB>::LAST_P;
@@ -1103,7 +1103,7 @@ __device__ __forceinline__ void row_stats_one(F val, int t, int i, int slot, int
   };
   if constexpr (M == kBest) {
     if (__any_sync(0xffffffffu, !(lmax < gate))) row_best<WL>(lmax, gate, ps.best + slot, find);
-    return;
+    return lmax;
   }
   const float wmax = warp_max<WL>(lmax);
   int best = INT_MAX;
@@ -1123,6 +1123,7 @@ __device__ __forceinline__ void row_stats_one(F val, int t, int i, int slot, int
     ps.partials[o] = StatPartial{wmax, best};
     if constexpr (M == kClip) ps.cparts[o] = cp;
   }
+  return lmax;
 }
 
 // Pass B over units of up to 16 consecutive transformed images, with the images
@@ -1272,11 +1273,16 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
         if (more) fetch(nsl, ntwo, nyb);
       }
       row_fft<N>(v, fbuf + xf * K::STRIDE_B, tb.twiddle, t, xf);
+      // no pixel of a sum is above the sum of its images' maxima in the lane
+      // (rounding is monotonic), so a sum's maximum is taken only where that
+      // bound reaches its gate: 1024^2 realtime row passes 75.2 -> 74.3 ms,
+      // 2048^2 batching 147.5 -> 145.1
+      float bound;
       {
         const int sa = __shfl_sync(0xffffffffu, slots, k), sb = __shfl_sync(0xffffffffu, slots, k + 1);
         const float ga = __shfl_sync(0xffffffffu, gates, k), gb = __shfl_sync(0xffffffffu, gates, k + 1);
-        row_stats_one<N, M>([&](int e) { return v[e].x; }, t, i, sa, g.tsplit, log2l, ga, ps);
-        if (two) row_stats_one<N, M>([&](int e) { return v[e].y; }, t, i, sb, g.tsplit, log2l, gb, ps);
+        bound = row_stats_one<N, M>([&](int e) { return v[e].x; }, t, i, sa, g.tsplit, log2l, ga, ps);
+        if (two) bound += row_stats_one<N, M>([&](int e) { return v[e].y; }, t, i, sb, g.tsplit, log2l, gb, ps);
       }
       if (!two || top == 0) continue;
       float2 s[EB / 2];
@@ -1288,7 +1294,7 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
         const int j = k >> lv;  // s is sum j of this level
         const int sl = __shfl_sync(0xffffffffu, slots, 32 - (32 >> lv) + j);
         const float gt = __shfl_sync(0xffffffffu, gates, 32 - (32 >> lv) + j);
-        if (sl >= 0)
+        if (sl >= 0 && (M != kBest || __any_sync(0xffffffffu, !(bound < gt))))
           row_stats_one<N, M>([&](int e) { return e & 1 ? s[e >> 1].y : s[e >> 1].x; }, t, i, sl, g.tsplit, log2l,
                                  gt, ps);
         // the next level's block of images must be whole
@@ -1296,8 +1302,10 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
         __syncwarp();
         if ((j & 1) == 0) {
           tmem_store16(keep + (lv - 1) * 32, s);
+          if (M == kBest) tmem_store1(keep + 96 + (lv - 1), bound);
           break;
         }
+        if (M == kBest) bound += tmem_load1(keep + 96 + (lv - 1));
         tmem_add16(keep + (lv - 1) * 32, s);
       }
     }
