@@ -13,6 +13,7 @@ from __future__ import annotations
 import ctypes
 import os
 import re
+import sys
 from typing import Optional, Sequence
 
 import numpy as np
@@ -290,12 +291,11 @@ def _ptr(x) -> int:
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        try:
-            import torch
-            if torch.cuda.is_available() and torch.cuda.is_initialized():
-                return torch.cuda.current_stream().cuda_stream
-        except ImportError:
-            pass
+        # a program that has not imported torch has no torch stream; asking the
+        # driver for its devices on every call costs microseconds
+        torch = sys.modules.get("torch")
+        if torch is not None and torch.cuda.is_initialized():
+            return torch.cuda.current_stream().cuda_stream
         return None
     if hasattr(stream, "cuda_stream"):
         return stream.cuda_stream
