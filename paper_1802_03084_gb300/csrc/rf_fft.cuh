@@ -339,8 +339,32 @@ __device__ __forceinline__ void pass_compute(float2 (&v)[EV], const float2* __re
 // exp(+2 pi i k r / (32 P)), k = j mod 32, from the pair table
 // tw2[(r / 2) 64 + 2 k + (r mod 2)]: one 16-byte load per pair of r,
 // consecutive across the transform's threads.
+// The first pass2_early of them are loaded by pass2_ahead, before the barrier
+// and the loads between the passes, when the transform's values are in shared
+// memory and their registers are free: eight for a short second pass (512^2
+// serving: column pass 3.09 -> 2.97 ms, row pass 4.37 -> 4.35), four for the
+// column pass's radix-32 ones (1024^2 realtime 54.0 -> 53.1, 2048^2 batching
+// 89.1 -> 88.5; eight: 53.4, 94.2), none for the row pass's, whose registers
+// the tile reads and sums fill (1024^2 74.2 -> 74.8 ms with four).
+constexpr int pass2_early(int P, bool PK) { return P < 32 ? 8 : (PK ? 4 : 0); }
+constexpr int pass2_slots(int P, bool PK) { return pass2_early(P, PK) > 0 ? pass2_early(P, PK) : 1; }
+template <int N, int P, bool PK>
+__device__ __forceinline__ void pass2_ahead(float4 (&w)[pass2_slots(P, PK)], const float2* __restrict__ tw2, int t) {
+  constexpr int E = FftShape<N>::E, T = FftShape<N>::T;
+#pragma unroll
+  for (int i = 0; i < pass2_early(P, PK); ++i) {
+    const int m = i / (P / 2), rp = i % (P / 2);
+    if (m < E / P) {
+      const float4* p = reinterpret_cast<const float4*>(tw2) + ((t + m * T) & (E - 1)) + rp * E;
+      asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
+                   : "=f"(w[i].x), "=f"(w[i].y), "=f"(w[i].z), "=f"(w[i].w)
+                   : "l"(p));
+    }
+  }
+}
 template <int N, int P, bool PK = false>
-__device__ __forceinline__ void pass2_compute(float2 (&v)[FftShape<N>::E], const float2* __restrict__ tw2, int t) {
+__device__ __forceinline__ void pass2_compute(float2 (&v)[FftShape<N>::E], const float2* __restrict__ tw2, int t,
+                                              const float4 (&ahead)[pass2_slots(P, PK)]) {
   constexpr int E = FftShape<N>::E;
   constexpr int T = FftShape<N>::T;
   static_assert(E == 32 && P % 2 == 0, "pair table of a radix-32 second pass");
@@ -350,7 +374,9 @@ __device__ __forceinline__ void pass2_compute(float2 (&v)[FftShape<N>::E], const
     const float4* w4 = reinterpret_cast<const float4*>(tw2) + k;
 #pragma unroll
     for (int rp = 0; rp < P / 2; ++rp) {
-      const float4 w = __ldg(w4 + rp * E);
+      const int i = m * (P / 2) + rp;
+      constexpr int NE = pass2_early(P, PK);
+      const float4 w = i < NE ? ahead[i < NE ? i : 0] : __ldg(w4 + rp * E);
       if (rp > 0) v[m * P + 2 * rp] = cmul(v[m * P + 2 * rp], make_float2(w.x, w.y));
       v[m * P + 2 * rp + 1] = cmul(v[m * P + 2 * rp + 1], make_float2(w.z, w.w));
     }
@@ -420,13 +446,15 @@ __device__ __forceinline__ void fft_inverse_from_regs(float2 (&v)[EV], float2* s
   } else {
     pass_compute<N, S::E, PK>(v, tw, t, 1);
     pass_store<N, S::E>(v, s, t, 1);
+    float4 ahead[pass2_slots(S::P2, PK)];
+    pass2_ahead<N, S::P2, PK>(ahead, tw + N, t);
     fft_sync<S::T>(xf);
     pass_load<N, S::P2>(v, s, t);
     if constexpr (S::NPASS == 2) {
-      pass2_compute<N, S::P2, PK>(v, tw + N, t);
+      pass2_compute<N, S::P2, PK>(v, tw + N, t, ahead);
     } else {
       fft_sync<S::T>(xf);
-      pass2_compute<N, S::E, PK>(v, tw + N, t);
+      pass2_compute<N, S::E, PK>(v, tw + N, t, ahead);
       pass_store<N, S::E>(v, s, t, S::E);
       fft_sync<S::T>(xf);
       pass_load<N, S::LAST_P>(v, s, t);
