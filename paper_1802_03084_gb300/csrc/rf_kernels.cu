@@ -542,7 +542,8 @@ __device__ __forceinline__ double parseval_sum(const float* __restrict__ cs, int
 // (mean = G(0, 0) / 2W; mean of I^2 = sum over the full plane of |G|^2 /
 // 4W^2), so that they are known before the row pass.  gate[i]: no raw maximum
 // below it reaches the threshold (threshold * sigma in raw units, lowered by
-// far more than its rounding).  clip[i]: the clipping window {mean, kClipSigmas
+// far more than its rounding; no pixel does where sigma is not above 0, as in
+// an empty image, whose every pixel would pass a gate of 0).  clip[i]: the clipping window {mean, kClipSigmas
 // sigma} of the raw image J = 2W I.
 __global__ void k_image_noise(int ncol, const float* __restrict__ colsq, const float* __restrict__ mean0,
                               const double* __restrict__ weight, int nimg, int img_base, double threshold,
@@ -562,7 +563,7 @@ __global__ void k_image_noise(int ncol, const float* __restrict__ colsq, const f
   const double sigma = sqrt(var);
   noise[i] = ImgNoise{mean, sigma};
   if (gate != nullptr) {
-    gate[i] = (float)(threshold * sigma * (2.0 * W) * (1.0 - 1e-5));
+    gate[i] = sigma > 0.0 && W > 0.0 ? (float)(threshold * sigma * (2.0 * W) * (1.0 - 1e-5)) : INFINITY;
     best[i] = 0;
   }
   if (clip != nullptr) {

@@ -46,3 +46,5 @@ def test_candidates_alone_equal_candidates_with_statistics(npix, nint, dts):
         cands = search(float(threshold))[0]
         assert 0 < len(cands) < len(snr)
     search(float(snr[len(snr) // 2]), rf.RF_NOISE_CLIPPED)
+    seg["vis"][:] = 0  # empty images: no noise, no candidate
+    assert len(search(1.0)[0]) == 0
