@@ -250,25 +250,32 @@ def cpu_baseline(spec, seg, seconds):
 
 
 # ------------------------------------------------------------ work counts --
-def dt1_fraction(plan, spec, nint):
-    """Fraction of the segment's images at dt = 1 (counted from the plan's
-    delay table and edge rule): those gather the stored samples, the others
-    the FP32 resampled series."""
+def transformed_images(plan, spec, nint, plain=False):
+    """How many of the segment's images are gridded and transformed (counted
+    from the plan's delay table and edge rule), and which fraction of those is
+    of width dt = 1: those gather the stored samples, the others the FP32
+    resampled series.  The batched form sums the images of a width 2 .. 16 times
+    (2 or 4 times above 2048^2) another one from that one's pixels."""
     import numpy as np
     maxd = plan.delays().max(axis=1)
+    levels = 0 if plain or spec.npix < 64 else (4 if spec.npix <= 2048 else 2)
+    widths, own = sorted(set(spec.dt_list)), []
+    while widths:
+        own.append(widths.pop(0))
+        widths = [w for w in widths if w not in [own[-1] << lv for lv in range(1, levels + 1)]]
     n = {}
-    for dt in spec.dt_list:
+    for dt in own:
         if spec.edge == "partial":
             n[dt] = len(maxd) * (nint // dt)
         else:
             n[dt] = int(np.sum(np.maximum(nint - maxd, 0) // dt))
     tot = sum(n.values())
-    return n.get(1, 0) / tot if tot else 1.0
+    return tot, n.get(1, 0) / tot if tot else 1.0
 
 
 def work_per_image(spec, info, frac_dt1):
-    """Algorithmic HBM bytes and FP32 flops per image of each imaging kernel
-    (columns beyond the longest baseline are pruned: ncol = iu_max + 1).
+    """Algorithmic HBM bytes and FP32 flops per transformed image of each imaging
+    kernel (columns beyond the longest baseline are pruned: ncol = iu_max + 1).
 
     grid_cells: one sample per gridding entry read (dt = 1: the stored
     sample, 4 B FP16 or 8 B FP32; dt > 1: the FP32 resampled sum, 8 B) and
@@ -277,11 +284,6 @@ def work_per_image(spec, info, frac_dt1):
     B) written; ncol length-N FFTs.
     rowfft_stats: T read once; N/2 length-N FFTs (two image rows per complex
     transform).  FFTs count 5 N log2 N flops.
-    image_fused (the column and row passes in one launch): the same bytes and
-    flops as grid_colfft and rowfft_stats together -- T counted written and
-    read once, as the byte model of a two-pass FFT does, although the fused
-    pass keeps it in an L2-resident ring (its DRAM traffic, from ncu, is far
-    lower).
     """
     N = spec.npix
     ncol = info.iu_max + 1
@@ -292,7 +294,6 @@ def work_per_image(spec, info, frac_dt1):
         "grid_cells": {"bytes": gather + 8 * info.n_cells, "flops": 0.0},
         "grid_colfft": {"bytes": 8 * info.n_cells + 8 * N * ncol, "flops": ncol * fft},
         "rowfft_stats": {"bytes": 8 * N * ncol, "flops": (N / 2) * fft},
-        "image_fused": {"bytes": 8 * info.n_cells + 16 * N * ncol, "flops": (ncol + N / 2) * fft},
     }
 
 
@@ -333,7 +334,7 @@ def source_hash():
 
 
 TRAFFIC_KERNELS = (("k_grid_cells", "grid_cells"), ("k_colfft", "grid_colfft"), ("k_rowfft_stats", "rowfft_stats"),
-                   ("k_image_fused", "image_fused"))
+                   ("k_rowfft_duo", "rowfft_stats"), ("k_rowfft_tree", "rowfft_stats"))
 _BYTE_UNITS = {"byte": 1.0, "kbyte": 1e3, "mbyte": 1e6, "gbyte": 1e9, "tbyte": 1e12}
 
 
@@ -369,9 +370,9 @@ def write_traffic(raw_csv, images_per_launch, command, workload, path=None):
     return doc
 
 
-def roofline(prof, spec, info, n_images, steps, frac_dt1, hbm_peak, peak_kind, sms, sm_mhz, step_ms):
+def roofline(prof, spec, info, n_transformed, steps, frac_dt1, hbm_peak, peak_kind, sms, sm_mhz, step_ms):
     """The dominant kernel's roofline on HBM: its algorithmic bytes per
-    launch (work_per_image x images per launch) over its average launch time
+    launch (work_per_image x transformed images per launch) over its average launch time
     (CUDA events around every launch in the timed region), against the
     measured copy bandwidth.  Its FP32 rate against the derived ALU peak, and
     the whole step's algorithmic bytes over the step time, ride along."""
@@ -382,7 +383,7 @@ def roofline(prof, spec, info, n_images, steps, frac_dt1, hbm_peak, peak_kind, s
         launches, ms = prof.get(name, (0, 0.0))
         if launches == 0:
             continue
-        imgs = n_images * steps / launches
+        imgs = n_transformed * steps / launches
         avg_s = ms / launches / 1e3
         per[name] = dict(launches=launches, total_ms=ms, avg_us=avg_s * 1e6, images_per_launch=imgs,
                          bytes_per_image=w["bytes"], gbs=w["bytes"] * imgs / avg_s / 1e9,
@@ -393,9 +394,7 @@ def roofline(prof, spec, info, n_images, steps, frac_dt1, hbm_peak, peak_kind, s
     dom = max(per, key=lambda k: per[k]["total_ms"])
     d = per[dom]
     traffic = load_traffic(dom, d["images_per_launch"])
-    # the step's bytes: gridding, then the fused pass or the two passes it replaces
-    step_kernels = ["grid_cells"] + (["image_fused"] if "image_fused" in per else ["grid_colfft", "rowfft_stats"])
-    step_bytes = sum(work[k]["bytes"] for k in step_kernels) * n_images
+    step_bytes = sum(w["bytes"] for w in work.values()) * n_transformed
     r = {"bound": "hbm", "achieved": round(d["gbs"], 1), "peak": hbm_peak, "unit": "GB/s",
          "frac": round(d["gbs"] / hbm_peak, 4), "traffic": traffic, "kernel": dom,
          "peak_source": f"MEASURED_PEAKS.json hbm_gbs ({peak_kind}, copy bandwidth)",
@@ -406,7 +405,7 @@ def roofline(prof, spec, info, n_images, steps, frac_dt1, hbm_peak, peak_kind, s
                  "frac": round(d["tflops"] / alu_peak, 4),
                  "peak_source": f"derived: {sms} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 flop x {sm_mhz:.0f} MHz",
                  "flops_model": "5 N log2 N per length-N complex FFT"},
-         "step": {"bytes_per_image": round(step_bytes / max(n_images, 1)),
+         "step": {"bytes_per_image": round(step_bytes / max(n_transformed, 1)), "transformed_images": n_transformed,
                   "gbs": round(step_bytes / (step_ms / 1e3) / 1e9, 1),
                   "frac": round(step_bytes / (step_ms / 1e3) / 1e9 / hbm_peak, 4)}}
     return r, per
@@ -686,7 +685,7 @@ def run_workload(args, config, rank, world, dist, local_rank, lite=False):
         plan.set_ring(args.ring)
     info = plan.info()
     n_images = plan.count_images(nint)
-    frac_dt1 = dt1_fraction(plan, spec, nint)
+    n_transformed, frac_dt1 = transformed_images(plan, spec, nint, args.form == "plain")
     warmup = max(args.warmup, 0)
     steps = args.steps if not lite else max(3, min(args.steps, 5))
     for _ in range(warmup):
@@ -726,7 +725,7 @@ def run_workload(args, config, rank, world, dist, local_rank, lite=False):
 
     hbm_peak, sm_max_mhz, peak_kind = peaks()
     sms = torch.cuda.get_device_properties(local_rank).multi_processor_count
-    roof, per_kernel = roofline(prof, spec, info, n_images, steps, frac_dt1, hbm_peak, peak_kind, sms,
+    roof, per_kernel = roofline(prof, spec, info, n_transformed, steps, frac_dt1, hbm_peak, peak_kind, sms,
                                 clk.get("sm_max_mhz") or sm_max_mhz, ms / steps)
     launches = sum(v[0] for k, v in prof.items() if k != "h2d_copy")
     value = job_rate(world, steps, n_images, ms)
