@@ -947,7 +947,7 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
   }
   // the periodicity row pass's tensor-copy tiles (one image's XB rows), at
   // N = 1024, where its transforms fit one warp
-  if (p->npix == 1024) encode_tile_map(p, p->tmap_P, p->d_T, p->tslots, xb);
+  if (p->npix == 1024) encode_tile_map(p, p->tmap_P, p->d_T, p->tslots, xb, true);
   if (p->pairs) {
     encode_tile_map(p, p->tmap_D, p->d_T, p->tslots, xb, true);
     if (half >= B) {
@@ -2107,8 +2107,8 @@ rf_status rf_periodicity_search(rf_plan* p, const void* vis, int32_t nint, int32
       const int ng = v.g1 - v.g0;
       const int np = v.p1 - v.p0;
       RF_CUDA(rf::launch_grid_cells(gp, tbp, d_grp, v.g0, ng, p->d_cellbuf, st));
-      RF_CUDA(rf::launch_colfft(gp, tbp, d_grp, v.g0, ng, v.i0, v.i0, p->d_cellbuf, p->d_T, p->d_colsq, p->d_mean0, false,
-                                st));
+      RF_CUDA(rf::launch_colfft(gp, tbp, d_grp, v.g0, ng, v.i0, v.i0, p->d_cellbuf, p->d_T, p->d_colsq, p->d_mean0,
+                                p->tmap_P.nbox > 0, st));
       RF_CUDA(rf::launch_rowfft_power(gp, tbp, p->d_T, d_pairs + v.p0, np, p->d_partials,
                                       p->tmap_P.nbox > 0 ? &p->tmap_P : nullptr, p->d_err, st));
       RF_CUDA(rf::launch_finalize_power(gp, p->d_partials, p->d_colsq, p->d_mean0, d_pairs + v.p0, np,

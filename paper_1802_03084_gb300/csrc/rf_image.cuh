@@ -1415,8 +1415,10 @@ inline int one_per_sm_smem(int smem, int row_smem, int smem_max) {
 // cp.async, or, where every transform fits one warp and tma_boxes > 0
 // (N = 1024), two tiles [rows][XB] of U and of Q rows, each filled by
 // tma_boxes tensor copies of tma_rows u rows from `tmap` ([slot][u][2N
-// floats], boxes of XB complex values, 64-byte rows swizzled by the hardware:
-// chunk c of row u at c ^ ((u >> 1) & 3)).  Then, as in the search's row
+// floats], boxes of XB complex values), with T in duo order: an 8-byte load of
+// 16 columns then meets 16 bank pairs (the hardware's 64-byte swizzle moves
+// 16-byte chunks and left two-way conflicts: 2048 pairs of
+// 1024^2 9.07 ms a call so, 8.67 this way).  Then, as in the search's row
 // pass, no block barrier is left: each warp waits for the tiles on an
 // mbarrier (bounded; a warp that gives up sets *err, waits once more and
 // leaves) and the last warp to read them issues the next item's copies.
@@ -1433,8 +1435,7 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* fbuf = reinterpret_cast<float2*>(smraw);                       // [XB][STRIDE_B]
   float4* tile = reinterpret_cast<float4*>(fbuf + K::XB * K::STRIDE_B);  // [ncol][CH]
-  // tensor-copy tiles of U and Q rows, [rows][4 chunks]: U 1024-byte
-  // aligned, Q 512 bytes after it (the 64-byte swizzle repeats every 8 rows)
+  // tensor-copy tiles of U and Q rows, [rows][XB]
   unsigned char* tu0 = smraw + K::XB * K::STRIDE_B * 8;
   tu0 += (1024u - (smem_u32(tu0) & 1023u)) & 1023u;
   const unsigned tsz = ((unsigned)(tma_boxes * tma_rows * K::XB * 8) + 511u) & ~511u;
@@ -1512,35 +1513,7 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
     const int y = t_row(iy, g.tsplit, log2l);
     float2 v[EB];
     if (PTMA && use_tma) {
-      // the U and Q tiles: complex value xf of u row u is half (xf & 1) of
-      // chunk (xf >> 1) ^ ((u >> 1) & 3); for u = t + 32 r (N - t - 32 r)
-      // the swizzle term is that of t (N - t)
-      const int rd_end = ncol > t ? (ncol - t + TB - 1) / TB : 0;
-      const int rm_beg = (N - ncol - t) / TB + 1;
-      auto at = [&](int u) { return (u * 4 + ((xf >> 1) ^ ((u >> 1) & 3))) * 2 + (xf & 1); };
-      const float2* pdu = tileU + at(t);
-      const float2* pdq = tileQ + at(t);
-      const float2* pmu = tileU + at(N - t);
-      const float2* pmq = tileQ + at(N - t);
-      constexpr int RS = TB * 4 * 2;  // float2 per 32 u rows
-#pragma unroll
-      for (int r = 0; r < EB / 2; ++r) {
-        float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
-        if (r < rd_end) {
-          a = pdu[r * RS];
-          b = pdq[r * RS];
-        }
-        v[r] = (r == 0 && t == 0) ? make_float2(a.x, b.x) : make_float2(a.x - b.y, a.y + b.x);
-      }
-#pragma unroll
-      for (int r = EB / 2; r < EB; ++r) {
-        float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
-        if (r >= rm_beg) {
-          a = pmu[-r * RS];
-          b = pmq[-r * RS];
-        }
-        v[r] = make_float2(a.x + b.y, b.x - a.y);
-      }
+      if constexpr (PTMA) row_zbuild_duo<N>(v, tileU, tileQ, t, xf, ncol);
     } else if constexpr (TB % K::CH == 0) {
       // as in the search's row pass: u = t + r T (or N - t - r T) has the
       // swizzle term of t (N - t), and the loads are predicated, not branched
@@ -1603,10 +1576,7 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
     for (int e = 0; e < EB; ++e) pa[e & 3] = fmaxf(pa[e & 3], fmaf(v[e].x, v[e].x, v[e].y * v[e].y));
     const float lmax = fmaxf(fmaxf(pa[0], pa[1]), fmaxf(pa[2], pa[3]));
     constexpr int WL = TB < 32 ? TB : 32;
-    constexpr unsigned MASK = 0xffffffffu;
-    float wmax = lmax;
-#pragma unroll
-    for (int off = WL / 2; off > 0; off >>= 1) wmax = fmaxf(wmax, __shfl_xor_sync(MASK, wmax, off));
+    const float wmax = warp_max<WL>(lmax);
     int best = INT_MAX;
     if (lmax == wmax) {
 #pragma unroll
@@ -1621,8 +1591,7 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
         }
     found:;
     }
-#pragma unroll
-    for (int off = WL / 2; off > 0; off >>= 1) best = min(best, __shfl_xor_sync(MASK, best, off));
+    best = warp_min<WL>(best);
     float mx = wmax;
     int mi = best;
     if (TB > 32) {
