@@ -94,11 +94,6 @@ __device__ __forceinline__ int ld_acquire_gpu(const int* p) {
   asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-// Orders this thread's generic-proxy global accesses before (and after)
-// async-proxy (tensor copy) accesses to global memory.
-__device__ __forceinline__ void fence_proxy_async_global() {
-  asm volatile("fence.proxy.async.global;" ::: "memory");
-}
 // Bounded wait until *p >= target (acquire), polling with a short sleep;
 // gives up after `polls` polls, or at once when *abort is set.
 __device__ __forceinline__ bool wait_count(const int* p, int target, const int* abort, int polls = 1 << 22) {
