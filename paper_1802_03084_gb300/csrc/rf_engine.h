@@ -198,13 +198,31 @@ struct ImgNoise {
 // and cparts are set together); or, where only candidates are wanted (best and
 // gate are set together), each image's largest pixel if it is not below its
 // gate: best[slot] starts at 0 and ends as the largest best_key of such pixels.
+// rms[slot] (plans with sums of 8 or 16 only): how bright an image is, raw
+// units (see may_pair); apart: how many units hold images that may not share
+// transforms, and which.
 struct PassStats {
   StatPartial* partials = nullptr;  // [slot][partials per image]
   const float2* clip = nullptr;
   ClipPartial* cparts = nullptr;    // [slot][partials per image]
   unsigned long long* best = nullptr;
   const float* gate = nullptr;
+  const float* rms = nullptr;
+  int* apart = nullptr;             // [1 + units of a wave]
 };
+
+// Whether two images, of RMS a and b, may share transforms (k_rowfft_duo): a
+// transform's FP32 rounding is relative to both, and one pixel that is not
+// finite spoils both.  At most 1.5 times apart (two images of noise are within
+// some percent), either's error is at most 1.3 times that of two rows of its
+// own; unlimited, a saturated integration put 0.2 sigma into its neighbour at
+// 10^6 times its brightness, and one NaN took the neighbour's candidate.
+constexpr float kPairContrast = 1.5f;
+#ifdef __CUDACC__
+__device__ __forceinline__ bool may_pair(float a, float b) {
+  return a <= kPairContrast * b && b <= kPairContrast * a && a + b < INFINITY;  // false for NaN
+}
+#endif
 
 // A pixel as a key: of two pixels the larger value has the larger key, of two
 // equal ones the lower index.  Never 0 (the value is not NaN).
@@ -321,10 +339,11 @@ cudaError_t launch_colfft(const SegmentGeom& g, const DevTables& tb, const Group
 // colsq, before the row pass.  gate[i] and best[i] (if not null): the raw pixel
 // value below which a maximum cannot make image i a candidate, and 0.  clip[i] (if not null): the
 // clipping window of the clipped noise in raw pixel units (the image times
-// 2W), {mean0[i], kClipSigmas * sigma over all pixels}.
+// 2W), {mean0[i], kClipSigmas * sigma over all pixels}.  rms[i] (if not null):
+// the raw image's RMS over all pixels, and *apart = 0 (see PassStats).
 cudaError_t launch_image_noise(const SegmentGeom& g, const float* colsq, const float* mean0, const double* weight,
                                int nimg, int img_base, double threshold, ImgNoise* noise, float* gate,
-                               unsigned long long* best, float2* clip, cudaStream_t st);
+                               unsigned long long* best, float2* clip, float* rms, int* apart, cudaStream_t st);
 
 // Row C2R (pass B) + statistics of `nimg` images in slots [0, nimg) whose
 // first image index is img_base.  Optionally writes the scaled images.

@@ -1137,10 +1137,15 @@ __device__ __forceinline__ float row_stats_one(F val, int t, int i, int slot, in
 // and one level more, which fits two levels of sums.  1024^2 realtime (widths 1,
 // 2, 4, 8): 94,700 images transformed and not 106,500, 164.3 -> 147.4 ms with
 // kBest; 2048^2 batching (1 .. 16) 295.3 -> 261.9 ms.
+// Units with two images that may not share a transform (may_pair) are listed at
+// their first row block and offer no best; a second launch (APART) takes the
+// listed ones again, such images each beside itself and once more together for
+// their sum only.  With both in one kernel, the registers of the rare case
+// took 2048^2 batching from 252 to 266 ms, 1024^2 realtime from 137.3 to 139.1.
 // T is read in duo order: with the tiles' rows of XB 8-byte values permuted by
 // column, a half-warp's loads meet 16 bank pairs (the hardware's swizzles move
 // 16-byte chunks: two-way conflicts).
-template <int N, RowMode M>
+template <int N, RowMode M, bool APART>
 __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
     k_rowfft_duo(SegmentGeom g, DevTables tb, const float2* __restrict__ Tbuf, const Unit* __restrict__ units,
                  int nunits, int img_base, int base_base, const PassStats ps,
@@ -1167,7 +1172,8 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
   const int tid = threadIdx.x, lane = tid & 31;
   const int ncol = g.ncol;
   constexpr int nrb = N / XB;
-  const int nitems = nunits * nrb;
+  const int nitems = (APART ? ps.apart[0] : nunits) * nrb;
+  if (APART && (int)blockIdx.x >= nitems) return;
   const int xf = tid / K::TB;
   const int t = tid - xf * K::TB;
   const int log2l = FftShape<N>::LOG2N - (g.tsplit > 1 ? __ffs(g.tsplit) - 1 : 0);
@@ -1211,8 +1217,11 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
 
   int item = blockIdx.x;
   // a unit's words, one a lane: base, n, img[0 .. 4]
-  auto load_unit = [&](int it) { return reinterpret_cast<const int*>(units + it / nrb)[lane & 7]; };
-  int cur = load_unit(item);  // the grid is at most the number of items
+  auto load_unit = [&](int it) {
+    const int u = APART ? ps.apart[1 + it / nrb] : it / nrb;
+    return reinterpret_cast<const int*>(units + u)[lane & 7];
+  };
+  int cur = load_unit(item);  // the grid (of the first launch) is at most the number of items
   bool failed = false;
   fetch(__shfl_sync(0xffffffffu, cur, 0) - base_base, __shfl_sync(0xffffffffu, cur, 1) > 1, (item % nrb) * XB);
   while (item < nitems && !failed) {
@@ -1226,6 +1235,16 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
     const int top = 31 - __clz((int)(__ballot_sync(0xffffffffu, cur >= 0) >> 2 & 31u) | 1);
     float gates = 0.f;
     if (M == kBest && slots >= 0) gates = ps.gate[slots];
+    unsigned apart;  // bit k: images k and k + 1 may not share a transform
+    {
+      const float rms = ll == 0 && slots >= 0 ? ps.rms[slots] : 0.f;
+      const float other = __shfl_xor_sync(0xffffffffu, rms, 1);
+      apart = __ballot_sync(0xffffffffu, (lane | 1) < n && !may_pair(rms, other));
+      if (!APART && apart != 0) {
+        gates = INFINITY;
+        if (y0 == 0 && tid == 0) ps.apart[1 + atomicAdd(ps.apart, 1)] = item / nrb;
+      }
+    }
     const int i = y0 + xf;
     for (int k = 0; k < n; k += 2) {
       if (use_tma) {
@@ -1244,6 +1263,17 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
       }
       const bool two = k + 1 < n;
       float2 v[EB];
+      const bool split = APART && (apart >> k & 1u);
+      if (split)
+#pragma unroll 1
+        for (int b = 0; b < 2; ++b) {
+          const float2* tile = b ? tileB : tileA;
+          row_zbuild_duo<N>(v, tile, tile, t, xf, ncol);
+          __syncwarp();  // the last transform's values are read
+          row_fft<N>(v, fbuf + xf * K::STRIDE_B, tb.twiddle, t, xf);
+          row_stats_one<N, M>([&](int e) { return v[e].x; }, t, i, __shfl_sync(0xffffffffu, slots, k + b), g.tsplit,
+                              log2l, __shfl_sync(0xffffffffu, gates, k + b), ps);
+        }
       row_zbuild_duo<N>(v, tileA, two ? tileB : tileA, t, xf, ncol);  // A alone: beside itself
       // the tiles are read: the unit's next images' (or the next item's first ones')
       const bool here = k + 2 < n;
@@ -1272,9 +1302,10 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
       // no pixel of a sum is above the sum of its images' maxima in the lane
       // (rounding is monotonic), so a sum's maximum is taken only where that
       // bound reaches its gate: 1024^2 realtime row passes 75.2 -> 74.3 ms,
-      // 2048^2 batching 147.5 -> 145.1
-      float bound;
-      {
+      // 2048^2 batching 147.5 -> 145.1.  The maxima of images that went through
+      // alone have other roundings: no bound.
+      float bound = INFINITY;
+      if (!split) {
         const int sa = __shfl_sync(0xffffffffu, slots, k), sb = __shfl_sync(0xffffffffu, slots, k + 1);
         const float ga = __shfl_sync(0xffffffffu, gates, k), gb = __shfl_sync(0xffffffffu, gates, k + 1);
         bound = row_stats_one<N, M>([&](int e) { return v[e].x; }, t, i, sa, g.tsplit, log2l, ga, ps);
@@ -1314,9 +1345,9 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
 }
 
 // The row-pass kernel of units at side N.
-template <int N, RowMode M, bool PAIRS>
+template <int N, RowMode M, bool PAIRS, bool APART = false>
 constexpr auto tree_kernel() {
-  if constexpr (PAIRS) return k_rowfft_duo<N, M>;
+  if constexpr (PAIRS) return k_rowfft_duo<N, M, APART>;
   else return k_rowfft_tree<N, M>;
 }
 
@@ -1717,13 +1748,13 @@ cudaError_t run_rowfft_stats(const SegmentGeom& g, const DevTables& tb, const fl
   return run_rowfft_stats_k<N, kParts>(g, tb, Tbuf, nimg, img_base, weight, ps, images, tm, err, st, pl);
 }
 
-template <int N, RowMode M, bool PAIRS>
+template <int N, RowMode M, bool PAIRS, bool APART = false>
 cudaError_t run_rowfft_tree_k(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Unit* units,
                               int nunits, int img_base, int base_base, const PassStats& ps, const TileMap* tm,
                               int* err, cudaStream_t st, const PassLaunch* pl) {
   using K = ImgCfg<N>;
   const int smem = K::SMEM_B_FIXED + (K::TILE_TMA ? 1024 : 0) + rowfft_tile_rows<N>(g.ncol) * K::CH * 16;
-  auto kern = tree_kernel<N, M, PAIRS>();
+  auto kern = tree_kernel<N, M, PAIRS, APART>();
   const int smem_max = max_dynamic_smem(kern);
   if (smem > smem_max) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
@@ -1738,7 +1769,7 @@ cudaError_t run_rowfft_tree_k(const SegmentGeom& g, const DevTables& tb, const f
   const long nitems = (long)nunits * (N / (PAIRS ? K::XB : K::RB));
   const long steps = unit_images(PAIRS) / (PAIRS ? 2 : 1);
   long grid = std::min<long>(nitems, (long)std::max(per_sm, 1) * sm_count());
-  if (pl != nullptr && pl->items_per_block > 0)
+  if (!APART && pl != nullptr && pl->items_per_block > 0)
     grid = std::max(grid, std::min<long>((steps * nitems + pl->items_per_block - 1) / pl->items_per_block,
                                          std::min<long>(nitems, INT_MAX)));
   const bool tma = K::TILE_TMA && tm != nullptr && tm->nbox > 0 && err != nullptr;
@@ -1753,10 +1784,16 @@ cudaError_t run_rowfft_tree(const SegmentGeom& g, const DevTables& tb, const flo
                             int nunits, bool pairs, int img_base, int base_base, const PassStats& ps,
                             const TileMap* tm, int* err, cudaStream_t st, const PassLaunch* pl) {
   static_assert(N >= kTreeMinNpix, "whole warps");
-#define RF_UNITS(M, P) run_rowfft_tree_k<N, M, P>(g, tb, Tbuf, units, nunits, img_base, base_base, ps, tm, err, st, pl)
+#define RF_UNITS(M, ...) \
+  run_rowfft_tree_k<N, M, __VA_ARGS__>(g, tb, Tbuf, units, nunits, img_base, base_base, ps, tm, err, st, pl)
   if (pairs) {
-    if constexpr (pairs_possible(N))
-      return ps.clip ? RF_UNITS(kClip, true) : (ps.best ? RF_UNITS(kBest, true) : RF_UNITS(kParts, true));
+    if constexpr (pairs_possible(N)) {
+      const cudaError_t e =
+          ps.clip ? RF_UNITS(kClip, true) : (ps.best ? RF_UNITS(kBest, true) : RF_UNITS(kParts, true));
+      if (e != cudaSuccess) return e;
+      return ps.clip ? RF_UNITS(kClip, true, true)
+                     : (ps.best ? RF_UNITS(kBest, true, true) : RF_UNITS(kParts, true, true));
+    }
     return cudaErrorInvalidValue;
   }
   return ps.clip ? RF_UNITS(kClip, false) : (ps.best ? RF_UNITS(kBest, false) : RF_UNITS(kParts, false));
