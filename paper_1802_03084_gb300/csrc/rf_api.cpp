@@ -2028,7 +2028,10 @@ rf_status rf_periodicity_search(rf_plan* p, const void* vis, int32_t nint, int32
     if ((int64_t)p->max_delay[d] + L <= nint) dms.push_back(d);
   const int K = kmax - kmin + 1;
   const int kpad = (K + 31) / 32 * 32;
-  const int B = p->shape.images_per_group;
+  // frequencies per block: its U and Q images have to fit one wave, which holds
+  // as little as one group (small RF_TUNE_WAVE_IMAGES, short segments, large images)
+  const int wave_cap = std::min(p->tslots, p->sslots);
+  const int B = std::min(p->shape.images_per_group, wave_cap / 2);
   const int nkb = (K + B - 1) / B;
   const size_t nrows = (size_t)p->nbl * p->nchan;
   const size_t per_dm = 2 * nrows * kpad * sizeof(float2);
@@ -2101,7 +2104,7 @@ rf_status rf_periodicity_search(rf_plan* p, const void* vis, int32_t nint, int32
     for (int j = 0; j < nb; ++j)
       for (int kb = 0; kb < nkb; ++kb) {
         const int n = std::min(B, K - kb * B);
-        if ((nimg + 2 * n) - w.i0 > std::min(p->tslots, p->sslots) || ((int)grp.size() + 2) - w.g0 > p->gslots_max) {
+        if ((nimg + 2 * n) - w.i0 > wave_cap || ((int)grp.size() + 2) - w.g0 > p->gslots_max) {
           w.g1 = (int)grp.size();
           w.i1 = nimg;
           w.p1 = (int)pairs.size();
