@@ -394,26 +394,24 @@ cudaError_t launch_grid_cells(const SegmentGeom& g, const DevTables& tb, const G
 // is summed from S in k_resample's order (or read from the resampled series),
 // then the warp adds its 32 entries' samples to their cells in entry order, as
 // grid_range does.  Those 12 images: 2.26 ms with the
-// resampling to 0.045 ms.
+// resampling to 0.045 ms.  Any plan's channels and ranges: the delays are read
+// where they lie, and the grid has one dimension.
 template <bool FP16>
 __global__ void __launch_bounds__(256) k_grid_single(SegmentGeom g, DevTables tb, const Group* __restrict__ groups,
                                                      int g_begin, const void* __restrict__ S, int direct,
                                                      float2* __restrict__ cellbuf) {
-  extern __shared__ int sdel[];  // [nchan] delays of this group's DM
-  const Group* __restrict__ gp = groups + g_begin + blockIdx.x;
+  const int nblk = (g.nranges + 7) / 8;  // blocks of eight ranges a group
+  const int gi = blockIdx.x / nblk;
+  const Group* __restrict__ gp = groups + g_begin + gi;
   const int s = gp->s, t0 = gp->t0;
-  {
-    const int* __restrict__ dl = tb.delays + (size_t)gp->d * g.nchan;
-    for (int c = threadIdx.x; c < g.nchan; c += blockDim.x) sdel[c] = dl[c];
-  }
-  __syncthreads();
+  const int* __restrict__ dl = tb.delays + (size_t)gp->d * g.nchan;
   const int lane = threadIdx.x & 31;
-  const int r = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int r = (blockIdx.x - gi * nblk) * 8 + (threadIdx.x >> 5);
   if (r >= g.nranges) return;
   const int2 rg = tb.ranges[r];
   const int dt = tb.dt_list[s];
   const unsigned char* __restrict__ Sb = reinterpret_cast<const unsigned char*>(S);
-  float2* __restrict__ out = cellbuf + (size_t)blockIdx.x * g.ncells * 32;
+  float2* __restrict__ out = cellbuf + (size_t)gi * g.ncells * 32;
   float2 acc = make_float2(0.f, 0.f);
   unsigned cur = 0xffffffffu;
   for (int base = rg.x; base < rg.y; base += 32) {
@@ -422,7 +420,7 @@ __global__ void __launch_bounds__(256) k_grid_single(SegmentGeom g, DevTables tb
     if (base + lane < rg.y) {
       const GridEntry e = tb.ent[base + lane];
       mycf = ((unsigned)e.cell & kCellMask) | ((unsigned)(e.cflags & 3) << 30);
-      const int del = sdel[e.cflags >> 2];
+      const int del = __ldg(dl + (e.cflags >> 2));
       const int t = t0 * dt + del;  // samples at or past nint are absent
       if (direct || dt == 1) {
         const size_t row = (size_t)e.bc * g.nint_pad;
@@ -466,11 +464,11 @@ __global__ void __launch_bounds__(256) k_grid_single(SegmentGeom g, DevTables tb
 cudaError_t launch_grid_single(const SegmentGeom& g, const DevTables& tb, const Group* groups, int g_begin,
                                int ngroups, const void* S, bool direct, float2* cellbuf, cudaStream_t st) {
   if (ngroups <= 0 || g.nranges <= 0) return cudaSuccess;
-  dim3 grid(ngroups, (g.nranges + 7) / 8);
+  const unsigned grid = (unsigned)ngroups * (unsigned)((g.nranges + 7) / 8);
   if (g.fp16)
-    k_grid_single<true><<<grid, 256, g.nchan * 4, st>>>(g, tb, groups, g_begin, S, direct ? 1 : 0, cellbuf);
+    k_grid_single<true><<<grid, 256, 0, st>>>(g, tb, groups, g_begin, S, direct ? 1 : 0, cellbuf);
   else
-    k_grid_single<false><<<grid, 256, g.nchan * 4, st>>>(g, tb, groups, g_begin, S, direct ? 1 : 0, cellbuf);
+    k_grid_single<false><<<grid, 256, 0, st>>>(g, tb, groups, g_begin, S, direct ? 1 : 0, cellbuf);
   return cudaGetLastError();
 }
 
