@@ -286,7 +286,6 @@ struct rf_plan {
   rf::ImgNoise* d_noise = nullptr;  // [sslots] mean and noise from the Parseval sums
   float* d_gate = nullptr;      // [sslots] least raw maximum of a candidate
   float* d_rms = nullptr;       // [sslots] raw RMS (plans with sums of 8 or 16)
-  int* d_apart = nullptr;       // 2 x [1 + tslots] units listed for the second row pass (the same plans)
   unsigned long long* d_best = nullptr;  // [sslots] largest pixel that reaches it
   float2* d_clip = nullptr;     // [sslots] clipping window (RF_NOISE_CLIPPED only)
   rf::ClipPartial* d_cparts = nullptr;  // kept-pixel partials (used with RF_NOISE_CLIPPED)
@@ -920,10 +919,7 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
   if (p->d_rms) {
     p->device_bytes -= (uint64_t)p->sslots * sizeof(float);
     p->dfree(p->d_rms);
-    p->device_bytes -= 2 * ((uint64_t)p->tslots + 1) * sizeof(int);
-    p->dfree(p->d_apart);
     p->d_rms = nullptr;
-    p->d_apart = nullptr;
   }
   if (p->d_best) {
     p->device_bytes -= (uint64_t)p->sslots * 8;
@@ -956,7 +952,6 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
   if ((s = p->dalloc(&p->d_gate, (size_t)p->sslots)) != RF_OK) return s;
   if ((s = p->dalloc(&p->d_best, (size_t)p->sslots)) != RF_OK) return s;
   if (p->pairs && (s = p->dalloc(&p->d_rms, (size_t)p->sslots)) != RF_OK) return s;
-  if (p->pairs && (s = p->dalloc(&p->d_apart, 2 * ((size_t)p->tslots + 1))) != RF_OK) return s;
   if ((s = p->dalloc(&p->d_cparts, (size_t)p->sslots * nrb)) != RF_OK) return s;
   if ((p->flags & RF_NOISE_CLIPPED) && (s = p->dalloc(&p->d_clip, (size_t)p->sslots)) != RF_OK) return s;
   const int xb = std::min(256 / (p->npix / 32), p->npix / 2);  // row pairs of a row-pass work item
@@ -1015,7 +1010,7 @@ uint64_t estimate_device_bytes(const rf_plan* p, int slots) {
        r(sslots, 4) + r(sslots, sizeof(rf::ImgNoise));
   b += r(sslots, sizeof(float)) + r(sslots, 8) + r((size_t)sslots * plan_partials(p), sizeof(rf::ClipPartial));
   if (p->flags & RF_NOISE_CLIPPED) b += r(sslots, sizeof(float2));
-  if (p->pairs) b += r(sslots, sizeof(float)) + r(2 * ((size_t)tslots + 1), sizeof(int));
+  if (p->pairs) b += r(sslots, sizeof(float));
   const size_t per_int = rows * p->npol * sizeof(float2);
   const size_t stage_nint = std::max<size_t>(1, std::min<size_t>(kStageBytes / per_int, (size_t)p->max_nint));
   b += r(stage_nint * per_int, 1);
@@ -1321,15 +1316,12 @@ rf_status finish_wave(rf_plan* p, const SegmentGeom& g, const Wave& w, const flo
   const bool only_cands = !clip && !d_stats && !im;
   float* gate = only_cands ? p->d_gate + slot0 : nullptr;
   unsigned long long* best = only_cands ? p->d_best + slot0 : nullptr;
-  const bool duo = wave_duo(p, w);
-  float* rms = duo ? p->d_rms + slot0 : nullptr;
-  int* apart = duo ? p->d_apart + (slot0 > 0 ? p->tslots + 1 : 0) : nullptr;
+  float* rms = wave_duo(p, w) ? p->d_rms + slot0 : nullptr;
   RF_TIMED(p->prof, K_IMAGE_NOISE, st,
            rf::launch_image_noise(g, colsq, mean0, p->d_weight, ni, w.img_begin, p->threshold, noise, gate, best,
-                                  cw, rms, apart, st));
+                                  cw, rms, st));
   rf::PassStats ps;
   ps.rms = rms;
-  ps.apart = apart;
   ps.partials = p->d_partials + slot0 * plan_partials(p);
   ps.gate = gate;
   ps.best = best;

@@ -199,8 +199,7 @@ struct ImgNoise {
 // gate are set together), each image's largest pixel if it is not below its
 // gate: best[slot] starts at 0 and ends as the largest best_key of such pixels.
 // rms[slot] (plans with sums of 8 or 16 only): how bright an image is, raw
-// units (see may_pair); apart: how many units hold images that may not share
-// transforms, and which.
+// units (see may_pair).
 struct PassStats {
   StatPartial* partials = nullptr;  // [slot][partials per image]
   const float2* clip = nullptr;
@@ -208,7 +207,6 @@ struct PassStats {
   unsigned long long* best = nullptr;
   const float* gate = nullptr;
   const float* rms = nullptr;
-  int* apart = nullptr;             // [1 + units of a wave]
 };
 
 // Whether two images, of RMS a and b, may share transforms (k_rowfft_duo): a
@@ -340,10 +338,10 @@ cudaError_t launch_colfft(const SegmentGeom& g, const DevTables& tb, const Group
 // value below which a maximum cannot make image i a candidate, and 0.  clip[i] (if not null): the
 // clipping window of the clipped noise in raw pixel units (the image times
 // 2W), {mean0[i], kClipSigmas * sigma over all pixels}.  rms[i] (if not null):
-// the raw image's RMS over all pixels, and *apart = 0 (see PassStats).
+// the raw image's RMS over all pixels (see PassStats).
 cudaError_t launch_image_noise(const SegmentGeom& g, const float* colsq, const float* mean0, const double* weight,
                                int nimg, int img_base, double threshold, ImgNoise* noise, float* gate,
-                               unsigned long long* best, float2* clip, float* rms, int* apart, cudaStream_t st);
+                               unsigned long long* best, float2* clip, float* rms, cudaStream_t st);
 
 // Row C2R (pass B) + statistics of `nimg` images in slots [0, nimg) whose
 // first image index is img_base.  Optionally writes the scaled images.

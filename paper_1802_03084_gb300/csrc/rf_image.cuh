@@ -22,6 +22,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 #include <utility>
 
 #include "rf_engine.h"
@@ -1137,15 +1138,16 @@ __device__ __forceinline__ float row_stats_one(F val, int t, int i, int slot, in
 // and one level more, which fits two levels of sums.  1024^2 realtime (widths 1,
 // 2, 4, 8): 94,700 images transformed and not 106,500, 164.3 -> 147.4 ms with
 // kBest; 2048^2 batching (1 .. 16) 295.3 -> 261.9 ms.
-// Units with two images that may not share a transform (may_pair) are listed at
-// their first row block and offer no best; a second launch (APART) takes the
-// listed ones again, such images each beside itself and once more together for
-// their sum only.  With both in one kernel, the registers of the rare case
-// took 2048^2 batching from 252 to 266 ms, 1024^2 realtime from 137.3 to 139.1.
+// Items with two images that may not share a transform (may_pair) offer no best;
+// the block takes them again after its other items, such images each beside
+// itself and once more together for their sum only.  Looking for them takes
+// 1024^2 realtime from 137.4 to 138.7 ms, 2048^2 batching from 253.3 to 254.0.  In
+// the loop of all items the registers of the rare case took them to 139.1 and 266
+// ms; a launch of its own took 8 us of a short search's 100.
 // T is read in duo order: with the tiles' rows of XB 8-byte values permuted by
 // column, a half-warp's loads meet 16 bank pairs (the hardware's swizzles move
 // 16-byte chunks: two-way conflicts).
-template <int N, RowMode M, bool APART>
+template <int N, RowMode M>
 __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
     k_rowfft_duo(SegmentGeom g, DevTables tb, const float2* __restrict__ Tbuf, const Unit* __restrict__ units,
                  int nunits, int img_base, int base_base, const PassStats ps,
@@ -1172,8 +1174,7 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
   const int tid = threadIdx.x, lane = tid & 31;
   const int ncol = g.ncol;
   constexpr int nrb = N / XB;
-  const int nitems = (APART ? ps.apart[0] : nunits) * nrb;
-  if (APART && (int)blockIdx.x >= nitems) return;
+  const int nitems = nunits * nrb;
   const int xf = tid / K::TB;
   const int t = tid - xf * K::TB;
   const int log2l = FftShape<N>::LOG2N - (g.tsplit > 1 ? __ffs(g.tsplit) - 1 : 0);
@@ -1215,139 +1216,155 @@ __global__ void __launch_bounds__(ImgCfg<N>::THREADS_B, 2)
     cp_async_commit();
   };
 
-  int item = blockIdx.x;
   // a unit's words, one a lane: base, n, img[0 .. 4]
-  auto load_unit = [&](int it) {
-    const int u = APART ? ps.apart[1 + it / nrb] : it / nrb;
-    return reinterpret_cast<const int*>(units + u)[lane & 7];
+  auto load_unit = [&](int it) { return reinterpret_cast<const int*>(units + it / nrb)[lane & 7]; };
+  // bit k: images k and k + 1 of the unit may not share a transform
+  auto apart_of = [&](int cur) {
+    const int n = __shfl_sync(0xffffffffu, cur, 1), img = __shfl_sync(0xffffffffu, cur, 2);
+    const float rms = lane < n ? ps.rms[img + lane - img_base] : 0.f;  // n <= 16
+    const float other = __shfl_xor_sync(0xffffffffu, rms, 1);
+    return __ballot_sync(0xffffffffu, (lane | 1) < n && !may_pair(rms, other));
   };
-  int cur = load_unit(item);  // the grid (of the first launch) is at most the number of items
-  bool failed = false;
-  fetch(__shfl_sync(0xffffffffu, cur, 0) - base_base, __shfl_sync(0xffffffffu, cur, 1) > 1, (item % nrb) * XB);
-  while (item < nitems && !failed) {
-    const int y0 = (item % nrb) * XB;
-    const int next = item + (int)gridDim.x;
-    const int nxt = next < nitems ? load_unit(next) : cur;
-    const int base = __shfl_sync(0xffffffffu, cur, 0), n = __shfl_sync(0xffffffffu, cur, 1);
-    const int first = __shfl_sync(0xffffffffu, cur, 2 + ll);
-    // this lane's image: its slot (-1: not searched) and gate; the highest level searched
-    const int slots = first >= 0 && (lj + 1) << ll <= n ? first + lj - img_base : -1;
-    const int top = 31 - __clz((int)(__ballot_sync(0xffffffffu, cur >= 0) >> 2 & 31u) | 1);
-    float gates = 0.f;
-    if (M == kBest && slots >= 0) gates = ps.gate[slots];
-    unsigned apart;  // bit k: images k and k + 1 may not share a transform
-    {
-      const float rms = ll == 0 && slots >= 0 ? ps.rms[slots] : 0.f;
-      const float other = __shfl_xor_sync(0xffffffffu, rms, 1);
-      apart = __ballot_sync(0xffffffffu, (lane | 1) < n && !may_pair(rms, other));
+  bool failed = false, again = false;
+  // every item of the block, or those with such images
+  auto items = [&](auto only_apart) {
+    constexpr bool APART = decltype(only_apart)::value;
+    int item = blockIdx.x, cur = load_unit(item);  // the grid is at most the number of items
+    auto advance = [&](int& it) {  // to the next item; its unit
+      int u = cur;
+      do {
+        it += (int)gridDim.x;
+        if (it >= nitems) break;
+        u = load_unit(it);
+      } while (APART && apart_of(u) == 0);
+      return u;
+    };
+    if (APART && apart_of(cur) == 0) cur = advance(item);
+    if (item < nitems)
+      fetch(__shfl_sync(0xffffffffu, cur, 0) - base_base, __shfl_sync(0xffffffffu, cur, 1) > 1, (item % nrb) * XB);
+    while (item < nitems && !failed) {
+      const int y0 = (item % nrb) * XB;
+      int next = item;
+      const int nxt = advance(next);
+      const int base = __shfl_sync(0xffffffffu, cur, 0), n = __shfl_sync(0xffffffffu, cur, 1);
+      const int first = __shfl_sync(0xffffffffu, cur, 2 + ll);
+      // this lane's image: its slot (-1: not searched) and gate; the highest level searched
+      const int slots = first >= 0 && (lj + 1) << ll <= n ? first + lj - img_base : -1;
+      const int top = 31 - __clz((int)(__ballot_sync(0xffffffffu, cur >= 0) >> 2 & 31u) | 1);
+      float gates = 0.f;
+      if (M == kBest && slots >= 0) gates = ps.gate[slots];
+      const unsigned apart = apart_of(cur);
       if (!APART && apart != 0) {
         gates = INFINITY;
-        if (y0 == 0 && tid == 0) ps.apart[1 + atomicAdd(ps.apart, 1)] = item / nrb;
+        again = true;
       }
-    }
-    const int i = y0 + xf;
-    for (int k = 0; k < n; k += 2) {
-      if (use_tma) {
-        // as in k_rowfft_stats: no copy is issued without this warp's count
-        // below, so the other warps' waits run out in turn
-        if (!__all_sync(0xffffffffu, mbar_wait(&tbar, phase))) {
-          if (lane == 0) atomicExch(err, 1);
-          mbar_wait(&tbar, phase);
-          failed = true;
-          break;
-        }
-        phase ^= 1u;
-      } else {
-        cp_async_wait_all();
-        __syncthreads();
-      }
-      const bool two = k + 1 < n;
-      float2 v[EB];
-      const bool split = APART && (apart >> k & 1u);
-      if (split)
-#pragma unroll 1
-        for (int b = 0; b < 2; ++b) {
-          const float2* tile = b ? tileB : tileA;
-          row_zbuild_duo<N>(v, tile, tile, t, xf, ncol);
-          __syncwarp();  // the last transform's values are read
-          row_fft<N>(v, fbuf + xf * K::STRIDE_B, tb.twiddle, t, xf);
-          row_stats_one<N, M>([&](int e) { return v[e].x; }, t, i, __shfl_sync(0xffffffffu, slots, k + b), g.tsplit,
-                              log2l, __shfl_sync(0xffffffffu, gates, k + b), ps);
-        }
-      row_zbuild_duo<N>(v, tileA, two ? tileB : tileA, t, xf, ncol);  // A alone: beside itself
-      // the tiles are read: the unit's next images' (or the next item's first ones')
-      const bool here = k + 2 < n;
-      const int nbase = __shfl_sync(0xffffffffu, nxt, 0), nn = __shfl_sync(0xffffffffu, nxt, 1);
-      const int nsl = (here ? base + k + 2 : nbase) - base_base;
-      const bool ntwo = here ? k + 3 < n : nn > 1;
-      const int nyb = here ? y0 : (next % nrb) * XB;
-      const bool more = here || next < nitems;
-      if (use_tma) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) {
-          __threadfence_block();
-          if (atomicAdd(&s_done, 1) == NWB - 1) {
-            s_done = 0;
-            __threadfence_block();
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            if (more) issue_tma(nsl, ntwo, nyb);
+      const int i = y0 + xf;
+      for (int k = 0; k < n; k += 2) {
+        if (use_tma) {
+          // as in k_rowfft_stats: no copy is issued without this warp's count
+          // below, so the other warps' waits run out in turn
+          if (!__all_sync(0xffffffffu, mbar_wait(&tbar, phase))) {
+            if (lane == 0) atomicExch(err, 1);
+            mbar_wait(&tbar, phase);
+            failed = true;
+            break;
           }
+          phase ^= 1u;
+        } else {
+          cp_async_wait_all();
+          __syncthreads();
         }
-      } else {
-        __syncthreads();
-        if (more) fetch(nsl, ntwo, nyb);
-      }
-      row_fft<N>(v, fbuf + xf * K::STRIDE_B, tb.twiddle, t, xf);
-      // no pixel of a sum is above the sum of its images' maxima in the lane
-      // (rounding is monotonic), so a sum's maximum is taken only where that
-      // bound reaches its gate: 1024^2 realtime row passes 75.2 -> 74.3 ms,
-      // 2048^2 batching 147.5 -> 145.1.  The maxima of images that went through
-      // alone have other roundings: no bound.
-      float bound = INFINITY;
-      if (!split) {
-        const int sa = __shfl_sync(0xffffffffu, slots, k), sb = __shfl_sync(0xffffffffu, slots, k + 1);
-        const float ga = __shfl_sync(0xffffffffu, gates, k), gb = __shfl_sync(0xffffffffu, gates, k + 1);
-        bound = row_stats_one<N, M>([&](int e) { return v[e].x; }, t, i, sa, g.tsplit, log2l, ga, ps);
-        if (two) bound += row_stats_one<N, M>([&](int e) { return v[e].y; }, t, i, sb, g.tsplit, log2l, gb, ps);
-      }
-      if (!two || top == 0) continue;
-      float2 s[EB / 2];
-#pragma unroll
-      for (int e = 0; e < EB / 2; ++e)
-        s[e] = make_float2(v[2 * e].x + v[2 * e].y, v[2 * e + 1].x + v[2 * e + 1].y);
+        const bool two = k + 1 < n;
+        float2 v[EB];
+        const bool split = APART && (apart >> k & 1u);
+        if (split)
 #pragma unroll 1
-      for (int lv = 1;; ++lv) {
-        const int j = k >> lv;  // s is sum j of this level
-        const int sl = __shfl_sync(0xffffffffu, slots, 32 - (32 >> lv) + j);
-        const float gt = __shfl_sync(0xffffffffu, gates, 32 - (32 >> lv) + j);
-        if (sl >= 0 && (M != kBest || __any_sync(0xffffffffu, !(bound < gt))))
-          row_stats_one<N, M>([&](int e) { return e & 1 ? s[e >> 1].y : s[e >> 1].x; }, t, i, sl, g.tsplit, log2l,
-                                 gt, ps);
-        // the next level's block of images must be whole
-        if (lv >= top || ((j | 1) + 1) << lv > n) break;
-        __syncwarp();
-        if ((j & 1) == 0) {
-          tmem_store16(keep + (lv - 1) * 32, s);
-          if (M == kBest) tmem_store1(keep + 96 + (lv - 1), bound);
-          break;
+          for (int b = 0; b < 2; ++b) {
+            const float2* tile = b ? tileB : tileA;
+            row_zbuild_duo<N>(v, tile, tile, t, xf, ncol);
+            __syncwarp();  // the last transform's values are read
+            row_fft<N>(v, fbuf + xf * K::STRIDE_B, tb.twiddle, t, xf);
+            row_stats_one<N, M>([&](int e) { return v[e].x; }, t, i, __shfl_sync(0xffffffffu, slots, k + b), g.tsplit,
+                                log2l, __shfl_sync(0xffffffffu, gates, k + b), ps);
+          }
+        row_zbuild_duo<N>(v, tileA, two ? tileB : tileA, t, xf, ncol);  // A alone: beside itself
+        // the tiles are read: the unit's next images' (or the next item's first ones')
+        const bool here = k + 2 < n;
+        const int nbase = __shfl_sync(0xffffffffu, nxt, 0), nn = __shfl_sync(0xffffffffu, nxt, 1);
+        const int nsl = (here ? base + k + 2 : nbase) - base_base;
+        const bool ntwo = here ? k + 3 < n : nn > 1;
+        const int nyb = here ? y0 : (next % nrb) * XB;
+        const bool more = here || next < nitems;
+        if (use_tma) {
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) {
+            __threadfence_block();
+            if (atomicAdd(&s_done, 1) == NWB - 1) {
+              s_done = 0;
+              __threadfence_block();
+              asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+              if (more) issue_tma(nsl, ntwo, nyb);
+            }
+          }
+        } else {
+          __syncthreads();
+          if (more) fetch(nsl, ntwo, nyb);
         }
-        if (M == kBest) bound += tmem_load1(keep + 96 + (lv - 1));
-        tmem_add16(keep + (lv - 1) * 32, s);
+        row_fft<N>(v, fbuf + xf * K::STRIDE_B, tb.twiddle, t, xf);
+        // no pixel of a sum is above the sum of its images' maxima in the lane
+        // (rounding is monotonic), so a sum's maximum is taken only where that
+        // bound reaches its gate: 1024^2 realtime row passes 75.2 -> 74.3 ms,
+        // 2048^2 batching 147.5 -> 145.1.  The maxima of images that went through
+        // alone have other roundings: no bound.
+        float bound = INFINITY;
+        if (!split) {
+          const int sa = __shfl_sync(0xffffffffu, slots, k), sb = __shfl_sync(0xffffffffu, slots, k + 1);
+          const float ga = __shfl_sync(0xffffffffu, gates, k), gb = __shfl_sync(0xffffffffu, gates, k + 1);
+          bound = row_stats_one<N, M>([&](int e) { return v[e].x; }, t, i, sa, g.tsplit, log2l, ga, ps);
+          if (two) bound += row_stats_one<N, M>([&](int e) { return v[e].y; }, t, i, sb, g.tsplit, log2l, gb, ps);
+        }
+        if (!two || top == 0) continue;
+        float2 s[EB / 2];
+#pragma unroll
+        for (int e = 0; e < EB / 2; ++e)
+          s[e] = make_float2(v[2 * e].x + v[2 * e].y, v[2 * e + 1].x + v[2 * e + 1].y);
+#pragma unroll 1
+        for (int lv = 1;; ++lv) {
+          const int j = k >> lv;  // s is sum j of this level
+          const int sl = __shfl_sync(0xffffffffu, slots, 32 - (32 >> lv) + j);
+          const float gt = __shfl_sync(0xffffffffu, gates, 32 - (32 >> lv) + j);
+          if (sl >= 0 && (M != kBest || __any_sync(0xffffffffu, !(bound < gt))))
+            row_stats_one<N, M>([&](int e) { return e & 1 ? s[e >> 1].y : s[e >> 1].x; }, t, i, sl, g.tsplit, log2l,
+                                gt, ps);
+          // the next level's block of images must be whole
+          if (lv >= top || ((j | 1) + 1) << lv > n) break;
+          __syncwarp();
+          if ((j & 1) == 0) {
+            tmem_store16(keep + (lv - 1) * 32, s);
+            if (M == kBest) tmem_store1(keep + 96 + (lv - 1), bound);
+            break;
+          }
+          if (M == kBest) bound += tmem_load1(keep + 96 + (lv - 1));
+          tmem_add16(keep + (lv - 1) * 32, s);
+        }
       }
+      item = next;
+      cur = nxt;
     }
-    item = next;
-    cur = nxt;
-  }
+  };
+  items(std::false_type{});
+  // every warp has read its last tile and, unless a wait ran out, seen every item
+  if (__syncthreads_and(!failed) && again) items(std::true_type{});
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
   __syncthreads();
   if (tid < 32) tmem_free(s_tmem, TCOLS);
 }
 
 // The row-pass kernel of units at side N.
-template <int N, RowMode M, bool PAIRS, bool APART = false>
+template <int N, RowMode M, bool PAIRS>
 constexpr auto tree_kernel() {
-  if constexpr (PAIRS) return k_rowfft_duo<N, M, APART>;
+  if constexpr (PAIRS) return k_rowfft_duo<N, M>;
   else return k_rowfft_tree<N, M>;
 }
 
@@ -1748,13 +1765,13 @@ cudaError_t run_rowfft_stats(const SegmentGeom& g, const DevTables& tb, const fl
   return run_rowfft_stats_k<N, kParts>(g, tb, Tbuf, nimg, img_base, weight, ps, images, tm, err, st, pl);
 }
 
-template <int N, RowMode M, bool PAIRS, bool APART = false>
+template <int N, RowMode M, bool PAIRS>
 cudaError_t run_rowfft_tree_k(const SegmentGeom& g, const DevTables& tb, const float2* Tbuf, const Unit* units,
                               int nunits, int img_base, int base_base, const PassStats& ps, const TileMap* tm,
                               int* err, cudaStream_t st, const PassLaunch* pl) {
   using K = ImgCfg<N>;
   const int smem = K::SMEM_B_FIXED + (K::TILE_TMA ? 1024 : 0) + rowfft_tile_rows<N>(g.ncol) * K::CH * 16;
-  auto kern = tree_kernel<N, M, PAIRS, APART>();
+  auto kern = tree_kernel<N, M, PAIRS>();
   const int smem_max = max_dynamic_smem(kern);
   if (smem > smem_max) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
@@ -1769,7 +1786,7 @@ cudaError_t run_rowfft_tree_k(const SegmentGeom& g, const DevTables& tb, const f
   const long nitems = (long)nunits * (N / (PAIRS ? K::XB : K::RB));
   const long steps = unit_images(PAIRS) / (PAIRS ? 2 : 1);
   long grid = std::min<long>(nitems, (long)std::max(per_sm, 1) * sm_count());
-  if (!APART && pl != nullptr && pl->items_per_block > 0)
+  if (pl != nullptr && pl->items_per_block > 0)
     grid = std::max(grid, std::min<long>((steps * nitems + pl->items_per_block - 1) / pl->items_per_block,
                                          std::min<long>(nitems, INT_MAX)));
   const bool tma = K::TILE_TMA && tm != nullptr && tm->nbox > 0 && err != nullptr;
@@ -1784,16 +1801,10 @@ cudaError_t run_rowfft_tree(const SegmentGeom& g, const DevTables& tb, const flo
                             int nunits, bool pairs, int img_base, int base_base, const PassStats& ps,
                             const TileMap* tm, int* err, cudaStream_t st, const PassLaunch* pl) {
   static_assert(N >= kTreeMinNpix, "whole warps");
-#define RF_UNITS(M, ...) \
-  run_rowfft_tree_k<N, M, __VA_ARGS__>(g, tb, Tbuf, units, nunits, img_base, base_base, ps, tm, err, st, pl)
+#define RF_UNITS(M, P) run_rowfft_tree_k<N, M, P>(g, tb, Tbuf, units, nunits, img_base, base_base, ps, tm, err, st, pl)
   if (pairs) {
-    if constexpr (pairs_possible(N)) {
-      const cudaError_t e =
-          ps.clip ? RF_UNITS(kClip, true) : (ps.best ? RF_UNITS(kBest, true) : RF_UNITS(kParts, true));
-      if (e != cudaSuccess) return e;
-      return ps.clip ? RF_UNITS(kClip, true, true)
-                     : (ps.best ? RF_UNITS(kBest, true, true) : RF_UNITS(kParts, true, true));
-    }
+    if constexpr (pairs_possible(N))
+      return ps.clip ? RF_UNITS(kClip, true) : (ps.best ? RF_UNITS(kBest, true) : RF_UNITS(kParts, true));
     return cudaErrorInvalidValue;
   }
   return ps.clip ? RF_UNITS(kClip, false) : (ps.best ? RF_UNITS(kBest, false) : RF_UNITS(kParts, false));

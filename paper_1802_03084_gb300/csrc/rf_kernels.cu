@@ -547,7 +547,7 @@ __global__ void k_image_noise(int ncol, const float* __restrict__ colsq, const f
                               const double* __restrict__ weight, int nimg, int img_base, double threshold,
                               ImgNoise* __restrict__ noise, float* __restrict__ gate,
                               unsigned long long* __restrict__ best, float2* __restrict__ clip,
-                              float* __restrict__ rms, int* __restrict__ apart) {
+                              float* __restrict__ rms) {
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (i >= nimg) return;
@@ -561,10 +561,7 @@ __global__ void k_image_noise(int ncol, const float* __restrict__ colsq, const f
   var = var > 0.0 ? var : 0.0;
   const double sigma = sqrt(var);
   noise[i] = ImgNoise{mean, sigma};
-  if (rms != nullptr) {
-    rms[i] = (float)sqrt(sq);
-    if (i == 0) *apart = 0;
-  }
+  if (rms != nullptr) rms[i] = (float)sqrt(sq);
   if (gate != nullptr) {
     gate[i] = sigma > 0.0 && W > 0.0 ? (float)(threshold * sigma * (2.0 * W) * (1.0 - 1e-5)) : INFINITY;
     best[i] = 0;
@@ -578,11 +575,10 @@ __global__ void k_image_noise(int ncol, const float* __restrict__ colsq, const f
 
 cudaError_t launch_image_noise(const SegmentGeom& g, const float* colsq, const float* mean0, const double* weight,
                                int nimg, int img_base, double threshold, ImgNoise* noise, float* gate,
-                               unsigned long long* best, float2* clip, float* rms, int* apart,
-                               cudaStream_t st) {
+                               unsigned long long* best, float2* clip, float* rms, cudaStream_t st) {
   if (nimg <= 0) return cudaSuccess;
   k_image_noise<<<(nimg + 7) / 8, 256, 0, st>>>(g.ncol, colsq, mean0, weight, nimg, img_base, threshold, noise, gate,
-                                                best, clip, rms, apart);
+                                                best, clip, rms);
   return cudaGetLastError();
 }
 
