@@ -305,12 +305,13 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
     // of |G|^2 over the full Hermitian plane, which counts this column
     // twice unless u = 0; its mean is G(0, 0) / (2 W).  Lane k is image k of
     // the part (two cells a step where the part is 16 images), so the cells of
-    // a sum of 2, 4, 8 or 16 images are xor-shuffles away; the warps' FP32
-    // sums meet in the first FFT buffer and are added in a fixed order: after
-    // the transforms, so that no barrier stands before those, unless the
+    // a sum of 2, 4, 8 or 16 images are xor-shuffles away.  FP32: a lane adds
+    // every 32nd cell, in U chains that take turns, and the chains and the
+    // warps' sums, which meet in the first FFT buffer, are added as a tree:
+    // after the transforms, so that no barrier stands before those, unless the
     // sums' registers would spill there (C::EARLY).
     constexpr int NL = N < kTreeMinNpix ? 0 : (pairs_possible(N) ? 4 : 2);
-    constexpr int NW = C::THREADS / 32, CPS = 32 / PI;
+    constexpr int NW = C::THREADS / 32, CPS = 32 / PI, U = 32 / (NW * CPS);
     const int warp = tid >> 5, kp = lane & (PI - 1);
     auto at = [&](int c, int k) {
       return R > 1 ? c * PI + 2 * ((k >> 1) ^ (c & (CPC - 1))) + (k & 1) : c * C::CELL_PITCH + k;
@@ -318,23 +319,32 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
     float a[NL + 1] = {};
     int top = 0;
     {
+      float ac[U][NL + 1] = {};
 #pragma unroll
       for (int lv = 1; lv <= NL; ++lv)
         if (gp->nsum[lv - 1] > 0) top = lv;
-#pragma unroll 2
-      for (int cb = warp * CPS; cb < ncells; cb += NW * CPS) {
-        const int c = cb + lane / PI;
-        float2 h = make_float2(0.f, 0.f);
-        if (c < ncells && kp < nk) h = cellv[at(c, kp)];
-        a[0] = fmaf(h.x, h.x, fmaf(h.y, h.y, a[0]));
+      for (int cb = warp * CPS; cb < ncells; cb += U * NW * CPS)
 #pragma unroll
-        for (int lv = 1; lv <= NL; ++lv)
-          if (lv <= top) {
-            h.x += __shfl_xor_sync(0xffffffffu, h.x, 1 << (lv - 1));
-            h.y += __shfl_xor_sync(0xffffffffu, h.y, 1 << (lv - 1));
-            a[lv] = fmaf(h.x, h.x, fmaf(h.y, h.y, a[lv]));
-          }
+        for (int u = 0; u < U; ++u) {
+          if (cb + u * NW * CPS >= ncells) break;
+          const int c = cb + u * NW * CPS + lane / PI;
+          float2 h = make_float2(0.f, 0.f);
+          if (c < ncells && kp < nk) h = cellv[at(c, kp)];
+          ac[u][0] = fmaf(h.x, h.x, fmaf(h.y, h.y, ac[u][0]));
+#pragma unroll
+          for (int lv = 1; lv <= NL; ++lv)
+            if (lv <= top) {
+              h.x += __shfl_xor_sync(0xffffffffu, h.x, 1 << (lv - 1));
+              h.y += __shfl_xor_sync(0xffffffffu, h.y, 1 << (lv - 1));
+              ac[u][lv] = fmaf(h.x, h.x, fmaf(h.y, h.y, ac[u][lv]));
+            }
+        }
+#pragma unroll
+      for (int lv = 0; lv <= NL; ++lv) {
+        a[lv] = ac[0][lv] + ac[1][lv];
+        if constexpr (U == 4) a[lv] += ac[2][lv] + ac[3][lv];
       }
+      static_assert(NW == 8 && (U == 2 || U == 4), "the trees");
       static_assert(CPS <= 2 && (1 << NL) <= PI && NL < NW && NW * (NL + 1) * 32 * 4 <= C::SMEM_FIXED,
                     "Parseval sums fit the FFT buffers, the sums' images one part, their levels the warps");
     }
@@ -353,8 +363,8 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, 2)
         const int k = kbase + lane, j = k >> lv;
         const int lim = lv == 0 ? gr.nimg : gp->nsum[lv - 1];
         if ((lane & ((1 << lv) - 1)) == 0 && j < lim) {
-          float acc = 0.f;
-          for (int w = 0; w < NW; ++w) acc += red[(lv * NW + w) * 32 + lane];
+          const float* __restrict__ rw = red + lv * NW * 32 + lane;
+          const float acc = ((rw[0] + rw[32]) + (rw[64] + rw[96])) + ((rw[128] + rw[160]) + (rw[192] + rw[224]));
           const size_t slot = (size_t)((lv == 0 ? gr.img0 : gp->isum[lv - 1]) + j - img_base);
           colsq[slot * g.ncol + col] = (col == 0 ? 1.f : 2.f) * acc;
           if (col == 0) {
