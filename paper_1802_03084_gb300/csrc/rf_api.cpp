@@ -288,7 +288,7 @@ struct rf_plan {
   float* d_rms = nullptr;       // [sslots] raw RMS (plans with sums of 8 or 16)
   unsigned long long* d_best = nullptr;  // [sslots] largest pixel that reaches it
   float2* d_clip = nullptr;     // [sslots] clipping window (RF_NOISE_CLIPPED only)
-  rf::ClipPartial* d_cparts = nullptr;  // kept-pixel partials (used with RF_NOISE_CLIPPED)
+  rf::ClipPartial* d_cparts = nullptr;  // kept-pixel partials (RF_NOISE_CLIPPED only)
   rf::PlainBuffers plain{};     // allocated on the first plain-form search
 
   // RF_TUNE_FUSED and RF_TUNE_RING: kept and reported, without effect
@@ -701,13 +701,27 @@ size_t plan_partials(const rf_plan* p) {
   return rf::unit_partials(p->shape, p->pairs);
 }
 
-// Transformed images and image records of a wave of `slots` images (two whole
-// groups at least, so that a half of either holds one, see run_waves_overlapped).
+// Transformed images and image records of a wave of `slots` images (a whole
+// group at least; waves overlap only where a half of either holds one, see
+// overlap_possible).
 int wave_tslots(const rf_plan* p, int slots) {
   if (!p->derived) return slots;
-  return std::max(2 * p->shape.images_per_group, std::min(slots, (int)std::ceil(slots * p->base_share)));
+  return std::max(p->shape.images_per_group, std::min(slots, (int)std::ceil(slots * p->base_share)));
 }
-int wave_sslots(const rf_plan* p, int slots) { return p->derived ? std::max(slots, 2 * group_images(p)) : slots; }
+int wave_sslots(const rf_plan* p, int slots) { return p->derived ? std::max(slots, group_images(p)) : slots; }
+
+// Units of the longest segment (every trial has its most images there).
+size_t count_units(const rf_plan* p) {
+  const int B = p->shape.images_per_group, step = rf::unit_images(p->pairs);
+  size_t n = 0;
+  for (int d = 0; d < p->ndm; ++d)
+    for (int s = 0; s < p->ndt; ++s)
+      if (p->sum_of[s] == s) {
+        const int nt = n_times(p, p->max_nint, d, s);
+        n += (size_t)(nt / B) * (B / step) + (nt % B + step - 1) / step;
+      }
+  return n;
+}
 
 // Default images per wave: the column-FFT scratch of its transformed images
 // within the budget.
@@ -952,8 +966,10 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
   if ((s = p->dalloc(&p->d_gate, (size_t)p->sslots)) != RF_OK) return s;
   if ((s = p->dalloc(&p->d_best, (size_t)p->sslots)) != RF_OK) return s;
   if (p->pairs && (s = p->dalloc(&p->d_rms, (size_t)p->sslots)) != RF_OK) return s;
-  if ((s = p->dalloc(&p->d_cparts, (size_t)p->sslots * nrb)) != RF_OK) return s;
-  if ((p->flags & RF_NOISE_CLIPPED) && (s = p->dalloc(&p->d_clip, (size_t)p->sslots)) != RF_OK) return s;
+  if (p->flags & RF_NOISE_CLIPPED) {
+    if ((s = p->dalloc(&p->d_clip, (size_t)p->sslots)) != RF_OK) return s;
+    if ((s = p->dalloc(&p->d_cparts, (size_t)p->sslots * nrb)) != RF_OK) return s;
+  }
   const int xb = std::min(256 / (p->npix / 32), p->npix / 2);  // row pairs of a row-pass work item
   encode_tile_map(p, p->tmap_T, p->d_T, p->tslots, 2 * xb);
   // the halves of d_T, each a wave's scratch when waves are overlapped
@@ -998,7 +1014,7 @@ uint64_t estimate_device_bytes(const rf_plan* p, int slots) {
   b += r(p->dt.size(), 8) + r(p->dt.size(), 4);
   const int64_t img_cap = std::max<int64_t>(count_images(p, p->max_nint), 1);
   b += r(img_cap, sizeof(int4)) + r(img_cap, sizeof(Group)) + r(img_cap, 8) + r(img_cap, sizeof(DevCand)) + 4 + 4;  // candidate count, error flag
-  if (p->derived) b += r(img_cap, sizeof(rf::Unit));
+  if (p->derived) b += r(count_units(p), sizeof(rf::Unit));
   const size_t per_slot = (size_t)p->ncol * N * sizeof(float2);
   if (slots <= 0) slots = default_slots(p, (size_t)img_cap);
   const int B = p->shape.images_per_group;
@@ -1008,8 +1024,9 @@ uint64_t estimate_device_bytes(const rf_plan* p, int slots) {
   b += r((size_t)tslots * per_slot, 1) + r((size_t)sslots * plan_partials(p), sizeof(StatPartial)) +
        r((size_t)gslots * std::max(p->n_cells, 1) * 32, sizeof(float2)) + r((size_t)sslots * p->ncol, 4) +
        r(sslots, 4) + r(sslots, sizeof(rf::ImgNoise));
-  b += r(sslots, sizeof(float)) + r(sslots, 8) + r((size_t)sslots * plan_partials(p), sizeof(rf::ClipPartial));
-  if (p->flags & RF_NOISE_CLIPPED) b += r(sslots, sizeof(float2));
+  b += r(sslots, sizeof(float)) + r(sslots, 8);
+  if (p->flags & RF_NOISE_CLIPPED)
+    b += r(sslots, sizeof(float2)) + r((size_t)sslots * plan_partials(p), sizeof(rf::ClipPartial));
   if (p->pairs) b += r(sslots, sizeof(float));
   const size_t per_int = rows * p->npol * sizeof(float2);
   const size_t stage_nint = std::max<size_t>(1, std::min<size_t>(kStageBytes / per_int, (size_t)p->max_nint));
@@ -1135,7 +1152,7 @@ rf_status alloc_device(rf_plan* p) {
   RF_CUDA(cudaMemset(p->d_err, 0, sizeof(int)));
 
   // column-FFT scratch, whole groups per wave
-  if (p->derived && (s = p->dalloc(&p->d_units, (size_t)p->img_cap)) != RF_OK) return s;
+  if (p->derived && (s = p->dalloc(&p->d_units, count_units(p))) != RF_OK) return s;
   if ((s = alloc_wave_scratch(p, default_slots(p, (size_t)p->img_cap))) != RF_OK) return s;
 
   // host->device staging of raw visibilities
