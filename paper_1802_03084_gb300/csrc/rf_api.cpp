@@ -288,7 +288,6 @@ struct rf_plan {
   float* d_rms = nullptr;       // [sslots] raw RMS (plans with sums of 8 or 16)
   unsigned long long* d_best = nullptr;  // [sslots] largest pixel that reaches it
   float2* d_clip = nullptr;     // [sslots] clipping window (RF_NOISE_CLIPPED only)
-  rf::ClipPartial* d_cparts = nullptr;  // kept-pixel partials (RF_NOISE_CLIPPED only)
   rf::PlainBuffers plain{};     // allocated on the first plain-form search
 
   // RF_TUNE_FUSED and RF_TUNE_RING: kept and reported, without effect
@@ -710,6 +709,16 @@ int wave_tslots(const rf_plan* p, int slots) {
 }
 int wave_sslots(const rf_plan* p, int slots) { return p->derived ? std::max(slots, group_images(p)) : slots; }
 
+// Cell sums of a wave's groups, 32 images a cell.  Under the clipped noise, which
+// overlapped waves exclude, the row pass's kept-pixel partials follow in the same
+// buffer once the column pass has read it.
+size_t cellbuf_len(const rf_plan* p, int gslots, int sslots) {
+  static_assert(sizeof(rf::ClipPartial) % sizeof(float2) == 0, "partials in units of cell sums");
+  const size_t cells = (size_t)gslots * std::max(p->n_cells, 1) * 32;
+  if (!(p->flags & RF_NOISE_CLIPPED)) return cells;
+  return std::max(cells, (size_t)sslots * plan_partials(p) * (sizeof(rf::ClipPartial) / sizeof(float2)));
+}
+
 // Units of the longest segment (every trial has its most images there).
 size_t count_units(const rf_plan* p) {
   const int B = p->shape.images_per_group, step = rf::unit_images(p->pairs);
@@ -910,7 +919,7 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
     p->d_partials = nullptr;
   }
   if (p->d_cellbuf) {
-    p->device_bytes -= (uint64_t)p->gslots_max * p->n_cells * 32 * sizeof(float2);
+    p->device_bytes -= cellbuf_len(p, p->gslots_max, p->sslots) * sizeof(float2);
     p->dfree(p->d_cellbuf);
     p->d_cellbuf = nullptr;
   }
@@ -945,11 +954,6 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
     p->dfree(p->d_clip);
     p->d_clip = nullptr;
   }
-  if (p->d_cparts) {
-    p->device_bytes -= (uint64_t)p->sslots * nrb * sizeof(rf::ClipPartial);
-    p->dfree(p->d_cparts);
-    p->d_cparts = nullptr;
-  }
   p->slots_max = slots;
   p->tslots = wave_tslots(p, slots);
   p->sslots = wave_sslots(p, slots);
@@ -959,17 +963,14 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
   rf_status s;
   if ((s = p->dalloc(&p->d_T, (size_t)p->tslots * per_slot)) != RF_OK) return s;
   if ((s = p->dalloc(&p->d_partials, (size_t)p->sslots * nrb)) != RF_OK) return s;
-  if ((s = p->dalloc(&p->d_cellbuf, (size_t)p->gslots_max * std::max(p->n_cells, 1) * 32)) != RF_OK) return s;
+  if ((s = p->dalloc(&p->d_cellbuf, cellbuf_len(p, p->gslots_max, p->sslots))) != RF_OK) return s;
   if ((s = p->dalloc(&p->d_colsq, (size_t)p->sslots * p->ncol)) != RF_OK) return s;
   if ((s = p->dalloc(&p->d_mean0, (size_t)p->sslots)) != RF_OK) return s;
   if ((s = p->dalloc(&p->d_noise, (size_t)p->sslots)) != RF_OK) return s;
   if ((s = p->dalloc(&p->d_gate, (size_t)p->sslots)) != RF_OK) return s;
   if ((s = p->dalloc(&p->d_best, (size_t)p->sslots)) != RF_OK) return s;
   if (p->pairs && (s = p->dalloc(&p->d_rms, (size_t)p->sslots)) != RF_OK) return s;
-  if (p->flags & RF_NOISE_CLIPPED) {
-    if ((s = p->dalloc(&p->d_clip, (size_t)p->sslots)) != RF_OK) return s;
-    if ((s = p->dalloc(&p->d_cparts, (size_t)p->sslots * nrb)) != RF_OK) return s;
-  }
+  if ((p->flags & RF_NOISE_CLIPPED) && (s = p->dalloc(&p->d_clip, (size_t)p->sslots)) != RF_OK) return s;
   const int xb = std::min(256 / (p->npix / 32), p->npix / 2);  // row pairs of a row-pass work item
   encode_tile_map(p, p->tmap_T, p->d_T, p->tslots, 2 * xb);
   // the halves of d_T, each a wave's scratch when waves are overlapped
@@ -1022,11 +1023,10 @@ uint64_t estimate_device_bytes(const rf_plan* p, int slots) {
   const int tslots = wave_tslots(p, slots), sslots = wave_sslots(p, slots);
   const int gslots = std::max(2 * ((tslots + B - 1) / B), 1);
   b += r((size_t)tslots * per_slot, 1) + r((size_t)sslots * plan_partials(p), sizeof(StatPartial)) +
-       r((size_t)gslots * std::max(p->n_cells, 1) * 32, sizeof(float2)) + r((size_t)sslots * p->ncol, 4) +
+       r(cellbuf_len(p, gslots, sslots), sizeof(float2)) + r((size_t)sslots * p->ncol, 4) +
        r(sslots, 4) + r(sslots, sizeof(rf::ImgNoise));
   b += r(sslots, sizeof(float)) + r(sslots, 8);
-  if (p->flags & RF_NOISE_CLIPPED)
-    b += r(sslots, sizeof(float2)) + r((size_t)sslots * plan_partials(p), sizeof(rf::ClipPartial));
+  if (p->flags & RF_NOISE_CLIPPED) b += r(sslots, sizeof(float2));
   if (p->pairs) b += r(sslots, sizeof(float));
   const size_t per_int = rows * p->npol * sizeof(float2);
   const size_t stage_nint = std::max<size_t>(1, std::min<size_t>(kStageBytes / per_int, (size_t)p->max_nint));
@@ -1343,7 +1343,7 @@ rf_status finish_wave(rf_plan* p, const SegmentGeom& g, const Wave& w, const flo
   ps.gate = gate;
   ps.best = best;
   ps.clip = cw;
-  ps.cparts = clip ? p->d_cparts + slot0 * plan_partials(p) : nullptr;
+  ps.cparts = clip ? reinterpret_cast<rf::ClipPartial*>(p->d_cellbuf) : nullptr;  // see cellbuf_len
   RF_TIMED(p->prof, K_ROWFFT_STATS, st, launch_row_pass(p, g, w, T, ps, tm, im, st, pl));
   RF_TIMED(p->prof, K_FINALIZE, st,
            rf::launch_finalize(g, ps, (int)nparts, noise, mean0, p->d_img_info, p->d_weight, ni, w.img_begin, p->threshold,

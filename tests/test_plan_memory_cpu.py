@@ -1,6 +1,7 @@
 """Device memory of plans whose widths are sums of others, as estimated before
 creation (the serving runtime admits by it): no more than the images of a wave
-need, and buffers of the clipped noise only under RF_NOISE_CLIPPED.
+need, and the clipped noise's partials only under RF_NOISE_CLIPPED, in the place
+of the cell sums.
 """
 
 import numpy as np
@@ -40,7 +41,11 @@ def test_one_group_where_a_wave_is_one_group(npix, dts):
 
 
 @pytest.mark.parametrize("npix,dts", [(256, [1]), (1024, [1, 2]), (2048, [1, 2, 4, 8])])
-def test_clipped_noise_buffers_only_with_the_flag(npix, dts):
+def test_clipped_noise_partials_lie_in_the_cell_buffer(npix, dts):
     with _plan(npix, dts) as plain, _plan(npix, dts, rf.RF_NOISE_CLIPPED) as clipped:
-        # a window an image and 16 bytes a row pair at least
-        assert _estimate(clipped, 64) - _estimate(plain, 64) >= 64 * (8 + npix // 2 * 16)
+        # beside a window an image: what the partials, 16 bytes a row pair or a
+        # row of an image, take beyond the cell sums of two to four groups
+        partials = 64 * npix // 2 * 16 * (2 if 8 in dts else 1) * (npix // 1024 if npix > 1024 else 1)
+        cells = plain.info().n_cells * 32 * 8
+        more = _estimate(clipped, 64) - _estimate(plain, 64) - 64 * 8
+        assert partials - 4 * cells <= more <= partials - 2 * cells
