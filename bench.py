@@ -65,8 +65,8 @@ def parse():
     ap.add_argument("--no-plain", action="store_true", help="skip timing the plain per-trial form")
     ap.add_argument("--no-autotune", action="store_true", help="keep the engine's default tuning")
     ap.add_argument("--fused", type=int, default=-1, choices=[-1, 0, 1],
-                    help="force the fused imaging pass off (0) or on (1); -1: the autotuner's or default choice")
-    ap.add_argument("--ring", type=int, default=0, help="chunk slots of the fused pass's ring (0: default)")
+                    help="kept for old command lines, without effect (see RF_TUNE_FUSED)")
+    ap.add_argument("--ring", type=int, default=0, help="kept for old command lines, without effect")
     ap.add_argument("--overlap", type=int, default=-1, choices=[-1, 0, 1],
                     help="force overlapped waves off (0) or on (1); -1: the autotuner's or default choice")
     ap.add_argument("--tune-cache", default=os.path.expanduser("~/.cache/realfast_gb300/tune.json"))

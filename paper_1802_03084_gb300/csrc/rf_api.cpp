@@ -100,12 +100,12 @@ struct BusyGuard {
 
 enum KernelKind {
   K_H2D = 0, K_INGEST, K_RESAMPLE, K_WEIGHTS, K_GRID_CELLS, K_GRID_COLFFT, K_ROWFFT_STATS, K_FINALIZE,
-  K_PLAIN_TRIAL, K_MEAN_SUBTRACT, K_IMAGE_NOISE, K_IMAGE_FUSED, K_NKINDS
+  K_PLAIN_TRIAL, K_MEAN_SUBTRACT, K_IMAGE_NOISE, K_NKINDS
 };
 const char* const kKindNames[K_NKINDS] = {"h2d_copy",    "ingest",       "resample",
                                            "weights",     "grid_cells",   "grid_colfft",
                                            "rowfft_stats", "finalize",    "plain_trial_chunk",
-                                           "mean_subtract", "image_noise", "image_fused"};
+                                           "mean_subtract", "image_noise"};
 
 // Event-pair timing of every launch a plan issues while profiling is on.
 struct Profiler {
@@ -222,7 +222,7 @@ struct rf_plan {
   std::vector<int32_t> ongrid_chan;
   int n_on = 0, iu_max = 0, iv_max = 0, ncol = 1, n_offgrid = 0;
   rf::ImageKernelShape shape{};
-  // Widths whose images are sums of two or four images of another width of
+  // Widths whose images are sums of 2, 4, 8 or 16 images of another width of
   // the plan (see build_widths): sum_of[s] is that width's index (s itself for
   // a width with transforms of its own), and sums[s][L - 1] the width made of
   // 2^L images of width s (-1: none).
@@ -393,13 +393,13 @@ int64_t count_images(const rf_plan* p, int nint) {
   return n;
 }
 
-// Chains of widths {b, 2 b, 4 b}: from the smallest width up, each one not yet
-// taken becomes a base, and the images of the widths twice and four times it
-// (the first entry of the list of each) are sums of its images.  Whenever an
+// Chains of widths {b, 2 b, 4 b, 8 b, 16 b} (up to 4 b above 2048^2): from the
+// smallest width up, each one not yet taken becomes a base, and the images of
+// the others (the first entry of the list of each) are sums of its images.  Whenever an
 // image of such a width is searched, so are the images that it is the sum of:
 // floor(x / 2 b) = floor(floor(x / b) / 2) for both edge rules and for a
-// stream's span.  Sums of eight would need 64 more registers a lane to be
-// kept than tensor memory has (see k_rowfft_tree).
+// stream's span.  What is kept for longer sums has no room in tensor memory
+// (see k_rowfft_duo and k_rowfft_tree).
 void build_widths(rf_plan* p) {
   const int n = p->ndt;
   p->sum_of.resize(n);
@@ -2223,14 +2223,14 @@ rf_status rf_selftest_bounded_wait(int32_t device, int32_t polls, int32_t* gave_
   DeviceGuard dg(device);
   if (!dg.ok) return fail(RF_ERR_CUDA, "cannot select device %d", device);
   int* d = nullptr;
-  RF_CUDA(cudaMalloc(&d, 2 * sizeof(int)));
+  RF_CUDA(cudaMalloc(&d, sizeof(int)));
   int h = 0;
-  cudaError_t e = cudaMemset(d, 0, 2 * sizeof(int));
+  cudaError_t e = cudaMemset(d, 0, sizeof(int));
   if (e == cudaSuccess) e = rf::launch_wait_selftest(polls, d, nullptr);
   if (e == cudaSuccess) e = cudaMemcpy(&h, d, sizeof(int), cudaMemcpyDeviceToHost);
   cudaFree(d);
   if (e != cudaSuccess) return fail(RF_ERR_CUDA, "bounded-wait check: %s", cudaGetErrorString(e));
-  *gave_up = h == 3 ? 1 : 0;  // both waits gave up
+  *gave_up = h;
   return RF_OK;
 }
 

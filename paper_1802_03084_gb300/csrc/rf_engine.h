@@ -285,13 +285,6 @@ struct SegmentGeom {
 // column's cells), leaving R transforms of length 1024.
 constexpr int col_split(int n) { return n >= 2048 ? n / 1024 : 1; }
 
-// Complex values per thread of the row pass at N = 2048: 32 (64 threads per
-// row pair, 256-thread blocks) or 16 (128 threads per row pair, 512-thread
-// blocks: twice the warps in the same shared memory, at 64 registers a
-// thread).  Both give the same images; 16 measured 36% slower on GB300
-// (48.0 against 35.2 ms per 8134-image launch), so 32 is built.
-#define RF_ROW_VALUES_2048 32
-
 // ---------------------------------------------------------------- launchers
 // All launchers return cudaSuccess or the launch error.
 
@@ -325,7 +318,7 @@ cudaError_t launch_grid_single(const SegmentGeom& g, const DevTables& tb, const 
 
 // Column FFTs (pass A2) of the same groups from cellbuf; writes
 // Tbuf[b][col][y], b = transformed-image index - base_base, and for every
-// image of the groups, sums of two and four included, the Parseval sums
+// image of the groups, sums of others included, the Parseval sums
 // colsq[slot][col] (weighted sum of |H|^2 over the column) and
 // mean0[slot] = Re H(u = 0, v = 0), slot = image index - img_base.  `duo`: in
 // the row order of k_rowfft_duo (duo_swizzle).

@@ -3,16 +3,18 @@
 // FFT + image statistics.
 //
 // The half-plane grid H[iv][iu] (iu = 0 .. iu_max) of an image is never
-// materialised in global memory.  Pass A (k_grid_colfft) builds one column of
-// H per transform directly in shared memory from the dedispersed, resampled
-// visibilities and runs the length-N inverse FFT along v; the result
-// T[iu][y] goes to a global (L2-resident) scratch.  Pass B (k_rowfft_stats)
-// takes two image rows y, y+1 per transform: with Z[u] = T[u][y] + i T[u][y+1]
-// on the Hermitian extension (Z[N-u] = conj T[u][y] + i conj T[u][y+1]),
-// one complex inverse FFT gives row y in the real part and row y+1 in the
-// imaginary part.  Pixel statistics (sum, sum of squares, max with lowest
-// index) are reduced in the same kernel; the image itself is written only
-// when a caller asks for it.
+// materialised in global memory: k_grid_cells (rf_kernels.cu) writes the sums of
+// its occupied cells.  Pass A (k_colfft) takes one column of them at a time, adds
+// up the image's noise (Parseval) and runs the length-N inverse FFT along v;
+// the result T[iu][y] goes to a global scratch, the size of a wave of images.
+// Pass B (k_rowfft_stats) takes two image rows y, y+1 per transform: with Z[u] =
+// T[u][y] + i T[u][y+1] on the Hermitian extension (Z[N-u] = conj T[u][y] + i conj
+// T[u][y+1]), one complex inverse FFT gives row y in the real part and row y+1 in
+// the imaginary part.  The maximum with its lowest index is reduced in the same
+// kernel (and under the clipped noise the sums over the kept pixels); the image
+// itself is written only when a caller asks for it.  k_rowfft_tree and
+// k_rowfft_duo are pass B for plans with widths whose images are sums of
+// another width's.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -51,19 +53,20 @@ struct ImgCfg {
   static constexpr int SMEM_A_FIXED = XA * fft_stride<N>() * 8;
   // pass B (row pass): EB values per thread, TB threads per transform, XB row
   // pairs (RB rows) per work item; the column-FFT tile of the next item is
-  // prefetched while the current one is transformed
-  static constexpr int EB = N == 2048 ? RF_ROW_VALUES_2048 : E;
-  static constexpr int TB = N / EB;
-  static constexpr int XB = cmin((EB == 32 ? 256 : 512) / TB, N / 2);
+  // prefetched while the current one is transformed.  (At 2048^2, 16 values
+  // a thread and twice the warps took 48.0 ms for 35.2 a wave of 8134 images.)
+  static constexpr int EB = E;
+  static constexpr int TB = T;
+  static constexpr int XB = cmin(256 / TB, N / 2);
   static constexpr int THREADS_B = TB * XB;
   static constexpr int RB = 2 * XB;
   static constexpr int PARTIALS = (N / 2) * (TB > 32 ? TB / 32 : 1);  // row-pass partials per image
   static constexpr int CH = XB;                                  // 16-byte chunks per tile row
   static constexpr int STRIDE = fft_stride<N>();
-  // N = 2048 (32 values a thread): each row-pair transform is split by one
+  // N = 2048: each row-pair transform is split by one
   // decimation-in-frequency step into two length-N/2 transforms, the even
   // and the odd pixels, one per warp of the transform (see row_zbuild)
-  static constexpr int RSPLIT = (N == 2048 && EB == 32) ? 2 : 1;
+  static constexpr int RSPLIT = N == 2048 ? 2 : 1;
   static constexpr int STRIDE_B = RSPLIT * fft_stride<N / RSPLIT>();  // float2 per row transform
   static constexpr int SMEM_B_FIXED = XB * STRIDE_B * 8;
   // N >= 1024: the row-pass tile arrives by tensor copies (TMA) whose
@@ -451,7 +454,7 @@ __device__ __forceinline__ void row_zbuild(float2 (&v)[ImgCfg<N>::EB], const flo
     // Y_s at u' = j + 32 r (lane j, r < 32): Z[u'] is a direct column or
     // zero, Z[u' + H] the mirror of column H - u' or zero.  For s = 1 the
     // factor exp(+2 pi i r / 64) of u' is applied here and exp(+2 pi i j / N)
-    // rides on the second-pass twiddles (see row_finish).
+    // rides on the second-pass twiddles (see row_fft).
     constexpr int H = N / 2;
     static_assert(EB == 32 && TB == 64 && 32 % (K::CH << K::SWZ_SH) == 0, "split row transform layout");
     const int s = t >> 5, j = t & 31;

@@ -310,12 +310,12 @@ cudaError_t run_noalloc(const float2* grid, double weight, const DeviceSetup& d,
                         rf_image_stat* out) {
   using K = ImgCfg<N>;
   // The column-FFT scratch holds one image of at most kMaxN, the partials
-  // area ImgCfg<kMaxN>::PARTIALS records; the Parseval sum of k_colfft_dense
-  // and the finalisation reduce within one warp per column, which holds
-  // while a transform fits one warp.
+  // area ImgCfg<kMaxN>::PARTIALS records; the Parseval sum of a column is
+  // reduced within a warp, in k_single_columns as in k_colfft_dense (below
+  // 64^2), which holds while a transform fits one.
   static_assert(N <= kMaxN, "image larger than the static scratch");
   static_assert(K::PARTIALS <= ImgCfg<kMaxN>::PARTIALS, "partials area too small");
-  static_assert(K::T <= 32, "the Parseval reduction of k_colfft_dense spans one warp");
+  static_assert(K::T <= 32, "the Parseval reduction of a column spans one warp");
   float2* T = reinterpret_cast<float2*>(d.scratch);
   StatPartial* partials = reinterpret_cast<StatPartial*>(d.scratch + kTBytes);
   float* colsq = reinterpret_cast<float*>(d.scratch + kTBytes + kPartialBytes);
