@@ -292,10 +292,12 @@ def _ptr(x) -> int:
 def _stream(stream) -> Optional[int]:
     if stream is None:
         # a program that has not imported torch has no torch stream; asking the
-        # driver for its devices on every call costs microseconds
-        torch = sys.modules.get("torch")
-        if torch is not None and torch.cuda.is_initialized():
-            return torch.cuda.current_stream().cuda_stream
+        # driver for its devices on every call costs microseconds.  While another
+        # thread imports torch, its module is there before its parts are.
+        cuda = getattr(sys.modules.get("torch"), "cuda", None)
+        initialized = getattr(cuda, "is_initialized", None)
+        if initialized is not None and initialized():
+            return cuda.current_stream().cuda_stream
         return None
     if hasattr(stream, "cuda_stream"):
         return stream.cuda_stream
