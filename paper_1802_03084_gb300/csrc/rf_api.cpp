@@ -971,7 +971,7 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
   if ((s = p->dalloc(&p->d_best, (size_t)p->sslots)) != RF_OK) return s;
   if (p->pairs && (s = p->dalloc(&p->d_rms, (size_t)p->sslots)) != RF_OK) return s;
   if ((p->flags & RF_NOISE_CLIPPED) && (s = p->dalloc(&p->d_clip, (size_t)p->sslots)) != RF_OK) return s;
-  const int xb = std::min(256 / (p->npix / 32), p->npix / 2);  // row pairs of a row-pass work item
+  const int xb = std::min(256 / std::max(p->npix / 32, 1), p->npix / 2);  // row pairs of a row-pass work item
   encode_tile_map(p, p->tmap_T, p->d_T, p->tslots, 2 * xb);
   // the halves of d_T, each a wave's scratch when waves are overlapped
   const int half = p->tslots / 2;
