@@ -54,6 +54,7 @@ constexpr uint32_t kKnownFlags = RF_STORE_FP16 | RF_EDGE_PARTIAL | RF_MEAN_SUBTR
 constexpr size_t kStageBytes = 256ull << 20;   // host->device chunk of raw visibilities
 constexpr size_t kTBudgetBytes = 4096ull << 20;  // column-FFT scratch per wave
 constexpr int kInlineCands = 512;                // candidates read back with their count
+constexpr int kRedoImages = 1024;                // sums imaged from their own samples at a time
 constexpr int kInlineStats = 16384;              // image records read back through page-locked memory
 constexpr int kRangeEntries = 64;                // target entries per gridding warp
 constexpr size_t kPeriodicBudgetBytes = 1ull << 30;  // transformed series per DM batch
@@ -100,12 +101,12 @@ struct BusyGuard {
 
 enum KernelKind {
   K_H2D = 0, K_INGEST, K_RESAMPLE, K_WEIGHTS, K_GRID_CELLS, K_GRID_COLFFT, K_ROWFFT_STATS, K_FINALIZE,
-  K_PLAIN_TRIAL, K_MEAN_SUBTRACT, K_IMAGE_NOISE, K_NKINDS
+  K_PLAIN_TRIAL, K_MEAN_SUBTRACT, K_IMAGE_NOISE, K_CHECK_SUMS, K_NKINDS
 };
 const char* const kKindNames[K_NKINDS] = {"h2d_copy",    "ingest",       "resample",
                                            "weights",     "grid_cells",   "grid_colfft",
                                            "rowfft_stats", "finalize",    "plain_trial_chunk",
-                                           "mean_subtract", "image_noise"};
+                                           "mean_subtract", "image_noise", "check_sums"};
 
 // Event-pair timing of every launch a plan issues while profiling is on.
 struct Profiler {
@@ -285,7 +286,11 @@ struct rf_plan {
   float* d_mean0 = nullptr;     // [slots] Re H(0, 0)
   rf::ImgNoise* d_noise = nullptr;  // [sslots] mean and noise from the Parseval sums
   float* d_gate = nullptr;      // [sslots] least raw maximum of a candidate
-  float* d_rms = nullptr;       // [sslots] raw RMS (plans with sums of 8 or 16)
+  float* d_rms = nullptr;       // [sslots] raw RMS (plans with sums)
+  int* d_redo = nullptr;        // [img_cap] sums to image from their own samples (plans with sums)
+  int4* d_redo_info = nullptr;  // [kRedoImages] lists of a chunk of them
+  Group* d_redo_groups = nullptr;
+  double* d_redo_weight = nullptr;
   unsigned long long* d_best = nullptr;  // [sslots] largest pixel that reaches it
   float2* d_clip = nullptr;     // [sslots] clipping window (RF_NOISE_CLIPPED only)
   rf::PlainBuffers plain{};     // allocated on the first plain-form search
@@ -969,7 +974,7 @@ rf_status alloc_wave_scratch(rf_plan* p, int slots) {
   if ((s = p->dalloc(&p->d_noise, (size_t)p->sslots)) != RF_OK) return s;
   if ((s = p->dalloc(&p->d_gate, (size_t)p->sslots)) != RF_OK) return s;
   if ((s = p->dalloc(&p->d_best, (size_t)p->sslots)) != RF_OK) return s;
-  if (p->pairs && (s = p->dalloc(&p->d_rms, (size_t)p->sslots)) != RF_OK) return s;
+  if (p->derived && (s = p->dalloc(&p->d_rms, (size_t)p->sslots)) != RF_OK) return s;
   if ((p->flags & RF_NOISE_CLIPPED) && (s = p->dalloc(&p->d_clip, (size_t)p->sslots)) != RF_OK) return s;
   const int xb = std::min(256 / std::max(p->npix / 32, 1), p->npix / 2);  // row pairs of a row-pass work item
   encode_tile_map(p, p->tmap_T, p->d_T, p->tslots, 2 * xb);
@@ -1014,8 +1019,9 @@ uint64_t estimate_device_bytes(const rf_plan* p, int slots) {
   }
   b += r(p->dt.size(), 8) + r(p->dt.size(), 4);
   const int64_t img_cap = std::max<int64_t>(count_images(p, p->max_nint), 1);
-  b += r(img_cap, sizeof(int4)) + r(img_cap, sizeof(Group)) + r(img_cap, 8) + r(img_cap, sizeof(DevCand)) + 4 + 4;  // candidate count, error flag
-  if (p->derived) b += r(count_units(p), sizeof(rf::Unit));
+  b += r(img_cap, sizeof(int4)) + r(img_cap, sizeof(Group)) + r(img_cap, 8) + r(img_cap, sizeof(DevCand)) + 12;  // counts, error flag
+  if (p->derived)
+    b += r(count_units(p), sizeof(rf::Unit)) + r(img_cap, 4) + kRedoImages * (sizeof(int4) + sizeof(Group) + 8);
   const size_t per_slot = (size_t)p->ncol * N * sizeof(float2);
   if (slots <= 0) slots = default_slots(p, (size_t)img_cap);
   const int B = p->shape.images_per_group;
@@ -1027,7 +1033,7 @@ uint64_t estimate_device_bytes(const rf_plan* p, int slots) {
        r(sslots, 4) + r(sslots, sizeof(rf::ImgNoise));
   b += r(sslots, sizeof(float)) + r(sslots, 8);
   if (p->flags & RF_NOISE_CLIPPED) b += r(sslots, sizeof(float2));
-  if (p->pairs) b += r(sslots, sizeof(float));
+  if (p->derived) b += r(sslots, sizeof(float));
   const size_t per_int = rows * p->npol * sizeof(float2);
   const size_t stage_nint = std::max<size_t>(1, std::min<size_t>(kStageBytes / per_int, (size_t)p->max_nint));
   b += r(stage_nint * per_int, 1);
@@ -1136,8 +1142,8 @@ rf_status alloc_device(rf_plan* p) {
   if ((s = p->dalloc(&p->d_groups, p->group_cap)) != RF_OK) return s;
   if ((s = p->dalloc(&p->d_weight, p->img_cap)) != RF_OK) return s;
   if ((s = p->dalloc(&p->d_cands, p->img_cap)) != RF_OK) return s;
-  if ((s = p->dalloc(&p->d_ncand, 2)) != RF_OK) return s;
-  p->d_err = p->d_ncand + 1;  // read back together
+  if ((s = p->dalloc(&p->d_ncand, 3)) != RF_OK) return s;  // candidates, sums to redo, error flag: read back together
+  p->d_err = p->d_ncand + 2;
   {
     const size_t head = 16 + (size_t)std::min(kInlineCands, p->img_cap) * sizeof(DevCand);
     const size_t at = (head + 15) / 16 * 16;
@@ -1152,7 +1158,13 @@ rf_status alloc_device(rf_plan* p) {
   RF_CUDA(cudaMemset(p->d_err, 0, sizeof(int)));
 
   // column-FFT scratch, whole groups per wave
-  if (p->derived && (s = p->dalloc(&p->d_units, count_units(p))) != RF_OK) return s;
+  if (p->derived) {
+    if ((s = p->dalloc(&p->d_units, count_units(p))) != RF_OK) return s;
+    if ((s = p->dalloc(&p->d_redo, (size_t)p->img_cap)) != RF_OK) return s;
+    if ((s = p->dalloc(&p->d_redo_info, kRedoImages)) != RF_OK) return s;
+    if ((s = p->dalloc(&p->d_redo_groups, kRedoImages)) != RF_OK) return s;
+    if ((s = p->dalloc(&p->d_redo_weight, kRedoImages)) != RF_OK) return s;
+  }
   if ((s = alloc_wave_scratch(p, default_slots(p, (size_t)p->img_cap))) != RF_OK) return s;
 
   // host->device staging of raw visibilities
@@ -1333,10 +1345,14 @@ rf_status finish_wave(rf_plan* p, const SegmentGeom& g, const Wave& w, const flo
   const bool only_cands = !clip && !d_stats && !im;
   float* gate = only_cands ? p->d_gate + slot0 : nullptr;
   unsigned long long* best = only_cands ? p->d_best + slot0 : nullptr;
-  float* rms = wave_duo(p, w) ? p->d_rms + slot0 : nullptr;
+  float* rms = units ? p->d_rms + slot0 : nullptr;
   RF_TIMED(p->prof, K_IMAGE_NOISE, st,
            rf::launch_image_noise(g, colsq, mean0, p->d_weight, ni, w.img_begin, p->threshold, noise, gate, best,
                                   cw, rms, st));
+  if (units)
+    RF_TIMED(p->prof, K_CHECK_SUMS, st,
+             rf::launch_check_sums(p->d_units + w.unit_begin, w.unit_end - w.unit_begin, w.img_begin, rms,
+                                   p->d_weight, p->d_ncand + 1, p->d_redo, st));
   rf::PassStats ps;
   ps.rms = rms;
   ps.partials = p->d_partials + slot0 * plan_partials(p);
@@ -1509,6 +1525,48 @@ rf_status run_plain(rf_plan* p, int nint, DevStat* d_stats, cudaStream_t st) {
   return RF_OK;
 }
 
+// Images the n sums that the waves have listed (see kSumCancel) from their
+// own samples, as listed trials, and adds their candidates and statistics to the
+// search's.  A copy and a wait for each chunk, where one is listed at all: noise
+// lists none.
+rf_status redo_sums(rf_plan* p, int nint, int n, DevStat* d_stats, cudaStream_t st) {
+  std::vector<int> redo(n);
+  RF_CUDA(cudaMemcpyAsync(redo.data(), p->d_redo, n * sizeof(int), cudaMemcpyDeviceToHost, st));
+  RF_CUDA(cudaStreamSynchronize(st));
+  std::sort(redo.begin(), redo.end());  // blocks listed them in any order
+  struct Lists {  // the search's own lists stay as they are
+    rf_plan* p;
+    explicit Lists(rf_plan* pl) : p(pl) { swap(); }
+    ~Lists() { swap(); }
+    void swap() {
+      std::swap(p->d_img_info, p->d_redo_info);
+      std::swap(p->d_groups, p->d_redo_groups);
+      std::swap(p->d_weight, p->d_redo_weight);
+    }
+  } lists(p);
+  const int per_wave = std::min(std::min(p->tslots, p->sslots), p->gslots_max);  // single-image groups
+  for (int k0 = 0; k0 < n; k0 += kRedoImages) {
+    const int m = std::min(kRedoImages, n - k0);
+    std::vector<int4> info(m);
+    std::vector<Group> grp(m);
+    for (int k = 0; k < m; ++k) {
+      info[k] = p->img_info[redo[k0 + k]];
+      grp[k] = Group{info[k].x, info[k].y, info[k].z, 1, k, k, {}, {}, {}};
+    }
+    RF_CUDA(cudaMemcpyAsync(p->d_img_info, info.data(), m * sizeof(int4), cudaMemcpyHostToDevice, st));
+    RF_CUDA(cudaMemcpyAsync(p->d_groups, grp.data(), m * sizeof(Group), cudaMemcpyHostToDevice, st));
+    std::vector<Wave> waves;
+    for (int k = 0; k < m; k += per_wave) {
+      const int e = std::min(m, k + per_wave);
+      waves.push_back(Wave{k, e, k, e, k, e, 0, 0});
+    }
+    const rf_status s = run_waves(p, nint, waves, m, d_stats, nullptr, st, Single::kDirect);
+    RF_CUDA(cudaStreamSynchronize(st));  // the lists are reused
+    if (s != RF_OK) return s;
+  }
+  return RF_OK;
+}
+
 // Sets the plan's t' span for one search and clears it on every exit.
 struct SpanGuard {
   rf_plan* p;
@@ -1558,7 +1616,7 @@ rf_status search_impl(rf_plan* p, const void* vis, int nint, void* stream, rf_ca
     }
     d_stats = p->d_stats;
   }
-  RF_CUDA(cudaMemsetAsync(p->d_ncand, 0, sizeof(int), st));
+  RF_CUDA(cudaMemsetAsync(p->d_ncand, 0, 2 * sizeof(int), st));
   if (nimg > 0) {
     if (p->form == RF_FORM_PLAIN)
       s = run_plain(p, nint, d_stats, st);
@@ -1574,22 +1632,22 @@ rf_status search_impl(rf_plan* p, const void* vis, int nint, void* stream, rf_ca
   const int head = std::min(kInlineCands, p->img_cap);
   const int* res = reinterpret_cast<const int*>(p->h_res);
   const DevCand* first = reinterpret_cast<const DevCand*>(p->h_res + 16);
-  RF_CUDA(cudaMemcpyAsync(p->h_res, p->d_ncand, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
-  RF_CUDA(cudaMemcpyAsync(p->h_res + 16, p->d_cands, head * sizeof(DevCand), cudaMemcpyDeviceToHost, st));
-  std::vector<DevStat> ds_far;
-  const DevStat* ds = nullptr;
-  if (d_stats && nimg > 0) {
-    if (p->h_stats) {
-      RF_CUDA(cudaMemcpyAsync(p->h_stats, d_stats, (size_t)nimg * sizeof(DevStat), cudaMemcpyDeviceToHost, st));
-      ds = p->h_stats;
-    } else {
-      ds_far.resize(nimg);
-      RF_CUDA(cudaMemcpyAsync(ds_far.data(), d_stats, (size_t)nimg * sizeof(DevStat), cudaMemcpyDeviceToHost, st));
-      ds = ds_far.data();
-    }
+  std::vector<DevStat> ds_far(d_stats && !p->h_stats ? nimg : 0);
+  DevStat* ds = p->h_stats ? p->h_stats : ds_far.data();
+  auto read_results = [&]() -> rf_status {
+    RF_CUDA(cudaMemcpyAsync(p->h_res, p->d_ncand, 3 * sizeof(int), cudaMemcpyDeviceToHost, st));
+    RF_CUDA(cudaMemcpyAsync(p->h_res + 16, p->d_cands, head * sizeof(DevCand), cudaMemcpyDeviceToHost, st));
+    if (d_stats && nimg > 0)
+      RF_CUDA(cudaMemcpyAsync(ds, d_stats, (size_t)nimg * sizeof(DevStat), cudaMemcpyDeviceToHost, st));
+    RF_CUDA(cudaStreamSynchronize(st));
+    return RF_OK;
+  };
+  if ((s = read_results()) != RF_OK) return s;
+  if (res[1] > 0 && !res[2] && nimg > 0) {
+    if ((s = redo_sums(p, nint, res[1], d_stats, st)) != RF_OK) return s;
+    if ((s = read_results()) != RF_OK) return s;
   }
-  RF_CUDA(cudaStreamSynchronize(st));
-  if (res[1]) {
+  if (res[2]) {
     cudaMemset(p->d_err, 0, sizeof(int));
     return fail(RF_ERR_TIMEOUT, "a bounded device-side wait for a tile copy gave up");
   }

@@ -198,8 +198,7 @@ struct ImgNoise {
 // and cparts are set together); or, where only candidates are wanted (best and
 // gate are set together), each image's largest pixel if it is not below its
 // gate: best[slot] starts at 0 and ends as the largest best_key of such pixels.
-// rms[slot] (plans with sums of 8 or 16 only): how bright an image is, raw
-// units (see may_pair).
+// rms[slot] (plans with sums): how bright an image is, raw units (see may_pair).
 struct PassStats {
   StatPartial* partials = nullptr;  // [slot][partials per image]
   const float2* clip = nullptr;
@@ -216,6 +215,13 @@ struct PassStats {
 // own; unlimited, a saturated integration put 0.2 sigma into its neighbour at
 // 10^6 times its brightness, and one NaN took the neighbour's candidate.
 constexpr float kPairContrast = 1.5f;
+// A sum of images carries the FP32 rounding of its parts' transforms.  Noise adds
+// up to the sum's own power; where the parts' power is more than kSumCancel times
+// that (mean-subtracted samples of a whole segment, interference that changes
+// sign), the rounding is more than twice that of a transform of the sum's own, in
+// the end all there is: a width as long as a mean-subtracted segment came out at
+// 10 to 16 sigma where its own transform gives the 4 to 5 of noise.
+constexpr double kSumCancel = 4.0;
 #ifdef __CUDACC__
 __device__ __forceinline__ bool may_pair(float a, float b) {
   return a <= kPairContrast * b && b <= kPairContrast * a && a + b < INFINITY;  // false for NaN
@@ -331,10 +337,16 @@ cudaError_t launch_colfft(const SegmentGeom& g, const DevTables& tb, const Group
 // value below which a maximum cannot make image i a candidate, and 0.  clip[i] (if not null): the
 // clipping window of the clipped noise in raw pixel units (the image times
 // 2W), {mean0[i], kClipSigmas * sigma over all pixels}.  rms[i] (if not null):
-// the raw image's RMS over all pixels (see PassStats).
+// the raw image's RMS over all pixels.
 cudaError_t launch_image_noise(const SegmentGeom& g, const float* colsq, const float* mean0, const double* weight,
                                int nimg, int img_base, double threshold, ImgNoise* noise, float* gate,
                                unsigned long long* best, float2* clip, float* rms, cudaStream_t st);
+
+// After it, where images are sums of others: sums of the units whose images cancel
+// (see kSumCancel) are listed in redo, *nredo of them (indices in the image list),
+// and lose their weight, so that the finalisation passes them over.
+cudaError_t launch_check_sums(const Unit* units, int nunits, int img_base, const float* rms, double* weight,
+                              int* nredo, int* redo, cudaStream_t st);
 
 // Row C2R (pass B) + statistics of `nimg` images in slots [0, nimg) whose
 // first image index is img_base.  Optionally writes the scaled images.

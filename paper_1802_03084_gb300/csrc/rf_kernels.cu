@@ -542,7 +542,7 @@ __device__ __forceinline__ double parseval_sum(const float* __restrict__ cs, int
 // below it reaches the threshold (threshold * sigma in raw units, lowered by
 // far more than its rounding; no pixel does where sigma is not above 0, as in
 // an empty image, whose every pixel would pass a gate of 0).  clip[i]: the clipping window {mean, kClipSigmas
-// sigma} of the raw image J = 2W I.
+// sigma} of the raw image J = 2W I.  rms[i]: its RMS.
 __global__ void k_image_noise(int ncol, const float* __restrict__ colsq, const float* __restrict__ mean0,
                               const double* __restrict__ weight, int nimg, int img_base, double threshold,
                               ImgNoise* __restrict__ noise, float* __restrict__ gate,
@@ -561,7 +561,7 @@ __global__ void k_image_noise(int ncol, const float* __restrict__ colsq, const f
   var = var > 0.0 ? var : 0.0;
   const double sigma = sqrt(var);
   noise[i] = ImgNoise{mean, sigma};
-  if (rms != nullptr) rms[i] = (float)sqrt(sq);
+  if (rms != nullptr) rms[i] = sqrtf((float)sq);
   if (gate != nullptr) {
     gate[i] = sigma > 0.0 && W > 0.0 ? (float)(threshold * sigma * (2.0 * W) * (1.0 - 1e-5)) : INFINITY;
     best[i] = 0;
@@ -579,6 +579,42 @@ cudaError_t launch_image_noise(const SegmentGeom& g, const float* colsq, const f
   if (nimg <= 0) return cudaSuccess;
   k_image_noise<<<(nimg + 7) / 8, 256, 0, st>>>(g.ncol, colsq, mean0, weight, nimg, img_base, threshold, noise, gate,
                                                 best, clip, rms);
+  return cudaGetLastError();
+}
+
+// One warp per unit: the sums whose images cancel.  (A launch of its own, some 2 us
+// a wave.  At the end of the row pass it took 25 us a wave, with a block per unit
+// for noise and sums, 1.64 ms of a 1024^2 realtime segment for 1.2.)
+__global__ void k_check_sums(const Unit* __restrict__ units, int nunits, int img_base, const float* __restrict__ rms,
+                             double* __restrict__ weight, int* __restrict__ nredo, int* __restrict__ redo) {
+  const int u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (u >= nunits) return;
+  // lanes 0 .. 15: the unit's images; 16 .. 23, 24 .. 27, 28 and 29, 30: place lj of its sums of 2^ll
+  const int ll = lane < 16 ? 0 : (lane < 24 ? 1 : (lane < 28 ? 2 : (lane < 30 ? 3 : 4)));
+  const int lj = lane - (32 - (32 >> ll));
+  const int word = reinterpret_cast<const int*>(units + u)[lane & 7];
+  const int n = __shfl_sync(0xffffffffu, word, 1), first = __shfl_sync(0xffffffffu, word, 2 + ll);
+  const bool have = first >= 0 && (lj + 1) << ll <= n;
+  const float r = have ? rms[first + lj - img_base] : 0.f;
+  const double own = (double)r * r;
+  double parts = lane < 16 ? own : 0.0;  // of the aligned 2^lv images of lane
+  bool cancels = false;
+#pragma unroll
+  for (int lv = 1; lv <= 4; ++lv) {
+    parts += __shfl_xor_sync(0xffffffffu, parts, 1 << (lv - 1));
+    const double mine = __shfl_sync(0xffffffffu, parts, (lj << lv) & 31);
+    if (ll == lv) cancels = have && mine > kSumCancel * own;
+  }
+  if (cancels) {
+    weight[first + lj] = 0.0;
+    redo[atomicAdd(nredo, 1)] = first + lj;
+  }
+}
+
+cudaError_t launch_check_sums(const Unit* units, int nunits, int img_base, const float* rms, double* weight,
+                              int* nredo, int* redo, cudaStream_t st) {
+  if (nunits <= 0) return cudaSuccess;
+  k_check_sums<<<(nunits + 3) / 4, 128, 0, st>>>(units, nunits, img_base, rms, weight, nredo, redo);
   return cudaGetLastError();
 }
 
