@@ -279,7 +279,9 @@ def work_per_image(spec, info, frac_dt1):
 
     grid_cells: one sample per gridding entry read (dt = 1: the stored
     sample, 4 B FP16 or 8 B FP32; dt > 1: the FP32 resampled sum, 8 B) and
-    one 8-byte cell value written per occupied cell.
+    one 8-byte cell value written per occupied cell.  Adjacent DM trials read
+    nearly the same samples, most of them from the first level cache, so only
+    the cells count as HBM bytes ("hbm") and the kernel has no HBM fraction.
     grid_colfft (the column FFTs): cells read, column-FFT output T (8 N ncol
     B) written; ncol length-N FFTs.
     rowfft_stats: T read once; N/2 length-N FFTs (two image rows per complex
@@ -291,9 +293,10 @@ def work_per_image(spec, info, frac_dt1):
     gather = (frac_dt1 * esz1 + (1.0 - frac_dt1) * 8) * info.n_entries
     fft = 5.0 * N * math.log2(N)
     return {
-        "grid_cells": {"bytes": gather + 8 * info.n_cells, "flops": 0.0},
-        "grid_colfft": {"bytes": 8 * info.n_cells + 8 * N * ncol, "flops": ncol * fft},
-        "rowfft_stats": {"bytes": 8 * N * ncol, "flops": (N / 2) * fft},
+        "grid_cells": {"bytes": gather + 8 * info.n_cells, "hbm": 8 * info.n_cells, "flops": 0.0},
+        "grid_colfft": {"bytes": 8 * info.n_cells + 8 * N * ncol, "hbm": 8 * info.n_cells + 8 * N * ncol,
+                        "flops": ncol * fft},
+        "rowfft_stats": {"bytes": 8 * N * ncol, "hbm": 8 * N * ncol, "flops": (N / 2) * fft},
     }
 
 
@@ -387,14 +390,14 @@ def roofline(prof, spec, info, n_transformed, steps, frac_dt1, hbm_peak, peak_ki
         avg_s = ms / launches / 1e3
         per[name] = dict(launches=launches, total_ms=ms, avg_us=avg_s * 1e6, images_per_launch=imgs,
                          bytes_per_image=w["bytes"], gbs=w["bytes"] * imgs / avg_s / 1e9,
-                         hbm_frac=w["bytes"] * imgs / avg_s / 1e9 / hbm_peak,
+                         hbm_frac=w["hbm"] * imgs / avg_s / 1e9 / hbm_peak if w["hbm"] == w["bytes"] else None,
                          tflops=w["flops"] * imgs / avg_s / 1e12)
     if not per:
         return None, per
     dom = max(per, key=lambda k: per[k]["total_ms"])
     d = per[dom]
     traffic = load_traffic(dom, d["images_per_launch"])
-    step_bytes = sum(w["bytes"] for w in work.values()) * n_transformed
+    step_bytes = sum(w["hbm"] for w in work.values()) * n_transformed
     r = {"bound": "hbm", "achieved": round(d["gbs"], 1), "peak": hbm_peak, "unit": "GB/s",
          "frac": round(d["gbs"] / hbm_peak, 4), "traffic": traffic, "kernel": dom,
          "peak_source": f"MEASURED_PEAKS.json hbm_gbs ({peak_kind}, copy bandwidth)",

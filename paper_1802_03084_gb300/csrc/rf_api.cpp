@@ -437,7 +437,7 @@ void build_widths(rf_plan* p) {
 // build_tables).  Counted, not 1 / dt summed: sweeps and remainders shorten the
 // trials of long widths more, and with a share some images short a search that
 // fits one wave ran a second one of a few images (64 integrations of two DM
-// trials at 64^2, widths 1 .. 8: 221 us a call and not 139).
+// trials at 64^2, widths 1 .. 8: 223 us a call and not 150).
 void count_base_share(rf_plan* p) {
   int64_t all = 0, base = 0;
   for (int d = 0; d < p->ndm; ++d)
